@@ -149,17 +149,43 @@ cudaError_t launch_correct(double* u, const float* e32, long long n, double inv_
                            cudaStream_t s);
 
 // ---------------------------------------------------------------------------
-// Single-CTA bottom solver for the levels of at most 16^3 cells (levels
-// 0 .. kBottomLevels-1): u, f, n, h, bc indexed by level (bc may be null when
-// fmg is false).  fmg = false: one V-cycle on levels top .. 0 of the
-// correction (u[top] starts at 0, f[top] holds the restricted defect);
-// fmg = true: Algorithm 2 up to level `top` from f[top].
-constexpr int kBottomLevels = 6;  // arrays of the bottom programs (levels up to 32^3)
-constexpr int kBottomTopN = 16;   // the single-grid driver hands levels <= 16^3 to one CTA
+// The coarse levels of a V-cycle, or of the FMG ladder, in one launch
+// (mg_coarse.cu).
+constexpr int kCoarseLevels = 8;  // levels the kernel's arguments hold
+constexpr int kDense = 64;        // cells of the level whose cycle is a matrix
+// Highest level (0: none) of the ladder g[0 .. levels-1] whose V-cycles the
+// kernel runs; the highest it runs Algorithm 2 up to; the level of kDense cells.
 template <typename T>
-cudaError_t launch_bottom(T* const* u, T* const* f, const int* n, const double* h, const Bc* bc,
-                          Bc hom, double omega, int pre, int post, int top, bool fmg,
-                          cudaStream_t s);
+int coarse_top(const Grid* g, int levels);
+template <typename T>
+int coarse_fmg_top(const Grid* g, int levels);
+int coarse_dense_level(const Grid* g, int levels);
+enum CoarseMode { COARSE_CYCLES = 0, COARSE_FMG = 1, COARSE_BASIS = 2 };
+// COARSE_CYCLES: `cycles` V-cycles on levels top .. 0 of u (level `top`, the
+// first from u = 0 when zero_guess) with rule bc[top] there and `hom` below.
+// COARSE_FMG: Algorithm 2 from f up to level `top`, rule bc[l] on level l.
+// COARSE_BASIS: the matrix of one V-cycle from zero on level top =
+// coarse_dense_level with rule bc[top] = hom, row by row into u.
+// g, h, bc by level; dense: that matrix, used on its level (null: not used).
+template <typename T>
+struct CoarseCall {
+  T* u;
+  const T* f;
+  const Grid* g;
+  const double* h;
+  const Bc* bc;
+  Bc hom;
+  double omega;
+  int pre, post, top, cycles;
+  bool zero_guess;
+  CoarseMode mode;
+  const T* dense;
+};
+template <typename T>
+cudaError_t launch_coarse(const CoarseCall<T>& q, cudaStream_t s);
+
+// Levels the batched solver's bottom programs hold (mg_bottom.cuh).
+constexpr int kBottomLevels = 6;
 
 // ---------------------------------------------------------------------------
 // Fused FP32 V-cycle legs (homogeneous rules only).  Each reads u_in and

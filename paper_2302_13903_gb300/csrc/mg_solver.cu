@@ -54,6 +54,7 @@ struct mg_ctx {
   float* u32[kMaxLevels] = {};
   float* u32b[kMaxLevels] = {};
   float* f32[kMaxLevels] = {};
+  void* dense = nullptr;       // matrix of the cycle on the level of kDense cells (FP64 or FP32)
   double* partials = nullptr;  // reduction partials
   int* iflag = nullptr;        // device flags: [0] fixed-point overflow, [1] tensor copy late
   long long* fxbuf = nullptr;  // second integer buffer of the fixed-point outer loop
@@ -179,6 +180,24 @@ bool mean_free(const mg_ctx* c) {
   return c->bc_kind == MG_BC_PERIODIC || c->bc_kind == MG_BC_ZEROGRAD;
 }
 
+// The ladder of a context for mg_coarse.cu.
+struct Ladder {
+  Grid g[kMaxLevels];
+  double h[kMaxLevels];
+  explicit Ladder(const mg_ctx* c) {
+    for (int l = 0; l < c->L; ++l) {
+      g[l] = level_grid(c, l);
+      h[l] = level_h(c, l);
+    }
+  }
+};
+
+// The level whose V-cycle from zero is one matrix (0: none).  FAS runs no
+// correction cycles.
+int dense_level(const mg_ctx* c) {
+  return c->opts.fas ? 0 : mg::coarse_dense_level(Ladder(c).g, c->L);
+}
+
 // The device arrays of a context (counted only, when c->dry).
 void alloc_hierarchy(mg_ctx* c) {
   const mg_bc bc = (mg_bc)c->bc_kind;
@@ -214,6 +233,8 @@ void alloc_hierarchy(mg_ctx* c) {
   c->partials = dalloc<double>(c, 3 * (size_t)c->partials_cap);
   c->scal = dalloc<double>(c, 64);
   c->iflag = dalloc<int>(c, 4);
+  if (dense_level(c) > 0)
+    c->dense = dalloc<char>(c, (size_t)mg::kDense * mg::kDense * (o.prec == MG_FP64 ? 8 : 4));
 }
 
 Bc physical_bc(const mg_ctx* c, int l) {
@@ -281,26 +302,41 @@ void collect_times(mg_ctx* c) {
 // ---------------------------------------------------------------------------
 // Cycles, templated on the level precision.
 
-// Highest level index the single-CTA bottom solver covers (<= 16^3 cells).
-int bottom_top(const mg_ctx* c) {
-  if (!is_cubic(c)) return 0;  // the single-CTA bottom solver takes cubes only
-  int t = 0;
-  while (t + 1 < c->L && t + 1 < mg::kBottomLevels && level_n(c, t + 1) <= mg::kBottomTopN) ++t;
-  return t;
+// Highest level whose V-cycles run in one cluster launch (0: none).
+template <typename T>
+int coarse_top(const mg_ctx* c) {
+  return mg::coarse_top<T>(Ladder(c).g, c->L);
 }
 
+// `cycles` V-cycles on level l <= coarse_top with rule bc_top there and `hom`
+// below, the first from u_l = 0 when zero_guess.
 template <typename T>
-void launch_bottom_levels(mg_ctx* c, T** u, T** f, int top, const Bc* bcs, const Bc& hom, bool fmg,
-                          cudaStream_t s) {
-  int n[mg::kBottomLevels];
-  double h[mg::kBottomLevels];
-  for (int l = 0; l <= top; ++l) {
-    n[l] = level_n(c, l);
-    h[l] = level_h(c, l);
-  }
-  check(c, mg::launch_bottom<T>(u, f, n, h, bcs, hom, c->opts.omega, c->opts.pre, c->opts.post,
-                                top, fmg, s),
-        "bottom");
+void coarse_vcycles(mg_ctx* c, T* u, const T* f, int l, const Bc& bc_top, const Bc& hom,
+                    int cycles, bool zero_guess, cudaStream_t s) {
+  const Ladder d(c);
+  Bc bcs[kMaxLevels];
+  bcs[l] = bc_top;
+  check(c, mg::launch_coarse<T>({u, f, d.g, d.h, bcs, hom, c->opts.omega, c->opts.pre,
+                                 c->opts.post, l, cycles, zero_guess, mg::COARSE_CYCLES,
+                                 static_cast<const T*>(c->dense)},
+                                s),
+        "coarse levels");
+}
+
+// Form the matrix of the cycle on the level of kDense cells: the correction
+// cycle's rule, smoothing steps and relaxation are the context's.
+template <typename T>
+void make_dense(mg_ctx* c, const Bc& hom) {
+  const Ladder d(c);
+  Bc bcs[kMaxLevels];
+  const int l = dense_level(c);
+  bcs[l] = hom;
+  check(c, mg::launch_coarse<T>({static_cast<T*>(c->dense), nullptr, d.g, d.h, bcs, hom,
+                                 c->opts.omega, c->opts.pre, c->opts.post, l, 1, true,
+                                 mg::COARSE_BASIS, nullptr},
+                                nullptr),
+        "coarse matrix");
+  check(c, cudaStreamSynchronize(nullptr), "sync");
 }
 
 // COARSEST on level 0 (Sec. 2.3.2): one cell is solved exactly; a level of
@@ -435,8 +471,6 @@ void vcycle_fused(mg_ctx* c, int l, const Bc& bc_top, const Bc& hom, bool zero_g
   Pyr<float> P = pyr<float>(c);
   if (l - 1 == 0)
     coarsest_solve<float>(c, P.u[0], P.f[0], hom, false, s);
-  else if (l - 1 <= bottom_top(c))
-    launch_bottom_levels<float>(c, P.u, P.f, l - 1, nullptr, hom, false, s);
   else
     vcycle<float>(c, P, l - 1, hom, hom, true, s);
   if (post >= 1) {  // 5-7
@@ -464,8 +498,6 @@ void coarse_correction(mg_ctx* c, int l, const Bc& hom, cudaStream_t s) {
   Pyr<float> P = pyr<float>(c);
   if (l - 1 == 0)
     coarsest_solve<float>(c, P.u[0], P.f[0], hom, false, s);
-  else if (l - 1 <= bottom_top(c))
-    launch_bottom_levels<float>(c, P.u, P.f, l - 1, nullptr, hom, false, s);
   else
     vcycle<float>(c, P, l - 1, hom, hom, true, s);
 }
@@ -520,6 +552,10 @@ void vcycle(mg_ctx* c, Pyr<T> P, int l, const Bc& bc_top, const Bc& hom, bool ze
             cudaStream_t s) {
   const Grid g = level_grid(c, l);
   const double h = level_h(c, l);
+  if (l <= coarse_top<T>(c)) {
+    coarse_vcycles<T>(c, P.u[l], P.f[l], l, bc_top, hom, 1, zero_guess, s);
+    return;
+  }
   if constexpr (std::is_same<T, float>::value) {
     // the fused up leg synthesises the coarse correction's ghosts with the
     // level's own rule, so it serves levels whose coarse rule is the same
@@ -537,8 +573,6 @@ void vcycle(mg_ctx* c, Pyr<T> P, int l, const Bc& bc_top, const Bc& hom, bool ze
   }
   if (l - 1 == 0)
     coarsest_solve<T>(c, P.u[0], P.f[0], hom, false, s);                               // 4.1
-  else if (l - 1 <= bottom_top(c))
-    launch_bottom_levels<T>(c, P.u, P.f, l - 1, nullptr, hom, false, s);                 // 4.2
   else
     vcycle<T>(c, P, l - 1, hom, hom, true, s);                                         // 4.2
   {
@@ -551,11 +585,16 @@ void vcycle(mg_ctx* c, Pyr<T> P, int l, const Bc& bc_top, const Bc& hom, bool ze
 // Algorithm 2 with rule bcs[l] on every level.
 template <typename T>
 void fmg(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s) {
-  const int lb = bottom_top(c);
+  const Ladder d(c);
+  const int lb = mg::coarse_fmg_top<T>(d.g, c->L);
   for (int l = c->L - 1; l > lb; --l)
     check(c, mg::launch_restrict<T>(P.f[l], P.f[l - 1], level_grid(c, l), s), "restrict");
-  if (lb > 0 || level_grid(c, 0).cells() == 1)
-    launch_bottom_levels<T>(c, P.u, P.f, lb, bcs, hom, true, s);  // levels 0 .. lb
+  if (lb > 0)  // levels 0 .. lb
+    check(c, mg::launch_coarse<T>({P.u[lb], P.f[lb], d.g, d.h, bcs, hom, c->opts.omega,
+                                   c->opts.pre, c->opts.post, lb, 1, true, mg::COARSE_FMG,
+                                   static_cast<const T*>(c->dense)},
+                                  s),
+          "coarse FMG");
   else
     coarsest_solve<T>(c, P.u[0], P.f[0], bcs[0], false, s);
   for (int l = lb + 1; l < c->L; ++l) {
@@ -762,6 +801,11 @@ void inner_solve_launches(mg_ctx* c, const Bc& hom, const Bc& coarse, int cycles
   Pyr<float> P = pyr<float>(c);
   Bc bcs[kMaxLevels];
   for (int l = 0; l < c->L; ++l) bcs[l] = hom;
+  if (!c->opts.inner_fmg && F >= 1 && F <= coarse_top<float>(c)) {
+    // the whole grid fits one cluster: every cycle in one launch
+    coarse_vcycles<float>(c, P.u[F], P.f[F], F, hom, coarse, cycles, true, s);
+    return;
+  }
   if (c->opts.inner_fmg) {
     fmg<float>(c, P, bcs, coarse, s);
   } else if (use_pairs(c) && pairs_ok(c, F, hom, coarse, cycles)) {
@@ -1614,6 +1658,11 @@ mg_status create_ctx(int nx, int ny, int nz, double dx, mg_bc bc, int face_mask,
     alloc_hierarchy(c);
     check(c, cudaMemset(c->iflag, 0, 4 * sizeof(int)), "clear flags");
     if (bc == MG_BC_MIXED) fill_mixed_faces(c);
+    if (c->dense) {
+      const Bc hom = correction_bc(c, physical_bc(c, L - 1));
+      if (o.prec == MG_FP64) make_dense<double>(c, hom);
+      else make_dense<float>(c, hom);
+    }
     check(c, cudaMallocHost(&c->pinned, 64 * sizeof(double)), "cudaMallocHost");
   } catch (const Fail& f) {
     mg_destroy(c);
