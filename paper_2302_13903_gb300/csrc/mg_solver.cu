@@ -90,11 +90,17 @@ struct mg_ctx {
   // replayed from then on; dropped when the launch shapes change.
   // Two graphs: [0] for 1 + inner_cycles V-cycles, [1] for the first outer
   // iteration's first_cycles when they differ.
+  // FP64: [2] the V-cycle below the finest level and [3] the FMG ladder below
+  // it, which touch the context's own arrays only.
   struct InnerGraph {
     cudaGraphExec_t exec = nullptr;
     long long launches = 0;  // kernels in the graph
     int runs = 0;
-  } inner[2];
+  } inner[4];
+  // stream of the solves given the legacy default stream, which cannot be
+  // captured, and the event that orders it after that stream
+  cudaStream_t own_stream = nullptr;
+  cudaEvent_t own_event = nullptr;
   // the autotuner timed the finest level's fused up-down pass faster than the
   // two legs it replaces (opts.leg_pairs = 0 then fuses them)
   bool pairs_faster = false;
@@ -297,6 +303,55 @@ void collect_times(mg_ctx* c) {
     }
   }
   c->pending_class.clear();
+}
+
+void drop_inner_graph(mg_ctx* c) {
+  for (auto& ig : c->inner) {
+    if (ig.exec) cudaGraphExecDestroy(ig.exec);
+    ig.exec = nullptr;
+    ig.runs = 0;
+  }
+}
+
+// `queue`, from its second run on as one CUDA graph launch: for work that is
+// the same launches on the context's own buffers every time.  Queued launch by
+// launch when `graphs` is false, on the legacy default stream, or inside a
+// capture the caller started.
+template <typename Queue>
+void replay(mg_ctx* c, mg_ctx::InnerGraph& ig, bool graphs, cudaStream_t s, Queue queue) {
+  if (ig.exec && graphs) {
+    check(c, cudaGraphLaunch(ig.exec, s), "graph");
+    mg::g_launches += ig.launches;
+    return;
+  }
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const bool capture = graphs && ig.runs >= 1 && s != nullptr &&
+                       cudaStreamIsCapturing(s, &cs) == cudaSuccess &&
+                       cs == cudaStreamCaptureStatusNone;
+  ++ig.runs;
+  if (!capture) {
+    queue();
+    return;
+  }
+  check(c, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal), "begin capture");
+  const long long before = mg::g_launches;
+  cudaGraph_t graph = nullptr;
+  try {
+    queue();
+  } catch (const Fail&) {
+    cudaStreamEndCapture(s, &graph);
+    if (graph) cudaGraphDestroy(graph);
+    throw;
+  }
+  check(c, cudaStreamEndCapture(s, &graph), "end capture");
+  const cudaError_t e = cudaGraphInstantiate(&ig.exec, graph, 0);
+  cudaGraphDestroy(graph);
+  if (e != cudaSuccess) {
+    ig.exec = nullptr;
+    check(c, e, "instantiate graph");
+  }
+  ig.launches = mg::g_launches - before;
+  check(c, cudaGraphLaunch(ig.exec, s), "graph");
 }
 
 // ---------------------------------------------------------------------------
@@ -573,6 +628,8 @@ void vcycle(mg_ctx* c, Pyr<T> P, int l, const Bc& bc_top, const Bc& hom, bool ze
   }
   if (l - 1 == 0)
     coarsest_solve<T>(c, P.u[0], P.f[0], hom, false, s);                               // 4.1
+  else if (std::is_same<T, double>::value && fin && l - 1 > coarse_top<T>(c))
+    replay(c, c->inner[2], true, s, [&]() { vcycle<T>(c, P, l - 1, hom, hom, true, s); });
   else
     vcycle<T>(c, P, l - 1, hom, hom, true, s);                                         // 4.2
   {
@@ -586,25 +643,31 @@ void vcycle(mg_ctx* c, Pyr<T> P, int l, const Bc& bc_top, const Bc& hom, bool ze
 template <typename T>
 void fmg(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s) {
   const Ladder d(c);
-  const int lb = mg::coarse_fmg_top<T>(d.g, c->L);
-  for (int l = c->L - 1; l > lb; --l)
-    check(c, mg::launch_restrict<T>(P.f[l], P.f[l - 1], level_grid(c, l), s), "restrict");
-  if (lb > 0)  // levels 0 .. lb
-    check(c, mg::launch_coarse<T>({P.u[lb], P.f[lb], d.g, d.h, bcs, hom, c->opts.omega,
-                                   c->opts.pre, c->opts.post, lb, 1, true, mg::COARSE_FMG,
-                                   static_cast<const T*>(c->dense)},
-                                  s),
-          "coarse FMG");
-  else
-    coarsest_solve<T>(c, P.u[0], P.f[0], bcs[0], false, s);
-  for (int l = lb + 1; l < c->L; ++l) {
+  const int F = c->L - 1, lb = mg::coarse_fmg_top<T>(d.g, c->L);
+  auto up = [&](int l) {
     {
-      KTimer t(c, MG_K_FMG_PROLONG, l == c->L - 1, s);
+      KTimer t(c, MG_K_FMG_PROLONG, l == F, s);
       check(c, mg::launch_prolong<T>(P.u[l - 1], P.u[l], level_grid(c, l), bcs[l - 1], 1, 0, s),
             "fmg_prolong");
     }
     vcycle<T>(c, P, l, bcs[l], hom, false, s);
-  }
+  };
+  auto below = [&]() {  // levels below the finest (or all, where the ladder's start is it)
+    for (int l = F; l > lb; --l)
+      check(c, mg::launch_restrict<T>(P.f[l], P.f[l - 1], level_grid(c, l), s), "restrict");
+    if (lb > 0)  // levels 0 .. lb
+      check(c, mg::launch_coarse<T>({P.u[lb], P.f[lb], d.g, d.h, bcs, hom, c->opts.omega,
+                                     c->opts.pre, c->opts.post, lb, 1, true, mg::COARSE_FMG,
+                                     static_cast<const T*>(c->dense)},
+                                    s),
+            "coarse FMG");
+    else
+      coarsest_solve<T>(c, P.u[0], P.f[0], bcs[0], false, s);
+    for (int l = lb + 1; l < F; ++l) up(l);
+  };
+  if (std::is_same<T, double>::value && lb < F) replay(c, c->inner[3], true, s, below);
+  else below();
+  if (lb < F) up(F);
 }
 
 // Algorithm 3 on level l >= 1 (FP64 path): every level solves the original
@@ -817,60 +880,17 @@ void inner_solve_launches(mg_ctx* c, const Bc& hom, const Bc& coarse, int cycles
   for (int q = 1; q < cycles; ++q) vcycle<float>(c, P, F, hom, coarse, false, s);
 }
 
-void drop_inner_graph(mg_ctx* c) {
-  for (auto& ig : c->inner) {
-    if (ig.exec) cudaGraphExecDestroy(ig.exec);
-    ig.exec = nullptr;
-    ig.runs = 0;
-  }
-}
-
 // V-cycles (or FMG and the V-cycles after it) of the inner solve of outer
 // iteration `it`.
 int inner_count(const mg_ctx* c, int it) {
   return (it == 0 && c->opts.first_cycles > 0) ? c->opts.first_cycles : 1 + c->opts.inner_cycles;
 }
 
-// The inner solve of `cycles` V-cycles, from its second run with that count
-// on as one CUDA graph launch (not while per-kernel timing is on, on the
-// legacy default stream, or inside a capture the caller started).  The
-// launches are the same every outer iteration: the same kernels, shapes and
-// buffers.
+// The inner solve of `cycles` V-cycles, as one CUDA graph launch from its
+// second run with that count on (not while per-kernel timing is on).
 void inner_solve(mg_ctx* c, const Bc& hom, const Bc& coarse, int cycles, cudaStream_t s) {
-  mg_ctx::InnerGraph& ig = c->inner[cycles == 1 + c->opts.inner_cycles ? 0 : 1];
-  if (ig.exec && !c->timing) {
-    check(c, cudaGraphLaunch(ig.exec, s), "inner solve graph");
-    mg::g_launches += ig.launches;
-    return;
-  }
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  const bool capture = !c->timing && ig.runs >= 1 && s != nullptr &&
-                       cudaStreamIsCapturing(s, &cs) == cudaSuccess &&
-                       cs == cudaStreamCaptureStatusNone;
-  ++ig.runs;
-  if (!capture) {
-    inner_solve_launches(c, hom, coarse, cycles, s);
-    return;
-  }
-  check(c, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal), "begin capture");
-  const long long before = mg::g_launches;
-  cudaGraph_t graph = nullptr;
-  try {
-    inner_solve_launches(c, hom, coarse, cycles, s);
-  } catch (const Fail&) {
-    cudaStreamEndCapture(s, &graph);
-    if (graph) cudaGraphDestroy(graph);
-    throw;
-  }
-  check(c, cudaStreamEndCapture(s, &graph), "end capture");
-  const cudaError_t e = cudaGraphInstantiate(&ig.exec, graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) {
-    ig.exec = nullptr;
-    check(c, e, "instantiate inner solve graph");
-  }
-  ig.launches = mg::g_launches - before;
-  check(c, cudaGraphLaunch(ig.exec, s), "inner solve graph");
+  replay(c, c->inner[cycles == 1 + c->opts.inner_cycles ? 0 : 1], !c->timing, s,
+         [&]() { inner_solve_launches(c, hom, coarse, cycles, s); });
 }
 
 mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol, double* phi,
@@ -1611,6 +1631,8 @@ mg_status mg_destroy(mg_ctx* c) {
   if (!c) return MG_OK;
   drop_inner_graph(c);
   for (cudaEvent_t e : c->events) cudaEventDestroy(e);
+  if (c->own_event) cudaEventDestroy(c->own_event);
+  if (c->own_stream) cudaStreamDestroy(c->own_stream);
   for (void* p : c->allocs) cudaFree(p);
   if (c->pinned) cudaFreeHost(c->pinned);
   delete c;
@@ -1751,6 +1773,21 @@ mg_status mg_required_bytes(int nx, int ny, int nz, mg_bc bc, const mg_opts* opt
   return MG_OK;
 }
 
+// The stream a solve given stream s runs on: s, or for the legacy default
+// stream (whose launches cannot be captured as a graph) the context's own,
+// ordered after what the default stream holds now.  The solve synchronises it
+// before it returns, so later work on any stream comes after it.
+static cudaStream_t capturable_stream(mg_ctx* c, cudaStream_t s) {
+  if (s != nullptr && s != cudaStreamLegacy) return s;
+  if (!c->own_stream) {
+    check(c, cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking), "stream");
+    check(c, cudaEventCreateWithFlags(&c->own_event, cudaEventDisableTiming), "event");
+  }
+  check(c, cudaEventRecord(c->own_event, s), "record");
+  check(c, cudaStreamWaitEvent(c->own_stream, c->own_event, 0), "wait");
+  return c->own_stream;
+}
+
 mg_status mg_solve(mg_ctx* c, const double* rho, double four_pi_G, double tol, double* phi,
                    double* hist, int hist_cap, int* n_hist, void* stream) {
   return mg_solve_gravity(c, rho, four_pi_G, tol, phi, nullptr, hist, hist_cap, n_hist, stream);
@@ -1773,6 +1810,7 @@ mg_status mg_solve_gravity(mg_ctx* c, const double* rho, double four_pi_G, doubl
   mg_status st;
   try {
     check(c, cudaSetDevice(c->device), "cudaSetDevice");
+    s = capturable_stream(c, s);
     if (c->opts.prec == MG_FP64)
       st = solve_fp64(c, rho, four_pi_G, tol, phi, g, hist, hist_cap, n_hist, s);
     else
