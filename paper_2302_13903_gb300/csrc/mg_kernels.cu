@@ -56,6 +56,237 @@ int grid_for(long long work) {
 }
 
 // ---------------------------------------------------------------------------
+// Level kernels for even sizes.  In FP64 an SM issues two operations per clock,
+// so what counts is the number of FP64 operations per cell and that no warp
+// runs two versions of them: a lane at a face selects what it loads (the
+// periodic image, or the ghost of Sec. 2.3.6) and then takes the same path as
+// the others.  A thread has a patch of 2 x 2 cells in (x, y), because the two
+// cells of one colour in it share the sum of the two others:
+//   j+1:  Y B      A and B of one colour: A's x and y neighbours inside the
+//   j  :  A X      patch are X and Y, and so are B's (or mirrored in x).
+
+// The neighbour of a cell across face q: ghost from the rule.
+template <typename T>
+__device__ __noinline__ T face_ghost(const T* u, T self, int q, int i, int j, int k, const Grid g,
+                                     const Bc bc) {
+  const int kind = face_kind(bc, q);
+  if (kind == BC_PERIODIC) {
+    const int hi = q & 1;
+    if (q < 2) i = hi ? 0 : g.nx - 1;
+    else if (q < 4) j = hi ? 0 : g.ny - 1;
+    else k = hi ? 0 : g.nz - 1;
+    return u[dev::at(g, i, j, k)];
+  }
+  if (kind == BC_ZEROGRAD) return self;
+  const T b = (T)dev::face_value(bc, g, q, (q < 2 ? j : i) + 1, (q < 4 ? k : j) + 1);
+  return T(2) * b - self;
+}
+
+// Neighbours of cell c = (i, j, k) along one axis: lower (q even) or upper.
+template <typename T, bool PER>
+struct Around {
+  const T* u;
+  const Grid& g;
+  const Bc& bc;
+  __device__ __forceinline__ T x(size_t c, int i, int j, int k, int hi) const {
+    const bool in = hi ? i < g.nx - 1 : i > 0;
+    if (PER) return u[in ? (hi ? c + 1 : c - 1) : (hi ? c + 1 - g.nx : c + g.nx - 1)];
+    return in ? u[hi ? c + 1 : c - 1] : face_ghost(u, u[c], hi, i, j, k, g, bc);
+  }
+  __device__ __forceinline__ T y(size_t c, int i, int j, int k, int hi) const {
+    const size_t sy = (size_t)g.nx, w = sy * (g.ny - 1);
+    const bool in = hi ? j < g.ny - 1 : j > 0;
+    if (PER) return u[in ? (hi ? c + sy : c - sy) : (hi ? c - w : c + w)];
+    return in ? u[hi ? c + sy : c - sy] : face_ghost(u, u[c], 2 + hi, i, j, k, g, bc);
+  }
+  __device__ __forceinline__ T z(size_t c, int i, int j, int k, int hi) const {
+    const size_t sz = (size_t)g.nx * g.ny, w = sz * (g.nz - 1);
+    const bool in = hi ? k < g.nz - 1 : k > 0;
+    if (PER) return u[in ? (hi ? c + sz : c - sz) : (hi ? c - w : c + w)];
+    return in ? u[hi ? c + sz : c - sz] : face_ghost(u, u[c], 4 + hi, i, j, k, g, bc);
+  }
+  // Neighbour sums of the patch's two cells of one colour: cell A of row j is
+  // 2 m + e, cell B of row j + 1 is 2 m + 1 - e (nine additions for both).
+  __device__ __forceinline__ void sums(int m, int j, int k, int e, size_t& ca, size_t& cb, T& sa,
+                                       T& sb) const {
+    const int ia = 2 * m + e, ib = 2 * m + 1 - e;
+    ca = dev::at(g, ia, j, k);
+    cb = dev::at(g, ib, j + 1, k);
+    const T p = u[dev::at(g, ib, j, k)] + u[dev::at(g, ia, j + 1, k)];
+    sa = (p + (x(ca, ia, j, k, e) + y(ca, ia, j, k, 0))) + (z(ca, ia, j, k, 0) + z(ca, ia, j, k, 1));
+    sb = (p + (x(cb, ib, j + 1, k, 1 - e) + y(cb, ib, j + 1, k, 1))) +
+         (z(cb, ib, j + 1, k, 0) + z(cb, ib, j + 1, k, 1));
+  }
+};
+
+// One colour of SMOOTH: 7.5 operations per updated cell.
+template <typename T, bool PER>
+__global__ void __launch_bounds__(kThreads) k_sor_patch(T* u, const T* f, Grid g, Bc bc, T cu, T cs,
+                                                        T cf, int colour) {
+  const int hx = g.nx >> 1, hy = g.ny >> 1;
+  const long long total = (long long)hx * hy * g.nz;
+  const dev::Split sp(hx, hy);
+  const Around<T, PER> n{u, g, bc};
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+       t += (long long)gridDim.x * blockDim.x) {
+    int m, jj, k;
+    sp(t, m, jj, k);
+    size_t ca, cb;
+    T sa, sb;
+    n.sums(m, 2 * jj, k, (k + colour) & 1, ca, cb, sa, sb);
+    const T va = cs * sa + (cu * u[ca] + cf * f[ca]);
+    const T vb = cs * sb + (cu * u[cb] + cf * f[cb]);
+    u[ca] = va;
+    u[cb] = vb;
+  }
+}
+
+// Partial sums of d^2, d = f - (sum_nb - 6 u) / h^2: 7.5 operations per cell.
+template <typename T, bool PER>
+__global__ void __launch_bounds__(kThreads) k_defect_norm(const T* u, const T* f, Grid g, Bc bc,
+                                                          T inv_h2, double* partials) {
+  const int hx = g.nx >> 1, hy = g.ny >> 1;
+  const long long total = (long long)hx * hy * g.nz;
+  const dev::Split sp(hx, hy);
+  const Around<T, PER> n{u, g, bc};
+  double acc = 0.0;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+       t += (long long)gridDim.x * blockDim.x) {
+    int m, jj, k;
+    sp(t, m, jj, k);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      size_t ca, cb;
+      T sa, sb;
+      n.sums(m, 2 * jj, k, e, ca, cb, sa, sb);
+      const T da = f[ca] - (sa - T(6) * u[ca]) * inv_h2;
+      const T db = f[cb] - (sb - T(6) * u[cb]) * inv_h2;
+      acc += (double)da * (double)da;
+      acc += (double)db * (double)db;
+    }
+  }
+  const double b = block_sum(acc);
+  if (threadIdx.x == 0) partials[blockIdx.x] = b;
+}
+
+// Defect of the eight children of each coarse cell, averaged (Algorithm 1,
+// steps 2-3).  Summed over the block, the neighbour sums are three times the
+// sum of the eight cells (each has three neighbours among them) plus the 24
+// cells around it: 40 operations per block where a defect per cell takes 72.
+// Two neighbouring lanes share a block, a plane each.
+template <typename T, bool PER>
+__global__ void __launch_bounds__(kThreads) k_defect_restrict_block(const T* u, const T* f, T* fc,
+                                                                    Grid g, Bc bc, T inv_h2) {
+  const Grid gc{g.nx / 2, g.ny / 2, g.nz / 2};
+  const long long work = 2 * gc.cells();
+  const dev::Split sp(gc.nx, gc.ny);
+  const Around<T, PER> n{u, g, bc};
+  for (long long t0 = blockIdx.x * (long long)blockDim.x; t0 < work;
+       t0 += (long long)gridDim.x * blockDim.x) {
+    const long long t = t0 + threadIdx.x;
+    const bool live = t < work;
+    const int d = (int)(t & 1);
+    int I, J, K;
+    sp(live ? t >> 1 : 0, I, J, K);
+    const int i = 2 * I, j = 2 * J, k = 2 * K + d;
+    const size_t c = dev::at(g, i, j, k), cy = c + g.nx;
+    const T own = (u[c] + u[c + 1]) + (u[cy] + u[cy + 1]);
+    const T fs = (f[c] + f[c + 1]) + (f[cy] + f[cy + 1]);
+    const T ox = (n.x(c, i, j, k, 0) + n.x(cy, i, j + 1, k, 0)) +
+                 (n.x(c + 1, i + 1, j, k, 1) + n.x(cy + 1, i + 1, j + 1, k, 1));
+    const T oy = (n.y(c, i, j, k, 0) + n.y(c + 1, i + 1, j, k, 0)) +
+                 (n.y(cy, i, j + 1, k, 1) + n.y(cy + 1, i + 1, j + 1, k, 1));
+    const T oz = (n.z(c, i, j, k, d) + n.z(c + 1, i + 1, j, k, d)) +
+                 (n.z(cy, i, j + 1, k, d) + n.z(cy + 1, i + 1, j + 1, k, d));
+    T v = fs - inv_h2 * (((ox + oy) + oz) - T(3) * own);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    if (live && !d) fc[t >> 1] = v * T(0.125);
+  }
+}
+
+// u += trilinear(uc) for a homogeneous coarse rule, over z-chunks of coarse
+// columns: the (x, y) interpolation of a coarse plane is formed once and kept
+// for the three pairs of fine planes that use it.  Interpolating 4 x by
+// 3 b + a (one operation) leaves a factor of 64 to the last, fused with the
+// addition to u: 26 operations per coarse cell and plane, where weights 1/4 and
+// 3/4 take 35.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_prolong_add(const T* uc, T* uf, Grid gf, Bc bc, int cz,
+                                                          long long items) {
+  const Grid gc{gf.nx / 2, gf.ny / 2, gf.nz / 2};
+  const dev::Split sp(gc.nx, gc.ny);
+  const size_t plane = (size_t)gf.nx * gf.ny, planec = (size_t)gc.nx * gc.ny;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < items;
+       t += (long long)gridDim.x * blockDim.x) {
+    int I, J, ch;
+    sp(t, I, J, ch);
+    const int K0 = ch * cz, K1 = min(K0 + cz, gc.nz);
+    // offset of the coarse neighbour on each side and whether it enters with
+    // a minus sign (the cell itself stands in for it at a wall)
+    int ox[3] = {0, 0, 0}, oy[3] = {0, 0, 0};
+    unsigned neg = 0;  // bits 0 x-, 1 x+, 2 y-, 3 y+
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+      const bool inx = hi ? I < gc.nx - 1 : I > 0, iny = hi ? J < gc.ny - 1 : J > 0;
+      const int kx = face_kind(bc, hi), ky = face_kind(bc, 2 + hi);
+      ox[2 * hi] = inx ? 2 * hi - 1 : kx == BC_PERIODIC ? (1 - 2 * hi) * (gc.nx - 1) : 0;
+      oy[2 * hi] = (iny ? 2 * hi - 1 : ky == BC_PERIODIC ? (1 - 2 * hi) * (gc.ny - 1) : 0) * gc.nx;
+      if (!inx && kx == BC_FIXED) neg |= 1u << hi;
+      if (!iny && ky == BC_FIXED) neg |= 4u << hi;
+    }
+    auto xy = [&](int K, T out[2][2]) {
+      bool nz = false;
+      if (K < 0 || K >= gc.nz) {
+        const int kz = face_kind(bc, K < 0 ? 4 : 5);
+        nz = kz == BC_FIXED;
+        K = (K < 0) == (kz == BC_PERIODIC) ? gc.nz - 1 : 0;
+      }
+      const T* p = uc + (size_t)K * planec + (size_t)J * gc.nx + I;
+      T vx[3][2];
+#pragma unroll
+      for (int y = 0; y < 3; ++y) {
+        T v[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          v[x] = p[ox[x] + oy[y]];
+          const bool n = (x != 1 && (neg >> (x >> 1) & 1)) != (y != 1 && (neg >> (2 + (y >> 1)) & 1));
+          if (n != nz) v[x] = -v[x];
+        }
+        vx[y][0] = T(3) * v[1] + v[0];
+        vx[y][1] = T(3) * v[1] + v[2];
+      }
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        out[0][x] = T(3) * vx[1][x] + vx[0][x];
+        out[1][x] = T(3) * vx[1][x] + vx[2][x];
+      }
+    };
+    T pm[2][2], p0[2][2], pp[2][2];
+    xy(K0 - 1, pm);
+    xy(K0, p0);
+    for (int K = K0; K < K1; ++K) {
+      xy(K + 1, pp);
+#pragma unroll
+      for (int y = 0; y < 2; ++y)
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          const size_t q = dev::at(gf, 2 * I + x, 2 * J + y, 2 * K);
+          uf[q] = T(1.0 / 64) * (T(3) * p0[y][x] + pm[y][x]) + uf[q];
+          uf[q + plane] = T(1.0 / 64) * (T(3) * p0[y][x] + pp[y][x]) + uf[q + plane];
+          pm[y][x] = p0[y][x];
+          p0[y][x] = pp[y][x];
+        }
+    }
+  }
+}
+
+bool even_sizes(const Grid& g) { return g.nx % 2 == 0 && g.ny % 2 == 0 && g.nz % 2 == 0; }
+bool homogeneous_rule(const Bc& bc) {
+  return bc.kind == BC_PERIODIC || bc.kind == BC_ZEROGRAD ||
+         (bc.kind == BC_FIXED && bc.value == 0.0) || (bc.kind == BC_MIXED && !bc.faces);
+}
+
+// ---------------------------------------------------------------------------
 // d = f - (sum_nb - 6u) / h^2; optional store and partial sums of d^2.
 template <typename T>
 __global__ void k_defect(const T* __restrict__ u, const T* __restrict__ f, T* __restrict__ d,
@@ -280,9 +511,16 @@ template <typename T>
 cudaError_t launch_sor(T* u, const T* f, Grid g, double h, Bc bc, double omega, int colour,
                        cudaStream_t s) {
   const long long work = (long long)(g.nx / 2) * g.ny * g.nz;
+  const T cu = (T)(1.0 - omega), cs = (T)(omega / 6.0), cf = (T)(-omega * h * h / 6.0);
   ++g_launches;
-  k_sor<T><<<grid_for(work), kThreads, 0, s>>>(u, f, g, bc, (T)(1.0 - omega), (T)(omega / 6.0),
-                                               (T)(-omega * h * h / 6.0), colour);
+  if (g.nx % 2 == 0 && g.ny % 2 == 0) {
+    if (bc.kind == BC_PERIODIC)
+      k_sor_patch<T, true><<<grid_for(work / 2), kThreads, 0, s>>>(u, f, g, bc, cu, cs, cf, colour);
+    else
+      k_sor_patch<T, false><<<grid_for(work / 2), kThreads, 0, s>>>(u, f, g, bc, cu, cs, cf, colour);
+  } else {
+    k_sor<T><<<grid_for(work), kThreads, 0, s>>>(u, f, g, bc, cu, cs, cf, colour);
+  }
   return cudaGetLastError();
 }
 
@@ -299,6 +537,14 @@ cudaError_t launch_defect(const T* u, const T* f, T* d, Grid g, double h, Bc bc,
                           cudaStream_t s) {
   ++g_launches;
   const int nb = partials ? reduce_blocks(g.cells()) : grid_for(g.cells());
+  if (partials && !d && g.nx % 2 == 0 && g.ny % 2 == 0) {
+    const T ih2 = (T)(1.0 / (h * h));
+    if (bc.kind == BC_PERIODIC)
+      k_defect_norm<T, true><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials);
+    else
+      k_defect_norm<T, false><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials);
+    return cudaGetLastError();
+  }
   k_defect<T><<<nb, kThreads, 0, s>>>(u, f, d, g, bc, (T)(1.0 / (h * h)), partials);
   return cudaGetLastError();
 }
@@ -307,8 +553,15 @@ template <typename T>
 cudaError_t launch_defect_restrict(const T* u, const T* f, T* fc, Grid g, double h, Bc bc,
                                    cudaStream_t s) {
   ++g_launches;
-  k_defect_restrict<T><<<grid_for(g.cells() / 8), kThreads, 0, s>>>(u, f, fc, g, bc,
-                                                                    (T)(1.0 / (h * h)));
+  const T ih2 = (T)(1.0 / (h * h));
+  if (!even_sizes(g))
+    k_defect_restrict<T><<<grid_for(g.cells() / 8), kThreads, 0, s>>>(u, f, fc, g, bc, ih2);
+  else if (bc.kind == BC_PERIODIC)
+    k_defect_restrict_block<T, true><<<grid_for(g.cells() / 4), kThreads, 0, s>>>(u, f, fc, g, bc,
+                                                                                  ih2);
+  else
+    k_defect_restrict_block<T, false><<<grid_for(g.cells() / 4), kThreads, 0, s>>>(u, f, fc, g, bc,
+                                                                                   ih2);
   return cudaGetLastError();
 }
 
@@ -323,14 +576,16 @@ template <typename T>
 cudaError_t launch_prolong(const T* uc, T* uf, Grid gf, Bc bc_coarse, int high_order, int add,
                            cudaStream_t s) {
   ++g_launches;
-  // z-chunks of coarse columns: 8 planes each while that leaves about 2^18
-  // work items (enough threads for the device), fewer on small levels
+  // z-chunks of coarse columns: 8 planes each while that leaves about 2^16
+  // work items (three FP64 warps per scheduler), fewer on small levels
   const long long cols = (long long)(gf.nx / 2) * (gf.ny / 2);
   const int cnz = gf.nz / 2;
   int cz = 8;
-  while (cz > 1 && cols * ((cnz + cz - 1) / cz) < (1LL << 18)) cz /= 2;
+  while (cz > 1 && cols * ((cnz + cz - 1) / cz) < (1LL << 16)) cz /= 2;
   const long long items = cols * ((cnz + cz - 1) / cz);
-  if (high_order)
+  if (!high_order && add && homogeneous_rule(bc_coarse))
+    k_prolong_add<T><<<grid_for(items), kThreads, 0, s>>>(uc, uf, gf, bc_coarse, cz, items);
+  else if (high_order)
     k_prolong<T, true><<<grid_for(items), kThreads, 0, s>>>(uc, uf, gf, bc_coarse, add, cz, items);
   else
     k_prolong<T, false><<<grid_for(items), kThreads, 0, s>>>(uc, uf, gf, bc_coarse, add, cz, items);
