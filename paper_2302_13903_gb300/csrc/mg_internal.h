@@ -309,6 +309,31 @@ cudaError_t launch_finish_fx_sum(const long long* psum, int nb, long long n, dou
                                  cudaStream_t s);
 
 // ---------------------------------------------------------------------------
+// The FP64 path's finest level in 64-bit fixed point (mg_fx64.cu).  Levels
+// with nx a multiple of 64, ny of 16 and nz even (fx64_ok); per-CTA sums in
+// arrays of fx64_blocks(g) entries (psum: pairs).
+bool fx64_ok(Grid g);
+int fx64_cz(Grid g);
+int fx64_blocks(Grid g);
+// u_out = SMOOTH(u_in); fc = the restricted defect times h^2 2^S; norm = sums
+// of (h^2 2^S defect)^2 over the red cells of u_in; psum = sums of u_in.
+cudaError_t launch_fx64_down(const long long* u_in, long long* u_out, const long long* F, double* fc,
+                             Grid g, const Bc& hom, double omega, double* norm, long long* psum,
+                             int* flag, cudaStream_t s);
+// u_out = SMOOTH(u_in + trilinear(ec)); norm = the same over the black cells of
+// u_out.  *flag |= 1 where |u_out| passes 2^59.
+cudaError_t launch_fx64_up(const long long* u_in, long long* u_out, const long long* F,
+                           const long long* ec, Grid g, const Bc& hom, double omega, double* norm,
+                           int* flag, cudaStream_t s);
+// In place: f becomes round(f c) less round(2 b 2^S) for each of the cell's
+// fixed and open faces (rule bc).
+cudaError_t launch_fx64_source(double* f, Grid g, const Bc& bc, double c, double two_pow_S,
+                               cudaStream_t s);
+// out[0] = sum of both arrays of nb partial sums.
+cudaError_t launch_fx64_norm(const double* red, const double* black, int nb, double* out,
+                             cudaStream_t s);
+
+// ---------------------------------------------------------------------------
 // Multipole boundary (App. A).
 
 // Upload the polynomial tables to this device's constant memory (once per

@@ -235,8 +235,13 @@ void alloc_hierarchy(mg_ctx* c) {
     const int nb = mg::fx_step_blocks(level_grid(c, F), 0);
     if (nb > c->partials_cap) c->partials_cap = nb;
   }
+  // the FP64 path's finest level in fixed point: a second integer buffer (phi
+  // itself is the first) and one more array of partial sums
+  const bool fx64 = o.prec == MG_FP64 && o.mode_fmg && !o.fas && !o.coarse_literal && o.pre == 1 &&
+                    o.post == 1 && L >= 2 && mg::fx64_ok(level_grid(c, F));
+  if (fx64) c->fxbuf = dalloc<long long>(c, level_grid(c, F).cells());
   // partials, then room for two integers per block of the fixed-point step
-  c->partials = dalloc<double>(c, 3 * (size_t)c->partials_cap);
+  c->partials = dalloc<double>(c, (fx64 ? 4 : 3) * (size_t)c->partials_cap);
   c->scal = dalloc<double>(c, 64);
   c->iflag = dalloc<int>(c, 4);
   if (dense_level(c) > 0)
@@ -639,20 +644,19 @@ void vcycle(mg_ctx* c, Pyr<T> P, int l, const Bc& bc_top, const Bc& hom, bool ze
   smooth_steps<T>(c, P, l, bc_top, c->opts.post, false, s);                            // 7
 }
 
-// Algorithm 2 with rule bcs[l] on every level.
+// Algorithm 2 with rule bcs[l] on every level, up to the prolongation to the
+// finest level F.  Returns false where the ladder's start is level F itself,
+// which is then done.
 template <typename T>
-void fmg(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s) {
+bool fmg_below(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s) {
   const Ladder d(c);
   const int F = c->L - 1, lb = mg::coarse_fmg_top<T>(d.g, c->L);
-  auto up = [&](int l) {
-    {
-      KTimer t(c, MG_K_FMG_PROLONG, l == F, s);
-      check(c, mg::launch_prolong<T>(P.u[l - 1], P.u[l], level_grid(c, l), bcs[l - 1], 1, 0, s),
-            "fmg_prolong");
-    }
-    vcycle<T>(c, P, l, bcs[l], hom, false, s);
+  auto prolong = [&](int l) {
+    KTimer t(c, MG_K_FMG_PROLONG, l == F, s);
+    check(c, mg::launch_prolong<T>(P.u[l - 1], P.u[l], level_grid(c, l), bcs[l - 1], 1, 0, s),
+          "fmg_prolong");
   };
-  auto below = [&]() {  // levels below the finest (or all, where the ladder's start is it)
+  auto below = [&]() {
     for (int l = F; l > lb; --l)
       check(c, mg::launch_restrict<T>(P.f[l], P.f[l - 1], level_grid(c, l), s), "restrict");
     if (lb > 0)  // levels 0 .. lb
@@ -663,11 +667,22 @@ void fmg(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s) {
             "coarse FMG");
     else
       coarsest_solve<T>(c, P.u[0], P.f[0], bcs[0], false, s);
-    for (int l = lb + 1; l < F; ++l) up(l);
+    for (int l = lb + 1; l < F; ++l) {
+      prolong(l);
+      vcycle<T>(c, P, l, bcs[l], hom, false, s);
+    }
   };
   if (std::is_same<T, double>::value && lb < F) replay(c, c->inner[3], true, s, below);
   else below();
-  if (lb < F) up(F);
+  if (lb >= F) return false;
+  prolong(F);
+  return true;
+}
+
+// Algorithm 2 with rule bcs[l] on every level.
+template <typename T>
+void fmg(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s) {
+  if (fmg_below<T>(c, P, bcs, hom, s)) vcycle<T>(c, P, c->L - 1, bcs[c->L - 1], hom, false, s);
 }
 
 // Algorithm 3 on level l >= 1 (FP64 path): every level solves the original
@@ -811,6 +826,110 @@ Bc correction_bc(const mg_ctx* c, const Bc& top) {
   return z;
 }
 
+// The V-cycles of the FP64 path with the finest level in 64-bit fixed point
+// (mg_fx64.cu): phi holds the FMG start, prolonged to the finest level, and
+// f64[F] the source.  Returns -1 where the values are not finite or phi leaves
+// the integers' range (then phi and f are to be formed again), else the status.
+int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, const Bc& bc,
+               const Bc& hom, double* hist, int hist_cap, int* n_hist, cudaStream_t s) {
+  const int F = c->L - 1;
+  const Grid g = level_grid(c, F);
+  const long long N = g.cells();
+  const double h = c->h, om = c->opts.omega;
+  // 2^S: |phi| < 2^55 (four bits of room before 2^59) and |h^2 f| < 2^58
+  check(c, mg::launch_absmax<double>(phi, N, c->partials, c->scal + 50, s), "max |phi|");
+  check(c, mg::launch_absmax<double>(c->f64[F], N, c->partials, c->scal + 51, s), "max |f|");
+  if (bc.kind == mg::BC_OPEN || bc.kind == mg::BC_MIXED)
+    check(c, mg::launch_absmax<double>(c->faces[F], (long long)mg::faces_count(g), c->partials,
+                                       c->scal + 52, s),
+          "max |b|");
+  check(c, cudaMemsetAsync(c->iflag, 0, sizeof(int), s), "clear flag");
+  check(c, cudaMemcpyAsync(c->pinned + 50, c->scal + 50, 3 * sizeof(double),
+                           cudaMemcpyDeviceToHost, s),
+        "read max");
+  check(c, cudaStreamSynchronize(s), "sync");
+  double mphi = c->pinned[50];
+  const double mfh = c->pinned[51] * h * h;
+  if (bc.kind == mg::BC_OPEN || bc.kind == mg::BC_MIXED) mphi = std::max(mphi, c->pinned[52]);
+  if (bc.kind == mg::BC_FIXED) mphi = std::max(mphi, std::fabs(bc.value));
+  if (!std::isfinite(fnorm) || !std::isfinite(mphi) || !std::isfinite(mfh) || mphi <= 0.0 ||
+      mfh <= 0.0)
+    return -1;
+  int ep = 0, ef = 0;
+  std::frexp(mphi, &ep);  // mphi < 2^ep
+  std::frexp(mfh, &ef);
+  const int S = std::min(55 - ep, 58 - ef);
+  if (S < -900 || S > 900) return -1;
+  const double two_S = std::ldexp(1.0, S);
+  long long *cur = reinterpret_cast<long long*>(phi), *alt = c->fxbuf;
+  const long long* FX = reinterpret_cast<const long long*>(c->f64[F]);
+  long long* ec = reinterpret_cast<long long*>(c->u64[F - 1]);
+  double *red = c->partials, *black = c->partials + 3 * (size_t)c->partials_cap;
+  long long* psum = reinterpret_cast<long long*>(c->partials + c->partials_cap);
+  const int nb = mg::fx64_blocks(g);
+  check(c, mg::launch_f64_to_fx(phi, N, 0.0, two_S, s), "phi -> fixed point");
+  check(c, mg::launch_fx64_source(c->f64[F], g, bc, h * h * two_S, two_S, s),
+        "h^2 f -> fixed point");
+  Pyr<double> P = pyr<double>(c);
+  const Grid gc = level_grid(c, F - 1);
+  StopRule rule{tol, c->opts.stall_ratio};
+  int n = 0, st = -1;
+  for (int cyc = -1;; ++cyc) {  // cycle -1 ends the FMG ladder
+    {
+      KTimer t(c, MG_K_FUSED_DOWN, true, s);
+      check(c, mg::launch_fx64_down(cur, alt, FX, c->f64[F - 1], g, hom, om, red, psum, c->iflag, s),
+            "down leg");
+    }
+    if (cyc >= 0) {  // the norm of the last cycle's phi (the leg above ran ahead of the test)
+      check(c, mg::launch_fx64_norm(red, black, nb, c->scal + 1, s), "norm");
+      check(c, cudaMemcpyAsync(c->pinned + 1, c->scal + 1, sizeof(double), cudaMemcpyDeviceToHost,
+                               s),
+            "read norm");
+      check(c, cudaMemcpyAsync(c->pinned + 60, c->iflag, sizeof(int), cudaMemcpyDeviceToHost, s),
+            "read flag");
+      check(c, cudaStreamSynchronize(s), "sync");
+      int flag = 0;
+      std::memcpy(&flag, c->pinned + 60, sizeof(int));
+      if (flag) return -1;
+      const double dn = std::sqrt(c->pinned[1] / (double)N) / (h * h * two_S);
+      if (n == 0 && fnorm == 0.0) fnorm = dn > 0.0 ? dn : 1.0;
+      const double r = dn / fnorm;
+      hist[n++] = r;
+      rule.record(r);
+      st = rule.decide(r, cyc, c->opts.max_cycles, n, hist_cap);
+      if (st >= 0) break;
+    }
+    // the correction of the scaled defect, then on phi's integer grid
+    if (F - 1 == 0) coarsest_solve<double>(c, P.u[0], P.f[0], hom, false, s);
+    else if (F - 1 > coarse_top<double>(c))
+      replay(c, c->inner[2], true, s,
+             [&]() { vcycle<double>(c, P, F - 1, hom, hom, true, s); });
+    else vcycle<double>(c, P, F - 1, hom, hom, true, s);
+    check(c, mg::launch_f64_to_fx(c->u64[F - 1], gc.cells(), 0.0, 1.0 / (h * h), s),
+          "correction -> fixed point");
+    KTimer t(c, MG_K_FUSED_UP, true, s);
+    check(c, mg::launch_fx64_up(alt, cur, FX, ec, g, hom, om, black, c->iflag, s), "up leg");
+  }
+  const long long* mean = nullptr;
+  if (mean_free(c)) {
+    check(c, mg::launch_finish_fx_sum(psum, nb, N, c->scal + 56, s), "finish sum phi");
+    mean = reinterpret_cast<const long long*>(c->scal + 57);
+  }
+  if (gacc) {
+    // it reads neighbours, so phi goes through the other buffer
+    KTimer t(c, MG_K_GRAVITY, true, s);
+    check(c, mg::launch_fx_finish_gravity(cur, reinterpret_cast<double*>(alt), gacc, g, bc, h, S,
+                                          mean, s),
+          "fixed point -> phi, g");
+    check(c, cudaMemcpyAsync(phi, alt, sizeof(double) * N, cudaMemcpyDeviceToDevice, s),
+          "copy phi");
+  } else {
+    check(c, mg::launch_fx_to_f64(cur, phi, N, S, mean, s), "fixed point -> phi");
+  }
+  *n_hist = n;
+  return st;
+}
+
 mg_status solve_fp64(mg_ctx* c, const double* rho, double four_pi_G, double tol, double* phi,
                      double* gacc, double* hist, int hist_cap, int* n_hist, cudaStream_t s) {
   const int F = c->L - 1;
@@ -827,7 +946,20 @@ mg_status solve_fp64(mg_ctx* c, const double* rho, double four_pi_G, double tol,
   const bool fas = c->opts.fas != 0;
   if (c->opts.mode_fmg) {
     if (fas) fmg_fas(c, bcs, hom, s);
-    else fmg<double>(c, P, bcs, hom, s);
+    else if (c->fxbuf && ((uintptr_t)phi & 15u) == 0) {
+      fmg_below<double>(c, P, bcs, hom, s);
+      const int st =
+          solve_fx64(c, fnorm, tol, phi, gacc, bcs[F], hom, hist, hist_cap, n_hist, s);
+      if (st >= 0) {
+        c->u64[F] = nullptr;
+        return (mg_status)st;
+      }
+      // outside the fixed-point range: everything again in FP64
+      fnorm = prepare_source(c, rho, four_pi_G, c->f64[F], true, s);
+      fmg<double>(c, P, bcs, hom, s);
+    } else {
+      fmg<double>(c, P, bcs, hom, s);
+    }
   }
   double dn = defect_rms(c, phi, c->f64[F], bcs[F], s);
   if (fnorm == 0.0) fnorm = dn > 0.0 ? dn : 1.0;

@@ -1,0 +1,123 @@
+"""The FP64 path's finest level in 64-bit fixed point (mg_fx64.cu) and the FP64
+level kernels, against the oracle.
+
+Whole solves with the same schedule differ from the oracle's in rounding order
+only: e_max <= 1e-11 as in the other same-schedule tests.  The shapes cover one
+tile and several, a z-chunk shorter than its halo's reach, ragged last chunks
+and tiles whose window wraps twice.  A source scaled by a power of two gives
+the same integers, so the same bits scaled.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle as orc
+import paper_2302_13903_gb300 as mg
+
+pytestmark = pytest.mark.gpu
+
+NO_STALL = 1e300
+P, F, Z = mg.PERIODIC, mg.FIXED, mg.ZEROGRAD
+RULES = {
+    "periodic": ((P,) * 6, (0,) * 6),
+    "fixed": ((F,) * 6, (0.4,) * 6),
+    "zerograd": ((Z,) * 6, (0,) * 6),
+    "x_walls": ((Z, F, P, P, P, P), (0, 0.3, 0, 0, 0, 0)),
+    "yz_walls": ((P, P, F, Z, Z, F), (0, 0, -0.5, 0, 0, 0.2)),
+}
+
+
+def source(dims, seed):
+    nx, ny, nz = dims
+    rho = np.random.default_rng(seed).standard_normal((nz, ny, nx))
+    return rho - rho.mean()
+
+
+def oracle_args(rule):
+    kinds, values = RULES[rule]
+    bc = kinds[0] if len(set(kinds)) == 1 else orc.PER_FACE
+    return bc, dict(bc_value=values[0],
+                    faces=orc.mixed_rule(kinds, values) if bc == orc.PER_FACE else None)
+
+
+def gpu(rho, rule, tol=0.0, phi=None, **kw):
+    kinds, values = RULES[rule]
+    nz, ny, nx = rho.shape
+    with mg.Solver((nx, ny, nz), 1.0 / nx, list(kinds), face_values=list(values), prec=mg.FP64,
+                   **kw) as s:
+        p, hist, st = s.solve(torch.from_numpy(rho).cuda(), 1.0, tol, phi=phi, raise_on_error=False)
+    return p.cpu().numpy(), hist, st
+
+
+@pytest.mark.parametrize("rule", sorted(RULES))
+@pytest.mark.parametrize("dims", [(64, 16, 16), (64, 64, 64), (128, 32, 16), (128, 128, 64)])
+def test_same_schedule(dims, rule):
+    rho = source(dims, sum(dims))
+    bc, kw = oracle_args(rule)
+    for k in (0, 2):
+        ref = orc.solve(rho, 1.0 / dims[0], bc, tol=0.0, max_cycles=k, stall_ratio=NO_STALL, **kw)
+        phi, hist, st = gpu(rho, rule, max_cycles=k, stall_ratio=NO_STALL)
+        assert st == ref.status and len(hist) == len(ref.hist)
+        assert np.abs(phi - ref.phi).max() <= 1e-11 * np.abs(ref.phi).max()
+        assert np.allclose(hist, ref.hist, rtol=1e-6, atol=1e-14)
+
+
+def test_power_of_two_scaling_is_exact_and_misaligned_phi_agrees():
+    rho = source((64, 32, 32), 3)
+    base, h0, _ = gpu(rho, "periodic", max_cycles=2, stall_ratio=NO_STALL)
+    for e in (-300, 300):
+        p, h, _ = gpu(rho * 2.0 ** e, "periodic", max_cycles=2, stall_ratio=NO_STALL)
+        assert np.array_equal(p, base * 2.0 ** e) and np.array_equal(h, h0)
+    # 8-byte aligned phi: the general FP64 kernels
+    odd = torch.zeros(rho.size + 1, dtype=torch.float64, device="cuda")[1:].view(rho.shape)
+    p, _, _ = gpu(rho, "periodic", phi=odd, max_cycles=2, stall_ratio=NO_STALL)
+    assert np.abs(p - base).max() <= 1e-12 * np.abs(base).max()
+
+
+def test_sources_outside_the_fixed_point_range():
+    rho = source((64, 64, 64), 5)
+    zero, hist, st = gpu(np.zeros_like(rho), "fixed", tol=1e-10)
+    ref = orc.solve(np.zeros_like(rho), 1.0 / 64, F, bc_value=0.4, tol=1e-10)
+    assert st == ref.status and np.abs(zero - ref.phi).max() <= 1e-11 * 0.4
+    phi, hist, st = gpu(np.zeros_like(rho), "periodic", tol=1e-10)
+    assert st == 0 and not phi.any()
+    bad = rho.copy()
+    bad[3, 4, 5] = np.nan
+    assert gpu(bad, "periodic", tol=1e-10)[2] == 5  # MG_ERR_DIVERGED
+    # relaxation far past the stable range: the oracle's status
+    ref = orc.solve(rho, 1.0 / 64, F, bc_value=0.4, tol=1e-10, omega=1.99)
+    assert gpu(rho, "fixed", tol=1e-10, omega=1.99)[2] == ref.status
+
+
+@pytest.mark.parametrize("rule", sorted(RULES))
+@pytest.mark.parametrize("dims", [(2, 2, 2), (6, 4, 2), (10, 6, 4), (64, 6, 10), (34, 2, 64)])
+@pytest.mark.parametrize("prec", [mg.FP64, mg.MIXED])
+def test_level_kernels_on_even_sizes(dims, rule, prec):
+    """SMOOTH, defect + restriction and prolongation on sizes that are even but
+    no powers of two; FP64 to 1e-13 of the largest output, FP32 to 2e-6, as the
+    operator tests on cubes."""
+    if len(set(RULES[rule][0])) > 1:
+        pytest.skip("the operators take one rule for all faces")
+    bc, kw = oracle_args(rule)
+    nx, ny, nz = dims
+    rng = np.random.default_rng(nx + ny + nz)
+    dt, tol = (np.float64, 1e-13) if prec == mg.FP64 else (np.float32, 2e-6)
+    u, f = (rng.standard_normal((nz, ny, nx)).astype(dt) for _ in range(2))
+    h = 0.125
+    gu, gf = (torch.from_numpy(a).cuda() for a in (u, f))
+    value = dict(bc_value=kw["bc_value"])
+
+    def close(got, ref):
+        assert np.abs(got.cpu().numpy() - ref).max() <= tol * max(1.0, np.abs(ref).max())
+
+    ud, fd = u.astype(np.float64), f.astype(np.float64)
+    close(mg.op_smooth(gu.clone(), gf, h, bc, **value),
+          orc.smooth(ud.copy(), fd, h, bc, **value))
+    d = orc.defect(ud, fd, h, bc, **value)
+    close(mg.op_defect_restrict(gu, gf, h, bc, **value), orc.restrict(d))
+    c = rng.standard_normal((nz, ny, nx)).astype(dt)
+    gc = torch.from_numpy(c).cuda()
+    fine = rng.standard_normal((2 * nz, 2 * ny, 2 * nx)).astype(dt)
+    got = mg.op_prolong(gc, bc, bc_value=0.0, add=True, uf=torch.from_numpy(fine).cuda())
+    ref = orc.prolong(c.astype(np.float64), bc, bc_value=0.0, add=True, uf=fine.astype(np.float64))
+    close(got, ref)
