@@ -29,6 +29,7 @@
 
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include "mg_convert.cuh"
 #include "mg_device.cuh"
@@ -37,7 +38,7 @@
 namespace mg {
 namespace {
 
-constexpr int TX = 64, TY = 16;
+constexpr int TY = 16;
 constexpr int kRing = 4;  // planes of the cp.async ring
 
 // omega / 6 = (hi + lo / 2^32) / 2^32.
@@ -54,7 +55,7 @@ struct Fx64Args {
   int cz;        // planes per CTA (even)
   Weight w;
   double* norm;  // per-CTA sum of R^2: red cells of u_in (down), black cells of u_out (up)
-  double* fc;           // down: coarse right-hand side, -sum of R / 8
+  double* fc;           // down: coarse right-hand side, -sum of R
   long long* psum;      // down: per-CTA exact sum of u_in, (hi, lo) pairs
   const long long* ec;  // up: coarse correction on the integer grid
   int* flag;            // |U| passed 2^59
@@ -73,42 +74,50 @@ __device__ __forceinline__ void cp16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp8(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// The window of a CTA: its tile and a halo of HX cells and HY rows.
-template <int HX, int HY>
+// The pairs of a CTA: its TX x TY tile and a halo of HX cells and HY rows.
+template <int TX_, int HX_, int HY_>
 struct Win {
+  static constexpr int TX = TX_, HX = HX_, HY = HY_;
   static constexpr int PW = (TX + 2 * HX) / 2;  // pairs per row
   static constexpr int RH = TY + 2 * HY;
   static constexpr int NT = PW * RH;
   static constexpr int PAD = PW + 1;  // so that every neighbour index is in range
   static constexpr int PLANE = NT + 2 * PAD;
 };
-using Down = Win<4, 3>;
-using Up = Win<2, 2>;
+// The down leg reads the raw black cells of one more row on either side: the
+// first 2 PW threads bring those in, so that no thread computes them.
+template <int TX>
+using Down = Win<TX, 4, 2>;
+template <int TX>
+using Up = Win<TX, 2, 2>;
 
+template <int NT, int NF>
 struct Ring {
-  template <int NT>
-  struct Of {
-    longlong2 u[kRing][NT];
-    longlong2 f[kRing][NT];
-  };
+  longlong2 u[kRing][NT];
+  longlong2 f[kRing][NT];
+  long long frame[kRing][NF];
 };
 
 // What a thread knows about its pair of columns.  Column P is the one that is
 // red in even planes, column Q the one that is red in odd planes.
 struct Pair {
-  int i0, j;       // cells (i0, j) and (i0 + 1, j), wrapped into the level
-  bool valid;      // inside the level
-  bool tile;       // written by this CTA
-  bool swap;       // P is cell i0 + 1
-  int xo;          // pair offset of P's neighbour outside the pair (Q's is -xo)
-  // walls (never with periodic axes): sign of the ghost, 0 where there is none
-  int wxp, wxq, wyl, wyh;
+  int i0, j;   // cells (i0, j) and (i0 + 1, j), wrapped into the level
+  bool valid;  // inside the level
+  bool tile;   // written by this CTA
+  bool swap;   // P is cell i0 + 1
+  int xo;      // pair offset of P's neighbour outside the pair (Q's is -xo)
+  int np, nq;  // 6 less the signs of the ghosts across x and y walls of P, Q
+  Weight w;    // the relaxation; 0 outside the level
 };
 
 __device__ __forceinline__ int wall_sign(int fk, int q) {
@@ -116,52 +125,66 @@ __device__ __forceinline__ int wall_sign(int fk, int q) {
   return kind == BC_PERIODIC ? 0 : kind == BC_ZEROGRAD ? 1 : -1;
 }
 
-template <typename W, int HX, int HY>
-__device__ __forceinline__ Pair make_pair_of(const Fx64Args& a, int t) {
+template <typename W>
+__device__ __forceinline__ Pair make_pair_of(const Fx64Args& a, int pm, int pr) {
   Pair p;
-  const int pm = t % W::PW, pr = t / W::PW;
-  int i = (int)blockIdx.x * TX + 2 * pm - HX, j = (int)blockIdx.y * TY + pr - HY;
-  p.tile = pm >= HX / 2 && pm < HX / 2 + TX / 2 && pr >= HY && pr < HY + TY;
+  int i = (int)blockIdx.x * W::TX + 2 * pm - W::HX, j = (int)blockIdx.y * TY + pr - W::HY;
+  p.tile = pm >= W::HX / 2 && pm < (W::HX + W::TX) / 2 && pr >= W::HY && pr < W::HY + TY;
   const bool px = (a.fk & 3) == BC_PERIODIC, py = ((a.fk >> 4) & 3) == BC_PERIODIC;
   p.valid = (px || (i >= 0 && i < a.g.nx)) && (py || (j >= 0 && j < a.g.ny));
   p.swap = j & 1;
   p.xo = p.swap ? 1 : -1;
   const int xl = i == 0 ? wall_sign(a.fk, 0) : 0, xh = i + 2 == a.g.nx ? wall_sign(a.fk, 1) : 0;
-  p.wxp = p.swap ? xh : xl;
-  p.wxq = p.swap ? xl : xh;
-  p.wyl = j == 0 ? wall_sign(a.fk, 2) : 0;
-  p.wyh = j == a.g.ny - 1 ? wall_sign(a.fk, 3) : 0;
-  // a level may be narrower than the window's reach: wrap by remainder
-  i = (i + 2 * a.g.nx) % a.g.nx;
-  j = (j + 2 * a.g.ny) % a.g.ny;
-  p.i0 = i;
-  p.j = j;
-  if (!p.valid) p.i0 = p.j = 0;
+  const int y = j == 0 ? wall_sign(a.fk, 2) : j == a.g.ny - 1 ? wall_sign(a.fk, 3) : 0;
+  p.np = 6 - (p.swap ? xh : xl) - y;
+  p.nq = 6 - (p.swap ? xl : xh) - y;
+  p.w = p.valid ? a.w : Weight{0, 0};
+  i = i < 0 ? i + a.g.nx : i >= a.g.nx ? i - a.g.nx : i;
+  j = j < 0 ? j + a.g.ny : j >= a.g.ny ? j - a.g.ny : j;
+  p.i0 = p.valid ? i : 0;
+  p.j = p.valid ? j : 0;
   return p;
 }
 
 __device__ __forceinline__ long long signed_by(int s, long long v) { return s < 0 ? -v : v; }
 
-// Sum of the six neighbours of a cell holding `self` whose colour's other
-// values of the plane are in `o` (at this thread's index); `mate` is the
-// pair's other cell, xo the offset of the neighbour outside the pair.
-template <bool WALLS, int PW>
-__device__ __forceinline__ long long sum6(const long long* o, long long self, long long mate, int xo,
-                                          int wx, const Pair& p, long long zl, long long zh, int wzl,
-                                          int wzh) {
-  long long x = o[xo], yl = o[-PW], yh = o[PW];
-  if (WALLS) {
-    if (wx) x = signed_by(wx, self);
-    if (p.wyl) yl = signed_by(p.wyl, self);
-    if (p.wyh) yh = signed_by(p.wyh, self);
-    if (wzl) zl = signed_by(wzl, self);
-    if (wzh) zh = signed_by(wzh, self);
-  }
-  return ((mate + x) + (yl + yh)) + (zl + zh);
+// (Sum of the six neighbours) - 6 self - F of a cell whose neighbours of the
+// plane are in o (at this thread's index); `mate` is the pair's other cell, xo
+// the offset of the neighbour outside the pair, zl and zh the planes below and
+// above.  A ghost across a wall is +-self: cells outside the level hold 0, and
+// n is 6 less the ghosts' signs.
+template <int PW>
+__device__ __forceinline__ long long residual(const long long* o, long long self, long long mate,
+                                              int xo, long long zl, long long zh, int n,
+                                              long long F) {
+  return (((mate + o[xo]) + (o[-PW] + o[PW])) + (zl + zh)) - n * self - F;
 }
 
+// Sum of squares of integers |R| < 2^63 in two floats (relative error about
+// 2^-44), scaled by 2^-24: FP32 and integer instructions only.  A conversion
+// and a multiply-add per cell on the FP64 units, 64 clocks of a scheduler each,
+// set the pace of the legs otherwise.
+struct Squares {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(long long r) {
+    // of |r|: its three parts then never cancel, so hi is |R| to 2^-24
+    const unsigned long long R = (unsigned long long)(r < 0 ? -r : r);
+    const float x2 = (float)(int)(R >> 40) * 0x1p28f;
+    const float x1 = (float)(int)((unsigned)(R >> 20) & 0xfffffu) * 0x1p8f;
+    const float x0 = (float)(int)((unsigned)R & 0xfffffu) * 0x1p-12f;
+    const float lo = x1 + x0, hi = x2 + lo;        // R 2^-12 = hi + rem
+    const float rem = ((x2 - hi) + x1) + x0;
+    const float q = hi * hi, e = fmaf(hi + hi, rem, fmaf(hi, hi, -q));
+    const float t = s + q, b = t - s;
+    c += ((s - (t - b)) + (q - b)) + e;
+    s = t;
+  }
+  __device__ __forceinline__ double total() const { return ((double)s + (double)c) * 0x1p24; }
+};
+
+// |v| at or past 2^59, by the high word.
 __device__ __forceinline__ bool too_large(long long v) {
-  return (unsigned long long)(v + (1LL << 59)) > (2ULL << 59);
+  return (unsigned)((int)(v >> 32) + (1 << 27)) >= (2u << 27);
 }
 
 // Block sum of doubles and of (hi, lo) integers into one partial per CTA.
@@ -205,27 +228,32 @@ __device__ __forceinline__ void block_sums(double v, long long s, bool sums, dou
   }
 }
 
-// Plane q of the level for a march that may leave it: wrapped, or -1 outside a wall.
+// Plane q of the level (-nz <= q < 2 nz) for a march that may leave it:
+// wrapped, or -1 outside a wall.
 __device__ __forceinline__ int plane_of(int q, int nz, bool pz) {
-  if (q >= 0 && q < nz) return q;
-  return pz ? (q + 2 * nz) % nz : -1;
+  const int k = q < 0 ? q + nz : q >= nz ? q - nz : q;
+  return pz || k == q ? k : -1;
 }
 
 // ---------------------------------------------------------------------------
-// Down leg: u_out = SMOOTH(u_in), fc = -(sum of R over the eight children) / 8
-// (the restricted defect times h^2 2^S).  Step q: plane q arrives; [A] red
+// Down leg: u_out = SMOOTH(u_in), fc = -(sum of R over the eight children) (8
+// times the restricted defect times h^2 2^S).  Step q: plane q arrives; [A] red
 // half-step of plane q - 1; [B] black half-step of q - 2, which is then final
 // and written, its black defects from the half-step's own R (the red
 // neighbours do not change again: R - 6 delta, and each ghost moves with the
-// cell); [C] red defects of q - 3.
-template <bool WALLS>
-__global__ void __launch_bounds__(Down::NT, 1) k_fx64_down(const __grid_constant__ Fx64Args a) {
-  using W = Down;
+// cell); [C] red defects of q - 3.  The march is unrolled by four, so that ring
+// slots and the registers of the four planes in hand are fixed: plane q is in
+// slot J, planes q - 1, q - 2, q - 3 in J - 1, J - 2, J - 3 (mod 4).
+template <bool WALLS, int TX>
+__global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
+    k_fx64_down(const __grid_constant__ Fx64Args a) {
+  using W = Down<TX>;
   extern __shared__ longlong2 fx64_smem[];
-  auto& ring = *reinterpret_cast<Ring::Of<W::NT>*>(fx64_smem);
-  long long* base = reinterpret_cast<long long*>(fx64_smem + 2 * kRing * W::NT);
+  using R = Ring<W::NT, 2 * W::PW>;
+  R& ring = *reinterpret_cast<R*>(fx64_smem);
+  long long* base = reinterpret_cast<long long*>(&ring + 1);
   const int t = threadIdx.x;
-  const Pair p = make_pair_of<W, 4, 3>(a, t);
+  const Pair p = make_pair_of<W>(a, t % W::PW, t / W::PW);
   // planes by colour and plane parity: raw black, red after [A], black after
   // [B]; then the odd rows' block sums
   long long* const raw = base + W::PAD + t;
@@ -233,132 +261,121 @@ __global__ void __launch_bounds__(Down::NT, 1) k_fx64_down(const __grid_constant
   long long* const blk = red + 2 * W::PLANE;
   long long* const odd = blk + 2 * W::PLANE;
   const bool pz = ((a.fk >> 8) & 3) == BC_PERIODIC;
+  const int wzl = WALLS ? wall_sign(a.fk, 4) : 0, wzh = WALLS ? wall_sign(a.fk, 5) : 0;
   const int nz = a.g.nz, z0 = (int)blockIdx.z * a.cz, z1 = min(z0 + a.cz, nz);
   const unsigned plane = (unsigned)a.g.nx * a.g.ny;
   const unsigned col = (unsigned)p.j * a.g.nx + p.i0;
-  auto issue = [&](int q) {
+  const unsigned colc = (unsigned)(p.j >> 1) * (a.g.nx >> 1) + (p.i0 >> 1);
+  const bool even_row = p.tile && !(p.j & 1), odd_row = p.j & 1;
+  // the frame: column of Q (black in even planes) and its distance to P's
+  const bool framed = t < 2 * W::PW;
+  const Pair fp = make_pair_of<W>(a, t % W::PW, t < W::PW ? -1 : W::RH);
+  const bool frame_in = framed && fp.valid;
+  const unsigned fcol = (unsigned)fp.j * a.g.nx + fp.i0 + (fp.swap ? 0 : 1);
+  const int fstep = fp.swap ? 1 : -1;
+  long long* const frame = raw + (t < W::PW ? -W::PW : W::NT - W::PW);
+  auto issue = [&](auto slot, int q) {
+    constexpr int s = decltype(slot)::value & 3;
     const int k = q <= z1 + 2 ? plane_of(q, nz, pz) : -1;
-    if (k >= 0 && p.valid) {
+    if (k >= 0 && (!WALLS || p.valid)) {
       const size_t o = (size_t)k * plane + col;
-      const int s = (q - z0 + 8) & (kRing - 1);
       cp16(&ring.u[s][t], a.u_in + o);
       cp16(&ring.f[s][t], a.F + o);
     }
+    if (k >= 0 && frame_in)  // odd slots hold even planes
+      cp8(&ring.frame[s][t], a.u_in + (size_t)k * plane + fcol + (s & 1 ? 0 : fstep));
     cp_commit();
   };
-  // values by plane: P, Q columns of planes a, b, c; what [C] needs of c - 1
-  long long uaP = 0, uaQ = 0, ubP = 0, ubQ = 0, ucP = 0, ucQ = 0, ud = 0;
-  long long faP = 0, faQ = 0, fbP = 0, fbQ = 0, fcr = 0;
-  long long acc = 0, done = 0, psum = 0;
-  double norm = 0.0;
+  long long uP[4] = {}, uQ[4] = {}, fP[4] = {}, fQ[4] = {};
+  long long ud = 0, acc = 0, done = 0, psum = 0;
+  const Weight w = WALLS ? p.w : a.w;
+  Squares norm;
   bool bad = false;
-  issue(z0 - 3);
-  issue(z0 - 2);
-  issue(z0 - 1);
-  // EVEN: plane q is even
-  auto step = [&](auto even, int q) {
-    constexpr bool EVEN = decltype(even)::value;
-    issue(q + 3);
-    cp_wait<3>();
-    const int s = (q - z0 + 8) & (kRing - 1);
-    longlong2 v = make_longlong2(0, 0), f = v;
-    if (p.valid && (!WALLS || plane_of(q, nz, pz) >= 0)) {
-      v = ring.u[s][t];
-      f = ring.f[s][t];
-    }
-    const long long uP = p.swap ? v.y : v.x, uQ = p.swap ? v.x : v.y;
-    const long long fP = p.swap ? f.y : f.x, fQ = p.swap ? f.x : f.y;
+  using std::integral_constant;
+  issue(integral_constant<int, 0>{}, z0 - 3);
+  issue(integral_constant<int, 1>{}, z0 - 2);
+  issue(integral_constant<int, 2>{}, z0 - 1);
+  auto step = [&](auto Jc, int q) {
+    constexpr int J = decltype(Jc)::value, A = (J + 3) & 3, B = (J + 2) & 3, C = (J + 1) & 3;
+    constexpr bool EVEN = J & 1;  // q is even (the march starts on an odd plane)
     constexpr int I0 = EVEN ? 0 : W::PLANE, I1 = EVEN ? W::PLANE : 0;  // parity of q, of q - 1
-    raw[I0] = EVEN ? uQ : uP;  // P is red in even planes
-    if (p.tile && q >= z0 && q < z1) psum += uP + uQ;
+    // the columns by what they are in planes of q's parity; in planes of the
+    // other parity red and black change places
+    long long(&uR)[4] = EVEN ? uP : uQ;
+    long long(&uB)[4] = EVEN ? uQ : uP;
+    long long(&fR)[4] = EVEN ? fP : fQ;
+    long long(&fB)[4] = EVEN ? fQ : fP;
+    const int xb = EVEN ? -p.xo : p.xo, nb = WALLS ? (EVEN ? p.nq : p.np) : 6;
+    issue(integral_constant<int, J + 3>{}, q + 3);
+    cp_wait<3>();
+    if (!WALLS || p.valid) {
+      const longlong2 v = ring.u[J][t], f = ring.f[J][t];
+      uP[J] = p.swap ? v.y : v.x;
+      uQ[J] = p.swap ? v.x : v.y;
+      fP[J] = p.swap ? f.y : f.x;
+      fQ[J] = p.swap ? f.x : f.y;
+    }
+    raw[I0] = uB[J];
+    if (framed) frame[I0] = frame_in ? ring.frame[J][t] : 0;
+    if (p.tile && q >= z0 && q < z1) psum += uP[J] + uQ[J];
     // the block whose last plane was q - 4: its even and odd row's sums
-    if (!EVEN && q - 5 >= z0 && q - 5 < z1 && p.tile && !(p.j & 1)) {
-      const long long sum = done + odd[W::PW];
-      const int K = (q - 5) >> 1;
-      a.fc[((size_t)K * (a.g.ny >> 1) + (p.j >> 1)) * (a.g.nx >> 1) + (p.i0 >> 1)] =
-          cvt::ll2d_pow2_rn(-sum, 3);
-    }
+    if (!EVEN && q - 5 >= z0 && q - 5 < z1 && even_row)
+      a.fc[(size_t)((q - 5) >> 1) * (plane >> 2) + colc] = cvt::ll2d_rn(-(done + odd[W::PW]));
     const int ka = q - 1, kb = q - 2, kc = q - 3;
-    // [A] plane q - 1 (the other parity): red is Q there when q is even
-    {
-      const int wl = WALLS && !pz && ka == 0 ? wall_sign(a.fk, 4) : 0;
-      const int wh = WALLS && !pz && ka == nz - 1 ? wall_sign(a.fk, 5) : 0;
-      long long& r = EVEN ? uaQ : uaP;
-      const long long R =
-          sum6<WALLS, W::PW>(raw + I1, r, EVEN ? uaP : uaQ, EVEN ? -p.xo : p.xo,
-                             EVEN ? p.wxq : p.wxp, p, EVEN ? ubQ : ubP, EVEN ? uQ : uP, wl, wh) -
-          6 * r - (EVEN ? faQ : faP);
-      if (p.tile && ka >= z0 && ka < z1) {
-        const double d = __ll2double_rn(R);
-        norm = fma(d, d, norm);
-      }
-      r += weigh(R, a.w);
-      red[I1] = r;
+    {  // [A]: red of plane q - 1 is in the columns uB
+      long long zl = uB[B], zh = uB[J];
+      int n = nb;
+      if (WALLS && wzl && ka == 0) zl = 0, n -= wzl;
+      if (WALLS && wzh && ka == nz - 1) zh = 0, n -= wzh;
+      const long long R = residual<W::PW>(raw + I1, uB[A], uR[A], xb, zl, zh, n, fB[A]);
+      if (p.tile && ka >= z0 && ka < z1) norm.add(R);
+      uB[A] += weigh(R, w);
+      red[I1] = uB[A];
     }
-    // [B] plane q - 2 (parity of q): black is Q there when q is even
     long long rb;
-    {
-      const int wl = WALLS && !pz && kb == 0 ? wall_sign(a.fk, 4) : 0;
-      const int wh = WALLS && !pz && kb == nz - 1 ? wall_sign(a.fk, 5) : 0;
-      long long& b = EVEN ? ubQ : ubP;
-      const long long R =
-          sum6<WALLS, W::PW>(red + I0, b, EVEN ? ubP : ubQ, EVEN ? -p.xo : p.xo,
-                             EVEN ? p.wxq : p.wxp, p, EVEN ? ucQ : ucP, EVEN ? uaQ : uaP, wl, wh) -
-          6 * b - (EVEN ? fbQ : fbP);
-      const long long d = weigh(R, a.w);
-      int n = 6;  // R moves by -d (6 - signs of the ghosts that move with the cell)
-      if (WALLS) n -= (EVEN ? p.wxq : p.wxp) + p.wyl + p.wyh + wl + wh;
-      b += d;
+    {  // [B]: black of plane q - 2 is in the columns uB
+      long long zl = uB[C], zh = uB[A];
+      int n = nb;  // R moves by -n d: the ghosts move with the cell
+      if (WALLS && wzl && kb == 0) zl = 0, n -= wzl;
+      if (WALLS && wzh && kb == nz - 1) zh = 0, n -= wzh;
+      const long long R = residual<W::PW>(red + I0, uB[B], uR[B], xb, zl, zh, n, fB[B]);
+      const long long d = weigh(R, w);
+      uB[B] += d;
       rb = R - n * d;
-      blk[I0] = b;
+      blk[I0] = uB[B];
       if (p.tile && kb >= z0 && kb < z1) {
-        bad |= too_large(ubP) || too_large(ubQ);
-        const size_t o = (size_t)kb * plane + col;
-        *reinterpret_cast<longlong2*>(a.u_out + o) =
-            p.swap ? make_longlong2(ubQ, ubP) : make_longlong2(ubP, ubQ);
+        bad |= too_large(uP[B]) || too_large(uQ[B]);
+        *reinterpret_cast<longlong2*>(a.u_out + (size_t)kb * plane + col) =
+            p.swap ? make_longlong2(uQ[B], uP[B]) : make_longlong2(uP[B], uQ[B]);
       }
     }
-    // [C] plane q - 3 (the other parity): red is Q there when q is even
-    {
-      const int wl = WALLS && !pz && kc == 0 ? wall_sign(a.fk, 4) : 0;
-      const int wh = WALLS && !pz && kc == nz - 1 ? wall_sign(a.fk, 5) : 0;
-      const long long r = EVEN ? ucQ : ucP;
-      const long long R =
-          sum6<WALLS, W::PW>(blk + I1, r, EVEN ? ucP : ucQ, EVEN ? -p.xo : p.xo,
-                             EVEN ? p.wxq : p.wxp, p, ud, EVEN ? ubQ : ubP, wl, wh) -
-          6 * r - fcr;
-      // planes kc (odd when q is even) and kb of blocks (2K, 2K + 1)
-      if (EVEN) {  // kc closes its block, kb opens the next
+    {  // [C]: red of plane q - 3 is in the columns uB
+      long long zl = ud, zh = uB[B];
+      int n = nb;
+      if (WALLS && wzl && kc == 0) zl = 0, n -= wzl;
+      if (WALLS && wzh && kc == nz - 1) zh = 0, n -= wzh;
+      const long long R = residual<W::PW>(blk + I1, uB[C], uR[C], xb, zl, zh, n, fB[C]);
+      // planes kc and kb of the blocks (2K, 2K + 1)
+      if (EVEN) {  // kc is odd and closes its block, kb opens the next
         done = acc + R;
         acc = rb;
-        if (p.j & 1) *odd = done;
+        if (odd_row) *odd = done;
       } else {
         acc += R + rb;
       }
     }
-    // the next plane's [C] needs the black of this q - 3 in the column of its red
-    ud = EVEN ? ucP : ucQ;
-    ucP = ubP;
-    ucQ = ubQ;
-    fcr = EVEN ? fbP : fbQ;
-    ubP = uaP;
-    ubQ = uaQ;
-    fbP = faP;
-    fbQ = faQ;
-    uaP = uP;
-    uaQ = uQ;
-    faP = fP;
-    faQ = fQ;
+    ud = uR[C];  // the next plane's [C] has its red in the other column
     __syncthreads();
   };
-  // z0 is even, so the march starts on an odd plane
-  for (int q = z0 - 3; q <= z1 + 3; q += 2) {
-    step(std::false_type{}, q);
-    step(std::true_type{}, q + 1);
+  for (int q = z0 - 3; q <= z1 + 3; q += 4) {
+    step(integral_constant<int, 0>{}, q);
+    step(integral_constant<int, 1>{}, q + 1);
+    step(integral_constant<int, 2>{}, q + 2);
+    step(integral_constant<int, 3>{}, q + 3);
   }
   cp_wait<0>();
   if (bad) atomicOr(a.flag, 1);
-  block_sums<W::NT>(norm, psum, true, a.norm, a.psum);
+  block_sums<W::NT>(norm.total(), psum, true, a.norm, a.psum);
 }
 
 // ---------------------------------------------------------------------------
@@ -366,34 +383,37 @@ __global__ void __launch_bounds__(Down::NT, 1) k_fx64_down(const __grid_constant
 // gets its correction; [A] red half-step of q - 1; [B] black half-step of
 // q - 2, then final and written.  The correction of a pair is interpolated
 // along y, then x, then z with weights 3 and 1 on the integer grid and rounded
-// once by the division by 64.
-template <bool WALLS>
-__global__ void __launch_bounds__(Up::NT, 1) k_fx64_up(const __grid_constant__ Fx64Args a) {
-  using W = Up;
+// once by the division by 64.  Unrolled by four as the down leg.
+template <bool WALLS, int TX>
+__global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
+    k_fx64_up(const __grid_constant__ Fx64Args a) {
+  using W = Up<TX>;
   extern __shared__ longlong2 fx64_smem[];
-  auto& ring = *reinterpret_cast<Ring::Of<W::NT>*>(fx64_smem);
-  long long* base = reinterpret_cast<long long*>(fx64_smem + 2 * kRing * W::NT);
+  using R = Ring<W::NT, 1>;
+  R& ring = *reinterpret_cast<R*>(fx64_smem);
+  long long* base = reinterpret_cast<long long*>(&ring + 1);
   const int t = threadIdx.x;
-  const Pair p = make_pair_of<W, 2, 2>(a, t);
+  const Pair p = make_pair_of<W>(a, t % W::PW, t / W::PW);
   long long* const raw = base + W::PAD + t;
   long long* const red = raw + 2 * W::PLANE;
   const bool pz = ((a.fk >> 8) & 3) == BC_PERIODIC;
+  const int wzl = WALLS ? wall_sign(a.fk, 4) : 0, wzh = WALLS ? wall_sign(a.fk, 5) : 0;
   const int nz = a.g.nz, z0 = (int)blockIdx.z * a.cz, z1 = min(z0 + a.cz, nz);
   const unsigned plane = (unsigned)a.g.nx * a.g.ny;
   const unsigned col = (unsigned)p.j * a.g.nx + p.i0;
-  auto issue = [&](int q) {
+  auto issue = [&](auto slot, int q) {
+    constexpr int s = decltype(slot)::value & 3;
     const int k = q <= z1 + 1 ? plane_of(q, nz, pz) : -1;
-    if (k >= 0 && p.valid) {
+    if (k >= 0 && (!WALLS || p.valid)) {
       const size_t o = (size_t)k * plane + col;
-      const int s = (q - z0 + 8) & (kRing - 1);
       cp16(&ring.u[s][t], a.u_in + o);
       cp16(&ring.f[s][t], a.F + o);
     }
     cp_commit();
   };
   // coarse columns m - 1, m, m + 1 of rows J and J': offsets and signs
-  const int nxc = a.g.nx >> 1, nyc = a.g.ny >> 1, nzc = nz >> 1, m = p.i0 >> 1, J = p.j >> 1;
-  int ml = m - 1, mh = m + 1, J2 = (p.j & 1) ? J + 1 : J - 1, sl = 1, sh = 1, sy = 1;
+  const int nxc = a.g.nx >> 1, nyc = a.g.ny >> 1, nzc = nz >> 1, m = p.i0 >> 1, J1 = p.j >> 1;
+  int ml = m - 1, mh = m + 1, J2 = (p.j & 1) ? J1 + 1 : J1 - 1, sl = 1, sh = 1, sy = 1, sz = 1;
   if (ml < 0) {
     const int s = wall_sign(a.fk, 0);
     ml = s ? 0 : nxc - 1;
@@ -410,15 +430,14 @@ __global__ void __launch_bounds__(Up::NT, 1) k_fx64_up(const __grid_constant__ F
     sy = s ? s : 1;
   }
   const unsigned planec = (unsigned)nxc * nyc;
-  const unsigned r1 = (unsigned)J * nxc, r2 = (unsigned)J2 * nxc;
+  const unsigned r1 = (unsigned)J1 * nxc, r2 = (unsigned)J2 * nxc;
   long long c1[3], c2[3];  // the next coarse plane's values, loaded ahead
-  int sz = 1;
   auto load_coarse = [&](int K) {
     int Kw = K;
     sz = 1;
     if (K < 0 || K >= nzc) {
       const int lo = K < 0, s = wall_sign(a.fk, lo ? 4 : 5);
-      Kw = s ? (lo ? 0 : nzc - 1) : (K + 2 * nzc) % nzc;
+      Kw = s ? (lo ? 0 : nzc - 1) : lo ? K + nzc : K - nzc;
       sz = s ? s : 1;
     }
     const long long* e = a.ec + (size_t)Kw * planec;
@@ -446,106 +465,101 @@ __global__ void __launch_bounds__(Up::NT, 1) k_fx64_up(const __grid_constant__ F
     }
   };
   long long em0, em1, e00, e01;  // coarse planes K - 1 and K
-  long long uaP = 0, uaQ = 0, ubP = 0, ubQ = 0, uc = 0;
-  long long faP = 0, faQ = 0, fbb = 0;
-  double norm = 0.0;
+  long long uP[4] = {}, uQ[4] = {}, fP[4] = {}, fQ[4] = {};
+  const Weight w = WALLS ? p.w : a.w;
+  Squares norm;
   bool bad = false;
-  issue(z0 - 2);
-  issue(z0 - 1);
-  issue(z0);
+  using std::integral_constant;
+  issue(integral_constant<int, 0>{}, z0 - 2);
+  issue(integral_constant<int, 1>{}, z0 - 1);
+  issue(integral_constant<int, 2>{}, z0);
   load_coarse((z0 >> 1) - 2);
   interp(em0, em1);
   load_coarse((z0 >> 1) - 1);
   interp(e00, e01);
   load_coarse(z0 >> 1);
-  auto step = [&](auto even, int q) {
-    constexpr bool EVEN = decltype(even)::value;
-    issue(q + 3);
+  auto step = [&](auto Jc, int q) {
+    constexpr int J = decltype(Jc)::value, A = (J + 3) & 3, B = (J + 2) & 3, C = (J + 1) & 3;
+    constexpr bool EVEN = !(J & 1);  // q is even (the march starts on an even plane)
+    constexpr int I0 = EVEN ? 0 : W::PLANE, I1 = EVEN ? W::PLANE : 0;
+    long long(&uR)[4] = EVEN ? uP : uQ;
+    long long(&uB)[4] = EVEN ? uQ : uP;
+    long long(&fB)[4] = EVEN ? fQ : fP;
+    const int xb = EVEN ? -p.xo : p.xo, nb = WALLS ? (EVEN ? p.nq : p.np) : 6;
+    issue(integral_constant<int, J + 3>{}, q + 3);
     cp_wait<3>();
-    const int s = (q - z0 + 8) & (kRing - 1);
-    longlong2 v = make_longlong2(0, 0), f = v;
-    if (p.valid && (!WALLS || plane_of(q, nz, pz) >= 0)) {
-      v = ring.u[s][t];
-      f = ring.f[s][t];
-    }
-    if (EVEN) {  // planes K - 1, K
-      v.x += (3 * e00 + em0 + 32) >> 6;
-      v.y += (3 * e01 + em1 + 32) >> 6;
+    long long d0, d1;  // the pair's correction
+    if (EVEN) {        // planes K - 1, K
+      d0 = 3 * e00 + em0;
+      d1 = 3 * e01 + em1;
     } else {  // planes K, K + 1
       long long p0, p1;
       interp(p0, p1);
-      v.x += (3 * e00 + p0 + 32) >> 6;
-      v.y += (3 * e01 + p1 + 32) >> 6;
+      d0 = 3 * e00 + p0;
+      d1 = 3 * e01 + p1;
       em0 = e00;
       em1 = e01;
       e00 = p0;
       e01 = p1;
       load_coarse(((q + 1) >> 1) + 1);
     }
-    const long long uP = p.swap ? v.y : v.x, uQ = p.swap ? v.x : v.y;
-    const long long fP = p.swap ? f.y : f.x, fQ = p.swap ? f.x : f.y;
-    constexpr int I0 = EVEN ? 0 : W::PLANE, I1 = EVEN ? W::PLANE : 0;
-    raw[I0] = EVEN ? uQ : uP;
-    const int ka = q - 1, kb = q - 2;
-    {
-      const int wl = WALLS && !pz && ka == 0 ? wall_sign(a.fk, 4) : 0;
-      const int wh = WALLS && !pz && ka == nz - 1 ? wall_sign(a.fk, 5) : 0;
-      long long& r = EVEN ? uaQ : uaP;
-      const long long R =
-          sum6<WALLS, W::PW>(raw + I1, r, EVEN ? uaP : uaQ, EVEN ? -p.xo : p.xo,
-                             EVEN ? p.wxq : p.wxp, p, EVEN ? ubQ : ubP, EVEN ? uQ : uP, wl, wh) -
-          6 * r - (EVEN ? faQ : faP);
-      r += weigh(R, a.w);
-      red[I1] = r;
+    if (!WALLS || p.valid) {
+      const longlong2 v = ring.u[J][t], f = ring.f[J][t];
+      const long long v0 = v.x + ((d0 + 32) >> 6), v1 = v.y + ((d1 + 32) >> 6);
+      uP[J] = p.swap ? v1 : v0;
+      uQ[J] = p.swap ? v0 : v1;
+      fP[J] = p.swap ? f.y : f.x;
+      fQ[J] = p.swap ? f.x : f.y;
     }
-    {
-      const int wl = WALLS && !pz && kb == 0 ? wall_sign(a.fk, 4) : 0;
-      const int wh = WALLS && !pz && kb == nz - 1 ? wall_sign(a.fk, 5) : 0;
-      long long& b = EVEN ? ubQ : ubP;
-      const long long R =
-          sum6<WALLS, W::PW>(red + I0, b, EVEN ? ubP : ubQ, EVEN ? -p.xo : p.xo,
-                             EVEN ? p.wxq : p.wxp, p, uc, EVEN ? uaQ : uaP, wl, wh) -
-          6 * b - fbb;
-      const long long d = weigh(R, a.w);
-      int n = 6;
-      if (WALLS) n -= (EVEN ? p.wxq : p.wxp) + p.wyl + p.wyh + wl + wh;
-      b += d;
+    raw[I0] = uB[J];
+    const int ka = q - 1, kb = q - 2;
+    {  // [A]: red of plane q - 1 is in the columns uB
+      long long zl = uB[B], zh = uB[J];
+      int n = nb;
+      if (WALLS && wzl && ka == 0) zl = 0, n -= wzl;
+      if (WALLS && wzh && ka == nz - 1) zh = 0, n -= wzh;
+      const long long R = residual<W::PW>(raw + I1, uB[A], uR[A], xb, zl, zh, n, fB[A]);
+      uB[A] += weigh(R, w);
+      red[I1] = uB[A];
+    }
+    {  // [B]: black of plane q - 2 is in the columns uB
+      long long zl = uB[C], zh = uB[A];
+      int n = nb;
+      if (WALLS && wzl && kb == 0) zl = 0, n -= wzl;
+      if (WALLS && wzh && kb == nz - 1) zh = 0, n -= wzh;
+      const long long R = residual<W::PW>(red + I0, uB[B], uR[B], xb, zl, zh, n, fB[B]);
+      const long long d = weigh(R, w);
+      uB[B] += d;
       if (p.tile && kb >= z0 && kb < z1) {
-        bad |= too_large(ubP) || too_large(ubQ);
-        const double x = __ll2double_rn(R - n * d);
-        norm = fma(x, x, norm);
-        const size_t o = (size_t)kb * plane + col;
-        *reinterpret_cast<longlong2*>(a.u_out + o) =
-            p.swap ? make_longlong2(ubQ, ubP) : make_longlong2(ubP, ubQ);
+        norm.add(R - n * d);
+        bad |= too_large(uP[B]) || too_large(uQ[B]);
+        *reinterpret_cast<longlong2*>(a.u_out + (size_t)kb * plane + col) =
+            p.swap ? make_longlong2(uQ[B], uP[B]) : make_longlong2(uP[B], uQ[B]);
       }
     }
-    // the next plane's [B] needs the red of this q - 2 in the column of its
-    // black, and the F of its black
-    uc = EVEN ? ubP : ubQ;
-    fbb = EVEN ? faP : faQ;
-    ubP = uaP;
-    ubQ = uaQ;
-    uaP = uP;
-    uaQ = uQ;
-    faP = fP;
-    faQ = fQ;
     __syncthreads();
   };
-  // z0 is even: the march starts on an even plane
-  for (int q = z0 - 2; q <= z1; q += 2) {
-    step(std::true_type{}, q);
-    step(std::false_type{}, q + 1);
+  for (int q = z0 - 2; q <= z1 + 1; q += 4) {
+    step(integral_constant<int, 0>{}, q);
+    step(integral_constant<int, 1>{}, q + 1);
+    step(integral_constant<int, 2>{}, q + 2);
+    step(integral_constant<int, 3>{}, q + 3);
   }
   cp_wait<0>();
   if (bad) atomicOr(a.flag, 1);
-  block_sums<W::NT>(norm, 0, false, a.norm, nullptr);
+  block_sums<W::NT>(norm.total(), 0, false, a.norm, nullptr);
 }
 
-template <typename W>
-constexpr size_t smem_bytes(int planes) {
-  return sizeof(Ring::Of<W::NT>) + (size_t)planes * W::PLANE * sizeof(long long);
+template <int TX>
+constexpr size_t down_smem() {
+  using W = Down<TX>;
+  return sizeof(Ring<W::NT, 2 * W::PW>) + 7 * (size_t)W::PLANE * sizeof(long long);
 }
-constexpr size_t kDownSmem = smem_bytes<Down>(7), kUpSmem = smem_bytes<Up>(4);
+template <int TX>
+constexpr size_t up_smem() {
+  using W = Up<TX>;
+  return sizeof(Ring<W::NT, 1>) + 4 * (size_t)W::PLANE * sizeof(long long);
+}
 
 // In place: f becomes F = round(f c) - sum over the cell's fixed and open
 // faces of round(2 b 2^S) (c2 = 2^(S+1)).
@@ -593,45 +607,53 @@ Weight weight_of(double omega) {
   return Weight{(int)hi, lo >= 2147483647.0 ? 2147483647 : (int)lo};
 }
 
-cudaError_t configure() {
+template <int TX>
+cudaError_t launch(const Fx64Args& a, bool down, cudaStream_t s) {
   static std::atomic<int> configured[64];
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && configured[dev].load()) return cudaSuccess;
-  struct {
-    const void* f;
-    size_t b;
-  } k[4] = {{(const void*)k_fx64_down<false>, kDownSmem},
-            {(const void*)k_fx64_down<true>, kDownSmem},
-            {(const void*)k_fx64_up<false>, kUpSmem},
-            {(const void*)k_fx64_up<true>, kUpSmem}};
-  for (auto& x : k) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(x.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)x.b);
+  if (dev < 0 || dev >= 64 || !configured[dev].load()) {
+    const cudaFuncAttribute most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_fx64_down<false, TX>, most, (int)down_smem<TX>());
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_fx64_down<true, TX>, most, (int)down_smem<TX>());
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fx64_up<false, TX>, most, (int)up_smem<TX>());
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fx64_up<true, TX>, most, (int)up_smem<TX>());
     if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) configured[dev].store(1);
   }
-  if (dev >= 0 && dev < 64) configured[dev].store(1);
-  return cudaSuccess;
+  const dim3 grid(a.g.nx / TX, a.g.ny / TY, (a.g.nz + a.cz - 1) / a.cz);
+  ++g_launches;
+  if (down && a.fk) k_fx64_down<true, TX><<<grid, Down<TX>::NT, down_smem<TX>(), s>>>(a);
+  else if (down) k_fx64_down<false, TX><<<grid, Down<TX>::NT, down_smem<TX>(), s>>>(a);
+  else if (a.fk) k_fx64_up<true, TX><<<grid, Up<TX>::NT, up_smem<TX>(), s>>>(a);
+  else k_fx64_up<false, TX><<<grid, Up<TX>::NT, up_smem<TX>(), s>>>(a);
+  return cudaGetLastError();
 }
+
+// Tile width: 64 cells, one CTA per SM, or on levels that would leave SMs
+// without one, 32 cells and two CTAs per SM (more halo, shorter chains).
+int tile_width(Grid g) { return g.cells() <= (1LL << 18) ? 32 : 64; }
 
 }  // namespace
 
 bool fx64_ok(Grid g) {
-  return g.nx % TX == 0 && g.ny % TY == 0 && g.nz % 2 == 0 && g.nz >= 16 &&
+  return g.nx % 64 == 0 && g.ny % TY == 0 && g.nz % 2 == 0 && g.nz >= 16 &&
          g.cells() <= (1LL << 30) && fx64_blocks(g) <= kPartials;
 }
 
-// Planes per CTA: the even count for which the last wave of CTAs (one per SM)
+// Planes per CTA: the even count for which the last wave of CTAs
 // is best filled, counting the six planes a chunk's halo costs; at most 128 (a
 // thread's exact sum of its columns' integers must stay below 2^63).
 int fx64_cz(Grid g) {
-  const long long cols = (long long)(g.nx / TX) * (g.ny / TY);
+  const int tx = tile_width(g), wave = sm_count() * (tx == 64 ? 1 : 2);
+  const long long cols = (long long)(g.nx / tx) * (g.ny / TY);
   int best = 0;
   long long least = 0;
   for (int cz = 4; cz <= 128 && cz <= g.nz; cz += 2) {
     const long long ctas = cols * ((g.nz + cz - 1) / cz);
     if (ctas > kPartials) continue;
-    const long long cost = (ctas + sm_count() - 1) / sm_count() * (cz + 6);
+    const long long cost = (ctas + wave - 1) / wave * (cz + 6);
     if (best == 0 || cost < least) {
       best = cz;
       least = cost;
@@ -643,7 +665,7 @@ int fx64_cz(Grid g) {
 int fx64_blocks(Grid g) {
   const int cz = fx64_cz(g);
   if (cz == 0) return 1 << 30;
-  return (int)((long long)(g.nx / TX) * (g.ny / TY) * ((g.nz + cz - 1) / cz));
+  return (int)((long long)(g.nx / tile_width(g)) * (g.ny / TY) * ((g.nz + cz - 1) / cz));
 }
 
 static int face_kinds_of(const Bc& hom) {
@@ -655,8 +677,6 @@ static int face_kinds_of(const Bc& hom) {
 cudaError_t launch_fx64_down(const long long* u_in, long long* u_out, const long long* F, double* fc,
                              Grid g, const Bc& hom, double omega, double* norm, long long* psum,
                              int* flag, cudaStream_t s) {
-  const cudaError_t e = configure();
-  if (e != cudaSuccess) return e;
   Fx64Args a{};
   a.u_in = u_in;
   a.u_out = u_out;
@@ -669,18 +689,12 @@ cudaError_t launch_fx64_down(const long long* u_in, long long* u_out, const long
   a.fc = fc;
   a.psum = psum;
   a.flag = flag;
-  const dim3 grid(g.nx / TX, g.ny / TY, (g.nz + a.cz - 1) / a.cz);
-  ++g_launches;
-  if (a.fk) k_fx64_down<true><<<grid, Down::NT, kDownSmem, s>>>(a);
-  else k_fx64_down<false><<<grid, Down::NT, kDownSmem, s>>>(a);
-  return cudaGetLastError();
+  return tile_width(g) == 64 ? launch<64>(a, true, s) : launch<32>(a, true, s);
 }
 
 cudaError_t launch_fx64_up(const long long* u_in, long long* u_out, const long long* F,
                            const long long* ec, Grid g, const Bc& hom, double omega, double* norm,
                            int* flag, cudaStream_t s) {
-  const cudaError_t e = configure();
-  if (e != cudaSuccess) return e;
   Fx64Args a{};
   a.u_in = u_in;
   a.u_out = u_out;
@@ -692,11 +706,7 @@ cudaError_t launch_fx64_up(const long long* u_in, long long* u_out, const long l
   a.norm = norm;
   a.ec = ec;
   a.flag = flag;
-  const dim3 grid(g.nx / TX, g.ny / TY, (g.nz + a.cz - 1) / a.cz);
-  ++g_launches;
-  if (a.fk) k_fx64_up<true><<<grid, Up::NT, kUpSmem, s>>>(a);
-  else k_fx64_up<false><<<grid, Up::NT, kUpSmem, s>>>(a);
-  return cudaGetLastError();
+  return tile_width(g) == 64 ? launch<64>(a, false, s) : launch<32>(a, false, s);
 }
 
 cudaError_t launch_fx64_source(double* f, Grid g, const Bc& bc, double c, double two_pow_S,

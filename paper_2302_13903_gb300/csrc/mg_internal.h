@@ -315,7 +315,7 @@ cudaError_t launch_finish_fx_sum(const long long* psum, int nb, long long n, dou
 bool fx64_ok(Grid g);
 int fx64_cz(Grid g);
 int fx64_blocks(Grid g);
-// u_out = SMOOTH(u_in); fc = the restricted defect times h^2 2^S; norm = sums
+// u_out = SMOOTH(u_in); fc = the restricted defect times 8 h^2 2^S; norm = sums
 // of (h^2 2^S defect)^2 over the red cells of u_in; psum = sums of u_in.
 cudaError_t launch_fx64_down(const long long* u_in, long long* u_out, const long long* F, double* fc,
                              Grid g, const Bc& hom, double omega, double* norm, long long* psum,

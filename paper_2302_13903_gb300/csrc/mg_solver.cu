@@ -905,7 +905,7 @@ int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, c
       replay(c, c->inner[2], true, s,
              [&]() { vcycle<double>(c, P, F - 1, hom, hom, true, s); });
     else vcycle<double>(c, P, F - 1, hom, hom, true, s);
-    check(c, mg::launch_f64_to_fx(c->u64[F - 1], gc.cells(), 0.0, 1.0 / (h * h), s),
+    check(c, mg::launch_f64_to_fx(c->u64[F - 1], gc.cells(), 0.0, 1.0 / (8.0 * h * h), s),
           "correction -> fixed point");
     KTimer t(c, MG_K_FUSED_UP, true, s);
     check(c, mg::launch_fx64_up(alt, cur, FX, ec, g, hom, om, black, c->iflag, s), "up leg");
