@@ -115,13 +115,14 @@ cudaError_t launch_coarsest(const T* f, T* u, double h, Bc bc, cudaStream_t s, b
 template <typename T>
 cudaError_t launch_fill(T* u, long long n, T v, cudaStream_t s);
 
-// FP64 source: f = four_pi_G * rho, partial sums of f into partials.
-cudaError_t launch_source(const double* rho, double* f, long long n, double four_pi_G,
+// FP64 source: f = four_pi_G * rho, partial sums of f (or of f^2) into partials.
+cudaError_t launch_source(const double* rho, double* f, long long n, double four_pi_G, bool squares,
                           double* partials, cudaStream_t s);
 // a[i] -= sum(partials[0..nb)) / n  (removes the mean; the sum is formed on
-// the device in a fixed order into *total_slot, a device scalar).
-cudaError_t launch_subtract_mean(double* a, long long n, const double* partials, int nb,
-                                 double* total_slot, cudaStream_t s);
+// the device in a fixed order into *total_slot, a device scalar).  squares:
+// partial sums of the new a^2 into partials (reduce_blocks(n) of them).
+cudaError_t launch_subtract_mean(double* a, long long n, double* partials, int nb,
+                                 double* total_slot, bool squares, cudaStream_t s);
 // Partial sums of a[i] (FP64) and of a[i]^2.
 template <typename T>
 cudaError_t launch_sum(const T* a, long long n, int squares, double* partials, cudaStream_t s);
@@ -250,12 +251,11 @@ int* down_tma_op_flag();
 // out[0] = max |a| (deterministic two-stage reduction through partials).
 template <typename T>
 cudaError_t launch_absmax(const T* a, long long n, double* partials, double* out, cudaStream_t s);
-// In place: double -> round((a - mu) * c) as int64.  out = q * c - m as
-// doubles (out may alias q), m = total[0] * cm when total is given.
-cudaError_t launch_f64_to_fx(double* a, long long n, double mu, double c, cudaStream_t s);
-// out[t] = (q[t] - *mean) 2^-S (mean may be null: 0); out may alias q.
+// In place: double -> round(a c) as int64.
+cudaError_t launch_f64_to_fx(double* a, long long n, double c, cudaStream_t s);
+// out[t] = (q[t] - *mean) 2^-S + b (mean may be null: 0); out may alias q.
 cudaError_t launch_fx_to_f64(const long long* q, double* out, long long n, int S,
-                             const long long* mean, cudaStream_t s);
+                             const long long* mean, double b, cudaStream_t s);
 // out[0] = sum rho, out[1] = max |rho| (n even; partials holds 2
 // reduce_blocks(n / 2) doubles); reads rho only.
 cudaError_t launch_convert(int kind, long long n, const void* in, void* out, cudaStream_t s);

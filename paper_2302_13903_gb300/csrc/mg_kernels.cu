@@ -16,6 +16,7 @@
 #include <atomic>
 #include <cstdint>
 
+#include "mg_convert.cuh"
 #include "mg_device.cuh"
 #include "mg_internal.h"
 
@@ -142,9 +143,11 @@ __global__ void __launch_bounds__(kThreads) k_sor_patch(T* u, const T* f, Grid g
 }
 
 // Partial sums of d^2, d = f - (sum_nb - 6 u) / h^2: 7.5 operations per cell.
-template <typename T, bool PER>
+// R32: also r32 = scale d, narrowed by integer arithmetic.
+template <typename T, bool PER, bool R32>
 __global__ void __launch_bounds__(kThreads) k_defect_norm(const T* u, const T* f, Grid g, Bc bc,
-                                                          T inv_h2, double* partials) {
+                                                          T inv_h2, double* partials, float* r32,
+                                                          double scale) {
   const int hx = g.nx >> 1, hy = g.ny >> 1;
   const long long total = (long long)hx * hy * g.nz;
   const dev::Split sp(hx, hy);
@@ -163,6 +166,10 @@ __global__ void __launch_bounds__(kThreads) k_defect_norm(const T* u, const T* f
       const T db = f[cb] - (sb - T(6) * u[cb]) * inv_h2;
       acc += (double)da * (double)da;
       acc += (double)db * (double)db;
+      if (R32) {
+        r32[ca] = cvt::d2f_rn((double)da * scale);
+        r32[cb] = cvt::d2f_rn((double)db * scale);
+      }
     }
   }
   const double b = block_sum(acc);
@@ -359,14 +366,17 @@ __global__ void k_add_const(double* __restrict__ u, long long n, double v) {
     u[t] += v;
 }
 
+// f = 4 pi G rho and partial sums of f, or of f^2 (SQ).
+template <bool SQ>
 __global__ void k_source(const double* __restrict__ rho, double* __restrict__ f, long long n,
                          double four_pi_G, double* __restrict__ partials) {
   double acc = 0.0;
+#pragma unroll 4
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
     const double v = four_pi_G * rho[t];
     f[t] = v;
-    acc += v;
+    acc = SQ ? fma(v, v, acc) : acc + v;
   }
   const double b = block_sum(acc);
   if (threadIdx.x == 0) partials[blockIdx.x] = b;
@@ -392,14 +402,28 @@ __global__ void k_finish_sum(const double* __restrict__ partials, int nb, double
   if (threadIdx.x == 0) out[0] = b;
 }
 
-// a -= total[0] / n (the total was formed on the device in a fixed order).
-__global__ void k_subtract_mean(double* __restrict__ a, long long n, const double* __restrict__ total) {
+// a -= total[0] / n (the total was formed on the device in a fixed order);
+// SQ: partial sums of the new a^2.
+template <bool SQ>
+__global__ void k_subtract_mean(double* __restrict__ a, long long n, const double* __restrict__ total,
+                                double* __restrict__ partials) {
   const double mean = total[0] / (double)n;
+  double acc = 0.0;
+#pragma unroll 4
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x)
-    a[t] -= mean;
+       t += (long long)gridDim.x * blockDim.x) {
+    const double v = a[t] - mean;
+    a[t] = v;
+    if (SQ) acc = fma(v, v, acc);
+  }
+  if (SQ) {
+    const double b = block_sum(acc);
+    if (threadIdx.x == 0) partials[blockIdx.x] = b;
+  }
 }
 
+// r32 = scale d with d = f - (sum_nb - 6 u) / h^2, partial sums of d^2: for
+// sizes that are not even.
 __global__ void k_outer_residual(const double* __restrict__ u, const double* __restrict__ f,
                                  float* __restrict__ r32, Grid g, Bc bc, double inv_h2,
                                  double scale, double* __restrict__ partials) {
@@ -540,9 +564,9 @@ cudaError_t launch_defect(const T* u, const T* f, T* d, Grid g, double h, Bc bc,
   if (partials && !d && g.nx % 2 == 0 && g.ny % 2 == 0) {
     const T ih2 = (T)(1.0 / (h * h));
     if (bc.kind == BC_PERIODIC)
-      k_defect_norm<T, true><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials);
+      k_defect_norm<T, true, false><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials, nullptr, 0.0);
     else
-      k_defect_norm<T, false><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials);
+      k_defect_norm<T, false, false><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials, nullptr, 0.0);
     return cudaGetLastError();
   }
   k_defect<T><<<nb, kThreads, 0, s>>>(u, f, d, g, bc, (T)(1.0 / (h * h)), partials);
@@ -606,19 +630,23 @@ cudaError_t launch_fill(T* u, long long n, T v, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_source(const double* rho, double* f, long long n, double four_pi_G,
+cudaError_t launch_source(const double* rho, double* f, long long n, double four_pi_G, bool squares,
                           double* partials, cudaStream_t s) {
   ++g_launches;
-  k_source<<<reduce_blocks(n), kThreads, 0, s>>>(rho, f, n, four_pi_G, partials);
+  if (squares) k_source<true><<<reduce_blocks(n), kThreads, 0, s>>>(rho, f, n, four_pi_G, partials);
+  else k_source<false><<<reduce_blocks(n), kThreads, 0, s>>>(rho, f, n, four_pi_G, partials);
   return cudaGetLastError();
 }
 
-cudaError_t launch_subtract_mean(double* a, long long n, const double* partials, int nb,
-                                 double* total_slot, cudaStream_t s) {
+cudaError_t launch_subtract_mean(double* a, long long n, double* partials, int nb,
+                                 double* total_slot, bool squares, cudaStream_t s) {
   ++g_launches;
   k_finish_sum<<<1, kThreads, 0, s>>>(partials, nb, total_slot);
   ++g_launches;
-  k_subtract_mean<<<grid_for(n), kThreads, 0, s>>>(a, n, total_slot);
+  if (squares)
+    k_subtract_mean<true><<<reduce_blocks(n), kThreads, 0, s>>>(a, n, total_slot, partials);
+  else
+    k_subtract_mean<false><<<grid_for(n), kThreads, 0, s>>>(a, n, total_slot, nullptr);
   return cudaGetLastError();
 }
 
@@ -657,8 +685,18 @@ cudaError_t launch_finish_sum(const double* partials, int nb, double* out, cudaS
 cudaError_t launch_outer_residual(const double* u, const double* f, float* r32, Grid g, double h,
                                   Bc bc, double scale, double* partials, cudaStream_t s) {
   ++g_launches;
-  k_outer_residual<<<reduce_blocks(g.cells()), kThreads, 0, s>>>(u, f, r32, g, bc, 1.0 / (h * h),
-                                                                 scale, partials);
+  const int nb = reduce_blocks(g.cells());
+  const double ih2 = 1.0 / (h * h);
+  if (g.nx % 2 == 0 && g.ny % 2 == 0) {
+    if (bc.kind == BC_PERIODIC)
+      k_defect_norm<double, true, true><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials, r32,
+                                                                scale);
+    else
+      k_defect_norm<double, false, true><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials, r32,
+                                                                 scale);
+  } else {
+    k_outer_residual<<<nb, kThreads, 0, s>>>(u, f, r32, g, bc, ih2, scale, partials);
+  }
   return cudaGetLastError();
 }
 

@@ -229,25 +229,103 @@ __global__ void k_raw_moments(const double* __restrict__ rho, Grid g, double h,
   }
 }
 
-__device__ double binom(int n, int k) {
-  double r = 1.0;
-  for (int q = 1; q <= k; ++q) r = r * (n - k + q) / q;
-  return r;
+// The same moments for an even number of planes, folded: with e and o the sum
+// and the difference of the values of a column at +-zeta, the moments along z
+// are sums of e, zeta^2 e, zeta^4 e and of zeta o, zeta^3 o: 3.5 FP64
+// operations per cell instead of 5, and no butterfly per row (25 more per 256
+// cells).  A block has 32 columns along x times 8 groups of `rows` rows, over
+// a chunk of zp pairs of planes; a thread folds y^b in per column and the
+// block adds x^a once at its end.
+constexpr int kMostPairs = 256;
+__global__ void __launch_bounds__(kThreads) k_folded_moments(const double* __restrict__ rho, Grid g,
+                                                             double h, int rows, int zp,
+                                                             double* __restrict__ partials) {
+  constexpr int kYZ = 15;  // y^b z^c with b + c <= 4
+  __shared__ double zt[kMostPairs][4];
+  __shared__ double acc[kYZ][kWarps][32];
+  const int half = g.nz >> 1, p0 = blockIdx.z * zp, p1 = min(p0 + zp, half);
+  for (int q = threadIdx.x; q < p1 - p0; q += kThreads) {
+    const double z = ((double)(p0 + q) + 0.5) * h;
+    zt[q][0] = z;
+    zt[q][1] = z * z;
+    zt[q][2] = z * z * z;
+    zt[q][3] = (z * z) * (z * z);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane, j0 = (blockIdx.y * kWarps + w) * rows;
+  const size_t plane = (size_t)g.nx * g.ny;
+  double t[kYZ];
+#pragma unroll
+  for (int q = 0; q < kYZ; ++q) t[q] = 0.0;
+  for (int r = 0; r < rows; ++r) {
+    const int j = j0 + r;
+    if (i >= g.nx || j >= g.ny) continue;
+    const double* up = rho + (size_t)(half + p0) * plane + (size_t)j * g.nx + i;
+    const double* lo = rho + (size_t)(half - 1 - p0) * plane + (size_t)j * g.nx + i;
+    double m[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int q = 0; q < p1 - p0; ++q) {
+      const double a = up[(size_t)q * plane], b = *(lo - (size_t)q * plane);
+      const double e = a + b, o = a - b;
+      m[0] += e;
+      m[1] = fma(zt[q][0], o, m[1]);
+      m[2] = fma(zt[q][1], e, m[2]);
+      m[3] = fma(zt[q][2], o, m[3]);
+      m[4] = fma(zt[q][3], e, m[4]);
+    }
+    const double y = ((double)j + 0.5 - 0.5 * g.ny) * h;
+    double yp = 1.0;
+    int q = 0;
+#pragma unroll
+    for (int b = 0; b <= 4; ++b) {
+#pragma unroll
+      for (int c = 0; c <= 4 - b; ++c, ++q) t[q] = fma(yp, m[c], t[q]);
+      yp *= y;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < kYZ; ++q) acc[q][w][lane] = t[q];
+  __syncthreads();
+  for (int q = w; q < kYZ; q += kWarps) {  // over the row groups
+    double s = 0.0;
+    for (int k = 0; k < kWarps; ++k) s += acc[q][k][lane];
+    acc[q][0][lane] = s;
+  }
+  __syncthreads();
+  const double x = i < g.nx ? ((double)i + 0.5 - 0.5 * g.nx) * h : 0.0;
+  const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  for (int m = w; m < kMono; m += kWarps) {
+    const int a = c_mono[m][0], b = c_mono[m][1], c = c_mono[m][2];
+    // y^b z^c: rows of 5, 4, 3, 2, 1 values
+    double v = acc[5 * b - b * (b - 1) / 2 + c][0][lane];
+    for (int p = 0; p < a; ++p) v *= x;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) partials[blk * kMono + m] = v;
+  }
 }
 
-// One block: reduce partials per monomial in block order, then the centre of
-// mass (thread 0), the moments about it (one monomial per thread) and Q_lm
-// (thread 0).
-__global__ void k_moments_finish(const double* __restrict__ partials, int nb, double h, int lmax,
+__device__ __forceinline__ double binom(int n, int k) {
+  constexpr unsigned char t[5][5] = {
+      {1, 0, 0, 0, 0}, {1, 1, 0, 0, 0}, {1, 2, 1, 0, 0}, {1, 3, 3, 1, 0}, {1, 4, 6, 4, 1}};
+  return (double)t[n][k];
+}
+
+// One block of kFinishThreads: reduce partials per monomial (a warp each, in a
+// fixed order), then the centre of mass (thread 0), the moments about it (one
+// monomial per thread) and Q_lm (one per thread).
+constexpr int kFinishThreads = 512;
+__global__ void __launch_bounds__(kFinishThreads) k_moments_finish(const double* __restrict__ partials, int nb, double h, int lmax,
                                  int use_com, double ox, double oy, double oz,
                                  double* __restrict__ out) {
   __shared__ double M[kMono];
   __shared__ double Cs[kMono];
   __shared__ double P[3][5];  // (-o)^p per axis, p = 0..4
-  for (int m = threadIdx.x; m < kMono; m += blockDim.x) {
+  for (int m = threadIdx.x >> 5; m < kMono; m += kFinishThreads / 32) {
     double t = 0.0;
-    for (int b = 0; b < nb; ++b) t += partials[(size_t)b * kMono + m];
-    M[m] = t;
+    for (int b = threadIdx.x & 31; b < nb; b += 32) t += partials[(size_t)b * kMono + m];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) M[m] = t;
   }
   __syncthreads();
   // M[0] = sum rho, M[1..3] = sum rho x, y, z (indices of (1,0,0), (0,1,0), (0,0,1))
@@ -280,27 +358,24 @@ __global__ void k_moments_finish(const double* __restrict__ partials, int nb, do
     Cs[q] = acc;
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  const double dv = h * h * h;
-  const double* C = Cs;
-  const double pi = 3.14159265358979323846;
-  double Q[kTerms];
-  for (int q = 0; q < kTerms; ++q) Q[q] = 0.0;
-  for (int t = 0; t < c_nterm; ++t) Q[c_term_lm[t]] += c_term_coef[t] * C[c_term_mono[t]];
-  for (int l = 0; l <= 4; ++l)
-    for (int m = -l; m <= l; ++m) {
-      const int q = l * l + m + l;
-      Q[q] = (l <= lmax) ? Q[q] * dv * sqrt(4.0 * pi / (2.0 * l + 1.0)) : 0.0;
-    }
-  for (int q = 0; q < kTerms; ++q) out[q] = Q[q];
-  out[28] = M[0] * dv;
+  const double dv = h * h * h, pi = 3.14159265358979323846;
+  if (threadIdx.x < kTerms) {
+    const int q = threadIdx.x, l = q == 0 ? 0 : q < 4 ? 1 : q < 9 ? 2 : q < 16 ? 3 : 4;
+    double Q = 0.0;
+    for (int t = 0; t < c_nterm; ++t)
+      if (c_term_lm[t] == q) Q += c_term_coef[t] * Cs[c_term_mono[t]];
+    out[q] = l <= lmax ? Q * dv * sqrt(4.0 * pi / (2.0 * l + 1.0)) : 0.0;
+  }
+  if (threadIdx.x == 0) out[28] = M[0] * dv;
 }
 
 // Potential of the expansion at every face point of a level.  The block first
 // folds the moments into the coefficient of each monomial of the potential's
 // degree-l parts (P_l = sqrt(4 pi / (2l + 1)) sum_m Q_lm r^l Y_lm, homogeneous
-// of degree l), so that a point costs the 35 monomials at compile-time
-// indices and one reciprocal square root: phi = -G sum_l P_l / r^(2l+1).
+// of degree l), so that phi = -G sum_l P_l(r) / r^(2l+1) = -(G / r) sum_l
+// P_l(r / r^2): one polynomial of degree 4 in r / r^2, by Horner's rule in x
+// of polynomials in y of polynomials in z (about 50 multiply-adds a point, where
+// the monomials one by one took 105 operations and their powers).
 __global__ void k_open_faces(Grid g, double h, const double* __restrict__ qo, int lmax, double G,
                              double* __restrict__ faces) {
   __shared__ double A[kMono];
@@ -336,30 +411,27 @@ __global__ void k_open_faces(Grid g, double h, const double* __restrict__ qo, in
     }
     x -= ox; y -= oy; z -= oz;
     const double r2 = x * x + y * y + z * z;
-    double xp[5], yp[5], zp[5];
-    xp[0] = yp[0] = zp[0] = 1.0;
+    const double ir = rsqrt(r2), ir2 = ir * ir;
+    x *= ir2; y *= ir2; z *= ir2;
+    // index of x^ea y^eb z^ec in the order of c_mono: degree, then a, then b
+    // descending
+    double px = 0.0;
 #pragma unroll
-    for (int p = 1; p < 5; ++p) { xp[p] = xp[p - 1] * x; yp[p] = yp[p - 1] * y; zp[p] = zp[p - 1] * z; }
-    // the monomials in the order of c_mono: degree, then a, then b descending
-    double P[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    int m = 0;
+    for (int ea = 4; ea >= 0; --ea) {
+      double py = 0.0;
 #pragma unroll
-    for (int d = 0; d <= 4; ++d)
+      for (int eb = 4 - ea; eb >= 0; --eb) {
+        double pz = 0.0;
 #pragma unroll
-      for (int ea = d; ea >= 0; --ea)
-#pragma unroll
-        for (int eb = d - ea; eb >= 0; --eb) {
-          P[d] += A[m] * (xp[ea] * yp[eb] * zp[d - ea - eb]);
-          ++m;
+        for (int ec = 4 - ea - eb; ec >= 0; --ec) {
+          const int d = ea + eb + ec, u = d - ea;
+          pz = fma(pz, z, A[d * (d + 1) * (d + 2) / 6 + u * (u + 1) / 2 + ec]);
         }
-    const double ir = 1.0 / sqrt(r2), ir2 = ir * ir;
-    double phi = 0.0, w = ir;  // 1 / r^(2l+1)
-#pragma unroll
-    for (int l = 0; l <= 4; ++l) {
-      phi += P[l] * w;
-      w *= ir2;
+        py = fma(py, y, pz);
+      }
+      px = fma(px, x, py);
     }
-    faces[t] = -G * phi;
+    faces[t] = -G * ir * px;
   }
 }
 
@@ -419,9 +491,31 @@ cudaError_t launch_raw_moments(const double* rho, Grid g, double h, double* part
                                cudaStream_t s) {
   cudaError_t e = upload_tables();
   if (e != cudaSuccess) return e;
+  // partials: nb * 35 doubles
+  constexpr long long most = kPartials / kMono;
+  if (g.nz % 2 == 0) {
+    // chunks of 64 pairs and 4 rows a thread; shorter chunks while the blocks
+    // are fewer than two per SM, longer ones where the partials would not fit
+    const int gx = (g.nx + 31) / 32, half = g.nz / 2;
+    int zp = 64, per = 4;
+    auto gy = [&]() { return (g.ny + kWarps * per - 1) / (kWarps * per); };
+    auto gz = [&]() { return (half + zp - 1) / zp; };
+    auto blocks = [&]() { return (long long)gx * gy() * gz(); };
+    while (zp > 8 && blocks() < 2LL * sm_count()) zp /= 2;
+    while (blocks() > most && (zp < kMostPairs || per < 64)) {
+      if (zp < kMostPairs) zp *= 2;
+      else per *= 2;
+    }
+    if (blocks() <= most) {
+      *nb_out = (int)blocks();
+      ++g_launches;
+      k_folded_moments<<<dim3(gx, gy(), gz()), kThreads, 0, s>>>(rho, g, h, per, zp, partials);
+      return cudaGetLastError();
+    }
+  }
   const long long rows = (long long)g.ny * g.nz;
   long long nb = (rows + kWarps - 1) / kWarps;
-  if (nb > kMaxReduceBlocks / 4) nb = kMaxReduceBlocks / 4;  // partials: nb * 35 doubles
+  if (nb > kMaxReduceBlocks / 4) nb = kMaxReduceBlocks / 4;
   *nb_out = (int)nb;
   ++g_launches;
   k_raw_moments<<<(int)nb, kThreads, 0, s>>>(rho, g, h, partials);
@@ -442,7 +536,7 @@ cudaError_t launch_moments_finish(const double* partials, int nb, double h, int 
   cudaError_t e = upload_tables();
   if (e != cudaSuccess) return e;
   ++g_launches;
-  k_moments_finish<<<1, 64, 0, s>>>(partials, nb, h, lmax, use_com, origin_in[0], origin_in[1],
+  k_moments_finish<<<1, kFinishThreads, 0, s>>>(partials, nb, h, lmax, use_com, origin_in[0], origin_in[1],
                                     origin_in[2], out);
   return cudaGetLastError();
 }

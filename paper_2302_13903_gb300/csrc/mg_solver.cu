@@ -768,11 +768,11 @@ double prepare_source(mg_ctx* c, const double* rho, double four_pi_G, double* f_
   const int nb = mg::reduce_blocks(N);
   {
     KTimer t(c, MG_K_SOURCE, true, s);
-    check(c, mg::launch_source(rho, f_fin, N, four_pi_G, c->partials, s), "source");
+    check(c, mg::launch_source(rho, f_fin, N, four_pi_G, !mean_free(c), c->partials, s), "source");
   }
   if (mean_free(c))
-    check(c, mg::launch_subtract_mean(f_fin, N, c->partials, nb, c->scal + 40, s), "subtract_mean");
-  check(c, mg::launch_sum<double>(f_fin, N, 1, c->partials, s), "sum f^2");
+    check(c, mg::launch_subtract_mean(f_fin, N, c->partials, nb, c->scal + 40, true, s),
+          "subtract_mean");
   check(c, mg::launch_finish_sum(c->partials, nb, c->scal + 0, s), "finish f^2");
   if (c->bc_kind == MG_BC_OPEN) {
     int nbm = 0;
@@ -793,7 +793,8 @@ void remove_mean(mg_ctx* c, double* u, cudaStream_t s) {
   if (!mean_free(c)) return;
   const long long N = level_grid(c, c->L - 1).cells();
   check(c, mg::launch_sum<double>(u, N, 0, c->partials, s), "sum phi");
-  check(c, mg::launch_subtract_mean(u, N, c->partials, mg::reduce_blocks(N), c->scal + 40, s),
+  check(c, mg::launch_subtract_mean(u, N, c->partials, mg::reduce_blocks(N), c->scal + 40,
+                                    false, s),
         "phi mean");
 }
 
@@ -867,7 +868,7 @@ int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, c
   double *red = c->partials, *black = c->partials + 3 * (size_t)c->partials_cap;
   long long* psum = reinterpret_cast<long long*>(c->partials + c->partials_cap);
   const int nb = mg::fx64_blocks(g);
-  check(c, mg::launch_f64_to_fx(phi, N, 0.0, two_S, s), "phi -> fixed point");
+  check(c, mg::launch_f64_to_fx(phi, N, two_S, s), "phi -> fixed point");
   check(c, mg::launch_fx64_source(c->f64[F], g, bc, h * h * two_S, two_S, s),
         "h^2 f -> fixed point");
   Pyr<double> P = pyr<double>(c);
@@ -905,7 +906,7 @@ int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, c
       replay(c, c->inner[2], true, s,
              [&]() { vcycle<double>(c, P, F - 1, hom, hom, true, s); });
     else vcycle<double>(c, P, F - 1, hom, hom, true, s);
-    check(c, mg::launch_f64_to_fx(c->u64[F - 1], gc.cells(), 0.0, 1.0 / (8.0 * h * h), s),
+    check(c, mg::launch_f64_to_fx(c->u64[F - 1], gc.cells(), 1.0 / (8.0 * h * h), s),
           "correction -> fixed point");
     KTimer t(c, MG_K_FUSED_UP, true, s);
     check(c, mg::launch_fx64_up(alt, cur, FX, ec, g, hom, om, black, c->iflag, s), "up leg");
@@ -924,7 +925,7 @@ int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, c
     check(c, cudaMemcpyAsync(phi, alt, sizeof(double) * N, cudaMemcpyDeviceToDevice, s),
           "copy phi");
   } else {
-    check(c, mg::launch_fx_to_f64(cur, phi, N, S, mean, s), "fixed point -> phi");
+    check(c, mg::launch_fx_to_f64(cur, phi, N, S, mean, 0.0, s), "fixed point -> phi");
   }
   *n_hist = n;
   return st;
@@ -1208,8 +1209,8 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
                                         mu * c2, s),
                 "h^2 f -> fixed point");
         else
-          check(c, mg::launch_f64_to_fx(f, N, 0.0, c2, s), "h^2 f -> fixed point");
-        if (!phi_zero) check(c, mg::launch_f64_to_fx(phi, N, 0.0, two_S, s), "phi -> fixed point");
+          check(c, mg::launch_f64_to_fx(f, N, c2, s), "h^2 f -> fixed point");
+        if (!phi_zero) check(c, mg::launch_f64_to_fx(phi, N, two_S, s), "phi -> fixed point");
         in_fx = true;
       }
       {
@@ -1255,9 +1256,8 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
     } else {
       // straight into the caller's pinned host phi when there is one
       double* out = c->host_phi ? c->host_phi : phi;
-      check(c, mg::launch_fx_to_f64(cur, out, N, S, mean, s), "fixed point -> phi");
+      check(c, mg::launch_fx_to_f64(cur, out, N, S, mean, b_shift, s), "fixed point -> phi");
       c->host_phi_written = c->host_phi != nullptr;
-      if (b_shift != 0.0) check(c, mg::launch_add_const(out, N, b_shift, s), "phi + b");
     }
     if (gacc && b_shift != 0.0) check(c, mg::launch_add_const(phi, N, b_shift, s), "phi + b");
     // both flags in one read: [0] overflow, [1] a tensor copy that was late
