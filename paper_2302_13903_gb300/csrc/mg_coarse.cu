@@ -557,6 +557,381 @@ __global__ void __launch_bounds__(kThreads<T>) k_coarse(const __grid_constant__ 
   else p.run_vcycles();
 }
 
+// ---------------------------------------------------------------------------
+// The same cycles in FP32 for a cube of 16^3 cells, the coarse end of every
+// cubic grid of the mixed path.  Here the sizes are compile-time constants and
+// a thread owns half a row of the 16^3 level (and the first 64 a row of 8^3)
+// for the whole call: its u and f stay in registers, the colours of a row are
+// kept apart (four red, four black per half row), and shared memory carries
+// only what the neighbouring rows read, in 16-byte loads: four per half-step
+// of four cells, and one shuffle for the cell across the half row's end.  A
+// half-step is about 45 instructions per thread where the general program
+// above spends about 240 on the same four cells (14-19 us per launch).
+//
+// Cell i = 2 m + e of row (j, k), e = (j + k) & 1, is red cell m of the row;
+// 2 m + 1 - e is black cell m.  A row's planes are padded so that the eight
+// lanes of a 16-byte phase (half row, j & 1, k & 1) hit different banks.
+
+struct CubeArgs {
+  float* u;
+  const float* f;
+  const float* dense;
+  float cu, cs;
+  float cf[2], ih2[2];  // levels 8^3, 16^3
+  int fk_top, fk;
+  int pre, post, cycles, zero_guess;
+};
+
+constexpr int kCubeThreads = 512;
+
+// Where a thread's row has its neighbour rows y-, y+, z-, z+: offset of that
+// row, or for a wall of the row itself with the ghost's sign.
+struct Rows {
+  int o[4];
+  float s[4];
+  bool wall[4];
+};
+
+template <int N, bool PER>
+__device__ __forceinline__ Rows rows_of(int fk, int j, int k, int sj, int sk, int tail) {
+  Rows r;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const bool hi = q & 1;
+    const int x = q < 2 ? j : k, kind = PER ? (int)BC_PERIODIC : fkind(fk, 2 + q);
+    const bool end = x == (hi ? N - 1 : 0);
+    r.wall[q] = !PER && end && kind != BC_PERIODIC;
+    r.s[q] = r.wall[q] && kind == BC_FIXED ? -1.f : 1.f;
+    const int y = r.wall[q] ? x : end ? (hi ? 0 : N - 1) : (hi ? x + 1 : x - 1);
+    r.o[q] = (q < 2 ? y * sj + k * sk : j * sj + y * sk) + tail;
+  }
+  return r;
+}
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// One colour of SMOOTH on four cells: own and oth the row's cells of that and
+// of the other colour, x[m] the neighbour along x outside the pair, so / ss
+// the shared arrays of the other and of the same colour.
+template <bool PER>
+__device__ __forceinline__ void relax4(float (&own)[4], const float (&oth)[4], const float (&x)[4],
+                                       const float (&f)[4], const float* so, const float* ss,
+                                       const Rows& r, float cu, float cs, float cf) {
+  float4 v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = ld4((PER || !r.wall[q] ? so : ss) + r.o[q]);
+  float s[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) s[m] = oth[m] + x[m];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+    for (int m = 0; m < 4; ++m) s[m] = PER ? s[m] + w[m] : fmaf(r.s[q], w[m], s[m]);
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) own[m] = cs * s[m] + (cu * own[m] + cf * f[m]);
+}
+
+// Defects summed over the pairs (2 m, 2 m + 1) of a row: xl, xr the cells
+// outside each pair along x.
+template <bool PER>
+__device__ __forceinline__ void pair_defects(float (&d)[4], const float (&red)[4],
+                                             const float (&blk)[4], const float (&xl)[4],
+                                             const float (&xr)[4], const float (&fr)[4],
+                                             const float (&fb)[4], const float* sr, const float* sb,
+                                             const Rows& r, float ih2) {
+  float s[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) s[m] = (xl[m] + xr[m]) - 5.f * (red[m] + blk[m]);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float4 a = ld4(sr + r.o[q]), b = ld4(sb + r.o[q]);
+    const float w[4] = {a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w};
+#pragma unroll
+    for (int m = 0; m < 4; ++m) s[m] = PER ? s[m] + w[m] : fmaf(r.s[q], w[m], s[m]);
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) d[m] = (fr[m] + fb[m]) - ih2 * s[m];
+}
+
+// The coarse rows a fine row (j, k) is interpolated from, with their weights
+// (times 16): its parent's, the nearer one along y, along z, and across.
+struct Parents {
+  int o[4];
+  float w[4];
+};
+template <int NC, bool PER>
+__device__ __forceinline__ Parents parents_of(int fk, int j, int k, int sj, int sk) {
+  const int J = j >> 1, K = k >> 1;
+  auto near = [&](int x, int hi, int q, float& s) {
+    const int y = hi ? x + 1 : x - 1, kind = PER ? (int)BC_PERIODIC : fkind(fk, q + hi);
+    s = 1.f;
+    if (y >= 0 && y < NC) return y;
+    if (kind == BC_PERIODIC) return hi ? 0 : NC - 1;
+    if (kind == BC_FIXED) s = -1.f;
+    return x;
+  };
+  float sy, sz;
+  const int J2 = near(J, j & 1, 2, sy), K2 = near(K, k & 1, 4, sz);
+  Parents p;
+  p.o[0] = J * sj + K * sk;
+  p.o[1] = J2 * sj + K * sk;
+  p.o[2] = J * sj + K2 * sk;
+  p.o[3] = J2 * sj + K2 * sk;
+  p.w[0] = 9.f;
+  p.w[1] = 3.f * sy;
+  p.w[2] = 3.f * sz;
+  p.w[3] = sy * sz;
+  return p;
+}
+
+template <bool PER>
+__global__ void __launch_bounds__(kCubeThreads) k_cube16(const __grid_constant__ CubeArgs a) {
+  constexpr int S16 = 144, S8 = 48;  // padded plane strides (floats)
+  __shared__ alignas(16) float sR[16 * S16], sB[16 * S16];
+  __shared__ alignas(16) float cR[8 * S8], cB[8 * S8], cfR[8 * S8], cfB[8 * S8];
+  __shared__ alignas(16) float nat[512], f4[kDense], u4[kDense];
+  const int t = threadIdx.x;
+  const int h = t & 1, j0 = t >> 1 & 1, k0 = t >> 2 & 1, J = t >> 3 & 7, K = t >> 6;
+  const int j = 2 * J + j0, k = 2 * K + k0;
+  const bool e = j0 != k0;
+  const int own = k * S16 + j * 8 + 4 * h;
+  const Rows rw = rows_of<16, PER>(a.fk_top, j, k, 8, S16, 4 * h);
+  // x walls of this half row (sign of the ghost, 0: none)
+  auto xsign = [&](int fk, int q) {
+    const int kind = PER ? (int)BC_PERIODIC : fkind(fk, q);
+    return kind == BC_PERIODIC ? 0.f : kind == BC_FIXED ? -1.f : 1.f;
+  };
+  const float wl = h == 0 ? xsign(a.fk_top, 0) : 0.f, wh = h == 1 ? xsign(a.fk_top, 1) : 0.f;
+  float md[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) md[q] = a.dense[8 * t + q];
+  float r[4], b[4], fr[4], fb[4];
+  // natural order to colours: cells 8 h .. 8 h + 7 of the row
+  const size_t g = ((size_t)k * 16 + j) * 16 + 8 * h;
+  auto split = [&](const float* p, float (&red)[4], float (&blk)[4]) {
+    const float4 lo = ld4(p), hi = ld4(p + 4);
+    const float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      red[m] = e ? v[2 * m + 1] : v[2 * m];
+      blk[m] = e ? v[2 * m] : v[2 * m + 1];
+    }
+  };
+  split(a.f + g, fr, fb);
+  if (a.zero_guess) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      r[m] = a.pre > 0 ? a.cf[1] * fr[m] : 0.f;
+      b[m] = 0.f;
+    }
+  } else {
+    split(a.u + g, r, b);
+  }
+  st4(sR + own, r);
+  st4(sB + own, b);
+  __syncthreads();
+  // the cell across the end of the half row that colour `own` reads: up: the
+  // other colour's m + 1 (from m = 3), else its m - 1 (from m = 0)
+  auto sweep16 = [&](float (&o)[4], const float (&n)[4], const float (&f)[4], float* so, float* sn,
+                     bool up) {
+    float got = __shfl_xor_sync(0xffffffffu, up ? n[0] : n[3], 1);
+    if (!PER) {
+      if (up && wh != 0.f) got = wh * o[3];
+      if (!up && wl != 0.f) got = wl * o[0];
+    }
+    float x[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) x[m] = up ? (m < 3 ? n[m + 1 & 3] : got) : (m > 0 ? n[m - 1 & 3] : got);
+    relax4<PER>(o, n, x, f, sn, so, rw, a.cu, a.cs, a.cf[1]);
+    st4(so + own, o);
+    __syncthreads();
+  };
+  auto smooth16 = [&](int steps, bool red0) {
+    for (int q = 0; q < steps; ++q) {
+      if (q > 0 || !red0) sweep16(r, b, fr, sR, sB, e);
+      sweep16(b, r, fb, sB, sR, !e);
+    }
+  };
+  // the 8^3 level: the first 64 threads have a row each
+  const int i8j = t & 1, i8k = t >> 1 & 1, J8 = t >> 2 & 3, K8 = t >> 4 & 3;
+  const int j8 = 2 * J8 + i8j, k8 = 2 * K8 + i8k;
+  const bool e8 = i8j != i8k;
+  const int own8 = k8 * S8 + j8 * 4;
+  const Rows rw8 = rows_of<8, PER>(a.fk, j8, k8, 4, S8, 0);
+  const float xl8 = xsign(a.fk, 0), xh8 = xsign(a.fk, 1);
+  float r8[4], b8[4], fr8[4], fb8[4];
+  auto bar64 = [&]() { asm volatile("bar.sync 1, 64;" ::: "memory"); };
+  auto sweep8 = [&](float (&o)[4], const float (&n)[4], const float (&f)[4], float* so, float* sn,
+                    bool up) {
+    float x[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const float hi = m < 3 ? n[m + 1 & 3] : xh8 != 0.f ? xh8 * o[3] : n[0];
+      const float lo = m > 0 ? n[m - 1 & 3] : xl8 != 0.f ? xl8 * o[0] : n[3];
+      x[m] = up ? hi : lo;
+    }
+    relax4<PER>(o, n, x, f, sn, so, rw8, a.cu, a.cs, a.cf[0]);
+    st4(so + own8, o);
+    bar64();
+  };
+  auto smooth8 = [&](int steps, bool red0) {
+    for (int q = 0; q < steps; ++q) {
+      if (q > 0 || !red0) sweep8(r8, b8, fr8, cR, cB, e8);
+      sweep8(b8, r8, fb8, cB, cR, !e8);
+    }
+  };
+  for (int cyc = 0; cyc < a.cycles; ++cyc) {
+    smooth16(a.pre, cyc == 0 && a.zero_guess);
+    {  // restrict to 8^3 (four lanes hold a block's rows)
+      float od[4], ev[4], xl[4], xr[4], d[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        od[m] = e ? r[m] : b[m];
+        ev[m] = e ? b[m] : r[m];
+      }
+      float l = __shfl_xor_sync(0xffffffffu, od[3], 1), u = __shfl_xor_sync(0xffffffffu, ev[0], 1);
+      if (!PER) {
+        if (wl != 0.f) l = wl * ev[0];
+        if (wh != 0.f) u = wh * od[3];
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        xl[m] = m > 0 ? od[m - 1 & 3] : l;
+        xr[m] = m < 3 ? ev[m + 1 & 3] : u;
+      }
+      pair_defects<PER>(d, r, b, xl, xr, fr, fb, sR, sB, rw, a.ih2[1]);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        d[m] += __shfl_xor_sync(0xffffffffu, d[m], 2);
+        d[m] += __shfl_xor_sync(0xffffffffu, d[m], 4);
+        d[m] *= 0.125f;
+      }
+      if (!j0 && !k0) {  // cells 4 h .. 4 h + 3 of coarse row (J, K)
+        const int o = K * S8 + J * 4 + 2 * h;
+        const bool ec = (J + K) & 1;
+        *reinterpret_cast<float2*>(cfR + o) = ec ? make_float2(d[1], d[3]) : make_float2(d[0], d[2]);
+        *reinterpret_cast<float2*>(cfB + o) = ec ? make_float2(d[0], d[2]) : make_float2(d[1], d[3]);
+      }
+    }
+    __syncthreads();
+    if (t < 64) {
+      const float4 x = ld4(cfR + own8), y = ld4(cfB + own8);
+      fr8[0] = x.x; fr8[1] = x.y; fr8[2] = x.z; fr8[3] = x.w;
+      fb8[0] = y.x; fb8[1] = y.y; fb8[2] = y.z; fb8[3] = y.w;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        r8[m] = a.pre > 0 ? a.cf[0] * fr8[m] : 0.f;
+        b8[m] = 0.f;
+      }
+      st4(cR + own8, r8);
+      st4(cB + own8, b8);
+      bar64();
+      smooth8(a.pre, true);
+      float od[4], ev[4], xl[4], xr[4], d[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        od[m] = e8 ? r8[m] : b8[m];
+        ev[m] = e8 ? b8[m] : r8[m];
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        xl[m] = m > 0 ? od[m - 1 & 3] : xl8 != 0.f ? xl8 * ev[0] : od[3];
+        xr[m] = m < 3 ? ev[m + 1 & 3] : xh8 != 0.f ? xh8 * od[3] : ev[0];
+      }
+      pair_defects<PER>(d, r8, b8, xl, xr, fr8, fb8, cR, cB, rw8, a.ih2[0]);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        d[m] += __shfl_xor_sync(0xffffffffu, d[m], 1);
+        d[m] += __shfl_xor_sync(0xffffffffu, d[m], 2);
+        d[m] *= 0.125f;
+      }
+      if (!i8j && !i8k) st4(f4 + (K8 * 4 + J8) * 4, d);
+    }
+    __syncthreads();
+    {  // the cycle of the levels from 4^3 down: eight lanes per row of the matrix
+      const float4 x = ld4(f4 + 8 * (t & 7)), y = ld4(f4 + 8 * (t & 7) + 4);
+      float v = (md[0] * x.x + md[1] * x.y) + (md[2] * x.z + md[3] * x.w);
+      v += (md[4] * y.x + md[5] * y.y) + (md[6] * y.z + md[7] * y.w);
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      v += __shfl_xor_sync(0xffffffffu, v, 4);
+      if ((t & 7) == 0) u4[t >> 3] = v;
+    }
+    __syncthreads();
+    if (t < 64) {
+      const Parents p = parents_of<4, PER>(a.fk, j8, k8, 4, 16);
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 c = ld4(u4 + p.o[q]);
+        v[0] = fmaf(p.w[q], c.x, v[0]);
+        v[1] = fmaf(p.w[q], c.y, v[1]);
+        v[2] = fmaf(p.w[q], c.z, v[2]);
+        v[3] = fmaf(p.w[q], c.w, v[3]);
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const float lo = m > 0 ? v[m - 1 & 3] : xl8 != 0.f ? xl8 * v[0] : v[3];
+        const float hi = m < 3 ? v[m + 1 & 3] : xh8 != 0.f ? xh8 * v[3] : v[0];
+        const float ev = (3.f * v[m] + lo) * 0.015625f, od = (3.f * v[m] + hi) * 0.015625f;
+        r8[m] += e8 ? od : ev;
+        b8[m] += e8 ? ev : od;
+      }
+      st4(cR + own8, r8);
+      st4(cB + own8, b8);
+      bar64();
+      smooth8(a.post, false);
+      float n0[4], n1[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        (m < 2 ? n0 : n1)[2 * m & 3] = e8 ? b8[m] : r8[m];
+        (m < 2 ? n0 : n1)[(2 * m & 3) + 1] = e8 ? r8[m] : b8[m];
+      }
+      st4(nat + (k8 * 8 + j8) * 8, n0);
+      st4(nat + (k8 * 8 + j8) * 8 + 4, n1);
+    }
+    __syncthreads();
+    {
+      const Parents p = parents_of<8, PER>(a.fk, j, k, 8, 64);
+      float v[8] = {};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 x = ld4(nat + p.o[q]), y = ld4(nat + p.o[q] + 4);
+        const float w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = fmaf(p.w[q], w[i], v[i]);
+      }
+      const float sl = xsign(a.fk, 0), sh = xsign(a.fk, 1);
+      const float lo0 = h ? v[3] : sl != 0.f ? sl * v[0] : v[7];
+      const float hi3 = h ? (sh != 0.f ? sh * v[7] : v[0]) : v[4];
+      float c[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) c[m] = h ? v[m + 4] : v[m];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const float lo = m > 0 ? c[m - 1 & 3] : lo0, hi = m < 3 ? c[m + 1 & 3] : hi3;
+        const float ev = (3.f * c[m] + lo) * 0.015625f, od = (3.f * c[m] + hi) * 0.015625f;
+        r[m] += e ? od : ev;
+        b[m] += e ? ev : od;
+      }
+    }
+    st4(sR + own, r);
+    st4(sB + own, b);
+    __syncthreads();
+    smooth16(a.post, false);
+  }
+  float4 lo, hi;
+  lo = e ? make_float4(b[0], r[0], b[1], r[1]) : make_float4(r[0], b[0], r[1], b[1]);
+  hi = e ? make_float4(b[2], r[2], b[3], r[3]) : make_float4(r[2], b[2], r[3], b[3]);
+  *reinterpret_cast<float4*>(a.u + g) = lo;
+  *reinterpret_cast<float4*>(a.u + g + 4) = hi;
+}
+
 int log2i(int n) {
   int l = 0;
   while ((1 << l) < n) ++l;
@@ -665,6 +1040,36 @@ cudaError_t launch_coarse(const CoarseCall<T>& q, cudaStream_t s) {
   if (top < 1 || top >= kCoarseLevels) return cudaErrorInvalidValue;
   const Grid* g = q.g;
   const double* h = q.h;
+  if constexpr (sizeof(T) == 4) {
+    // (the FP32 path's rules are homogeneous)
+    const Bc& b = q.bc[top];
+    const bool plain = b.kind != BC_OPEN && (b.kind != BC_FIXED || b.value == 0.0) &&
+                       (b.kind != BC_MIXED || !b.faces);
+    if (q.mode == COARSE_CYCLES && plain && q.dense && g[top].nx == 16 && g[top].ny == 16 &&
+        g[top].nz == 16 && (((uintptr_t)q.u | (uintptr_t)q.f) & 15u) == 0) {
+      CubeArgs a{};
+      a.u = q.u;
+      a.f = q.f;
+      a.dense = q.dense;
+      a.cu = (float)(1.0 - q.omega);
+      a.cs = (float)(q.omega / 6.0);
+      for (int l = 0; l < 2; ++l) {
+        const double hl = h[top - 1 + l];
+        a.cf[l] = (float)(-q.omega * hl * hl / 6.0);
+        a.ih2[l] = (float)(1.0 / (hl * hl));
+      }
+      a.fk_top = face_kinds(b);
+      a.fk = face_kinds(q.hom);
+      a.pre = q.pre;
+      a.post = q.post;
+      a.cycles = q.cycles;
+      a.zero_guess = q.zero_guess ? 1 : 0;
+      ++g_launches;
+      if (a.fk_top == 0 && a.fk == 0) k_cube16<true><<<1, kCubeThreads, 0, s>>>(a);
+      else k_cube16<false><<<1, kCubeThreads, 0, s>>>(a);
+      return cudaGetLastError();
+    }
+  }
   const bool one_cta = q.mode != COARSE_CYCLES;
   CoarseArgs<T> a{};
   a.swap_yz = !one_cta && swap_for(g[top]);
