@@ -1437,6 +1437,12 @@ void autotune(mg_ctx* c, cudaStream_t s) {
     for (int l = 1; l <= F; ++l) {
       const Grid g = level_grid(c, l);
       if (!c->u32b[l] || !mg::fused_ok(g, hom)) continue;
+      // a level whose u (both buffers) and f stay in L2 from leg to leg is
+      // timed with them there: flushed, the launch that moves the fewest bytes
+      // wins, which at 128^3 was the up-down pass (29.5 us against 21 us for
+      // the two legs inside a solve)
+      const bool resident = 12 * (size_t)g.cells() <= (size_t)prop.l2CacheSize / 4 * 3;
+      void* const cold = resident ? nullptr : flush;
       for (int z : {0, 1, 2}) {  // zero-fill the level's buffers once
         float* buf = z == 0 ? c->u32[l] : z == 1 ? c->u32b[l] : c->f32[l];
         check(c, cudaMemsetAsync(buf, 0, sizeof(float) * g.cells(), s), "zero");
@@ -1464,7 +1470,7 @@ void autotune(mg_ctx* c, cudaStream_t s) {
               const int cz = cand_i < 32 ? 8 * (1 + (cand_i >> 2)) : 4;
               const mg::TileCfg cand{tx, cz, ty};
               if (cz > g.nz || !mg::fused_cfg_ok(g, cand)) continue;
-              const float ms = time_launches(c, s, reps, flush, flush_bytes, [&]() {
+              const float ms = time_launches(c, s, reps, cold, flush_bytes, [&]() {
                 if (kind == TUNE_DOWN)
                   return mg::launch_fused_down(c->u32[l], c->u32b[l], c->f32[l], c->f32[l - 1], g,
                                                h, hom, om, false, s, cand);
@@ -1504,7 +1510,7 @@ void autotune(mg_ctx* c, cudaStream_t s) {
             int bcz = 0;
             for (int cz = 8; cz <= 64; cz += 8) {
               if (cz > g.nz || !mg::fused_cfg_ok(g, mg::TileCfg{64, cz, ty})) continue;
-              const float ms = time_launches(c, s, reps, flush, flush_bytes, [&]() { return run(cz); });
+              const float ms = time_launches(c, s, reps, cold, flush_bytes, [&]() { return run(cz); });
               if (ms < best) {
                 best = ms;
                 bcz = cz;
@@ -1515,8 +1521,8 @@ void autotune(mg_ctx* c, cudaStream_t s) {
           auto second_faster = [&](auto run_a, auto run_b) {
             float a = 0.f, b = 0.f;
             for (int r = 0; r < 3; ++r) {
-              a += time_launches(c, s, reps, flush, flush_bytes, run_a);
-              b += time_launches(c, s, reps, flush, flush_bytes, run_b);
+              a += time_launches(c, s, reps, cold, flush_bytes, run_a);
+              b += time_launches(c, s, reps, cold, flush_bytes, run_b);
             }
             return b < a;
           };
@@ -1579,7 +1585,7 @@ void autotune(mg_ctx* c, cudaStream_t s) {
             for (int cz : {16, 32, 64, 128}) {
               const mg::TileCfg cand{64, cz, ty};
               if (cz > g.nz || !mg::updown_cfg_ok(g, cand)) continue;
-              const float ms = time_launches(c, s, reps, flush, flush_bytes, [&]() {
+              const float ms = time_launches(c, s, reps, cold, flush_bytes, [&]() {
                 return mg::launch_fused_updown(c->u32[l], c->u32b[l], c->f32[l], c->u32[l - 1],
                                                c->f32[l - 1], g, h, hom, om, s, cand);
               });
@@ -1599,16 +1605,16 @@ void autotune(mg_ctx* c, cudaStream_t s) {
         if (whit != g_tune.end()) {
           c->pairs_faster = whit->second.cz == 1;
         } else {
-          const float ud_ms = time_launches(c, s, reps, flush, flush_bytes, [&]() {
+          const float ud_ms = time_launches(c, s, reps, cold, flush_bytes, [&]() {
             return mg::launch_fused_updown(c->u32[l], c->u32b[l], c->f32[l], c->u32[l - 1],
                                            c->f32[l - 1], g, h, hom, om, s, best);
           });
           const float legs_ms =
-              time_launches(c, s, reps, flush, flush_bytes, [&]() {
+              time_launches(c, s, reps, cold, flush_bytes, [&]() {
                 return mg::launch_fused_down(c->u32[l], c->u32b[l], c->f32[l], c->f32[l - 1], g,
                                              h, hom, om, false, s, c->cfg_down[l]);
               }) +
-              time_launches(c, s, reps, flush, flush_bytes, [&]() {
+              time_launches(c, s, reps, cold, flush_bytes, [&]() {
                 return mg::launch_fused_up(c->u32[l], c->u32b[l], c->f32[l], c->u32[l - 1], g, h,
                                            hom, om, s, c->cfg_up[l]);
               });
