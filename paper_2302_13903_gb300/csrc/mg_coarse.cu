@@ -548,6 +548,7 @@ struct Prog {
 
 template <typename T, bool PER, int MODE>
 __global__ void __launch_bounds__(kThreads<T>) k_coarse(const __grid_constant__ CoarseArgs<T> a) {
+  dev::after_previous();
   extern __shared__ double coarse_smem[];
   __shared__ Slab<T> slabs[2][kCoarseLevels];
   Prog<T, PER> p(a, reinterpret_cast<T*>(coarse_smem), slabs);
@@ -691,6 +692,7 @@ __device__ __forceinline__ Parents parents_of(int fk, int j, int k, int sj, int 
 
 template <bool PER>
 __global__ void __launch_bounds__(kCubeThreads) k_cube16(const __grid_constant__ CubeArgs a) {
+  dev::after_previous();
   constexpr int S16 = 144, S8 = 48;  // padded plane strides (floats)
   __shared__ alignas(16) float sR[16 * S16], sB[16 * S16];
   __shared__ alignas(16) float cR[8 * S8], cB[8 * S8], cfR[8 * S8], cfB[8 * S8];
@@ -1065,8 +1067,8 @@ cudaError_t launch_coarse(const CoarseCall<T>& q, cudaStream_t s) {
       a.cycles = q.cycles;
       a.zero_guess = q.zero_guess ? 1 : 0;
       ++g_launches;
-      if (a.fk_top == 0 && a.fk == 0) k_cube16<true><<<1, kCubeThreads, 0, s>>>(a);
-      else k_cube16<false><<<1, kCubeThreads, 0, s>>>(a);
+      if (a.fk_top == 0 && a.fk == 0) launch_after(k_cube16<true>, 1, kCubeThreads, 0, s, a);
+      else launch_after(k_cube16<false>, 1, kCubeThreads, 0, s, a);
       return cudaGetLastError();
     }
   }
@@ -1115,7 +1117,9 @@ cudaError_t launch_coarse(const CoarseCall<T>& q, cudaStream_t s) {
   bool any = false;
   for (int l = 0; l <= top; ++l) any = any || a.lev[l].dist;
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = any ? kCluster : 1;
   attr[0].val.clusterDim.y = 1;
@@ -1125,7 +1129,7 @@ cudaError_t launch_coarse(const CoarseCall<T>& q, cudaStream_t s) {
   cfg.dynamicSmemBytes = (size_t)values * sizeof(T);
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   ++g_launches;
   if (q.mode == COARSE_FMG)
     return per ? launch_mode<T, true, COARSE_FMG>(cfg, a) : launch_mode<T, false, COARSE_FMG>(cfg, a);

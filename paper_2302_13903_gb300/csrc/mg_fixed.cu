@@ -61,6 +61,7 @@ __device__ __forceinline__ double block_reduce(double v) {
 // load, four loads in flight per thread.
 template <bool VEC>
 __global__ void k_absmax(const float* __restrict__ a, long long n, double* __restrict__ partials) {
+  dev::after_previous();
   float m = 0.f;
   auto take = [&](float x) {
     const float v = x < 0.f ? -x : x;
@@ -107,6 +108,7 @@ __global__ void k_absmax(const float* __restrict__ a, long long n, double* __res
 template <bool PAIRS>
 __global__ void k_absmax_bits(const unsigned long long* __restrict__ a, long long n,
                               double* __restrict__ partials) {
+  dev::after_previous();
   unsigned long long m = 0;
   auto take = [&](unsigned long long x) {
     x &= 0x7fffffffffffffffULL;
@@ -141,6 +143,7 @@ __global__ void k_absmax_bits(const unsigned long long* __restrict__ a, long lon
 }
 
 __global__ void k_finish_max(const double* __restrict__ partials, int nb, double* out) {
+  dev::after_previous();
   double m = 0.0;
   for (int t = threadIdx.x; t < nb; t += blockDim.x) m = fmax(m, partials[t]);
   m = block_reduce<true>(m);
@@ -185,6 +188,7 @@ inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 template <bool PAIRS, bool ADD>
 __global__ void k_fx_to_f64(const long long* q, double* out, long long n, int S,
                             const long long* __restrict__ mean, double b) {
+  dev::after_previous();
   const long long M = mean ? mean[0] : 0;
   stream8<PAIRS>(reinterpret_cast<const unsigned long long*>(q),
                  reinterpret_cast<unsigned long long*>(out), n, [&](unsigned long long v) {
@@ -196,6 +200,7 @@ __global__ void k_fx_to_f64(const long long* q, double* out, long long n, int S,
 // In place: the double a[t] becomes the integer round(a[t] c).
 template <bool PAIRS>
 __global__ void k_f64_to_fx(double* a, long long n, double c) {
+  dev::after_previous();
   unsigned long long* q = reinterpret_cast<unsigned long long*>(a);
   stream8<PAIRS>(q, q, n, [&](unsigned long long v) {
     return (unsigned long long)cvt::d2ll_rn(__longlong_as_double((long long)v) * c);
@@ -281,6 +286,7 @@ __device__ __forceinline__ double exact_value(const ExactSum& a) {
 __global__ void k_rho_stats(const double2* __restrict__ rho, long long n2,
                             double* __restrict__ sum, double* __restrict__ mx,
                             double2* __restrict__ copy) {
+  dev::after_previous();
   ExactSum acc;
   unsigned long long m = 0;
   auto take = [&](const double2 r) {
@@ -328,6 +334,7 @@ __global__ void k_rho_stats(const double2* __restrict__ rho, long long n2,
 __global__ void k_rho_to_r32(const double2* __restrict__ rho, float2* __restrict__ r32,
                              long long n2, float a_arg, float b_arg, const double* __restrict__ ab,
                              double* __restrict__ sum, double* __restrict__ mx) {
+  dev::after_previous();
   const float a = ab ? (float)ab[0] : a_arg, b = ab ? (float)ab[1] : b_arg;
   float acc = 0.f, m = 0.f;
 #pragma unroll 4
@@ -351,6 +358,7 @@ __global__ void k_rho_to_r32(const double2* __restrict__ rho, float2* __restrict
 template <bool PAIRS>
 __global__ void k_rho_to_fx(const double* __restrict__ rho, long long* __restrict__ q, long long n,
                             double a, double b) {
+  dev::after_previous();
   stream8<PAIRS>(reinterpret_cast<const unsigned long long*>(rho),
                  reinterpret_cast<unsigned long long*>(q), n, [&](unsigned long long v) {
                    return (unsigned long long)cvt::d2ll_rn(fma(a, __longlong_as_double(v), -b));
@@ -359,6 +367,7 @@ __global__ void k_rho_to_fx(const double* __restrict__ rho, long long* __restric
 
 __global__ void k_finish_sum_max(const double* __restrict__ sum, const double* __restrict__ mx,
                                  int nb, double* __restrict__ out) {
+  dev::after_previous();
   double a = 0.0, m = 0.0;
   for (int t = threadIdx.x; t < nb; t += blockDim.x) {
     a += sum[t];
@@ -376,6 +385,7 @@ __global__ void k_finish_sum_max(const double* __restrict__ sum, const double* _
 // value above 2^60, past which neighbour sums could overflow.
 __global__ void k_fx_correct(long long* __restrict__ phi, const float* __restrict__ e, long long n,
                              float c, int* __restrict__ flag) {
+  dev::after_previous();
   bool bad = false;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
@@ -502,6 +512,7 @@ __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
               float* __restrict__ r32, Grid g, FxBc bc, float factor, int cz,
               double* __restrict__ partials, long long* __restrict__ psum,
               int* __restrict__ flag) {
+  dev::after_previous();
   __shared__ long long P[2][FX_H][FX_W];
   extern __shared__ long long fx_dyn[];
   FxRing& ring = *reinterpret_cast<FxRing*>(fx_dyn);
@@ -672,6 +683,7 @@ __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
 // sum as a double; out[1]: the mean's bits as a long long.
 __global__ void k_finish_fx_sum(const long long* __restrict__ psum, int nb, int log2n,
                                 double* __restrict__ out) {
+  dev::after_previous();
   __shared__ long long sh[kThreads], sl[kThreads];
   long long h = 0, l = 0;
   for (int t = threadIdx.x; t < nb; t += blockDim.x) {
@@ -714,6 +726,7 @@ __global__ void k_finish_fx_sum(const long long* __restrict__ psum, int nb, int 
 __global__ void k_fx_finish_gravity(const long long* __restrict__ q, double* __restrict__ phi,
                                     double* __restrict__ g, Grid gr, FxBc bc, int S,
                                     double cg, const long long* __restrict__ mean) {
+  dev::after_previous();
   const long long M = mean ? mean[0] : 0;
   const long long N = gr.cells();
   const dev::Split sp(gr.nx, gr.ny);
@@ -744,15 +757,15 @@ cudaError_t launch_absmax(const T* a, long long n, double* partials, double* out
   ++g_launches;
   if constexpr (sizeof(T) == 8) {
     const unsigned long long* q = reinterpret_cast<const unsigned long long*>(a);
-    if (aligned16(a)) k_absmax_bits<true><<<nb, kThreads, 0, s>>>(q, n, partials);
-    else k_absmax_bits<false><<<nb, kThreads, 0, s>>>(q, n, partials);
+    if (aligned16(a)) launch_after(k_absmax_bits<true>, nb, kThreads, 0, s, q, n, partials);
+    else launch_after(k_absmax_bits<false>, nb, kThreads, 0, s, q, n, partials);
   } else if (aligned16(a)) {
-    k_absmax<true><<<nb, kThreads, 0, s>>>(a, n, partials);
+    launch_after(k_absmax<true>, nb, kThreads, 0, s, a, n, partials);
   } else {
-    k_absmax<false><<<nb, kThreads, 0, s>>>(a, n, partials);
+    launch_after(k_absmax<false>, nb, kThreads, 0, s, a, n, partials);
   }
   ++g_launches;
-  k_finish_max<<<1, kThreads, 0, s>>>(partials, nb, out);
+  launch_after(k_finish_max, 1, kThreads, 0, s, partials, nb, out);
   return cudaGetLastError();
 }
 template cudaError_t launch_absmax<double>(const double*, long long, double*, double*, cudaStream_t);
@@ -760,8 +773,8 @@ template cudaError_t launch_absmax<float>(const float*, long long, double*, doub
 
 cudaError_t launch_f64_to_fx(double* a, long long n, double c, cudaStream_t s) {
   ++g_launches;
-  if (aligned16(a)) k_f64_to_fx<true><<<grid_for(n / 8), kThreads, 0, s>>>(a, n, c);
-  else k_f64_to_fx<false><<<grid_for(n), kThreads, 0, s>>>(a, n, c);
+  if (aligned16(a)) launch_after(k_f64_to_fx<true>, grid_for(n / 8), kThreads, 0, s, a, n, c);
+  else launch_after(k_f64_to_fx<false>, grid_for(n), kThreads, 0, s, a, n, c);
   return cudaGetLastError();
 }
 
@@ -770,15 +783,16 @@ cudaError_t launch_fx_to_f64(const long long* q, double* out, long long n, int S
   ++g_launches;
   const bool pairs = aligned16(q) && aligned16(out), add = b != 0.0;
   const int blocks = grid_for(pairs ? n / 8 : n);
-  if (pairs && add) k_fx_to_f64<true, true><<<blocks, kThreads, 0, s>>>(q, out, n, S, mean, b);
-  else if (pairs) k_fx_to_f64<true, false><<<blocks, kThreads, 0, s>>>(q, out, n, S, mean, b);
-  else if (add) k_fx_to_f64<false, true><<<blocks, kThreads, 0, s>>>(q, out, n, S, mean, b);
-  else k_fx_to_f64<false, false><<<blocks, kThreads, 0, s>>>(q, out, n, S, mean, b);
+  if (pairs && add) launch_after(k_fx_to_f64<true, true>, blocks, kThreads, 0, s, q, out, n, S, mean, b);
+  else if (pairs) launch_after(k_fx_to_f64<true, false>, blocks, kThreads, 0, s, q, out, n, S, mean, b);
+  else if (add) launch_after(k_fx_to_f64<false, true>, blocks, kThreads, 0, s, q, out, n, S, mean, b);
+  else launch_after(k_fx_to_f64<false, false>, blocks, kThreads, 0, s, q, out, n, S, mean, b);
   return cudaGetLastError();
 }
 
 template <int KIND>
 __global__ void k_convert(const void* __restrict__ in, void* __restrict__ out, long long n) {
+  dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
     if (KIND == 0) static_cast<long long*>(out)[t] = cvt::d2ll_rn(static_cast<const double*>(in)[t]);
@@ -793,11 +807,11 @@ cudaError_t launch_convert(int kind, long long n, const void* in, void* out, cud
   if (n == 0) return cudaSuccess;
   ++g_launches;
   switch (kind) {
-    case 0: k_convert<0><<<grid_for(n), kThreads, 0, s>>>(in, out, n); break;
-    case 1: k_convert<1><<<grid_for(n), kThreads, 0, s>>>(in, out, n); break;
-    case 2: k_convert<2><<<grid_for(n), kThreads, 0, s>>>(in, out, n); break;
-    case 3: k_convert<3><<<grid_for(n), kThreads, 0, s>>>(in, out, n); break;
-    case 4: k_convert<4><<<grid_for(n), kThreads, 0, s>>>(in, out, n); break;
+    case 0: launch_after(k_convert<0>, grid_for(n), kThreads, 0, s, in, out, n); break;
+    case 1: launch_after(k_convert<1>, grid_for(n), kThreads, 0, s, in, out, n); break;
+    case 2: launch_after(k_convert<2>, grid_for(n), kThreads, 0, s, in, out, n); break;
+    case 3: launch_after(k_convert<3>, grid_for(n), kThreads, 0, s, in, out, n); break;
+    case 4: launch_after(k_convert<4>, grid_for(n), kThreads, 0, s, in, out, n); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -810,10 +824,9 @@ cudaError_t launch_rho_stats(const double* rho, long long n, double* partials, d
   // at most 2^14 values per thread in the exact sums (2^32 cells, 34 GB of rho)
   if (n > (long long)nb * kThreads * 16384) return cudaErrorInvalidValue;
   ++g_launches;
-  k_rho_stats<<<nb, kThreads, 0, s>>>(reinterpret_cast<const double2*>(rho), n / 2, partials,
-                                      partials + nb, nullptr);
+  launch_after(k_rho_stats, nb, kThreads, 0, s, reinterpret_cast<const double2*>(rho), n / 2, partials, partials + nb, nullptr);
   ++g_launches;
-  k_finish_sum_max<<<1, kThreads, 0, s>>>(partials, partials + nb, nb, out);
+  launch_after(k_finish_sum_max, 1, kThreads, 0, s, partials, partials + nb, nb, out);
   return cudaGetLastError();
 }
 
@@ -823,10 +836,9 @@ cudaError_t launch_rho_stats_copy(const double* host_rho, double* dev, long long
   const int nb = reduce_blocks(n / 2);
   if (n > (long long)nb * kThreads * 16384) return cudaErrorInvalidValue;
   ++g_launches;
-  k_rho_stats<<<nb, kThreads, 0, s>>>(reinterpret_cast<const double2*>(host_rho), n / 2, partials,
-                                      partials + nb, reinterpret_cast<double2*>(dev));
+  launch_after(k_rho_stats, nb, kThreads, 0, s, reinterpret_cast<const double2*>(host_rho), n / 2, partials, partials + nb, reinterpret_cast<double2*>(dev));
   ++g_launches;
-  k_finish_sum_max<<<1, kThreads, 0, s>>>(partials, partials + nb, nb, out);
+  launch_after(k_finish_sum_max, 1, kThreads, 0, s, partials, partials + nb, nb, out);
   return cudaGetLastError();
 }
 
@@ -837,6 +849,7 @@ cudaError_t launch_rho_stats_copy(const double* host_rho, double* dev, long long
 // operation in the order the host would take them.
 __global__ void k_source_scale(const double* __restrict__ st, long long n, double four_pi_G,
                                int has_mean, double* __restrict__ out) {
+  dev::after_previous();
   const double mu = has_mean ? __dmul_rn(four_pi_G, __ddiv_rn(st[0], (double)n)) : 0.0;
   const double bound = __dadd_rn(__dmul_rn(fabs(four_pi_G), st[1]), fabs(mu));
   const double scale = bound > 0.0 ? __ddiv_rn(1.0, bound) : 1.0;
@@ -849,7 +862,7 @@ __global__ void k_source_scale(const double* __restrict__ st, long long n, doubl
 cudaError_t launch_source_scale(const double* st, long long n, double four_pi_G, bool has_mean,
                                 double* out, cudaStream_t s) {
   ++g_launches;
-  k_source_scale<<<1, 1, 0, s>>>(st, n, four_pi_G, has_mean ? 1 : 0, out);
+  launch_after(k_source_scale, 1, 1, 0, s, st, n, four_pi_G, has_mean ? 1 : 0, out);
   return cudaGetLastError();
 }
 
@@ -859,11 +872,9 @@ cudaError_t launch_rho_to_r32(const double* rho, float* r32, long long n, double
   if (n % 2) return cudaErrorInvalidValue;
   const int nb = reduce_blocks(n / 2);
   ++g_launches;
-  k_rho_to_r32<<<nb, kThreads, 0, s>>>(reinterpret_cast<const double2*>(rho),
-                                       reinterpret_cast<float2*>(r32), n / 2, (float)a, (float)b,
-                                       ab_dev, partials, partials + nb);
+  launch_after(k_rho_to_r32, nb, kThreads, 0, s, reinterpret_cast<const double2*>(rho), reinterpret_cast<float2*>(r32), n / 2, (float)a, (float)b, ab_dev, partials, partials + nb);
   ++g_launches;
-  k_finish_sum_max<<<1, kThreads, 0, s>>>(partials, partials + nb, nb, out);
+  launch_after(k_finish_sum_max, 1, kThreads, 0, s, partials, partials + nb, nb, out);
   return cudaGetLastError();
 }
 
@@ -871,16 +882,16 @@ cudaError_t launch_rho_to_fx(const double* rho, long long* q, long long n, doubl
                              cudaStream_t s) {
   ++g_launches;
   if (aligned16(rho) && aligned16(q))
-    k_rho_to_fx<true><<<grid_for(n / 8), kThreads, 0, s>>>(rho, q, n, a, b);
+    launch_after(k_rho_to_fx<true>, grid_for(n / 8), kThreads, 0, s, rho, q, n, a, b);
   else
-    k_rho_to_fx<false><<<grid_for(n), kThreads, 0, s>>>(rho, q, n, a, b);
+    launch_after(k_rho_to_fx<false>, grid_for(n), kThreads, 0, s, rho, q, n, a, b);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fx_correct(long long* phi, const float* e, long long n, float c, int* flag,
                               cudaStream_t s) {
   ++g_launches;
-  k_fx_correct<<<grid_for(n), kThreads, 0, s>>>(phi, e, n, c, flag);
+  launch_after(k_fx_correct, grid_for(n), kThreads, 0, s, phi, e, n, c, flag);
   return cudaGetLastError();
 }
 
@@ -968,8 +979,7 @@ cudaError_t launch_fx_step(const long long* phi_in, long long* phi_out, const fl
     configured[dev].store(1);
   }
   const Kf kf = kfs[pm][zero_in ? 1 : 0];
-  kf<<<grid, FX_TX * FX_TY, kFxSmem, s>>>(phi_in, phi_out, e, c, F, r32, g, b, factor, cz,
-                                          partials, psum, flag);
+  launch_after(kf, grid, FX_TX * FX_TY, kFxSmem, s, phi_in, phi_out, e, c, F, r32, g, b, factor, cz, partials, psum, flag);
   return cudaGetLastError();
 }
 
@@ -979,8 +989,7 @@ cudaError_t launch_fx_finish_gravity(const long long* q, double* phi, double* g,
   const double two_pow_S = std::ldexp(1.0, S);
   const FxBc b = fx_bc(bc, two_pow_S);
   ++g_launches;
-  k_fx_finish_gravity<<<grid_for(gr.cells()), kThreads, 0, s>>>(
-      q, phi, g, gr, b, S, 1.0 / (2.0 * h * two_pow_S), mean);
+  launch_after(k_fx_finish_gravity, grid_for(gr.cells()), kThreads, 0, s, q, phi, g, gr, b, S, 1.0 / (2.0 * h * two_pow_S), mean);
   return cudaGetLastError();
 }
 
@@ -990,7 +999,7 @@ cudaError_t launch_finish_fx_sum(const long long* psum, int nb, long long n, dou
   while ((1LL << log2n) < n) ++log2n;
   if ((1LL << log2n) != n) return cudaErrorInvalidValue;  // levels have 2^k cells
   ++g_launches;
-  k_finish_fx_sum<<<1, kThreads, 0, s>>>(psum, nb, log2n, out);
+  launch_after(k_finish_fx_sum, 1, kThreads, 0, s, psum, nb, log2n, out);
   return cudaGetLastError();
 }
 

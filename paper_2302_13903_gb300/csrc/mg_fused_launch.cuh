@@ -31,7 +31,7 @@ inline cudaError_t launch_t(const float* ui, float* uo, const float* f, const fl
   }
   dim3 grid(p.nx / TX, p.ny / TY, (p.nz + p.cz - 1) / p.cz);
   ++g_launches;
-  k_fused<MODE, ZERO, PM, TX, TY><<<grid, S_::NT, S_::SMEM, s>>>(ui, uo, f, ec, fc, p);
+  launch_after(k_fused<MODE, ZERO, PM, TX, TY>, grid, S_::NT, S_::SMEM, s, ui, uo, f, ec, fc, p);
   return cudaGetLastError();
 }
 

@@ -39,6 +39,7 @@ __global__ void __maxnreg__((fused::fused_max_regs<fused::kDown, 32>()))
                      const float* __restrict__ f, float* __restrict__ fc, FusedParams p,
                      const __grid_constant__ CUtensorMap tmu,
                      const __grid_constant__ CUtensorMap tmf, int* err) {
+  dev::after_previous();
   extern __shared__ float4 smem_tma[];
   // tensor copies land on 128-byte boundaries: round the base up (the launch
   // gives 128 bytes more than the shape needs)
@@ -56,6 +57,7 @@ __global__ void __maxnreg__((fused::fused_max_regs<fused::kUp, 16>()))
                    const float* __restrict__ f, const float* __restrict__ ec, FusedParams p,
                    const __grid_constant__ CUtensorMap tmu,
                    const __grid_constant__ CUtensorMap tmf, int* err) {
+  dev::after_previous();
   extern __shared__ float4 smem_tma[];
   const unsigned off = (unsigned)__cvta_generic_to_shared(smem_tma);
   float4* base = smem_tma + ((128u - (off & 127u)) & 127u) / 16u;
@@ -148,9 +150,9 @@ cudaError_t launch_fused_down_tma(const float* u_in, float* u_out, const float* 
   const dim3 grid(g.nx / 64, g.ny / 32, (g.nz + p.cz - 1) / p.cz);
   ++g_launches;
   if (zero_guess)
-    k_fused_down_tma<true><<<grid, S32::NT, bytes, s>>>(u_in, u_out, f, fc, p, mu, mf, err);
+    launch_after(k_fused_down_tma<true>, grid, S32::NT, bytes, s, u_in, u_out, f, fc, p, mu, mf, err);
   else
-    k_fused_down_tma<false><<<grid, S32::NT, bytes, s>>>(u_in, u_out, f, fc, p, mu, mf, err);
+    launch_after(k_fused_down_tma<false>, grid, S32::NT, bytes, s, u_in, u_out, f, fc, p, mu, mf, err);
   return cudaGetLastError();
 }
 
@@ -188,7 +190,7 @@ cudaError_t launch_fused_up_tma(const float* u_in, float* u_out, const float* f,
   if (attr != cudaSuccess) return attr;
   const dim3 grid(g.nx / 64, g.ny / 16, (g.nz + p.cz - 1) / p.cz);
   ++g_launches;
-  k_fused_up_tma<<<grid, SUp::NT, bytes, s>>>(u_in, u_out, f, ec, p, mu, mf, err);
+  launch_after(k_fused_up_tma, grid, SUp::NT, bytes, s, u_in, u_out, f, ec, p, mu, mf, err);
   return cudaGetLastError();
 }
 

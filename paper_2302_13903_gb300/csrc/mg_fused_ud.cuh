@@ -305,6 +305,7 @@ __global__ void __maxnreg__((updown_max_regs<TY>()))
     k_updown(const float* __restrict__ u_in, float* __restrict__ u_out,
              const float* __restrict__ f, const float* __restrict__ ec, float* __restrict__ fc,
              FusedParams p) {
+  dev::after_previous();
   extern __shared__ float4 smem[];
   updown_tile<PM, TX, TY>(u_in, u_out, f, ec, fc, p, blockIdx.x, blockIdx.y, blockIdx.z, smem);
 }

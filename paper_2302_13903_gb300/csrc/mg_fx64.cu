@@ -247,6 +247,7 @@ __device__ __forceinline__ int plane_of(int q, int nz, bool pz) {
 template <bool WALLS, int TX>
 __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     k_fx64_down(const __grid_constant__ Fx64Args a) {
+  dev::after_previous();
   using W = Down<TX>;
   extern __shared__ longlong2 fx64_smem[];
   using R = Ring<W::NT, 2 * W::PW>;
@@ -387,6 +388,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
 template <bool WALLS, int TX>
 __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
     k_fx64_up(const __grid_constant__ Fx64Args a) {
+  dev::after_previous();
   using W = Up<TX>;
   extern __shared__ longlong2 fx64_smem[];
   using R = Ring<W::NT, 1>;
@@ -564,6 +566,7 @@ constexpr size_t up_smem() {
 // In place: f becomes F = round(f c) - sum over the cell's fixed and open
 // faces of round(2 b 2^S) (c2 = 2^(S+1)).
 __global__ void k_fx64_source(double* f, Grid g, Bc bc, double c, double c2) {
+  dev::after_previous();
   long long* q = reinterpret_cast<long long*>(f);
   const dev::Split sp(g.nx, g.ny);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < g.cells();
@@ -587,6 +590,7 @@ __global__ void k_fx64_source(double* f, Grid g, Bc bc, double c, double c2) {
 
 // out[0] = sum of a[0 .. n) + sum of b[0 .. nb), in a fixed order.
 __global__ void k_fx64_norm(const double* a, int n, const double* b, int nb, double* out) {
+  dev::after_previous();
   __shared__ double ws[8];
   double s = 0.0;
   for (int t = threadIdx.x; t < n; t += blockDim.x) s += a[t];
@@ -624,10 +628,10 @@ cudaError_t launch(const Fx64Args& a, bool down, cudaStream_t s) {
   }
   const dim3 grid(a.g.nx / TX, a.g.ny / TY, (a.g.nz + a.cz - 1) / a.cz);
   ++g_launches;
-  if (down && a.fk) k_fx64_down<true, TX><<<grid, Down<TX>::NT, down_smem<TX>(), s>>>(a);
-  else if (down) k_fx64_down<false, TX><<<grid, Down<TX>::NT, down_smem<TX>(), s>>>(a);
-  else if (a.fk) k_fx64_up<true, TX><<<grid, Up<TX>::NT, up_smem<TX>(), s>>>(a);
-  else k_fx64_up<false, TX><<<grid, Up<TX>::NT, up_smem<TX>(), s>>>(a);
+  if (down && a.fk) launch_after(k_fx64_down<true, TX>, grid, Down<TX>::NT, down_smem<TX>(), s, a);
+  else if (down) launch_after(k_fx64_down<false, TX>, grid, Down<TX>::NT, down_smem<TX>(), s, a);
+  else if (a.fk) launch_after(k_fx64_up<true, TX>, grid, Up<TX>::NT, up_smem<TX>(), s, a);
+  else launch_after(k_fx64_up<false, TX>, grid, Up<TX>::NT, up_smem<TX>(), s, a);
   return cudaGetLastError();
 }
 
@@ -714,14 +718,14 @@ cudaError_t launch_fx64_source(double* f, Grid g, const Bc& bc, double c, double
   long long b = (g.cells() + 255) / 256;
   if (b > sm_count() * 64LL) b = sm_count() * 64LL;
   ++g_launches;
-  k_fx64_source<<<(int)b, 256, 0, s>>>(f, g, bc, c, 2.0 * two_pow_S);
+  launch_after(k_fx64_source, (int)b, 256, 0, s, f, g, bc, c, 2.0 * two_pow_S);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fx64_norm(const double* red, const double* black, int nb, double* out,
                              cudaStream_t s) {
   ++g_launches;
-  k_fx64_norm<<<1, 256, 0, s>>>(red, nb, black, nb, out);
+  launch_after(k_fx64_norm, 1, 256, 0, s, red, nb, black, nb, out);
   return cudaGetLastError();
 }
 

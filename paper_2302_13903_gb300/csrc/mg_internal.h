@@ -80,6 +80,29 @@ int sm_count();
 // resets and reads it around one solve on one thread).
 extern thread_local long long g_launches;
 
+#ifdef __CUDACC__
+// Launch a kernel that begins with dev::after_previous() so that it may be
+// placed while the kernel before it in the stream still runs: small launches,
+// whose latency counts (above four CTAs per SM the launch is ordinary: there
+// the early placement gained nothing and cost the FP64 solves of 256^3 and
+// 512^3 0.7-1.3 %).
+template <typename... K, typename... A>
+cudaError_t launch_after(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                         A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = (long long)grid.x * grid.y * grid.z <= 4LL * sm_count() ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+#endif
+
 // Number of blocks used by the deterministic two-stage reductions for an
 // array of `n` elements; partial buffers need this many doubles.
 int reduce_blocks(long long n);

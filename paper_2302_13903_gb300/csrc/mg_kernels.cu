@@ -56,6 +56,17 @@ int grid_for(long long work) {
   return (int)b;
 }
 
+// Threads per block of a level kernel with `work` items: 256, or 64 where blocks
+// of 256 would leave SMs, and with them FP64 units, without one (32^3: 32
+// blocks on 152 SMs).
+int threads_for(long long work) { return work < 256LL * sm_count() ? 64 : kThreads; }
+int blocks_for(long long work) {
+  const int t = threads_for(work);
+  long long b = (work + t - 1) / t;
+  if (b > sm_count() * 64LL) b = sm_count() * 64LL;
+  return b < 1 ? 1 : (int)b;
+}
+
 // ---------------------------------------------------------------------------
 // Level kernels for even sizes.  In FP64 an SM issues two operations per clock,
 // so what counts is the number of FP64 operations per cell and that no warp
@@ -124,6 +135,7 @@ struct Around {
 template <typename T, bool PER>
 __global__ void __launch_bounds__(kThreads) k_sor_patch(T* u, const T* f, Grid g, Bc bc, T cu, T cs,
                                                         T cf, int colour) {
+  dev::after_previous();
   const int hx = g.nx >> 1, hy = g.ny >> 1;
   const long long total = (long long)hx * hy * g.nz;
   const dev::Split sp(hx, hy);
@@ -148,6 +160,7 @@ template <typename T, bool PER, bool R32>
 __global__ void __launch_bounds__(kThreads) k_defect_norm(const T* u, const T* f, Grid g, Bc bc,
                                                           T inv_h2, double* partials, float* r32,
                                                           double scale) {
+  dev::after_previous();
   const int hx = g.nx >> 1, hy = g.ny >> 1;
   const long long total = (long long)hx * hy * g.nz;
   const dev::Split sp(hx, hy);
@@ -184,6 +197,7 @@ __global__ void __launch_bounds__(kThreads) k_defect_norm(const T* u, const T* f
 template <typename T, bool PER>
 __global__ void __launch_bounds__(kThreads) k_defect_restrict_block(const T* u, const T* f, T* fc,
                                                                     Grid g, Bc bc, T inv_h2) {
+  dev::after_previous();
   const Grid gc{g.nx / 2, g.ny / 2, g.nz / 2};
   const long long work = 2 * gc.cells();
   const dev::Split sp(gc.nx, gc.ny);
@@ -220,6 +234,7 @@ __global__ void __launch_bounds__(kThreads) k_defect_restrict_block(const T* u, 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_prolong_add(const T* uc, T* uf, Grid gf, Bc bc, int cz,
                                                           long long items) {
+  dev::after_previous();
   const Grid gc{gf.nx / 2, gf.ny / 2, gf.nz / 2};
   const dev::Split sp(gc.nx, gc.ny);
   const size_t plane = (size_t)gf.nx * gf.ny, planec = (size_t)gc.nx * gc.ny;
@@ -298,6 +313,7 @@ bool homogeneous_rule(const Bc& bc) {
 template <typename T>
 __global__ void k_defect(const T* __restrict__ u, const T* __restrict__ f, T* __restrict__ d,
                          Grid g, Bc bc, T inv_h2, double* __restrict__ partials) {
+  dev::after_previous();
   const long long total = g.cells();
   double acc = 0.0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
@@ -318,18 +334,21 @@ __global__ void k_defect(const T* __restrict__ u, const T* __restrict__ f, T* __
 
 template <typename T>
 __global__ void k_sor(T* u, const T* f, Grid g, Bc bc, T cu, T cs, T cf, int colour) {
+  dev::after_previous();
   dev::sor_range(u, f, g, bc, cu, cs, cf, colour, blockIdx.x * (long long)blockDim.x + threadIdx.x,
                  (long long)gridDim.x * blockDim.x);
 }
 
 template <typename T>
 __global__ void k_sor_red_zero(T* u, const T* f, Grid g, T cf) {
+  dev::after_previous();
   dev::sor_red_zero_range(u, f, g, cf, blockIdx.x * (long long)blockDim.x + threadIdx.x,
                           (long long)gridDim.x * blockDim.x);
 }
 
 template <typename T>
 __global__ void k_defect_restrict(const T* u, const T* f, T* fc, Grid g, Bc bc, T inv_h2) {
+  dev::after_previous();
   dev::defect_restrict_range(u, f, fc, g, bc, inv_h2,
                              blockIdx.x * (long long)blockDim.x + threadIdx.x,
                              (long long)gridDim.x * blockDim.x);
@@ -337,12 +356,14 @@ __global__ void k_defect_restrict(const T* u, const T* f, T* fc, Grid g, Bc bc, 
 
 template <typename T>
 __global__ void k_restrict(const T* uf, T* uc, Grid gf) {
+  dev::after_previous();
   dev::restrict_range(uf, uc, gf, blockIdx.x * (long long)blockDim.x + threadIdx.x,
                       (long long)gridDim.x * blockDim.x);
 }
 
 template <typename T, bool HIGH>
 __global__ void k_prolong(const T* uc, T* uf, Grid gf, Bc bc, int add, int cz, long long items) {
+  dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < items;
        t += (long long)gridDim.x * blockDim.x)
     dev::prolong_zchunk<T, HIGH>(uc, uf, gf, bc, add, t, cz);
@@ -350,17 +371,20 @@ __global__ void k_prolong(const T* uc, T* uf, Grid gf, Bc bc, int add, int cz, l
 
 template <typename T>
 __global__ void k_coarsest(const T* f, T* u, double h, Bc bc, bool keep) {
+  dev::after_previous();
   if (threadIdx.x == 0 && blockIdx.x == 0) dev::coarsest_one(f, u, h, bc, keep);
 }
 
 template <typename T>
 __global__ void k_fill(T* __restrict__ u, long long n, T v) {
+  dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     u[t] = v;
 }
 
 __global__ void k_add_const(double* __restrict__ u, long long n, double v) {
+  dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     u[t] += v;
@@ -370,6 +394,7 @@ __global__ void k_add_const(double* __restrict__ u, long long n, double v) {
 template <bool SQ>
 __global__ void k_source(const double* __restrict__ rho, double* __restrict__ f, long long n,
                          double four_pi_G, double* __restrict__ partials) {
+  dev::after_previous();
   double acc = 0.0;
 #pragma unroll 4
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
@@ -385,6 +410,7 @@ __global__ void k_source(const double* __restrict__ rho, double* __restrict__ f,
 template <typename T>
 __global__ void k_sum(const T* __restrict__ a, long long n, int squares,
                       double* __restrict__ partials) {
+  dev::after_previous();
   double acc = 0.0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
@@ -396,6 +422,7 @@ __global__ void k_sum(const T* __restrict__ a, long long n, int squares,
 }
 
 __global__ void k_finish_sum(const double* __restrict__ partials, int nb, double* __restrict__ out) {
+  dev::after_previous();
   double acc = 0.0;
   for (int t = threadIdx.x; t < nb; t += blockDim.x) acc += partials[t];
   const double b = block_sum(acc);
@@ -407,6 +434,7 @@ __global__ void k_finish_sum(const double* __restrict__ partials, int nb, double
 template <bool SQ>
 __global__ void k_subtract_mean(double* __restrict__ a, long long n, const double* __restrict__ total,
                                 double* __restrict__ partials) {
+  dev::after_previous();
   const double mean = total[0] / (double)n;
   double acc = 0.0;
 #pragma unroll 4
@@ -427,6 +455,7 @@ __global__ void k_subtract_mean(double* __restrict__ a, long long n, const doubl
 __global__ void k_outer_residual(const double* __restrict__ u, const double* __restrict__ f,
                                  float* __restrict__ r32, Grid g, Bc bc, double inv_h2,
                                  double scale, double* __restrict__ partials) {
+  dev::after_previous();
   const long long total = g.cells();
   double acc = 0.0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
@@ -445,6 +474,7 @@ __global__ void k_outer_residual(const double* __restrict__ u, const double* __r
 
 __global__ void k_scale_to_f32(const double* __restrict__ a, float* __restrict__ b, long long n,
                                double scale) {
+  dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     b[t] = (float)(scale * a[t]);
@@ -452,6 +482,7 @@ __global__ void k_scale_to_f32(const double* __restrict__ a, float* __restrict__
 
 __global__ void k_correct(double* __restrict__ u, const float* __restrict__ e, long long n,
                           double inv_scale) {
+  dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     u[t] += inv_scale * (double)e[t];
@@ -461,6 +492,7 @@ __global__ void k_correct(double* __restrict__ u, const float* __restrict__ e, l
 // Laplacian with the level's own rule) and the start value u = ur.
 __global__ void k_fas_rhs(const double* __restrict__ ur, double* __restrict__ f,
                           double* __restrict__ u, Grid g, Bc bc, double inv_h2) {
+  dev::after_previous();
   const long long total = g.cells();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -475,6 +507,7 @@ __global__ void k_fas_rhs(const double* __restrict__ ur, double* __restrict__ f,
 
 // Algorithm 3 step 7: u -= ur (the coarse-grid correction).
 __global__ void k_sub(double* __restrict__ u, const double* __restrict__ ur, long long n) {
+  dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     u[t] -= ur[t];
@@ -485,6 +518,7 @@ __global__ void k_sub(double* __restrict__ u, const double* __restrict__ ur, lon
 // neighbours outside the level from the rule; g = [g_x | g_y | g_z].
 __global__ void k_gravity(const double* __restrict__ u, double* __restrict__ g, Grid gr, Bc bc,
                           double h) {
+  dev::after_previous();
   const long long total = gr.cells();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -539,11 +573,11 @@ cudaError_t launch_sor(T* u, const T* f, Grid g, double h, Bc bc, double omega, 
   ++g_launches;
   if (g.nx % 2 == 0 && g.ny % 2 == 0) {
     if (bc.kind == BC_PERIODIC)
-      k_sor_patch<T, true><<<grid_for(work / 2), kThreads, 0, s>>>(u, f, g, bc, cu, cs, cf, colour);
+      launch_after(k_sor_patch<T, true>, blocks_for(work / 2), threads_for(work / 2), 0, s, u, f, g, bc, cu, cs, cf, colour);
     else
-      k_sor_patch<T, false><<<grid_for(work / 2), kThreads, 0, s>>>(u, f, g, bc, cu, cs, cf, colour);
+      launch_after(k_sor_patch<T, false>, blocks_for(work / 2), threads_for(work / 2), 0, s, u, f, g, bc, cu, cs, cf, colour);
   } else {
-    k_sor<T><<<grid_for(work), kThreads, 0, s>>>(u, f, g, bc, cu, cs, cf, colour);
+    launch_after(k_sor<T>, grid_for(work), kThreads, 0, s, u, f, g, bc, cu, cs, cf, colour);
   }
   return cudaGetLastError();
 }
@@ -552,7 +586,7 @@ template <typename T>
 cudaError_t launch_sor_red_zero(T* u, const T* f, Grid g, double h, double omega,
                                 cudaStream_t s) {
   ++g_launches;
-  k_sor_red_zero<T><<<grid_for(g.cells()), kThreads, 0, s>>>(u, f, g, (T)(-omega * h * h / 6.0));
+  launch_after(k_sor_red_zero<T>, blocks_for(g.cells()), threads_for(g.cells()), 0, s, u, f, g, (T)(-omega * h * h / 6.0));
   return cudaGetLastError();
 }
 
@@ -564,12 +598,12 @@ cudaError_t launch_defect(const T* u, const T* f, T* d, Grid g, double h, Bc bc,
   if (partials && !d && g.nx % 2 == 0 && g.ny % 2 == 0) {
     const T ih2 = (T)(1.0 / (h * h));
     if (bc.kind == BC_PERIODIC)
-      k_defect_norm<T, true, false><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials, nullptr, 0.0);
+      launch_after(k_defect_norm<T, true, false>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials, nullptr, 0.0);
     else
-      k_defect_norm<T, false, false><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials, nullptr, 0.0);
+      launch_after(k_defect_norm<T, false, false>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials, nullptr, 0.0);
     return cudaGetLastError();
   }
-  k_defect<T><<<nb, kThreads, 0, s>>>(u, f, d, g, bc, (T)(1.0 / (h * h)), partials);
+  launch_after(k_defect<T>, nb, kThreads, 0, s, u, f, d, g, bc, (T)(1.0 / (h * h)), partials);
   return cudaGetLastError();
 }
 
@@ -579,20 +613,18 @@ cudaError_t launch_defect_restrict(const T* u, const T* f, T* fc, Grid g, double
   ++g_launches;
   const T ih2 = (T)(1.0 / (h * h));
   if (!even_sizes(g))
-    k_defect_restrict<T><<<grid_for(g.cells() / 8), kThreads, 0, s>>>(u, f, fc, g, bc, ih2);
+    launch_after(k_defect_restrict<T>, grid_for(g.cells() / 8), kThreads, 0, s, u, f, fc, g, bc, ih2);
   else if (bc.kind == BC_PERIODIC)
-    k_defect_restrict_block<T, true><<<grid_for(g.cells() / 4), kThreads, 0, s>>>(u, f, fc, g, bc,
-                                                                                  ih2);
+    launch_after(k_defect_restrict_block<T, true>, blocks_for(g.cells() / 4), threads_for(g.cells() / 4), 0, s, u, f, fc, g, bc, ih2);
   else
-    k_defect_restrict_block<T, false><<<grid_for(g.cells() / 4), kThreads, 0, s>>>(u, f, fc, g, bc,
-                                                                                   ih2);
+    launch_after(k_defect_restrict_block<T, false>, blocks_for(g.cells() / 4), threads_for(g.cells() / 4), 0, s, u, f, fc, g, bc, ih2);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_restrict(const T* uf, T* uc, Grid gf, cudaStream_t s) {
   ++g_launches;
-  k_restrict<T><<<grid_for(gf.cells() / 8), kThreads, 0, s>>>(uf, uc, gf);
+  launch_after(k_restrict<T>, grid_for(gf.cells() / 8), kThreads, 0, s, uf, uc, gf);
   return cudaGetLastError();
 }
 
@@ -608,77 +640,77 @@ cudaError_t launch_prolong(const T* uc, T* uf, Grid gf, Bc bc_coarse, int high_o
   while (cz > 1 && cols * ((cnz + cz - 1) / cz) < (1LL << 16)) cz /= 2;
   const long long items = cols * ((cnz + cz - 1) / cz);
   if (!high_order && add && homogeneous_rule(bc_coarse))
-    k_prolong_add<T><<<grid_for(items), kThreads, 0, s>>>(uc, uf, gf, bc_coarse, cz, items);
+    launch_after(k_prolong_add<T>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf, bc_coarse, cz, items);
   else if (high_order)
-    k_prolong<T, true><<<grid_for(items), kThreads, 0, s>>>(uc, uf, gf, bc_coarse, add, cz, items);
+    launch_after(k_prolong<T, true>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf, bc_coarse, add, cz, items);
   else
-    k_prolong<T, false><<<grid_for(items), kThreads, 0, s>>>(uc, uf, gf, bc_coarse, add, cz, items);
+    launch_after(k_prolong<T, false>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf, bc_coarse, add, cz, items);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_coarsest(const T* f, T* u, double h, Bc bc, cudaStream_t s, bool keep) {
   ++g_launches;
-  k_coarsest<T><<<1, 32, 0, s>>>(f, u, h, bc, keep);
+  launch_after(k_coarsest<T>, 1, 32, 0, s, f, u, h, bc, keep);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_fill(T* u, long long n, T v, cudaStream_t s) {
   ++g_launches;
-  k_fill<T><<<grid_for(n), kThreads, 0, s>>>(u, n, v);
+  launch_after(k_fill<T>, grid_for(n), kThreads, 0, s, u, n, v);
   return cudaGetLastError();
 }
 
 cudaError_t launch_source(const double* rho, double* f, long long n, double four_pi_G, bool squares,
                           double* partials, cudaStream_t s) {
   ++g_launches;
-  if (squares) k_source<true><<<reduce_blocks(n), kThreads, 0, s>>>(rho, f, n, four_pi_G, partials);
-  else k_source<false><<<reduce_blocks(n), kThreads, 0, s>>>(rho, f, n, four_pi_G, partials);
+  if (squares) launch_after(k_source<true>, reduce_blocks(n), kThreads, 0, s, rho, f, n, four_pi_G, partials);
+  else launch_after(k_source<false>, reduce_blocks(n), kThreads, 0, s, rho, f, n, four_pi_G, partials);
   return cudaGetLastError();
 }
 
 cudaError_t launch_subtract_mean(double* a, long long n, double* partials, int nb,
                                  double* total_slot, bool squares, cudaStream_t s) {
   ++g_launches;
-  k_finish_sum<<<1, kThreads, 0, s>>>(partials, nb, total_slot);
+  launch_after(k_finish_sum, 1, kThreads, 0, s, partials, nb, total_slot);
   ++g_launches;
   if (squares)
-    k_subtract_mean<true><<<reduce_blocks(n), kThreads, 0, s>>>(a, n, total_slot, partials);
+    launch_after(k_subtract_mean<true>, reduce_blocks(n), kThreads, 0, s, a, n, total_slot, partials);
   else
-    k_subtract_mean<false><<<grid_for(n), kThreads, 0, s>>>(a, n, total_slot, nullptr);
+    launch_after(k_subtract_mean<false>, grid_for(n), kThreads, 0, s, a, n, total_slot, nullptr);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_sum(const T* a, long long n, int squares, double* partials, cudaStream_t s) {
   ++g_launches;
-  k_sum<T><<<reduce_blocks(n), kThreads, 0, s>>>(a, n, squares, partials);
+  launch_after(k_sum<T>, reduce_blocks(n), kThreads, 0, s, a, n, squares, partials);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fas_rhs(const double* ur, double* f, double* u, Grid g, double h, Bc bc,
                            cudaStream_t s) {
   ++g_launches;
-  k_fas_rhs<<<grid_for(g.cells()), kThreads, 0, s>>>(ur, f, u, g, bc, 1.0 / (h * h));
+  launch_after(k_fas_rhs, grid_for(g.cells()), kThreads, 0, s, ur, f, u, g, bc, 1.0 / (h * h));
   return cudaGetLastError();
 }
 
 cudaError_t launch_sub(double* u, const double* ur, long long n, cudaStream_t s) {
   ++g_launches;
-  k_sub<<<grid_for(n), kThreads, 0, s>>>(u, ur, n);
+  launch_after(k_sub, grid_for(n), kThreads, 0, s, u, ur, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gravity(const double* u, double* g, Grid gr, double h, Bc bc, cudaStream_t s) {
   ++g_launches;
-  k_gravity<<<grid_for(gr.cells()), kThreads, 0, s>>>(u, g, gr, bc, h);
+  launch_after(k_gravity, grid_for(gr.cells()), kThreads, 0, s, u, g, gr, bc, h);
   return cudaGetLastError();
 }
 
 cudaError_t launch_finish_sum(const double* partials, int nb, double* out, cudaStream_t s) {
   ++g_launches;
-  k_finish_sum<<<1, kThreads, 0, s>>>(partials, nb, out);
+  launch_after(k_finish_sum, 1, kThreads, 0, s, partials, nb, out);
   return cudaGetLastError();
 }
 
@@ -689,34 +721,32 @@ cudaError_t launch_outer_residual(const double* u, const double* f, float* r32, 
   const double ih2 = 1.0 / (h * h);
   if (g.nx % 2 == 0 && g.ny % 2 == 0) {
     if (bc.kind == BC_PERIODIC)
-      k_defect_norm<double, true, true><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials, r32,
-                                                                scale);
+      launch_after(k_defect_norm<double, true, true>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials, r32, scale);
     else
-      k_defect_norm<double, false, true><<<nb, kThreads, 0, s>>>(u, f, g, bc, ih2, partials, r32,
-                                                                 scale);
+      launch_after(k_defect_norm<double, false, true>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials, r32, scale);
   } else {
-    k_outer_residual<<<nb, kThreads, 0, s>>>(u, f, r32, g, bc, ih2, scale, partials);
+    launch_after(k_outer_residual, nb, kThreads, 0, s, u, f, r32, g, bc, ih2, scale, partials);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_add_const(double* u, long long n, double v, cudaStream_t s) {
   ++g_launches;
-  k_add_const<<<grid_for(n), kThreads, 0, s>>>(u, n, v);
+  launch_after(k_add_const, grid_for(n), kThreads, 0, s, u, n, v);
   return cudaGetLastError();
 }
 
 cudaError_t launch_scale_to_f32(const double* a, float* b, long long n, double scale,
                                cudaStream_t s) {
   ++g_launches;
-  k_scale_to_f32<<<grid_for(n), kThreads, 0, s>>>(a, b, n, scale);
+  launch_after(k_scale_to_f32, grid_for(n), kThreads, 0, s, a, b, n, scale);
   return cudaGetLastError();
 }
 
 cudaError_t launch_correct(double* u, const float* e32, long long n, double inv_scale,
                            cudaStream_t s) {
   ++g_launches;
-  k_correct<<<grid_for(n), kThreads, 0, s>>>(u, e32, n, inv_scale);
+  launch_after(k_correct, grid_for(n), kThreads, 0, s, u, e32, n, inv_scale);
   return cudaGetLastError();
 }
 
