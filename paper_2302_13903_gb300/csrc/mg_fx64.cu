@@ -3,7 +3,7 @@
 // An SM issues two FP64 operations per clock, so a V(1,1) cycle's 25-30 FP64
 // operations per cell take several times as long as its bytes.  Here phi and
 // h^2 f of the finest level are 64-bit integers scaled by 2^S with |phi| <
-// 2^55: a quantum of at most 2^-54 max|phi|, against the 2^-53 of a double.
+// 2^54: a quantum of at most 2^-53 max|phi|, the spacing of doubles there.
 // With U and F those integers,
 //   R = (sum of the six neighbours of U) - 6 U - F       (exactly)
 //   SMOOTH: U += round(R omega / 6)                      (Eqs. rbsor1-rbsor2)
@@ -12,6 +12,11 @@
 // once.  omega / 6 is a 64-bit fraction.  A face's value b enters the ghost 2 b - u as a
 // constant and is folded into F (F - round(2 b 2^S)) when F is formed, so the
 // sweeps run the homogeneous rule.
+//
+// The levels below, down to 64^3, hold the correction on the same grid with two
+// guard bits (2^(S+2)): with h_c = 2 h their right-hand side is F_c = -(sum of
+// R) / 2 in quanta of their own, so no scale has to be found, and a correction
+// is known to a quarter of a quantum of the phi it is added to.
 //
 // Two z-marching kernels, like the FP32 legs: down = one SMOOTH and the
 // restricted defect, up = the prolonged correction and one SMOOTH.  A CTA
@@ -55,10 +60,13 @@ struct Fx64Args {
   int cz;        // planes per CTA (even)
   Weight w;
   double* norm;  // per-CTA sum of R^2: red cells of u_in (down), black cells of u_out (up)
-  double* fc;           // down: coarse right-hand side, -sum of R
+  double* fc;           // down: coarse right-hand side, -sum of R, as doubles,
+  long long* fci;       //   or on the coarse level's integer grid (fc null)
+  int shift;            // down: -sum of R 2^shift is F there; up: ec has `shift` guard bits
   long long* psum;      // down: per-CTA exact sum of u_in, (hi, lo) pairs
   const long long* ec;  // up: coarse correction on the integer grid
-  int* flag;            // |U| passed 2^59
+  int limit;            // log2 of the largest |U|
+  int* flag;            // |U| or |F| of the coarse level passed its limit
 };
 
 // round(R w), halves up, for w = (hi + lo / 2^32) / 2^32 < 1/3 and |R| < 2^63:
@@ -182,9 +190,9 @@ struct Squares {
   __device__ __forceinline__ double total() const { return ((double)s + (double)c) * 0x1p24; }
 };
 
-// |v| at or past 2^59, by the high word.
-__device__ __forceinline__ bool too_large(long long v) {
-  return (unsigned)((int)(v >> 32) + (1 << 27)) >= (2u << 27);
+// |v| at or past 2^32 m, by the high word.
+__device__ __forceinline__ bool too_large(long long v, int m) {
+  return (unsigned)((int)(v >> 32) + m) >= 2u * m;
 }
 
 // Block sum of doubles and of (hi, lo) integers into one partial per CTA.
@@ -244,7 +252,8 @@ __device__ __forceinline__ int plane_of(int q, int nz, bool pz) {
 // cell); [C] red defects of q - 3.  The march is unrolled by four, so that ring
 // slots and the registers of the four planes in hand are fixed: plane q is in
 // slot J, planes q - 1, q - 2, q - 3 in J - 1, J - 2, J - 3 (mod 4).
-template <bool WALLS, int TX>
+// COARSE: a correction level, from u = 0 and without the norm and the sum.
+template <bool WALLS, int TX, bool COARSE>
 __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     k_fx64_down(const __grid_constant__ Fx64Args a) {
   dev::after_previous();
@@ -280,16 +289,17 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     const int k = q <= z1 + 2 ? plane_of(q, nz, pz) : -1;
     if (k >= 0 && (!WALLS || p.valid)) {
       const size_t o = (size_t)k * plane + col;
-      cp16(&ring.u[s][t], a.u_in + o);
+      if (!COARSE) cp16(&ring.u[s][t], a.u_in + o);
       cp16(&ring.f[s][t], a.F + o);
     }
-    if (k >= 0 && frame_in)  // odd slots hold even planes
+    if (!COARSE && k >= 0 && frame_in)  // odd slots hold even planes
       cp8(&ring.frame[s][t], a.u_in + (size_t)k * plane + fcol + (s & 1 ? 0 : fstep));
     cp_commit();
   };
   long long uP[4] = {}, uQ[4] = {}, fP[4] = {}, fQ[4] = {};
   long long ud = 0, acc = 0, done = 0, psum = 0;
   const Weight w = WALLS ? p.w : a.w;
+  const int most = 1 << (a.limit - 32);
   Squares norm;
   bool bad = false;
   using std::integral_constant;
@@ -310,26 +320,38 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     issue(integral_constant<int, J + 3>{}, q + 3);
     cp_wait<3>();
     if (!WALLS || p.valid) {
-      const longlong2 v = ring.u[J][t], f = ring.f[J][t];
+      const longlong2 v = COARSE ? make_longlong2(0, 0) : ring.u[J][t], f = ring.f[J][t];
       uP[J] = p.swap ? v.y : v.x;
       uQ[J] = p.swap ? v.x : v.y;
       fP[J] = p.swap ? f.y : f.x;
       fQ[J] = p.swap ? f.x : f.y;
     }
-    raw[I0] = uB[J];
-    if (framed) frame[I0] = frame_in ? ring.frame[J][t] : 0;
-    if (p.tile && q >= z0 && q < z1) psum += uP[J] + uQ[J];
+    if (!COARSE) {
+      raw[I0] = uB[J];
+      if (framed) frame[I0] = frame_in ? ring.frame[J][t] : 0;
+      if (p.tile && q >= z0 && q < z1) psum += uP[J] + uQ[J];
+    }
     // the block whose last plane was q - 4: its even and odd row's sums
-    if (!EVEN && q - 5 >= z0 && q - 5 < z1 && even_row)
-      a.fc[(size_t)((q - 5) >> 1) * (plane >> 2) + colc] = cvt::ll2d_rn(-(done + odd[W::PW]));
+    if (!EVEN && q - 5 >= z0 && q - 5 < z1 && even_row) {
+      const long long sum = -(done + odd[W::PW]);
+      const size_t o = (size_t)((q - 5) >> 1) * (plane >> 2) + colc;
+      if (a.fci) {
+        const long long f = a.shift >= 0 ? sum << a.shift : (sum + 1) >> 1;
+        a.fci[o] = f;
+        bad |= too_large(f, 1 << 27) || too_large(sum, 1 << 26);
+      } else {
+        a.fc[o] = cvt::ll2d_rn(sum);
+      }
+    }
     const int ka = q - 1, kb = q - 2, kc = q - 3;
     {  // [A]: red of plane q - 1 is in the columns uB
       long long zl = uB[B], zh = uB[J];
       int n = nb;
       if (WALLS && wzl && ka == 0) zl = 0, n -= wzl;
       if (WALLS && wzh && ka == nz - 1) zh = 0, n -= wzh;
-      const long long R = residual<W::PW>(raw + I1, uB[A], uR[A], xb, zl, zh, n, fB[A]);
-      if (p.tile && ka >= z0 && ka < z1) norm.add(R);
+      const long long R =
+          COARSE ? -fB[A] : residual<W::PW>(raw + I1, uB[A], uR[A], xb, zl, zh, n, fB[A]);
+      if (!COARSE && p.tile && ka >= z0 && ka < z1) norm.add(R);
       uB[A] += weigh(R, w);
       red[I1] = uB[A];
     }
@@ -345,7 +367,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
       rb = R - n * d;
       blk[I0] = uB[B];
       if (p.tile && kb >= z0 && kb < z1) {
-        bad |= too_large(uP[B]) || too_large(uQ[B]);
+        bad |= too_large(uP[B], most) || too_large(uQ[B], most);
         *reinterpret_cast<longlong2*>(a.u_out + (size_t)kb * plane + col) =
             p.swap ? make_longlong2(uQ[B], uP[B]) : make_longlong2(uP[B], uQ[B]);
       }
@@ -376,7 +398,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
   }
   cp_wait<0>();
   if (bad) atomicOr(a.flag, 1);
-  block_sums<W::NT>(norm.total(), psum, true, a.norm, a.psum);
+  if (!COARSE) block_sums<W::NT>(norm.total(), psum, true, a.norm, a.psum);
 }
 
 // ---------------------------------------------------------------------------
@@ -385,7 +407,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
 // q - 2, then final and written.  The correction of a pair is interpolated
 // along y, then x, then z with weights 3 and 1 on the integer grid and rounded
 // once by the division by 64.  Unrolled by four as the down leg.
-template <bool WALLS, int TX>
+template <bool WALLS, int TX, bool COARSE>
 __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
     k_fx64_up(const __grid_constant__ Fx64Args a) {
   dev::after_previous();
@@ -469,6 +491,9 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
   long long em0, em1, e00, e01;  // coarse planes K - 1 and K
   long long uP[4] = {}, uQ[4] = {}, fP[4] = {}, fQ[4] = {};
   const Weight w = WALLS ? p.w : a.w;
+  const int most = 1 << (a.limit - 32);
+  const int bits = 6 + a.shift;
+  const long long half = 1LL << (bits - 1);
   Squares norm;
   bool bad = false;
   using std::integral_constant;
@@ -507,7 +532,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
     }
     if (!WALLS || p.valid) {
       const longlong2 v = ring.u[J][t], f = ring.f[J][t];
-      const long long v0 = v.x + ((d0 + 32) >> 6), v1 = v.y + ((d1 + 32) >> 6);
+      const long long v0 = v.x + ((d0 + half) >> bits), v1 = v.y + ((d1 + half) >> bits);
       uP[J] = p.swap ? v1 : v0;
       uQ[J] = p.swap ? v0 : v1;
       fP[J] = p.swap ? f.y : f.x;
@@ -533,8 +558,8 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
       const long long d = weigh(R, w);
       uB[B] += d;
       if (p.tile && kb >= z0 && kb < z1) {
-        norm.add(R - n * d);
-        bad |= too_large(uP[B]) || too_large(uQ[B]);
+        if (!COARSE) norm.add(R - n * d);
+        bad |= too_large(uP[B], most) || too_large(uQ[B], most);
         *reinterpret_cast<longlong2*>(a.u_out + (size_t)kb * plane + col) =
             p.swap ? make_longlong2(uQ[B], uP[B]) : make_longlong2(uP[B], uQ[B]);
       }
@@ -549,7 +574,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
   }
   cp_wait<0>();
   if (bad) atomicOr(a.flag, 1);
-  block_sums<W::NT>(norm.total(), 0, false, a.norm, nullptr);
+  if (!COARSE) block_sums<W::NT>(norm.total(), 0, false, a.norm, nullptr);
 }
 
 template <int TX>
@@ -588,13 +613,13 @@ __global__ void k_fx64_source(double* f, Grid g, Bc bc, double c, double c2) {
   }
 }
 
-// out[0] = sum of a[0 .. n) + sum of b[0 .. nb), in a fixed order.
-__global__ void k_fx64_norm(const double* a, int n, const double* b, int nb, double* out) {
+// out[0] = sum of a[0 .. n) + sum of b[0 .. n), in a fixed order; out[1] = *flag.
+__global__ void k_fx64_norm(const double* a, const double* b, int n, const int* flag, double* out) {
   dev::after_previous();
   __shared__ double ws[8];
   double s = 0.0;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) s += a[t];
-  for (int t = threadIdx.x; t < nb; t += blockDim.x) s += b[t];
+#pragma unroll 4
+  for (int t = threadIdx.x; t < n; t += 256) s += a[t] + b[t];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
   __syncthreads();
@@ -602,6 +627,7 @@ __global__ void k_fx64_norm(const double* a, int n, const double* b, int nb, dou
     double r = 0.0;
     for (int w = 0; w < 8; ++w) r += ws[w];
     out[0] = r;
+    out[1] = (double)*flag;
   }
 }
 
@@ -611,28 +637,30 @@ Weight weight_of(double omega) {
   return Weight{(int)hi, lo >= 2147483647.0 ? 2147483647 : (int)lo};
 }
 
-template <int TX>
-cudaError_t launch(const Fx64Args& a, bool down, cudaStream_t s) {
-  static std::atomic<int> configured[64];
+template <typename K>
+cudaError_t launch_leg(K* kernel, std::atomic<int>* configured, size_t smem, int threads, int tx,
+                       const Fx64Args& a, cudaStream_t s) {
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !configured[dev].load()) {
-    const cudaFuncAttribute most = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(k_fx64_down<false, TX>, most, (int)down_smem<TX>());
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_fx64_down<true, TX>, most, (int)down_smem<TX>());
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fx64_up<false, TX>, most, (int)up_smem<TX>());
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fx64_up<true, TX>, most, (int)up_smem<TX>());
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev].store(1);
   }
-  const dim3 grid(a.g.nx / TX, a.g.ny / TY, (a.g.nz + a.cz - 1) / a.cz);
+  const dim3 grid(a.g.nx / tx, a.g.ny / TY, (a.g.nz + a.cz - 1) / a.cz);
   ++g_launches;
-  if (down && a.fk) launch_after(k_fx64_down<true, TX>, grid, Down<TX>::NT, down_smem<TX>(), s, a);
-  else if (down) launch_after(k_fx64_down<false, TX>, grid, Down<TX>::NT, down_smem<TX>(), s, a);
-  else if (a.fk) launch_after(k_fx64_up<true, TX>, grid, Up<TX>::NT, up_smem<TX>(), s, a);
-  else launch_after(k_fx64_up<false, TX>, grid, Up<TX>::NT, up_smem<TX>(), s, a);
-  return cudaGetLastError();
+  const cudaError_t e = launch_after(kernel, grid, threads, smem, s, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <bool WALLS, int TX, bool COARSE>
+cudaError_t launch(const Fx64Args& a, bool down, cudaStream_t s) {
+  static std::atomic<int> configured[2][64];
+  return down ? launch_leg(k_fx64_down<WALLS, TX, COARSE>, configured[0], down_smem<TX>(),
+                           Down<TX>::NT, TX, a, s)
+              : launch_leg(k_fx64_up<WALLS, TX, COARSE>, configured[1], up_smem<TX>(), Up<TX>::NT,
+                           TX, a, s);
 }
 
 // Tile width: 64 cells, one CTA per SM, or on levels that would leave SMs
@@ -678,39 +706,31 @@ static int face_kinds_of(const Bc& hom) {
   return fk;
 }
 
-cudaError_t launch_fx64_down(const long long* u_in, long long* u_out, const long long* F, double* fc,
-                             Grid g, const Bc& hom, double omega, double* norm, long long* psum,
-                             int* flag, cudaStream_t s) {
+cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s) {
   Fx64Args a{};
-  a.u_in = u_in;
-  a.u_out = u_out;
-  a.F = F;
-  a.g = g;
-  a.fk = face_kinds_of(hom);
-  a.cz = fx64_cz(g);
-  a.w = weight_of(omega);
-  a.norm = norm;
-  a.fc = fc;
-  a.psum = psum;
-  a.flag = flag;
-  return tile_width(g) == 64 ? launch<64>(a, true, s) : launch<32>(a, true, s);
-}
-
-cudaError_t launch_fx64_up(const long long* u_in, long long* u_out, const long long* F,
-                           const long long* ec, Grid g, const Bc& hom, double omega, double* norm,
-                           int* flag, cudaStream_t s) {
-  Fx64Args a{};
-  a.u_in = u_in;
-  a.u_out = u_out;
-  a.F = F;
-  a.g = g;
-  a.fk = face_kinds_of(hom);
-  a.cz = fx64_cz(g);
-  a.w = weight_of(omega);
-  a.norm = norm;
-  a.ec = ec;
-  a.flag = flag;
-  return tile_width(g) == 64 ? launch<64>(a, false, s) : launch<32>(a, false, s);
+  a.u_in = q.u_in;
+  a.u_out = q.u_out;
+  a.F = q.F;
+  a.g = q.g;
+  a.fk = face_kinds_of(q.hom);
+  a.cz = fx64_cz(q.g);
+  a.w = weight_of(q.omega);
+  a.norm = q.norm;
+  a.fc = q.fc;
+  a.fci = q.fci;
+  a.shift = q.shift;
+  a.psum = q.psum;
+  a.ec = q.ec;
+  // with |ec| < 2^56 and its sums of weight 64 below 2^62
+  a.limit = q.coarse ? 56 : 59;
+  a.flag = q.flag;
+  const bool wide = tile_width(q.g) == 64;
+  if (q.coarse) {
+    if (a.fk) return wide ? launch<true, 64, true>(a, down, s) : launch<true, 32, true>(a, down, s);
+    return wide ? launch<false, 64, true>(a, down, s) : launch<false, 32, true>(a, down, s);
+  }
+  if (a.fk) return wide ? launch<true, 64, false>(a, down, s) : launch<true, 32, false>(a, down, s);
+  return wide ? launch<false, 64, false>(a, down, s) : launch<false, 32, false>(a, down, s);
 }
 
 cudaError_t launch_fx64_source(double* f, Grid g, const Bc& bc, double c, double two_pow_S,
@@ -722,10 +742,10 @@ cudaError_t launch_fx64_source(double* f, Grid g, const Bc& bc, double c, double
   return cudaGetLastError();
 }
 
-cudaError_t launch_fx64_norm(const double* red, const double* black, int nb, double* out,
-                             cudaStream_t s) {
+cudaError_t launch_fx64_norm(const double* red, const double* black, int nb, const int* flag,
+                             double* out, cudaStream_t s) {
   ++g_launches;
-  launch_after(k_fx64_norm, 1, 256, 0, s, red, nb, black, nb, out);
+  launch_after(k_fx64_norm, 1, 256, 0, s, red, black, nb, flag, out);
   return cudaGetLastError();
 }
 

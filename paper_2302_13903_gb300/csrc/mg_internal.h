@@ -69,6 +69,12 @@ mg_status solve_host_copies(mg_ctx* c, const double* rho, double four_pi_G, doub
                             double* phi, double* hist, int hist_cap, int* n_hist,
                             cudaStream_t s, double* copy_ms = nullptr);
 
+// Device bytes the first mg_solve of a context of this shape adds to what
+// mg_create allocated (mg_required_bytes): the FP64 path's integer buffers.
+size_t solve_buffer_bytes(int nx, int ny, int nz, const mg_opts& opts);
+// Solves of this context do without them (in FP64 throughout).
+void no_solve_buffers(mg_ctx* c);
+
 // Record the message mg_last_error(NULL) returns on this thread (entry points
 // that have no context report their failures through it).
 void set_last_error(const std::string& msg);
@@ -338,23 +344,38 @@ cudaError_t launch_finish_fx_sum(const long long* psum, int nb, long long n, dou
 bool fx64_ok(Grid g);
 int fx64_cz(Grid g);
 int fx64_blocks(Grid g);
-// u_out = SMOOTH(u_in); fc = the restricted defect times 8 h^2 2^S; norm = sums
-// of (h^2 2^S defect)^2 over the red cells of u_in; psum = sums of u_in.
-cudaError_t launch_fx64_down(const long long* u_in, long long* u_out, const long long* F, double* fc,
-                             Grid g, const Bc& hom, double omega, double* norm, long long* psum,
-                             int* flag, cudaStream_t s);
-// u_out = SMOOTH(u_in + trilinear(ec)); norm = the same over the black cells of
-// u_out.  *flag |= 1 where |u_out| passes 2^59.
-cudaError_t launch_fx64_up(const long long* u_in, long long* u_out, const long long* F,
-                           const long long* ec, Grid g, const Bc& hom, double omega, double* norm,
-                           int* flag, cudaStream_t s);
+// down: u_out = SMOOTH(u_in); fc = the restricted defect times 8 h^2 2^S, or
+// fci = that divided by 8 times 2^(3 + shift), F of an integer coarse level;
+// norm = sums of (h^2 2^S defect)^2 over the red cells of u_in; psum = sums of
+// u_in.  up: u_out = SMOOTH(u_in + trilinear(ec) 2^-shift); norm = the same
+// over the black cells of u_out.  coarse: a correction level, down from u_in =
+// 0, no norms and sums.  *flag |= 1 where |u_out| passes 2^59 (coarse 2^56) or
+// fci its range.
+constexpr int kFx64Guard = 2;  // guard bits of the integer correction levels
+struct Fx64Leg {
+  const long long* u_in;
+  long long* u_out;
+  const long long* F;
+  Grid g;
+  Bc hom;
+  double omega;
+  bool coarse;
+  int shift;
+  double* fc;
+  long long* fci;
+  const long long* ec;
+  double* norm;
+  long long* psum;
+  int* flag;
+};
+cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s);
 // In place: f becomes round(f c) less round(2 b 2^S) for each of the cell's
 // fixed and open faces (rule bc).
 cudaError_t launch_fx64_source(double* f, Grid g, const Bc& bc, double c, double two_pow_S,
                                cudaStream_t s);
-// out[0] = sum of both arrays of nb partial sums.
-cudaError_t launch_fx64_norm(const double* red, const double* black, int nb, double* out,
-                             cudaStream_t s);
+// out[0] = sum of both arrays of nb partial sums, out[1] = *flag.
+cudaError_t launch_fx64_norm(const double* red, const double* black, int nb, const int* flag,
+                             double* out, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Multipole boundary (App. A).

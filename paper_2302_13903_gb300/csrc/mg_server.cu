@@ -56,6 +56,7 @@ struct Request {
   mg_request req{};
   Key key;
   size_t need = 0;
+  bool plain = false;  // solve without the FP64 path's integer buffers
   Clock::time_point t_submit, t_start, t_done;
   bool done = false;
   int waiters = 0;       // threads in mg_server_wait on this ticket
@@ -168,6 +169,7 @@ mg_status create_hier(mg_server* S, const Request* r, cudaStream_t stream, Hier*
                            r->req.face_value, &o, &h->ctx);
     else
       st = mg_create(r->req.nx, r->req.ny, r->req.nz, r->req.dx, r->req.bc, &o, &h->ctx);
+    if (st == MG_OK && r->plain) mg::no_solve_buffers(h->ctx);
     if (st == MG_OK) mg_ctx_autotune(h->ctx, stream);  // shapes, cached per process
   }
   if (st != MG_OK) {
@@ -432,6 +434,11 @@ mg_status mg_server_submit(mg_server* S, const mg_request* q, long long* ticket)
   if (q->per_face) need += 4 * sizeof(double) * 6 * (size_t)(q->nx + 2) * (q->nx + 2) / 3;
   Request* r = new Request;
   r->req = *q;
+  // the FP64 path's integer buffers count in the budget too; where they do not
+  // fit it beside the hierarchy, its solves do without them
+  const size_t extra = mg::solve_buffer_bytes(q->nx, q->ny, q->nz, o);
+  r->plain = need + extra > S->pool.budget();
+  if (!r->plain) need += extra;
   r->key.n = q->nx;
   r->key.bc = q->per_face ? (int)MG_BC_MIXED : (int)q->bc;
   r->key.lmax = !q->per_face && q->bc == MG_BC_OPEN ? q->lmax : 0;

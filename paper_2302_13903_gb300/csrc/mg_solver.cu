@@ -49,6 +49,8 @@ struct mg_ctx {
   double* f64[kMaxLevels] = {};
   double* faces[kMaxLevels] = {};  // open / fixed-face boundary values per level
   double* ur64[kMaxLevels] = {};   // FAS: restricted potential per coarse level
+  long long* ub64[kMaxLevels] = {};  // second buffer of the integer correction levels
+  bool fx64_tried = false;           // whether those buffers were asked for
   // FP32 hierarchy (mixed precision); u32b is the second buffer of levels the
   // fused kernels handle (they read one buffer and write the other).
   float* u32[kMaxLevels] = {};
@@ -204,6 +206,36 @@ int dense_level(const mg_ctx* c) {
   return c->opts.fas ? 0 : mg::coarse_dense_level(Ladder(c).g, c->L);
 }
 
+// Whether the FP64 path's upper levels may run in fixed point (mg_fx64.cu).
+bool fx64_wanted(const mg_ctx* c) {
+  const mg_opts& o = c->opts;
+  return o.prec == MG_FP64 && o.mode_fmg && !o.fas && !o.coarse_literal && o.pre == 1 &&
+         o.post == 1 && c->L >= 2 && mg::fx64_ok(level_grid(c, c->L - 1));
+}
+
+// The integer levels' second buffers (the first ones are phi's own storage and
+// the FP64 levels'), 9.1 bytes per finest cell: allocated by the first solve
+// that uses them and kept; where they do not fit, the solve runs in FP64.
+bool fx64_buffers(mg_ctx* c) {
+  if (c->fxbuf) return true;
+  if (c->fx64_tried || !fx64_wanted(c)) return false;
+  c->fx64_tried = true;
+  const size_t had = c->allocs.size(), bytes = c->bytes;
+  try {
+    for (int l = c->L - 2; l > 0 && mg::fx64_ok(level_grid(c, l)); --l)
+      c->ub64[l] = dalloc<long long>(c, level_grid(c, l).cells());
+    c->fxbuf = dalloc<long long>(c, level_grid(c, c->L - 1).cells());
+  } catch (const Fail&) {
+    for (; c->allocs.size() > had; c->allocs.pop_back()) cudaFree(c->allocs.back());
+    c->bytes = bytes;
+    for (long long*& p : c->ub64) p = nullptr;
+    c->fxbuf = nullptr;
+    c->err.clear();
+    return false;
+  }
+  return true;
+}
+
 // The device arrays of a context (counted only, when c->dry).
 void alloc_hierarchy(mg_ctx* c) {
   const mg_bc bc = (mg_bc)c->bc_kind;
@@ -235,17 +267,14 @@ void alloc_hierarchy(mg_ctx* c) {
     const int nb = mg::fx_step_blocks(level_grid(c, F), 0);
     if (nb > c->partials_cap) c->partials_cap = nb;
   }
-  // the FP64 path's finest level in fixed point: a second integer buffer (phi
-  // itself is the first) and one more array of partial sums
-  const bool fx64 = o.prec == MG_FP64 && o.mode_fmg && !o.fas && !o.coarse_literal && o.pre == 1 &&
-                    o.post == 1 && L >= 2 && mg::fx64_ok(level_grid(c, F));
-  if (fx64) c->fxbuf = dalloc<long long>(c, level_grid(c, F).cells());
+  const bool fx64 = fx64_wanted(c);
   // partials, then room for two integers per block of the fixed-point step
   c->partials = dalloc<double>(c, (fx64 ? 4 : 3) * (size_t)c->partials_cap);
-  c->scal = dalloc<double>(c, 64);
-  c->iflag = dalloc<int>(c, 4);
-  if (dense_level(c) > 0)
-    c->dense = dalloc<char>(c, (size_t)mg::kDense * mg::kDense * (o.prec == MG_FP64 ? 8 : 4));
+  // scalars, then the flags, then the dense matrix
+  const size_t dense = dense_level(c) > 0 ? (size_t)mg::kDense * mg::kDense : 0;
+  c->scal = dalloc<double>(c, 66 + dense);
+  c->iflag = reinterpret_cast<int*>(c->scal + 64);
+  c->dense = dense ? c->scal + 66 : nullptr;
 }
 
 Bc physical_bc(const mg_ctx* c, int l) {
@@ -396,7 +425,6 @@ void make_dense(mg_ctx* c, const Bc& hom) {
                                  mg::COARSE_BASIS, nullptr},
                                 nullptr),
         "coarse matrix");
-  check(c, cudaStreamSynchronize(nullptr), "sync");
 }
 
 // COARSEST on level 0 (Sec. 2.3.2): one cell is solved exactly; a level of
@@ -827,17 +855,57 @@ Bc correction_bc(const mg_ctx* c, const Bc& top) {
   return z;
 }
 
-// The V-cycles of the FP64 path with the finest level in 64-bit fixed point
-// (mg_fx64.cu): phi holds the FMG start, prolonged to the finest level, and
-// f64[F] the source.  Returns -1 where the values are not finite or phi leaves
+// The FP64 levels below an integer level of spacing h: the V-cycle from f64[l]
+// (the defect restricted from the level above, times 8 h^2 and that level's
+// scale) and its correction on that level's integer grid.
+void fp64_correction(mg_ctx* c, int l, const Bc& hom, double h, cudaStream_t s) {
+  Pyr<double> P = pyr<double>(c);
+  if (l == 0) coarsest_solve<double>(c, P.u[0], P.f[0], hom, false, s);
+  else vcycle<double>(c, P, l, hom, hom, true, s);
+  check(c, mg::launch_f64_to_fx(c->u64[l], level_grid(c, l).cells(), 1.0 / (8.0 * h * h), s),
+        "correction -> fixed point");
+}
+
+// The correction of level l < F of the integer FP64 path from F in f64[l] into
+// u64[l] (both as integers with kFx64Guard guard bits): the levels with a
+// second buffer as integers, the ones below in FP64.
+void fx64_correction(mg_ctx* c, int l, const Bc& hom, cudaStream_t s) {
+  const Grid g = level_grid(c, l);
+  const double h = level_h(c, l);
+  auto q = [](double* p) { return reinterpret_cast<long long*>(p); };
+  mg::Fx64Leg leg{};
+  leg.F = q(c->f64[l]);
+  leg.g = g;
+  leg.hom = hom;
+  leg.omega = c->opts.omega;
+  leg.coarse = true;
+  leg.flag = c->iflag;
+  leg.u_out = c->ub64[l];
+  leg.shift = -1;
+  const bool below = c->ub64[l - 1] != nullptr;
+  leg.fc = below ? nullptr : c->f64[l - 1];
+  leg.fci = below ? q(c->f64[l - 1]) : nullptr;
+  check(c, mg::launch_fx64(leg, true, s), "down leg");
+  if (below) fx64_correction(c, l - 1, hom, s);
+  else fp64_correction(c, l - 1, hom, h, s);
+  leg.u_in = c->ub64[l];
+  leg.u_out = q(c->u64[l]);
+  leg.ec = q(c->u64[l - 1]);
+  leg.shift = 0;
+  check(c, mg::launch_fx64(leg, false, s), "up leg");
+}
+
+// The V-cycles of the FP64 path with the levels from 64^3 up in 64-bit fixed
+// point (mg_fx64.cu): phi holds the FMG start, prolonged to the finest level,
+// and f64[F] the source.  Returns -1 where the values are not finite or leave
 // the integers' range (then phi and f are to be formed again), else the status.
 int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, const Bc& bc,
                const Bc& hom, double* hist, int hist_cap, int* n_hist, cudaStream_t s) {
   const int F = c->L - 1;
   const Grid g = level_grid(c, F);
   const long long N = g.cells();
-  const double h = c->h, om = c->opts.omega;
-  // 2^S: |phi| < 2^55 (four bits of room before 2^59) and |h^2 f| < 2^58
+  const double h = c->h;
+  // 2^S: |phi| < 2^54 (five bits of room before 2^59) and |h^2 f| < 2^55
   check(c, mg::launch_absmax<double>(phi, N, c->partials, c->scal + 50, s), "max |phi|");
   check(c, mg::launch_absmax<double>(c->f64[F], N, c->partials, c->scal + 51, s), "max |f|");
   if (bc.kind == mg::BC_OPEN || bc.kind == mg::BC_MIXED)
@@ -859,39 +927,44 @@ int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, c
   int ep = 0, ef = 0;
   std::frexp(mphi, &ep);  // mphi < 2^ep
   std::frexp(mfh, &ef);
-  const int S = std::min(55 - ep, 58 - ef);
+  const int S = std::min(54 - ep, 55 - ef);
   if (S < -900 || S > 900) return -1;
   const double two_S = std::ldexp(1.0, S);
   long long *cur = reinterpret_cast<long long*>(phi), *alt = c->fxbuf;
-  const long long* FX = reinterpret_cast<const long long*>(c->f64[F]);
-  long long* ec = reinterpret_cast<long long*>(c->u64[F - 1]);
   double *red = c->partials, *black = c->partials + 3 * (size_t)c->partials_cap;
-  long long* psum = reinterpret_cast<long long*>(c->partials + c->partials_cap);
   const int nb = mg::fx64_blocks(g);
   check(c, mg::launch_f64_to_fx(phi, N, two_S, s), "phi -> fixed point");
   check(c, mg::launch_fx64_source(c->f64[F], g, bc, h * h * two_S, two_S, s),
         "h^2 f -> fixed point");
-  Pyr<double> P = pyr<double>(c);
-  const Grid gc = level_grid(c, F - 1);
+  const bool below = c->ub64[F - 1] != nullptr;
+  mg::Fx64Leg leg{};
+  leg.F = reinterpret_cast<const long long*>(c->f64[F]);
+  leg.g = g;
+  leg.hom = hom;
+  leg.omega = c->opts.omega;
+  leg.fc = below ? nullptr : c->f64[F - 1];
+  leg.fci = below ? reinterpret_cast<long long*>(c->f64[F - 1]) : nullptr;
+  leg.ec = reinterpret_cast<const long long*>(c->u64[F - 1]);
+  leg.psum = reinterpret_cast<long long*>(c->partials + c->partials_cap);
+  leg.flag = c->iflag;
   StopRule rule{tol, c->opts.stall_ratio};
   int n = 0, st = -1;
   for (int cyc = -1;; ++cyc) {  // cycle -1 ends the FMG ladder
     {
       KTimer t(c, MG_K_FUSED_DOWN, true, s);
-      check(c, mg::launch_fx64_down(cur, alt, FX, c->f64[F - 1], g, hom, om, red, psum, c->iflag, s),
-            "down leg");
+      leg.u_in = cur;
+      leg.u_out = alt;
+      leg.norm = red;
+      leg.shift = mg::kFx64Guard - 1;
+      check(c, mg::launch_fx64(leg, true, s), "down leg");
     }
     if (cyc >= 0) {  // the norm of the last cycle's phi (the leg above ran ahead of the test)
-      check(c, mg::launch_fx64_norm(red, black, nb, c->scal + 1, s), "norm");
-      check(c, cudaMemcpyAsync(c->pinned + 1, c->scal + 1, sizeof(double), cudaMemcpyDeviceToHost,
-                               s),
-            "read norm");
-      check(c, cudaMemcpyAsync(c->pinned + 60, c->iflag, sizeof(int), cudaMemcpyDeviceToHost, s),
-            "read flag");
+      check(c, mg::launch_fx64_norm(red, black, nb, c->iflag, c->scal + 1, s), "norm");
+      check(c, cudaMemcpyAsync(c->pinned + 1, c->scal + 1, 2 * sizeof(double),
+                               cudaMemcpyDeviceToHost, s),
+            "read norm and flag");
       check(c, cudaStreamSynchronize(s), "sync");
-      int flag = 0;
-      std::memcpy(&flag, c->pinned + 60, sizeof(int));
-      if (flag) return -1;
+      if (c->pinned[2] != 0.0) return -1;
       const double dn = std::sqrt(c->pinned[1] / (double)N) / (h * h * two_S);
       if (n == 0 && fnorm == 0.0) fnorm = dn > 0.0 ? dn : 1.0;
       const double r = dn / fnorm;
@@ -900,20 +973,20 @@ int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, c
       st = rule.decide(r, cyc, c->opts.max_cycles, n, hist_cap);
       if (st >= 0) break;
     }
-    // the correction of the scaled defect, then on phi's integer grid
-    if (F - 1 == 0) coarsest_solve<double>(c, P.u[0], P.f[0], hom, false, s);
-    else if (F - 1 > coarse_top<double>(c))
-      replay(c, c->inner[2], true, s,
-             [&]() { vcycle<double>(c, P, F - 1, hom, hom, true, s); });
-    else vcycle<double>(c, P, F - 1, hom, hom, true, s);
-    check(c, mg::launch_f64_to_fx(c->u64[F - 1], gc.cells(), 1.0 / (8.0 * h * h), s),
-          "correction -> fixed point");
+    replay(c, c->inner[1], true, s, [&]() {
+      if (below) fx64_correction(c, F - 1, hom, s);
+      else fp64_correction(c, F - 1, hom, h, s);
+    });
     KTimer t(c, MG_K_FUSED_UP, true, s);
-    check(c, mg::launch_fx64_up(alt, cur, FX, ec, g, hom, om, black, c->iflag, s), "up leg");
+    leg.u_in = alt;
+    leg.u_out = cur;
+    leg.norm = black;
+    leg.shift = below ? mg::kFx64Guard : 0;
+    check(c, mg::launch_fx64(leg, false, s), "up leg");
   }
   const long long* mean = nullptr;
   if (mean_free(c)) {
-    check(c, mg::launch_finish_fx_sum(psum, nb, N, c->scal + 56, s), "finish sum phi");
+    check(c, mg::launch_finish_fx_sum(leg.psum, nb, N, c->scal + 56, s), "finish sum phi");
     mean = reinterpret_cast<const long long*>(c->scal + 57);
   }
   if (gacc) {
@@ -947,7 +1020,7 @@ mg_status solve_fp64(mg_ctx* c, const double* rho, double four_pi_G, double tol,
   const bool fas = c->opts.fas != 0;
   if (c->opts.mode_fmg) {
     if (fas) fmg_fas(c, bcs, hom, s);
-    else if (c->fxbuf && ((uintptr_t)phi & 15u) == 0) {
+    else if (((uintptr_t)phi & 15u) == 0 && fx64_buffers(c)) {
       fmg_below<double>(c, P, bcs, hom, s);
       const int st =
           solve_fx64(c, fnorm, tol, phi, gacc, bcs[F], hom, hist, hist_cap, n_hist, s);
@@ -1661,6 +1734,25 @@ void autotune(mg_ctx* c, cudaStream_t s) {
 
 }  // namespace
 
+size_t mg::solve_buffer_bytes(int nx, int ny, int nz, const mg_opts& o) {
+  if (!dims_ok(nx, ny, nz)) return 0;
+  mg_ctx c;
+  c.n = nx;
+  c.ny = ny;
+  c.nz = nz;
+  c.opts = o;
+  const int m = std::min(nx, std::min(ny, nz));
+  c.L = 1;
+  while ((m >> (c.L - 1)) > 1) ++c.L;
+  if (c.L > kMaxLevels || !fx64_wanted(&c)) return 0;
+  size_t cells = 0;
+  for (int l = c.L - 1; l > 0 && mg::fx64_ok(level_grid(&c, l)); --l)
+    cells += (size_t)level_grid(&c, l).cells();
+  return cells * sizeof(long long);
+}
+
+void mg::no_solve_buffers(mg_ctx* c) { c->fx64_tried = true; }
+
 extern "C" {
 
 void mg_opts_init(mg_opts* o) {
@@ -1824,6 +1916,7 @@ mg_status create_ctx(int nx, int ny, int nz, double dx, mg_bc bc, int face_mask,
       else make_dense<float>(c, hom);
     }
     check(c, cudaMallocHost(&c->pinned, 64 * sizeof(double)), "cudaMallocHost");
+    check(c, cudaStreamSynchronize(nullptr), "sync");
   } catch (const Fail& f) {
     mg_destroy(c);
     return f.st;

@@ -50,7 +50,8 @@ def gpu(rho, rule, tol=0.0, phi=None, **kw):
 
 
 @pytest.mark.parametrize("rule", sorted(RULES))
-@pytest.mark.parametrize("dims", [(64, 16, 16), (64, 64, 64), (128, 32, 16), (128, 128, 64)])
+@pytest.mark.parametrize("dims", [(64, 16, 16), (64, 64, 64), (128, 32, 16), (128, 128, 64),
+                                  (256, 64, 64)])
 def test_same_schedule(dims, rule):
     rho = source(dims, sum(dims))
     bc, kw = oracle_args(rule)
