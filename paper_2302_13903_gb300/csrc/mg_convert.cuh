@@ -44,6 +44,22 @@ __device__ __forceinline__ long long d2ll_rn(double x) {
   return neg ? (long long)(0 - a) : (long long)a;
 }
 
+// binary64 x times 2^S -> int64 (the exponent raised by S, no FP64 operation);
+// saturates as d2ll_rn, NaN gives 0.
+__device__ __forceinline__ long long d2ll_pow2_rn(double x, int S) {
+  const uint64_t u = (uint64_t)__double_as_longlong(x);
+  const int e = (int)((u >> 52) & 0x7ff);
+  const uint64_t frac = u & 0xFFFFFFFFFFFFFULL;
+  const bool neg = (u >> 63) != 0;
+  if (e == 0x7ff && frac) return 0;
+  if (e == 0) return 0;  // |x| < 2^-1022
+  const int k = e - 1075 + S;
+  if (e == 0x7ff || k >= 11) return neg ? (long long)0x8000000000000000ULL : 0x7fffffffffffffffLL;
+  const uint64_t m = frac | (1ULL << 52);
+  const uint64_t a = k >= 0 ? (m << k) : shr_rne(m, -k);
+  return neg ? (long long)(0 - a) : (long long)a;
+}
+
 // int64 -> binary64.
 __device__ __forceinline__ double ll2d_rn(long long v) {
   if (v == 0) return 0.0;

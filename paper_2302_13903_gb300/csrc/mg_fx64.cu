@@ -588,28 +588,124 @@ constexpr size_t up_smem() {
   return sizeof(Ring<W::NT, 1>) + 4 * (size_t)W::PLANE * sizeof(long long);
 }
 
-// In place: f becomes F = round(f c) - sum over the cell's fixed and open
-// faces of round(2 b 2^S) (c2 = 2^(S+1)).
-__global__ void k_fx64_source(double* f, Grid g, Bc bc, double c, double c2) {
+// F = round(a rho - b) less round(2 b_face 2^S) for each of the cell's fixed and
+// open faces (c2 = 2^(S+1)), b = c *mu; per-block sums of F^2 without the
+// faces' part (the norm of f).
+__global__ void __launch_bounds__(256) k_fx64_source(const double* __restrict__ rho,
+                                                     long long* __restrict__ F, Grid g, Bc bc,
+                                                     double a, double c, const double* mu, double c2,
+                                                     double* __restrict__ partials) {
   dev::after_previous();
-  long long* q = reinterpret_cast<long long*>(f);
   const dev::Split sp(g.nx, g.ny);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < g.cells();
-       t += (long long)gridDim.x * blockDim.x) {
-    int i, j, k;
-    sp(t, i, j, k);
-    long long v = cvt::d2ll_rn(f[t] * c);
-    if (i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1) {
-      for (int s = 0; s < 6; ++s) {
-        const int kind = face_kind(bc, s);
-        if (kind != BC_FIXED && kind != BC_OPEN) continue;
-        const int x = s < 2 ? i : s < 4 ? j : k, n = s < 2 ? g.nx : s < 4 ? g.ny : g.nz;
-        if (x != ((s & 1) ? n - 1 : 0)) continue;
-        v -= __double2ll_rn(dev::face_value(bc, g, s, (s < 2 ? j : i) + 1, (s < 4 ? k : j) + 1) *
-                            c2);
+  const double b = c * mu[0];
+  const bool faces = bc.kind != BC_PERIODIC && bc.kind != BC_ZEROGRAD;
+  Squares sum;
+#pragma unroll 4
+  for (long long t = blockIdx.x * 256LL + threadIdx.x; t < g.cells(); t += gridDim.x * 256LL) {
+    long long v = cvt::d2ll_rn(fma(a, rho[t], -b));
+    sum.add(v);
+    if (faces) {
+      int i, j, k;
+      sp(t, i, j, k);
+      if (i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1) {
+        for (int s = 0; s < 6; ++s) {
+          const int kind = face_kind(bc, s);
+          if (kind != BC_FIXED && kind != BC_OPEN) continue;
+          const int x = s < 2 ? i : s < 4 ? j : k, n = s < 2 ? g.nx : s < 4 ? g.ny : g.nz;
+          if (x != ((s & 1) ? n - 1 : 0)) continue;
+          v -= __double2ll_rn(
+              dev::face_value(bc, g, s, (s < 2 ? j : i) + 1, (s < 4 ? k : j) + 1) * c2);
+        }
       }
     }
-    q[t] = v;
+    F[t] = v;
+  }
+  __shared__ double ws[8];
+  double d = sum.total();
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = d;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) d += ws[w];
+    partials[blockIdx.x] = d;
+  }
+}
+
+// fc = 4 pi G (mean of rho over the eight children) - *mu: the source of the
+// next level, straight from rho (one FP64 operation per cell).
+__global__ void __launch_bounds__(256) k_fx64_restrict(const double* __restrict__ rho,
+                                                       double* __restrict__ fc, Grid g, double c,
+                                                       const double* mu) {
+  dev::after_previous();
+  const Grid gc{g.nx / 2, g.ny / 2, g.nz / 2};
+  const dev::Split sp(gc.nx, gc.ny);
+  const double m = mu[0];
+  const size_t sy = g.nx, sz = (size_t)g.nx * g.ny;
+  for (long long t = blockIdx.x * 256LL + threadIdx.x; t < gc.cells(); t += gridDim.x * 256LL) {
+    int I, J, K;
+    sp(t, I, J, K);
+    const double* p = rho + dev::at(g, 2 * I, 2 * J, 2 * K);
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double* x = p + (q & 1) * sy + (q >> 1) * sz;
+      v[q] = x[0] + x[1];
+    }
+    fc[t] = fma(0.125 * c, (v[0] + v[1]) + (v[2] + v[3]), -m);
+  }
+}
+
+// phi = I' u (Sec. 2.3.1) on the integer grid, from the coarse level's doubles:
+// weights 5, 30, -3 over 32 along x, y, z, rounded after each axis.  A thread
+// marches up a chunk of cz coarse planes of one coarse column.
+__global__ void __launch_bounds__(256) k_fx64_prolong(const double* uc, long long* __restrict__ out,
+                                                      Grid g, Bc bc, int S, int cz,
+                                                      long long items) {
+  dev::after_previous();
+  const Grid gc{g.nx / 2, g.ny / 2, g.nz / 2};
+  const dev::Split sp(gc.nx, gc.ny);
+  const size_t plane = (size_t)g.nx * g.ny;
+  auto pair = [](long long a, long long b, long long c, long long& even, long long& odd) {
+    const long long t = 30 * b + (a + c) + 16, d = 4 * (a - c);
+    even = (t + d) >> 5;
+    odd = (t - d) >> 5;
+  };
+  for (long long t = blockIdx.x * 256LL + threadIdx.x; t < items; t += gridDim.x * 256LL) {
+    int I, J, ch;
+    sp(t, I, J, ch);
+    auto xy = [&](int K, long long o[2][2]) {
+      long long v[3][2];
+#pragma unroll
+      for (int y = 0; y < 3; ++y) {
+        long long e[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+          e[x] = cvt::d2ll_pow2_rn(dev::fetch(uc, I + x - 1, J + y - 1, K, gc, bc), S);
+        pair(e[0], e[1], e[2], v[y][0], v[y][1]);
+      }
+#pragma unroll
+      for (int x = 0; x < 2; ++x) pair(v[0][x], v[1][x], v[2][x], o[0][x], o[1][x]);
+    };
+    const int K0 = ch * cz, K1 = min(K0 + cz, gc.nz);
+    long long pm[2][2], p0[2][2], pp[2][2];
+    xy(K0 - 1, pm);
+    xy(K0, p0);
+    for (int K = K0; K < K1; ++K) {
+      xy(K + 1, pp);
+#pragma unroll
+      for (int y = 0; y < 2; ++y) {
+        long long lo[2], hi[2];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          pair(pm[y][x], p0[y][x], pp[y][x], lo[x], hi[x]);
+          pm[y][x] = p0[y][x];
+          p0[y][x] = pp[y][x];
+        }
+        const size_t q = dev::at(g, 2 * I, 2 * J + y, 2 * K);
+        *reinterpret_cast<longlong2*>(out + q) = make_longlong2(lo[0], lo[1]);
+        *reinterpret_cast<longlong2*>(out + q + plane) = make_longlong2(hi[0], hi[1]);
+      }
+    }
   }
 }
 
@@ -733,12 +829,35 @@ cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s) {
   return wide ? launch<false, 64, false>(a, down, s) : launch<false, 32, false>(a, down, s);
 }
 
-cudaError_t launch_fx64_source(double* f, Grid g, const Bc& bc, double c, double two_pow_S,
-                               cudaStream_t s) {
-  long long b = (g.cells() + 255) / 256;
-  if (b > sm_count() * 64LL) b = sm_count() * 64LL;
+cudaError_t launch_fx64_source(const double* rho, long long* F, Grid g, const Bc& bc,
+                               double four_pi_G, const double* mu, double c, double two_pow_S,
+                               double* partials, cudaStream_t s) {
   ++g_launches;
-  launch_after(k_fx64_source, (int)b, 256, 0, s, f, g, bc, c, 2.0 * two_pow_S);
+  launch_after(k_fx64_source, reduce_blocks(g.cells()), 256, 0, s, rho, F, g, bc, four_pi_G * c, c,
+               mu, 2.0 * two_pow_S, partials);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fx64_restrict(const double* rho, double* fc, Grid g, double four_pi_G,
+                                 const double* mu, cudaStream_t s) {
+  const long long b = (g.cells() / 8 + 255) / 256;
+  ++g_launches;
+  launch_after(k_fx64_restrict, (int)(b < 64LL * sm_count() ? b : 64LL * sm_count()), 256, 0, s, rho,
+               fc, g, four_pi_G, mu);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fx64_prolong(const double* uc, long long* phi, Grid g, const Bc& bc, int S,
+                                cudaStream_t s) {
+  // chunks of 8 coarse planes while that leaves four blocks per SM
+  const long long cols = (long long)(g.nx / 2) * (g.ny / 2);
+  const int nzc = g.nz / 2;
+  int cz = 8;
+  while (cz > 1 && cols * ((nzc + cz - 1) / cz) < 1024LL * sm_count()) cz /= 2;
+  const long long items = cols * ((nzc + cz - 1) / cz), b = (items + 255) / 256;
+  ++g_launches;
+  launch_after(k_fx64_prolong, (int)(b < 64LL * sm_count() ? b : 64LL * sm_count()), 256, 0, s, uc,
+               phi, g, bc, S, cz, items);
   return cudaGetLastError();
 }
 

@@ -155,7 +155,8 @@ cudaError_t launch_subtract_mean(double* a, long long n, double* partials, int n
 // Partial sums of a[i] (FP64) and of a[i]^2.
 template <typename T>
 cudaError_t launch_sum(const T* a, long long n, int squares, double* partials, cudaStream_t s);
-// out[0] = sum(partials[0..nb)) in a fixed order.
+// out[0] = sum(partials[0..nb)) in a fixed order (out may be page-locked host
+// memory).
 cudaError_t launch_finish_sum(const double* partials, int nb, double* out, cudaStream_t s);
 // FAS (Algorithm 3): f += L ur and u = ur (step 5); u -= ur (step 7).
 cudaError_t launch_fas_rhs(const double* ur, double* f, double* u, Grid g, double h, Bc bc,
@@ -369,10 +370,18 @@ struct Fx64Leg {
   int* flag;
 };
 cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s);
-// In place: f becomes round(f c) less round(2 b 2^S) for each of the cell's
-// fixed and open faces (rule bc).
-cudaError_t launch_fx64_source(double* f, Grid g, const Bc& bc, double c, double two_pow_S,
-                               cudaStream_t s);
+// F = round((4 pi G rho - *mu) c) less round(2 b 2^S) for each of the cell's
+// fixed and open faces (rule bc); reduce_blocks partial sums of F^2 without
+// the faces' part.
+cudaError_t launch_fx64_source(const double* rho, long long* F, Grid g, const Bc& bc,
+                               double four_pi_G, const double* mu, double c, double two_pow_S,
+                               double* partials, cudaStream_t s);
+// fc = restriction of 4 pi G rho - *mu.
+cudaError_t launch_fx64_restrict(const double* rho, double* fc, Grid g, double four_pi_G,
+                                 const double* mu, cudaStream_t s);
+// phi = round(I' uc 2^S), coarse ghosts from rule bc.
+cudaError_t launch_fx64_prolong(const double* uc, long long* phi, Grid g, const Bc& bc, int S,
+                                cudaStream_t s);
 // out[0] = sum of both arrays of nb partial sums, out[1] = *flag.
 cudaError_t launch_fx64_norm(const double* red, const double* black, int nb, const int* flag,
                              double* out, cudaStream_t s);

@@ -424,7 +424,8 @@ __global__ void k_sum(const T* __restrict__ a, long long n, int squares,
 __global__ void k_finish_sum(const double* __restrict__ partials, int nb, double* __restrict__ out) {
   dev::after_previous();
   double acc = 0.0;
-  for (int t = threadIdx.x; t < nb; t += blockDim.x) acc += partials[t];
+#pragma unroll 8
+  for (int t = threadIdx.x; t < nb; t += kThreads) acc += partials[t];
   const double b = block_sum(acc);
   if (threadIdx.x == 0) out[0] = b;
 }

@@ -93,7 +93,8 @@ struct mg_ctx {
   // Two graphs: [0] for 1 + inner_cycles V-cycles, [1] for the first outer
   // iteration's first_cycles when they differ.
   // FP64: [2] the V-cycle below the finest level and [3] the FMG ladder below
-  // it, which touch the context's own arrays only.
+  // it, [1] and [0] the same where the finest level is in fixed point; they
+  // touch the context's own arrays only.
   struct InnerGraph {
     cudaGraphExec_t exec = nullptr;
     long long launches = 0;  // kernels in the graph
@@ -103,6 +104,7 @@ struct mg_ctx {
   // captured, and the event that orders it after that stream
   cudaStream_t own_stream = nullptr;
   cudaEvent_t own_event = nullptr;
+  cudaEvent_t ready = nullptr;  // mg_create's device work, until the first solve has waited for it
   // the autotuner timed the finest level's fused up-down pass faster than the
   // two legs it replaces (opts.leg_pairs = 0 then fuses them)
   bool pairs_faster = false;
@@ -672,20 +674,24 @@ void vcycle(mg_ctx* c, Pyr<T> P, int l, const Bc& bc_top, const Bc& hom, bool ze
   smooth_steps<T>(c, P, l, bc_top, c->opts.post, false, s);                            // 7
 }
 
-// Algorithm 2 with rule bcs[l] on every level, up to the prolongation to the
-// finest level F.  Returns false where the ladder's start is level F itself,
-// which is then done.
+// u_l = I' u_{l-1}, the start of level l in Algorithm 2.
 template <typename T>
-bool fmg_below(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s) {
+void fmg_prolong(mg_ctx* c, Pyr<T> P, int l, const Bc* bcs, cudaStream_t s) {
+  KTimer t(c, MG_K_FMG_PROLONG, l == c->L - 1, s);
+  check(c, mg::launch_prolong<T>(P.u[l - 1], P.u[l], level_grid(c, l), bcs[l - 1], 1, 0, s),
+        "fmg_prolong");
+}
+
+// Algorithm 2 with rule bcs[l] on the levels below the finest level F, from f
+// of level F, or of F - 1 when `restricted`.  Returns false where the ladder's
+// start is level F itself, which is then done.
+template <typename T>
+bool fmg_below(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, bool restricted,
+               cudaStream_t s) {
   const Ladder d(c);
   const int F = c->L - 1, lb = mg::coarse_fmg_top<T>(d.g, c->L);
-  auto prolong = [&](int l) {
-    KTimer t(c, MG_K_FMG_PROLONG, l == F, s);
-    check(c, mg::launch_prolong<T>(P.u[l - 1], P.u[l], level_grid(c, l), bcs[l - 1], 1, 0, s),
-          "fmg_prolong");
-  };
   auto below = [&]() {
-    for (int l = F; l > lb; --l)
+    for (int l = restricted ? F - 1 : F; l > lb; --l)
       check(c, mg::launch_restrict<T>(P.f[l], P.f[l - 1], level_grid(c, l), s), "restrict");
     if (lb > 0)  // levels 0 .. lb
       check(c, mg::launch_coarse<T>({P.u[lb], P.f[lb], d.g, d.h, bcs, hom, c->opts.omega,
@@ -696,21 +702,24 @@ bool fmg_below(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s
     else
       coarsest_solve<T>(c, P.u[0], P.f[0], bcs[0], false, s);
     for (int l = lb + 1; l < F; ++l) {
-      prolong(l);
+      fmg_prolong<T>(c, P, l, bcs, s);
       vcycle<T>(c, P, l, bcs[l], hom, false, s);
     }
   };
-  if (std::is_same<T, double>::value && lb < F) replay(c, c->inner[3], true, s, below);
-  else below();
-  if (lb >= F) return false;
-  prolong(F);
-  return true;
+  if (std::is_same<T, double>::value && lb < F)
+    replay(c, c->inner[restricted ? 0 : 3], true, s, below);
+  else
+    below();
+  return lb < F;
 }
 
 // Algorithm 2 with rule bcs[l] on every level.
 template <typename T>
 void fmg(mg_ctx* c, Pyr<T> P, const Bc* bcs, const Bc& hom, cudaStream_t s) {
-  if (fmg_below<T>(c, P, bcs, hom, s)) vcycle<T>(c, P, c->L - 1, bcs[c->L - 1], hom, false, s);
+  const int F = c->L - 1;
+  if (!fmg_below<T>(c, P, bcs, hom, false, s)) return;
+  fmg_prolong<T>(c, P, F, bcs, s);
+  vcycle<T>(c, P, F, bcs[F], hom, false, s);
 }
 
 // Algorithm 3 on level l >= 1 (FP64 path): every level solves the original
@@ -760,13 +769,12 @@ void fmg_fas(mg_ctx* c, const Bc* bcs, const Bc& hom, cudaStream_t s) {
   }
 }
 
-// Fixed-order sums of squares -> host.
-double read_scalar(mg_ctx* c, int slot, cudaStream_t s) {
-  check(c, cudaMemcpyAsync(c->pinned + slot, c->scal + slot, sizeof(double),
-                           cudaMemcpyDeviceToHost, s),
-        "read norm");
+// The sum of nb partial sums, in a fixed order, written to page-locked host
+// memory by the kernel that forms it (a copy behind it costs 3-4 us).
+double read_sum(mg_ctx* c, int nb, cudaStream_t s) {
+  check(c, mg::launch_finish_sum(c->partials, nb, c->pinned, s), "finish sum");
   check(c, cudaStreamSynchronize(s), "sync");
-  return c->pinned[slot];
+  return c->pinned[0];
 }
 
 struct StopRule {
@@ -787,6 +795,25 @@ struct StopRule {
   }
 };
 
+// The open rule's values at the face points of the finest level, or of all.
+void open_boundary(mg_ctx* c, const double* rho, double four_pi_G, bool all_levels_faces,
+                   cudaStream_t s) {
+  const int F = c->L - 1;
+  const Grid gf = level_grid(c, F);
+  if (c->bc_kind == MG_BC_OPEN) {
+    int nbm = 0;
+    check(c, mg::launch_raw_moments(rho, gf, c->h, c->partials, &nbm, s), "moments");
+    check(c, mg::launch_moments_finish(c->partials, nbm, c->h, c->opts.lmax, c->opts.use_com,
+                                       c->opts.origin, c->scal + 2, s),
+          "moments_finish");
+    const double G = four_pi_G / (4.0 * 3.14159265358979323846);
+    for (int l = all_levels_faces ? 0 : F; l <= F; ++l)
+      check(c, mg::launch_open_faces(level_grid(c, l), level_h(c, l), c->scal + 2, c->opts.lmax,
+                                     G, c->faces[l], s),
+            "open_faces");
+  }
+}
+
 // Source, mean removal, norm of f, and the open-boundary values.
 double prepare_source(mg_ctx* c, const double* rho, double four_pi_G, double* f_fin,
                       bool all_levels_faces, cudaStream_t s) {
@@ -801,20 +828,10 @@ double prepare_source(mg_ctx* c, const double* rho, double four_pi_G, double* f_
   if (mean_free(c))
     check(c, mg::launch_subtract_mean(f_fin, N, c->partials, nb, c->scal + 40, true, s),
           "subtract_mean");
-  check(c, mg::launch_finish_sum(c->partials, nb, c->scal + 0, s), "finish f^2");
-  if (c->bc_kind == MG_BC_OPEN) {
-    int nbm = 0;
-    check(c, mg::launch_raw_moments(rho, gf, c->h, c->partials, &nbm, s), "moments");
-    check(c, mg::launch_moments_finish(c->partials, nbm, c->h, c->opts.lmax, c->opts.use_com,
-                                       c->opts.origin, c->scal + 2, s),
-          "moments_finish");
-    const double G = four_pi_G / (4.0 * 3.14159265358979323846);
-    for (int l = all_levels_faces ? 0 : F; l <= F; ++l)
-      check(c, mg::launch_open_faces(level_grid(c, l), level_h(c, l), c->scal + 2, c->opts.lmax,
-                                     G, c->faces[l], s),
-            "open_faces");
-  }
-  return std::sqrt(read_scalar(c, 0, s) / (double)N);
+  check(c, mg::launch_finish_sum(c->partials, nb, c->pinned, s), "finish f^2");
+  open_boundary(c, rho, four_pi_G, all_levels_faces, s);
+  check(c, cudaStreamSynchronize(s), "sync");
+  return std::sqrt(c->pinned[0] / (double)N);
 }
 
 void remove_mean(mg_ctx* c, double* u, cudaStream_t s) {
@@ -835,8 +852,7 @@ double defect_rms(mg_ctx* c, const double* u, const double* f, const Bc& bc, cud
     check(c, mg::launch_defect<double>(u, f, nullptr, g, level_h(c, F), bc, c->partials, s),
           "defect norm");
   }
-  check(c, mg::launch_finish_sum(c->partials, nb, c->scal + 1, s), "finish d^2");
-  return std::sqrt(read_scalar(c, 1, s) / (double)g.cells());
+  return std::sqrt(read_sum(c, nb, s) / (double)g.cells());
 }
 
 // The rule of the coarse correction levels below a level with rule `top`:
@@ -895,34 +911,45 @@ void fx64_correction(mg_ctx* c, int l, const Bc& hom, cudaStream_t s) {
   check(c, mg::launch_fx64(leg, false, s), "up leg");
 }
 
-// The V-cycles of the FP64 path with the levels from 64^3 up in 64-bit fixed
-// point (mg_fx64.cu): phi holds the FMG start, prolonged to the finest level,
-// and f64[F] the source.  Returns -1 where the values are not finite or leave
-// the integers' range (then phi and f are to be formed again), else the status.
-int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, const Bc& bc,
-               const Bc& hom, double* hist, int hist_cap, int* n_hist, cudaStream_t s) {
+// The FP64 solve from an FMG start with the levels from 64^3 up in 64-bit fixed
+// point (mg_fx64.cu).  The finest level's source and start are never formed
+// as doubles.  Returns -1 where the values are not finite or leave the
+// integers' range (nothing but phi is lost then), else the status.
+int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, double* phi,
+               double* gacc, const Bc* bcs, const Bc& hom, double* hist, int hist_cap, int* n_hist,
+               cudaStream_t s) {
   const int F = c->L - 1;
-  const Grid g = level_grid(c, F);
+  const Grid g = level_grid(c, F), gc = level_grid(c, F - 1);
+  const Bc& bc = bcs[F];
   const long long N = g.cells();
   const double h = c->h;
-  // 2^S: |phi| < 2^54 (five bits of room before 2^59) and |h^2 f| < 2^55
-  check(c, mg::launch_absmax<double>(phi, N, c->partials, c->scal + 50, s), "max |phi|");
-  check(c, mg::launch_absmax<double>(c->f64[F], N, c->partials, c->scal + 51, s), "max |f|");
+  {
+    KTimer t(c, MG_K_SOURCE, true, s);
+    check(c, mg::launch_rho_stats(rho, N, c->partials, c->scal + 0, s), "source stats");
+  }
+  double* const mu = c->scal + 32;  // the mean of f, or 0
+  check(c, mg::launch_source_scale(c->scal + 0, N, four_pi_G, mean_free(c), mu, s), "source mean");
+  check(c, mg::launch_fx64_restrict(rho, c->f64[F - 1], g, four_pi_G, mu, s), "restrict");
+  open_boundary(c, rho, four_pi_G, true, s);
+  check(c, cudaMemsetAsync(c->scal + 50, 0, 2 * sizeof(double), s), "zero");
+  fmg_below<double>(c, pyr<double>(c), bcs, hom, true, s);
+  // 2^S: |phi| < 2^54 (five bits of room before 2^59) and |h^2 f| < 2^55; I'
+  // raises max |u| by (38 / 32)^3 < 2 at most
+  check(c, mg::launch_absmax<double>(c->u64[F - 1], gc.cells(), c->partials, c->scal + 50, s),
+        "max |phi|");
   if (bc.kind == mg::BC_OPEN || bc.kind == mg::BC_MIXED)
     check(c, mg::launch_absmax<double>(c->faces[F], (long long)mg::faces_count(g), c->partials,
-                                       c->scal + 52, s),
+                                       c->scal + 51, s),
           "max |b|");
   check(c, cudaMemsetAsync(c->iflag, 0, sizeof(int), s), "clear flag");
-  check(c, cudaMemcpyAsync(c->pinned + 50, c->scal + 50, 3 * sizeof(double),
-                           cudaMemcpyDeviceToHost, s),
-        "read max");
+  check(c, cudaMemcpyAsync(c->pinned, c->scal, 64 * sizeof(double), cudaMemcpyDeviceToHost, s),
+        "read scalars");
   check(c, cudaStreamSynchronize(s), "sync");
-  double mphi = c->pinned[50];
-  const double mfh = c->pinned[51] * h * h;
-  if (bc.kind == mg::BC_OPEN || bc.kind == mg::BC_MIXED) mphi = std::max(mphi, c->pinned[52]);
+  double mphi = std::max(2.0 * c->pinned[50], c->pinned[51]);
   if (bc.kind == mg::BC_FIXED) mphi = std::max(mphi, std::fabs(bc.value));
-  if (!std::isfinite(fnorm) || !std::isfinite(mphi) || !std::isfinite(mfh) || mphi <= 0.0 ||
-      mfh <= 0.0)
+  const double mfh = h * h * (std::fabs(four_pi_G) * c->pinned[1] + std::fabs(c->pinned[32]));
+  if (!std::isfinite(mphi) || !std::isfinite(mfh) || !std::isfinite(c->pinned[0]) ||
+      mphi <= 0.0 || mfh <= 0.0)
     return -1;
   int ep = 0, ef = 0;
   std::frexp(mphi, &ep);  // mphi < 2^ep
@@ -933,9 +960,15 @@ int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, c
   long long *cur = reinterpret_cast<long long*>(phi), *alt = c->fxbuf;
   double *red = c->partials, *black = c->partials + 3 * (size_t)c->partials_cap;
   const int nb = mg::fx64_blocks(g);
-  check(c, mg::launch_f64_to_fx(phi, N, two_S, s), "phi -> fixed point");
-  check(c, mg::launch_fx64_source(c->f64[F], g, bc, h * h * two_S, two_S, s),
+  check(c, mg::launch_fx64_source(rho, reinterpret_cast<long long*>(c->f64[F]), g, bc, four_pi_G, mu,
+                                  h * h * two_S, two_S, c->partials, s),
         "h^2 f -> fixed point");
+  check(c, mg::launch_finish_sum(c->partials, mg::reduce_blocks(N), c->pinned, s), "finish f^2");
+  {
+    KTimer t(c, MG_K_FMG_PROLONG, true, s);
+    check(c, mg::launch_fx64_prolong(c->u64[F - 1], cur, g, bcs[F - 1], S, s), "fmg_prolong");
+  }
+  double fnorm = -1.0;  // read with the first defect norm
   const bool below = c->ub64[F - 1] != nullptr;
   mg::Fx64Leg leg{};
   leg.F = reinterpret_cast<const long long*>(c->f64[F]);
@@ -959,13 +992,11 @@ int solve_fx64(mg_ctx* c, double fnorm, double tol, double* phi, double* gacc, c
       check(c, mg::launch_fx64(leg, true, s), "down leg");
     }
     if (cyc >= 0) {  // the norm of the last cycle's phi (the leg above ran ahead of the test)
-      check(c, mg::launch_fx64_norm(red, black, nb, c->iflag, c->scal + 1, s), "norm");
-      check(c, cudaMemcpyAsync(c->pinned + 1, c->scal + 1, 2 * sizeof(double),
-                               cudaMemcpyDeviceToHost, s),
-            "read norm and flag");
+      check(c, mg::launch_fx64_norm(red, black, nb, c->iflag, c->pinned + 1, s), "norm");
       check(c, cudaStreamSynchronize(s), "sync");
       if (c->pinned[2] != 0.0) return -1;
-      const double dn = std::sqrt(c->pinned[1] / (double)N) / (h * h * two_S);
+      const double unit = h * h * two_S, dn = std::sqrt(c->pinned[1] / (double)N) / unit;
+      if (n == 0) fnorm = std::sqrt(c->pinned[0] / (double)N) / unit;
       if (n == 0 && fnorm == 0.0) fnorm = dn > 0.0 ? dn : 1.0;
       const double r = dn / fnorm;
       hist[n++] = r;
@@ -1013,27 +1044,21 @@ mg_status solve_fp64(mg_ctx* c, const double* rho, double four_pi_G, double tol,
           "H2D rho");
   c->u64[F] = phi;
   Pyr<double> P = pyr<double>(c);
-  double fnorm = prepare_source(c, rho, four_pi_G, c->f64[F], true, s);
   Bc bcs[kMaxLevels];
   for (int l = 0; l < c->L; ++l) bcs[l] = physical_bc(c, l);
   const Bc hom = correction_bc(c, bcs[F]);
   const bool fas = c->opts.fas != 0;
+  if ((((uintptr_t)phi | (uintptr_t)rho) & 15u) == 0 && fx64_buffers(c)) {
+    const int st = solve_fx64(c, rho, four_pi_G, tol, phi, gacc, bcs, hom, hist, hist_cap, n_hist, s);
+    if (st >= 0) {
+      c->u64[F] = nullptr;
+      return (mg_status)st;
+    }
+  }
+  double fnorm = prepare_source(c, rho, four_pi_G, c->f64[F], true, s);
   if (c->opts.mode_fmg) {
     if (fas) fmg_fas(c, bcs, hom, s);
-    else if (((uintptr_t)phi & 15u) == 0 && fx64_buffers(c)) {
-      fmg_below<double>(c, P, bcs, hom, s);
-      const int st =
-          solve_fx64(c, fnorm, tol, phi, gacc, bcs[F], hom, hist, hist_cap, n_hist, s);
-      if (st >= 0) {
-        c->u64[F] = nullptr;
-        return (mg_status)st;
-      }
-      // outside the fixed-point range: everything again in FP64
-      fnorm = prepare_source(c, rho, four_pi_G, c->f64[F], true, s);
-      fmg<double>(c, P, bcs, hom, s);
-    } else {
-      fmg<double>(c, P, bcs, hom, s);
-    }
+    else fmg<double>(c, P, bcs, hom, s);
   }
   double dn = defect_rms(c, phi, c->f64[F], bcs[F], s);
   if (fnorm == 0.0) fnorm = dn > 0.0 ? dn : 1.0;
@@ -1180,8 +1205,7 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
     } else {
       check(c, mg::launch_outer_residual(phi, f, c->f32[F], g, c->h, bc, scale, c->partials, s),
             "outer residual");
-      check(c, mg::launch_finish_sum(c->partials, nb, c->scal + 1, s), "finish r^2");
-      rn = std::sqrt(read_scalar(c, 1, s) / (double)N);
+      rn = std::sqrt(read_sum(c, nb, s) / (double)N);
     }
     if (fnorm == 0.0) {
       fnorm = rn > 0.0 ? rn : 1.0;
@@ -1242,8 +1266,7 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
       KTimer t(c, MG_K_OUTER_RESIDUAL, true, s);
       check(c, mg::launch_outer_residual(phi, f, c->f32[F], g, c->h, bc, scale, c->partials, s),
             "outer residual");
-      check(c, mg::launch_finish_sum(c->partials, nb, c->scal + 1, s), "finish r^2");
-      rn = std::sqrt(read_scalar(c, 1, s) / (double)N);
+      rn = std::sqrt(read_sum(c, nb, s) / (double)N);
     } else {
       if (it == 0) {
         // S such that |phi| < 2^55 and |h^2 f| < 2^58 on the integer grid;
@@ -1297,8 +1320,7 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
       }
       phi_zero = false;
       std::swap(cur, alt);
-      check(c, mg::launch_finish_sum(c->partials, nbs, c->scal + 1, s), "finish r^2");
-      rn = std::sqrt(read_scalar(c, 1, s) / (double)N) / scale;
+      rn = std::sqrt(read_sum(c, nbs, s) / (double)N) / scale;
     }
     const double r = rn / fnorm;
     hist[n++] = r;
@@ -1809,6 +1831,7 @@ mg_status mg_ctx_autotune(mg_ctx* c, void* stream) {
   try {
     check(c, cudaSetDevice(c->device), "cudaSetDevice");
     drop_inner_graph(c);  // the launch shapes may change
+    if (c->ready) check(c, cudaStreamWaitEvent((cudaStream_t)stream, c->ready, 0), "wait");
     autotune(c, (cudaStream_t)stream);
   } catch (const Fail& f) {
     cudaStreamSynchronize((cudaStream_t)stream);
@@ -1862,6 +1885,7 @@ mg_status mg_destroy(mg_ctx* c) {
   drop_inner_graph(c);
   for (cudaEvent_t e : c->events) cudaEventDestroy(e);
   if (c->own_event) cudaEventDestroy(c->own_event);
+  if (c->ready) cudaEventDestroy(c->ready);
   if (c->own_stream) cudaStreamDestroy(c->own_stream);
   for (void* p : c->allocs) cudaFree(p);
   if (c->pinned) cudaFreeHost(c->pinned);
@@ -1915,8 +1939,9 @@ mg_status create_ctx(int nx, int ny, int nz, double dx, mg_bc bc, int face_mask,
       if (o.prec == MG_FP64) make_dense<double>(c, hom);
       else make_dense<float>(c, hom);
     }
+    check(c, cudaEventCreateWithFlags(&c->ready, cudaEventDisableTiming), "event");
+    check(c, cudaEventRecord(c->ready, nullptr), "record");
     check(c, cudaMallocHost(&c->pinned, 64 * sizeof(double)), "cudaMallocHost");
-    check(c, cudaStreamSynchronize(nullptr), "sync");
   } catch (const Fail& f) {
     mg_destroy(c);
     return f.st;
@@ -2042,6 +2067,11 @@ mg_status mg_solve_gravity(mg_ctx* c, const double* rho, double four_pi_G, doubl
   try {
     check(c, cudaSetDevice(c->device), "cudaSetDevice");
     s = capturable_stream(c, s);
+    if (c->ready) {
+      check(c, cudaStreamWaitEvent(s, c->ready, 0), "wait");
+      cudaEventDestroy(c->ready);
+      c->ready = nullptr;
+    }
     if (c->opts.prec == MG_FP64)
       st = solve_fp64(c, rho, four_pi_G, tol, phi, g, hist, hist_cap, n_hist, s);
     else
