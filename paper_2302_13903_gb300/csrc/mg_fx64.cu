@@ -62,7 +62,7 @@ struct Fx64Args {
   double* norm;  // per-CTA sum of R^2: red cells of u_in (down), black cells of u_out (up)
   double* fc;           // down: coarse right-hand side, -sum of R, as doubles,
   long long* fci;       //   or on the coarse level's integer grid (fc null)
-  int shift;            // down: -sum of R 2^shift is F there; up: ec has `shift` guard bits
+  int shift;            // down: -sum of R 2^shift is F there
   long long* psum;      // down: per-CTA exact sum of u_in, (hi, lo) pairs
   const long long* ec;  // up: coarse correction on the integer grid
   int limit;            // log2 of the largest |U|
@@ -124,8 +124,7 @@ struct Pair {
   bool tile;   // written by this CTA
   bool swap;   // P is cell i0 + 1
   int xo;      // pair offset of P's neighbour outside the pair (Q's is -xo)
-  int np, nq;  // 6 less the signs of the ghosts across x and y walls of P, Q
-  Weight w;    // the relaxation; 0 outside the level
+  int n;       // 6 less the signs of the ghosts across x and y walls of P, of Q << 8
 };
 
 __device__ __forceinline__ int wall_sign(int fk, int q) {
@@ -144,9 +143,7 @@ __device__ __forceinline__ Pair make_pair_of(const Fx64Args& a, int pm, int pr) 
   p.xo = p.swap ? 1 : -1;
   const int xl = i == 0 ? wall_sign(a.fk, 0) : 0, xh = i + 2 == a.g.nx ? wall_sign(a.fk, 1) : 0;
   const int y = j == 0 ? wall_sign(a.fk, 2) : j == a.g.ny - 1 ? wall_sign(a.fk, 3) : 0;
-  p.np = 6 - (p.swap ? xh : xl) - y;
-  p.nq = 6 - (p.swap ? xl : xh) - y;
-  p.w = p.valid ? a.w : Weight{0, 0};
+  p.n = (6 - (p.swap ? xh : xl) - y) | (6 - (p.swap ? xl : xh) - y) << 8;
   i = i < 0 ? i + a.g.nx : i >= a.g.nx ? i - a.g.nx : i;
   j = j < 0 ? j + a.g.ny : j >= a.g.ny ? j - a.g.ny : j;
   p.i0 = p.valid ? i : 0;
@@ -298,7 +295,8 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
   };
   long long uP[4] = {}, uQ[4] = {}, fP[4] = {}, fQ[4] = {};
   long long ud = 0, acc = 0, done = 0, psum = 0;
-  const Weight w = WALLS ? p.w : a.w;
+  // outside the level cells stay 0
+  auto delta = [&](long long R) { return !WALLS || p.valid ? weigh(R, a.w) : 0; };
   const int most = 1 << (a.limit - 32);
   Squares norm;
   bool bad = false;
@@ -316,7 +314,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     long long(&uB)[4] = EVEN ? uQ : uP;
     long long(&fR)[4] = EVEN ? fP : fQ;
     long long(&fB)[4] = EVEN ? fQ : fP;
-    const int xb = EVEN ? -p.xo : p.xo, nb = WALLS ? (EVEN ? p.nq : p.np) : 6;
+    const int xb = EVEN ? -p.xo : p.xo, nb = WALLS ? (EVEN ? p.n >> 8 : p.n & 255) : 6;
     issue(integral_constant<int, J + 3>{}, q + 3);
     cp_wait<3>();
     if (!WALLS || p.valid) {
@@ -352,7 +350,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
       const long long R =
           COARSE ? -fB[A] : residual<W::PW>(raw + I1, uB[A], uR[A], xb, zl, zh, n, fB[A]);
       if (!COARSE && p.tile && ka >= z0 && ka < z1) norm.add(R);
-      uB[A] += weigh(R, w);
+      uB[A] += delta(R);
       red[I1] = uB[A];
     }
     long long rb;
@@ -362,7 +360,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
       if (WALLS && wzl && kb == 0) zl = 0, n -= wzl;
       if (WALLS && wzh && kb == nz - 1) zh = 0, n -= wzh;
       const long long R = residual<W::PW>(red + I0, uB[B], uR[B], xb, zl, zh, n, fB[B]);
-      const long long d = weigh(R, w);
+      const long long d = delta(R);
       uB[B] += d;
       rb = R - n * d;
       blk[I0] = uB[B];
@@ -407,7 +405,8 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
 // q - 2, then final and written.  The correction of a pair is interpolated
 // along y, then x, then z with weights 3 and 1 on the integer grid and rounded
 // once by the division by 64.  Unrolled by four as the down leg.
-template <bool WALLS, int TX, bool COARSE>
+// GUARD: ec's guard bits.
+template <bool WALLS, int TX, bool COARSE, int GUARD>
 __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
     k_fx64_up(const __grid_constant__ Fx64Args a) {
   dev::after_previous();
@@ -490,10 +489,11 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
   };
   long long em0, em1, e00, e01;  // coarse planes K - 1 and K
   long long uP[4] = {}, uQ[4] = {}, fP[4] = {}, fQ[4] = {};
-  const Weight w = WALLS ? p.w : a.w;
+  // outside the level cells stay 0
+  auto delta = [&](long long R) { return !WALLS || p.valid ? weigh(R, a.w) : 0; };
   const int most = 1 << (a.limit - 32);
-  const int bits = 6 + a.shift;
-  const long long half = 1LL << (bits - 1);
+  constexpr int bits = 6 + GUARD;
+  constexpr long long half = 1LL << (bits - 1);
   Squares norm;
   bool bad = false;
   using std::integral_constant;
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
     long long(&uR)[4] = EVEN ? uP : uQ;
     long long(&uB)[4] = EVEN ? uQ : uP;
     long long(&fB)[4] = EVEN ? fQ : fP;
-    const int xb = EVEN ? -p.xo : p.xo, nb = WALLS ? (EVEN ? p.nq : p.np) : 6;
+    const int xb = EVEN ? -p.xo : p.xo, nb = WALLS ? (EVEN ? p.n >> 8 : p.n & 255) : 6;
     issue(integral_constant<int, J + 3>{}, q + 3);
     cp_wait<3>();
     long long d0, d1;  // the pair's correction
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
       if (WALLS && wzl && ka == 0) zl = 0, n -= wzl;
       if (WALLS && wzh && ka == nz - 1) zh = 0, n -= wzh;
       const long long R = residual<W::PW>(raw + I1, uB[A], uR[A], xb, zl, zh, n, fB[A]);
-      uB[A] += weigh(R, w);
+      uB[A] += delta(R);
       red[I1] = uB[A];
     }
     {  // [B]: black of plane q - 2 is in the columns uB
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
       if (WALLS && wzl && kb == 0) zl = 0, n -= wzl;
       if (WALLS && wzh && kb == nz - 1) zh = 0, n -= wzh;
       const long long R = residual<W::PW>(red + I0, uB[B], uR[B], xb, zl, zh, n, fB[B]);
-      const long long d = weigh(R, w);
+      const long long d = delta(R);
       uB[B] += d;
       if (p.tile && kb >= z0 && kb < z1) {
         if (!COARSE) norm.add(R - n * d);
@@ -750,13 +750,19 @@ cudaError_t launch_leg(K* kernel, std::atomic<int>* configured, size_t smem, int
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// guard: up from a level with guard bits to one without.
 template <bool WALLS, int TX, bool COARSE>
-cudaError_t launch(const Fx64Args& a, bool down, cudaStream_t s) {
-  static std::atomic<int> configured[2][64];
-  return down ? launch_leg(k_fx64_down<WALLS, TX, COARSE>, configured[0], down_smem<TX>(),
-                           Down<TX>::NT, TX, a, s)
-              : launch_leg(k_fx64_up<WALLS, TX, COARSE>, configured[1], up_smem<TX>(), Up<TX>::NT,
-                           TX, a, s);
+cudaError_t launch(const Fx64Args& a, bool down, bool guard, cudaStream_t s) {
+  static std::atomic<int> configured[3][64];
+  if (down)
+    return launch_leg(k_fx64_down<WALLS, TX, COARSE>, configured[0], down_smem<TX>(), Down<TX>::NT,
+                      TX, a, s);
+  if constexpr (!COARSE)
+    if (guard)
+      return launch_leg(k_fx64_up<WALLS, TX, false, kFx64Guard>, configured[2], up_smem<TX>(),
+                        Up<TX>::NT, TX, a, s);
+  return launch_leg(k_fx64_up<WALLS, TX, COARSE, 0>, configured[1], up_smem<TX>(), Up<TX>::NT, TX,
+                    a, s);
 }
 
 // Tile width: 64 cells, one CTA per SM, or on levels that would leave SMs
@@ -820,13 +826,13 @@ cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s) {
   // with |ec| < 2^56 and its sums of weight 64 below 2^62
   a.limit = q.coarse ? 56 : 59;
   a.flag = q.flag;
-  const bool wide = tile_width(q.g) == 64;
+  const bool wide = tile_width(q.g) == 64, gd = !down && q.shift != 0;
   if (q.coarse) {
-    if (a.fk) return wide ? launch<true, 64, true>(a, down, s) : launch<true, 32, true>(a, down, s);
-    return wide ? launch<false, 64, true>(a, down, s) : launch<false, 32, true>(a, down, s);
+    if (a.fk) return wide ? launch<true, 64, true>(a, down, gd, s) : launch<true, 32, true>(a, down, gd, s);
+    return wide ? launch<false, 64, true>(a, down, gd, s) : launch<false, 32, true>(a, down, gd, s);
   }
-  if (a.fk) return wide ? launch<true, 64, false>(a, down, s) : launch<true, 32, false>(a, down, s);
-  return wide ? launch<false, 64, false>(a, down, s) : launch<false, 32, false>(a, down, s);
+  if (a.fk) return wide ? launch<true, 64, false>(a, down, gd, s) : launch<true, 32, false>(a, down, gd, s);
+  return wide ? launch<false, 64, false>(a, down, gd, s) : launch<false, 32, false>(a, down, gd, s);
 }
 
 cudaError_t launch_fx64_source(const double* rho, long long* F, Grid g, const Bc& bc,
