@@ -1048,7 +1048,12 @@ mg_status solve_fp64(mg_ctx* c, const double* rho, double four_pi_G, double tol,
   for (int l = 0; l < c->L; ++l) bcs[l] = physical_bc(c, l);
   const Bc hom = correction_bc(c, bcs[F]);
   const bool fas = c->opts.fas != 0;
-  if ((((uintptr_t)phi | (uintptr_t)rho) & 15u) == 0 && fx64_buffers(c)) {
+  // the integer path writes phi before it knows that the values fit, and starts
+  // again from rho where they do not: not for a phi that shares rho's memory
+  const uintptr_t pr = (uintptr_t)rho, pp = (uintptr_t)phi;
+  const size_t bytes = sizeof(double) * level_grid(c, F).cells();
+  const bool apart = pr + bytes <= pp || pp + bytes <= pr;
+  if (((pp | pr) & 15u) == 0 && apart && fx64_buffers(c)) {
     const int st = solve_fx64(c, rho, four_pi_G, tol, phi, gacc, bcs, hom, hist, hist_cap, n_hist, s);
     if (st >= 0) {
       c->u64[F] = nullptr;

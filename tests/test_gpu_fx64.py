@@ -90,6 +90,18 @@ def test_sources_outside_the_fixed_point_range():
     assert gpu(rho, "fixed", tol=1e-10, omega=1.99)[2] == ref.status
 
 
+def test_in_place_is_the_general_path():
+    """rho and phi the same array: the general FP64 kernels, as for a misaligned phi."""
+    rho = source((64, 32, 32), 4)
+    odd = torch.zeros(rho.size + 1, dtype=torch.float64, device="cuda")[1:].view(rho.shape)
+    ref, h0, _ = gpu(rho, "fixed", phi=odd, max_cycles=2, stall_ratio=NO_STALL)
+    both = torch.from_numpy(rho).cuda()
+    with mg.Solver((64, 32, 32), 1.0 / 64, [F] * 6, face_values=[0.4] * 6, prec=mg.FP64,
+                   max_cycles=2, stall_ratio=NO_STALL) as s:
+        p, h, _ = s.solve(both, 1.0, 0.0, phi=both, raise_on_error=False)
+    assert np.array_equal(p.cpu().numpy(), ref) and np.array_equal(h, h0)
+
+
 @pytest.mark.parametrize("rule", sorted(RULES))
 @pytest.mark.parametrize("dims", [(2, 2, 2), (6, 4, 2), (10, 6, 4), (64, 6, 10), (34, 2, 64)])
 @pytest.mark.parametrize("prec", [mg.FP64, mg.MIXED])
