@@ -434,12 +434,14 @@ mg_status mg_batch_create(int n, const int *dims, const double *dx, const mg_bc 
  * g, four_pi_G[g] and tol[g] its constants (host arrays of n).  rho_dev[g] =
  * NULL leaves slot g out of this solve (phi_dev[g] is not touched, status[g]
  * = MG_OK, n_hist[g] = 0); at least one grid must be given.  A grid's result
- * does not depend on the other slots.  One persistent
- * cooperative kernel runs every phase of every grid; the first call captures
- * the upload of the per-grid arguments, the kernel and the download of the
- * results as a CUDA graph (so make it outside any capture of your own) and
- * later calls replay it; each grid stops by the
- * rule of mg_solve (Sec. 2.3.7).  hist (host, n * hist_cap, may be NULL)
+ * does not depend on the other slots.  Grids of one size, rule and spacing
+ * form a class; the classes run side by side on streams of the batch's own,
+ * ordered after `stream`, a launch per phase and class, each outer iteration
+ * after a class's first as a CUDA graph (so make the call outside any capture
+ * of your own).  After mg_batch_set_blocks or mg_batch_set_barrier_limit, and
+ * for more than 24 classes, one persistent cooperative kernel runs every phase
+ * of every grid instead, captured by the first call and replayed by later
+ * ones: the same bits.  Each grid stops by the rule of mg_solve (Sec. 2.3.7).  hist (host, n * hist_cap, may be NULL)
  * receives each grid's ||d||/||f|| after every outer iteration, n_hist[g] the
  * count, status[g] its result.  Returns MG_OK when every grid converged, else
  * the first failing grid's status, MG_ERR_TIMEOUT if a grid-wide barrier wait
@@ -453,12 +455,14 @@ mg_status mg_batch_destroy(mg_batch *batch);
 /* Total cells of the finest levels of the batch. */
 long long mg_batch_cells(const mg_batch *batch);
 
-/* 1 when the solve runs as a captured CUDA graph (captured on the first
- * mg_batch_solve and replayed after), 0 when it is launched directly. */
+/* 1 when the last mg_batch_solve replayed CUDA graphs, 0 when it was launched
+ * directly. */
 int mg_batch_graph(const mg_batch *batch);
 
-/* Device time of the last mg_batch_solve by phase kind, in milliseconds
- * (from the GPU's global timer at each grid-wide barrier): ms_by_type[k] for
+/* Device time of the last mg_batch_solve by phase kind, in milliseconds (from
+ * the GPU's global timer at each grid-wide barrier of the persistent kernel,
+ * else the whole solve's time by the shares of the kinds, whose launches
+ * overlap, in the thread-clocks spent): ms_by_type[k] for
  * k < n_types in the order source, mean, first residual, norms of the
  * source and first residual, fused down leg, bottom levels, fused up leg, max |e|,
  * fixed-point scale, conversion to fixed point, outer step (correction and
@@ -467,14 +471,14 @@ int mg_batch_graph(const mg_batch *batch);
  * Synchronises the device.  Errors: MG_ERR_ARG, MG_ERR_CUDA. */
 mg_status mg_batch_phase_ms(mg_batch *batch, double *ms_by_type, int n_types);
 
-/* CTAs of the persistent launch: 0 (default) as many as fit on the device at
- * once, else at most that many (fewer CTAs leave SMs to other streams' work,
- * for a batch of small grids).  Takes effect at the next mg_batch_solve,
+/* CTAs of the persistent launch: 0 (default) no limit, else at most that many
+ * (fewer CTAs leave SMs to other streams' work, for a batch of small grids).  Takes effect at the next mg_batch_solve,
  * which captures its CUDA graph again.  Errors: MG_ERR_ARG (blocks < 0). */
 mg_status mg_batch_set_blocks(mg_batch *batch, int blocks);
 
 /* Limit of one wait at the persistent kernel's grid-wide barriers, in GPU
- * clock cycles (default 4e9, about 2 s at 2 GHz); a wait that runs out makes
+ * clock cycles (default 4e9, about 2 s at 2 GHz; any other value chooses that
+ * kernel); a wait that runs out makes
  * every block return and mg_batch_solve report MG_ERR_TIMEOUT, leaving the
  * batch usable.  Takes effect at the next mg_batch_solve, which captures its
  * CUDA graph again.  Errors: MG_ERR_ARG (cycles < 0). */

@@ -591,7 +591,7 @@ def faces_count(nx, ny, nz):
 
 
 class Batch:
-    """Many independent grids solved by one persistent launch (mg_batch_*)."""
+    """Many independent grids solved together (mg_batch_*)."""
 
     def __init__(self, sizes, dxs, bcs, fixed_values=None, **opts):
         self.n = len(sizes)
@@ -651,7 +651,7 @@ class Batch:
         return st, [hist[g, : nh[g]].copy() for g in range(n)], sts
 
     def set_blocks(self, blocks):
-        """CTAs of the persistent launch (0: all that fit)."""
+        """CTAs of the persistent launch (0: no limit)."""
         st = lib().mg_batch_set_blocks(self.ptr, int(blocks))
         if st != 0:
             raise MGError(st, lib().mg_batch_last_error(self.ptr).decode())

@@ -1,4 +1,6 @@
-// mg_batch.cu -- many independent grids solved by one persistent launch.
+// mg_batch.cu -- many independent grids solved together: in stages, a launch per
+// phase and class of like grids (see "Staged solve" below), or by one
+// persistent launch, as follows.
 //
 // Each grid is solved by the mixed-precision method of the single-grid path:
 // an FP64 outer defect-correction loop (source, residual, correction and
@@ -30,6 +32,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "../../include/mg.h"
@@ -52,6 +55,7 @@ static_assert(fused::Shape<fused::kUp, 64, 16, 4, kPad>::SMEM <= kSmem &&
                   fused::Shape<fused::kUp, 32, 16, 4, kPad>::SMEM <= kSmem,
               "an up-leg tile needs more shared memory than the CTA has");
 constexpr int kMaxL = 16;
+constexpr int kMaxClasses = 24;  // streams of a staged solve
 constexpr int kChunk = 32768;   // cells per chunk item
 constexpr int kFusedMinN = 32;  // levels of at least 32^3 use the fused tiles
 constexpr int kCz = 64;         // z-chunk of fused tiles
@@ -99,6 +103,8 @@ enum PhaseType : int {
   PH_PMEAN,        // grid: mean of phi
   PH_PSUB          // chunk: phi = PHI 2^-S - mean (fixed point) or phi -= mean
 };
+constexpr int kPhaseTypes = PH_PSUB + 1;
+constexpr int kBottomThreads = 512;  // of a bottom CTA of its own (staged solve)
 
 struct Phase {
   int type;
@@ -132,6 +138,7 @@ struct Ctl {
   int max_cycles, inner_zero;
   double stall_ratio;
   long long bar_cycles;  // a barrier wait gives up after this many clock cycles
+  unsigned long long* work;  // staged: [type] thread-clocks spent, then first start, last end (ns)
 };
 
 __device__ bool grid_barrier(const Ctl& c) {
@@ -612,6 +619,120 @@ __device__ void fin_item(const Ctl& c, GridDev& g, int gi) {
   }
 }
 
+// The phases that are one thread's work on one grid (index gi).
+__device__ void grid_item(const Ctl& c, GridDev& g, int type, int gi) {
+  const double N = (double)g.n * g.n * g.n;
+  switch (type) {
+    case PH_MEANFIN:
+      g.mean = (g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD) ? g.fpg * (chunk_total(c, g) / N) : 0.0;
+      // max |f - mean| <= |4 pi G| max |rho| + |mean|: the scale of r32 and of 2^S
+      g.maxf = fabs(g.fpg) * chunk_max(c, g) + fabs(g.mean);
+      g.scale = g.maxf > 0.0 ? 1.0 / g.maxf : 1.0;
+      break;
+    case PH_R0FIN: {
+      double fs = 0.0, rs = 0.0;  // sums of ((f - mean) sc)^2 and (r0 sc)^2
+      for (int q = 0; q < g.nchunk; ++q) {
+        fs += c.part[g.chunk0 + q];
+        rs += c.part2[g.chunk0 + q];
+      }
+      g.fnorm = sqrt(fs / N) / g.scale;
+      g.rn = sqrt(rs / N) / g.scale;
+      if (g.fnorm == 0.0) g.fnorm = g.rn > 0.0 ? g.rn : 1.0;
+      if (g.rn == 0.0) {  // phi = 0 is exact
+        g.active = 0;
+        g.status = MG_OK;
+        if (c.hist_cap > 0) c.hist[(size_t)gi * c.hist_cap] = 0.0;
+        g.nh = 1;
+      }
+      break;
+    }
+    case PH_SETFX: setfx_item(c, g); break;
+    case PH_PMEAN: {
+      double m = 0.0;
+      if (g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD) {
+        if (g.in_fx) {  // exact integer total, independent of the chunking
+          long long th = 0, tl = 0;
+          for (int q = 0; q < g.nchunk; ++q) {
+            th += c.ipart[2 * (g.chunk0 + q)];
+            tl += c.ipart[2 * (g.chunk0 + q) + 1];
+          }
+          m = ((double)th * 4294967296.0 + (double)tl) / (N * g.two_S);
+          // the same mean as an integer, exactly: the 128-bit sum th 2^32 + tl
+          // over N = 2^(3 lg) cells, rounded (ties up)
+          const int k = 3 * (g.L - 1);
+          const unsigned long long t = (unsigned long long)th << 32;
+          unsigned long long lo = t + (unsigned long long)tl;
+          long long hi = (th >> 32) + (tl < 0 ? -1 : 0) + (lo < t ? 1 : 0);
+          if (k > 0) {
+            const unsigned long long lo2 = lo + (1ULL << (k - 1));
+            hi += lo2 < lo ? 1 : 0;
+            g.imean = (long long)((lo2 >> k) | ((unsigned long long)hi << (64 - k)));
+          } else {
+            g.imean = (long long)lo;
+          }
+        }  // otherwise phi = 0 exactly (the grid stopped at its first residual)
+      }
+      g.mean = m;
+      break;
+    }
+  }
+}
+
+// Whether grid g takes part in a phase of this type.
+__device__ __forceinline__ bool runs(const GridDev& g, int type) {
+  const bool has_mean = g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD;
+  return !g.skip && (type == PH_PSUM ? has_mean : (type > PH_PSUM || g.active));
+}
+
+// The levels of at most 16^3 of one V-cycle, by one CTA, in its dynamic shared
+// memory (kBottomBytes): a chain of some 25 dependent passes over at most 4096
+// cells, so what counts is the latency of a load.
+constexpr size_t kBottomBytes = 2 * (4096 + 512 + 64 + 8 + 1) * sizeof(float);
+static_assert(kBottomBytes <= kSmem, "the bottom levels exceed the CTA's smem");
+
+__device__ void bottom_item(const Ctl& c, const GridDev& g, int cycle, float4* smem) {
+  // the arguments in shared memory: their per-level arrays are indexed by a
+  // run-time level, which in each thread's own copy would put them in local
+  // memory
+  __shared__ bottom::BottomArgs<float> a;
+  const int top = level_of(g, min(g.n, kFusedMinN / 2));
+  if (threadIdx.x == 0) {
+    for (int l = 0; l < kBottomLevels; ++l) {
+      const bool used = l <= top;
+      a.u[l] = used ? g.u32[l] : nullptr;
+      a.f[l] = used ? g.f32[l] : nullptr;
+      a.n[l] = used ? (g.n >> (g.L - 1 - l)) : 0;
+      a.h[l] = used ? g.h * (double)(1 << (g.L - 1 - l)) : 0.0;
+      a.bc[l] = hom_bc(g);
+    }
+    a.hom = hom_bc(g);
+    a.omega = c.omega;
+    a.pre = 1;
+    a.post = 1;
+    a.top = top;
+    a.fmg = 0;
+    bottom::set_coefficients(a);
+  }
+  __syncthreads();
+  const bool zg = (top < g.L - 1) || (cycle == 0 && c.inner_zero);
+  bottom::in_shared(a, reinterpret_cast<float*>(smem), !zg, [&](const bottom::BottomArgs<float>& b) {
+    bottom::vcycle<float, false>(b, top, b.hom, zg);
+  });
+}
+
+// The constants of a leg on level l (n^3 cells) of grid g.
+__host__ __device__ inline fused::FusedParams leg_params(int n, int bc, double hl, double omega) {
+  fused::FusedParams fp;
+  fp.nx = fp.ny = fp.nz = n;
+  fp.sx0 = fp.sx1 = fp.sy0 = fp.sy1 = fp.sz0 = fp.sz1 = bc == BC_ZEROGRAD ? 1.f : -1.f;
+  fp.cu = (float)(1.0 - omega);
+  fp.cs = (float)(omega / 6.0);
+  fp.cf = (float)(-omega * hl * hl / 6.0);
+  fp.inv_h2 = (float)(1.0 / (hl * hl));
+  fp.cz = kCz < n ? kCz : n;
+  return fp;
+}
+
 // One tile item of a fused leg on level l: tiles TX x 16 cells, the chunk's
 // planes; the down leg starts from zero on coarse levels and, when asked, on
 // the finest.
@@ -660,81 +781,22 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(Ctl c) {
       if (it >= P.count) break;
       const Item I = c.items[P.first + it];
       GridDev& g = c.grids[I.grid];
-      const bool has_mean = g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD;
-      const bool run =
-          !g.skip && (P.type == PH_PSUM ? has_mean : (P.type > PH_PSUM || g.active));
-      if (!run) continue;
+      if (!runs(g, P.type)) continue;
       switch (P.type) {
         case PH_SRC: chunk_item<PH_SRC>(c, g, I.a); break;
         case PH_R0: chunk_item<PH_R0>(c, g, I.a); break;
         case PH_EMAX: chunk_item<PH_EMAX>(c, g, I.a); break;
         case PH_TOFX: chunk_item<PH_TOFX>(c, g, I.a); break;
-        case PH_SETFX:
-          if (threadIdx.x == 0) setfx_item(c, g);
-          break;
         case PH_FXSTEP:
           fx_tile_item(c, g, I, P.cycle != 0, smem);
           break;
         case PH_PSUM: chunk_item<PH_PSUM>(c, g, I.a); break;
         case PH_PSUB: chunk_item<PH_PSUB>(c, g, I.a); break;
         case PH_MEANFIN:
-          if (threadIdx.x == 0) {
-            const double N = (double)g.n * g.n * g.n;
-            g.mean = (g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD) ? g.fpg * (chunk_total(c, g) / N)
-                                                                  : 0.0;
-            // max |f - mean| <= |4 pi G| max |rho| + |mean|: the scale of r32 and of 2^S
-            g.maxf = fabs(g.fpg) * chunk_max(c, g) + fabs(g.mean);
-            g.scale = g.maxf > 0.0 ? 1.0 / g.maxf : 1.0;
-          }
-          break;
         case PH_PMEAN:
-          if (threadIdx.x == 0) {
-            const double N = (double)g.n * g.n * g.n;
-            double m = 0.0;
-            if (g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD) {
-              if (g.in_fx) {  // exact integer total, independent of the chunking
-                long long th = 0, tl = 0;
-                for (int q = 0; q < g.nchunk; ++q) {
-                  th += c.ipart[2 * (g.chunk0 + q)];
-                  tl += c.ipart[2 * (g.chunk0 + q) + 1];
-                }
-                m = ((double)th * 4294967296.0 + (double)tl) / (N * g.two_S);
-                // the same mean as an integer, exactly: the 128-bit sum th 2^32 + tl
-                // over N = 2^(3 lg) cells, rounded (ties up)
-                const int k = 3 * (g.L - 1);
-                const unsigned long long t = (unsigned long long)th << 32;
-                unsigned long long lo = t + (unsigned long long)tl;
-                long long hi = (th >> 32) + (tl < 0 ? -1 : 0) + (lo < t ? 1 : 0);
-                if (k > 0) {
-                  const unsigned long long lo2 = lo + (1ULL << (k - 1));
-                  hi += lo2 < lo ? 1 : 0;
-                  g.imean = (long long)((lo2 >> k) | ((unsigned long long)hi << (64 - k)));
-                } else {
-                  g.imean = (long long)lo;
-                }
-              }  // otherwise phi = 0 exactly (the grid stopped at its first residual)
-            }
-            g.mean = m;
-          }
-          break;
         case PH_R0FIN:
-          if (threadIdx.x == 0) {
-            const double N = (double)g.n * g.n * g.n;
-            double fs = 0.0, rs = 0.0;  // sums of ((f - mean) sc)^2 and (r0 sc)^2
-            for (int q = 0; q < g.nchunk; ++q) {
-              fs += c.part[g.chunk0 + q];
-              rs += c.part2[g.chunk0 + q];
-            }
-            g.fnorm = sqrt(fs / N) / g.scale;
-            g.rn = sqrt(rs / N) / g.scale;
-            if (g.fnorm == 0.0) g.fnorm = g.rn > 0.0 ? g.rn : 1.0;
-            if (g.rn == 0.0) {  // phi = 0 is exact
-              g.active = 0;
-              g.status = MG_OK;
-              if (c.hist_cap > 0) c.hist[(size_t)I.grid * c.hist_cap] = 0.0;
-              g.nh = 1;
-            }
-          }
+        case PH_SETFX:
+          if (threadIdx.x == 0) grid_item(c, g, P.type, I.grid);
           break;
         case PH_FIN:
           if (threadIdx.x == 0) {
@@ -742,46 +804,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(Ctl c) {
             if (g.active) atomicAdd(&c.active_left[ph], 1);
           }
           break;
-        case PH_BOTTOM: {
-          // the arguments in shared memory: their per-level arrays are indexed
-          // by a run-time level, which in each thread's own copy would put
-          // them in local memory
-          __shared__ bottom::BottomArgs<float> a;
-          const int top = level_of(g, min(g.n, kFusedMinN / 2));
-          if (threadIdx.x == 0) {
-            for (int l = 0; l < kBottomLevels; ++l) {
-              const bool used = l <= top;
-              a.u[l] = used ? g.u32[l] : nullptr;
-              a.f[l] = used ? g.f32[l] : nullptr;
-              a.n[l] = used ? (g.n >> (g.L - 1 - l)) : 0;
-              a.h[l] = used ? g.h * (double)(1 << (g.L - 1 - l)) : 0.0;
-              a.bc[l] = hom_bc(g);
-            }
-            a.hom = hom_bc(g);
-            a.omega = c.omega;
-            a.pre = 1;
-            a.post = 1;
-            a.top = top;
-            a.fmg = 0;
-            bottom::set_coefficients(a);
-          }
-          __syncthreads();
-          const bool zg = (top < g.L - 1) || (P.cycle == 0 && c.inner_zero);
-          bottom::vcycle<float, false>(a, top, a.hom, zg);
-          break;
-        }
+        case PH_BOTTOM: bottom_item(c, g, P.cycle, smem); break;
         case PH_DOWN:
         case PH_UP: {
           const int l = level_of(g, P.n);
           const double hl = g.h * (double)(1 << (g.L - 1 - l));
-          fused::FusedParams fp;
-          fp.nx = fp.ny = fp.nz = P.n;
-          fp.sx0 = fp.sx1 = fp.sy0 = fp.sy1 = fp.sz0 = fp.sz1 = g.bc == BC_ZEROGRAD ? 1.f : -1.f;
-          fp.cu = (float)(1.0 - c.omega);
-          fp.cs = (float)(c.omega / 6.0);
-          fp.cf = (float)(-c.omega * hl * hl / 6.0);
-          fp.inv_h2 = (float)(1.0 / (hl * hl));
-          fp.cz = kCz < P.n ? kCz : P.n;
+          const fused::FusedParams fp = leg_params(P.n, g.bc, hl, c.omega);
           const bool per = g.bc == BC_PERIODIC;
           if (P.n >= 64)
             tile_leg<64>(P.type == PH_DOWN, per, g, l, P.cycle == 0 && c.inner_zero, fp, I, smem);
@@ -801,6 +829,120 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(Ctl c) {
       ph = q - 1;
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// Staged solve: each phase a launch of its own, for the grids of one class
+// (same size, rule and spacing), the classes side by side on streams.  The
+// persistent kernel gives every phase one block shape, 128 registers and two
+// CTAs per SM, and its legs ran at 0.35-0.40 of the HBM peak; as their own
+// kernels they have the single-grid legs' shapes (an up leg of three CTAs per
+// SM) and constants, and one class's last wave is filled by the others.  The
+// items are the persistent kernel's programs: the same bits.
+
+// What the phase cost, for the shares in mg_batch_phase_ms.
+struct Meter {
+  unsigned long long* w;
+  int type;
+  long long t0;
+  __device__ Meter(const Ctl& c, int type_) {
+    w = c.work;
+    type = type_;
+    t0 = clock64();
+    if (threadIdx.x == 0 && type == PH_SRC) atomicMin(w + kPhaseTypes, global_ns());
+  }
+  __device__ void stop() {
+    if (threadIdx.x != 0) return;
+    atomicAdd(w + type, (unsigned long long)(clock64() - t0) * blockDim.x);
+    if (type == PH_PSUB) atomicMax(w + kPhaseTypes + 1, global_ns());
+  }
+};
+
+template <int TYPE>
+__global__ void __launch_bounds__(kThreads) k_stage_chunks(const __grid_constant__ Ctl c,
+                                                           const int* grids) {
+  dev::after_previous();
+  GridDev& g = c.grids[grids[blockIdx.y]];
+  if (!runs(g, TYPE)) return;
+  Meter m(c, TYPE);
+  chunk_item<TYPE>(c, g, blockIdx.x);
+  m.stop();
+}
+
+__global__ void k_stage_grid(const __grid_constant__ Ctl c, const int* grids, int type) {
+  dev::after_previous();
+  const int gi = grids[blockIdx.x];
+  GridDev& g = c.grids[gi];
+  if (!runs(g, type)) return;
+  Meter m(c, type);
+  if (threadIdx.x == 0) grid_item(c, g, type, gi);
+  m.stop();
+}
+
+// The stopping rule of a class's grids; the number still active goes to
+// page-locked memory, where the host reads it.
+__global__ void k_stage_fin(const __grid_constant__ Ctl c, const int* grids, int count, int* left) {
+  dev::after_previous();
+  Meter m(c, PH_FIN);
+  int n = 0;
+  for (int q = threadIdx.x; q < count; q += blockDim.x) {
+    GridDev& g = c.grids[grids[q]];
+    if (!runs(g, PH_FIN)) continue;
+    fin_item(c, g, grids[q]);
+    n += g.active;
+  }
+  __shared__ int total;
+  if (threadIdx.x == 0) total = 0;
+  __syncthreads();
+  atomicAdd(&total, n);
+  __syncthreads();
+  m.stop();
+  if (threadIdx.x == 0) {
+    *reinterpret_cast<volatile int*>(left) = total;
+    __threadfence_system();
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_stage_fx(const __grid_constant__ Ctl c,
+                                                       const int* grids, int n, int zero_in) {
+  dev::after_previous();
+  extern __shared__ float4 smem[];
+  GridDev& g = c.grids[grids[blockIdx.y]];
+  if (!runs(g, PH_FXSTEP)) return;
+  Meter m(c, PH_FXSTEP);
+  const int nx = n / fx_tx(n), ny = n / fx_ty(n), t = blockIdx.x;
+  fx_tile_item(c, g, Item{0, t % nx, t / nx % ny, t / (nx * ny)}, zero_in != 0, smem);
+  m.stop();
+}
+
+__global__ void __launch_bounds__(kBottomThreads) k_stage_bottom(const __grid_constant__ Ctl c,
+                                                                 const int* grids, int cycle) {
+  dev::after_previous();
+  extern __shared__ float4 smem[];
+  const GridDev& g = c.grids[grids[blockIdx.x]];
+  if (!runs(g, PH_BOTTOM)) return;
+  Meter m(c, PH_BOTTOM);
+  bottom_item(c, g, cycle, smem);
+  m.stop();
+}
+
+template <int MODE, bool ZERO, int PM, int TX>
+__global__ void __maxnreg__((fused::fused_max_regs<MODE, 16, PM>()))
+    k_stage_leg(const __grid_constant__ Ctl c, const int* grids, int l,
+                const __grid_constant__ fused::FusedParams p) {
+  dev::after_previous();
+  extern __shared__ float4 smem[];
+  const GridDev& g = c.grids[grids[blockIdx.y]];
+  constexpr int type = MODE == fused::kDown ? PH_DOWN : PH_UP;
+  if (!runs(g, type)) return;
+  Meter m(c, type);
+  const int nx = p.nx / TX, ny = p.nx / 16, t = blockIdx.x;
+  constexpr bool UP = MODE == fused::kUp;
+  fused::fused_tile<MODE, ZERO, PM, TX, 16>(UP ? g.u32b[l] : g.u32[l], UP ? g.u32[l] : g.u32b[l],
+                                            g.f32[l], UP ? g.u32[l - 1] : nullptr,
+                                            UP ? nullptr : g.f32[l - 1], p, t % nx, t / nx % ny,
+                                            t / (nx * ny), smem);
+  m.stop();
 }
 
 }  // namespace batch
@@ -843,6 +985,25 @@ struct mg_batch {
   size_t bytes = 0;
   std::string err;
   long long bar_cycles = kBarrierCycles;  // limit of one grid-wide barrier wait
+  // staged solve: the grids by size, rule and spacing, largest first
+  struct Class {
+    int n, bc, L;
+    double h;
+    int first, count;  // its grids in d_class
+    cudaStream_t s = nullptr;
+    cudaEvent_t ev = nullptr;
+    cudaGraphExec_t iter = nullptr;  // an outer iteration after the first
+    long long launches = 0;          // kernels in it
+    int done = 0;                    // outer iterations queued in this solve
+    bool last = false;               // its final phases are queued
+  };
+  std::vector<Class> classes;
+  int* d_class = nullptr;
+  unsigned long long* d_work = nullptr;
+  int* h_left = nullptr;  // pinned: grids of each class still active
+  cudaEvent_t start = nullptr;
+  bool start_ok = false;    // the streams, events and h_left are there
+  bool staged = false;      // whether the last solve was staged
 };
 
 namespace {
@@ -867,6 +1028,13 @@ void free_batch(mg_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   if (b->cap) cudaStreamDestroy(b->cap);
+  for (auto& k : b->classes) {
+    if (k.iter) cudaGraphExecDestroy(k.iter);
+    if (k.ev) cudaEventDestroy(k.ev);
+    if (k.s) cudaStreamDestroy(k.s);
+  }
+  if (b->start) cudaEventDestroy(b->start);
+  if (b->h_left) cudaFreeHost(b->h_left);
   for (void* p : b->allocs) cudaFree(p);
   if (b->h_grids) cudaFreeHost(b->h_grids);
   if (b->h_hist) cudaFreeHost(b->h_hist);
@@ -944,16 +1112,8 @@ void build_phases(mg_batch* b, std::vector<Phase>& phases, std::vector<Item>& it
   add_chunk_phase(PH_PSUB);
 }
 
-// The device work of one solve, in stream order.
-cudaError_t enqueue_solve(mg_batch* b, cudaStream_t s) {
-  cudaError_t e = cudaMemcpyAsync(b->d_grids, b->h_grids, sizeof(GridDev) * b->ngrids,
-                                  cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counters, 0, sizeof(unsigned) * b->nphases, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned) * 2, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_err, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_active, 0, sizeof(int) * b->nphases, s);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(b->d_ptime, 0, sizeof(unsigned long long) * (b->nphases + 1), s);
+// The arguments every phase takes.
+Ctl control(const mg_batch* b) {
   Ctl c;
   c.phases = b->d_phases;
   c.items = b->d_items;
@@ -977,6 +1137,21 @@ cudaError_t enqueue_solve(mg_batch* b, cudaStream_t s) {
   c.inner_zero = b->opts.inner_fmg ? 0 : 1;
   c.stall_ratio = b->opts.stall_ratio;
   c.bar_cycles = b->bar_cycles;
+  c.work = b->d_work;
+  return c;
+}
+
+// The device work of one solve, in stream order.
+cudaError_t enqueue_solve(mg_batch* b, cudaStream_t s) {
+  cudaError_t e = cudaMemcpyAsync(b->d_grids, b->h_grids, sizeof(GridDev) * b->ngrids,
+                                  cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counters, 0, sizeof(unsigned) * b->nphases, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned) * 2, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_err, 0, sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_active, 0, sizeof(int) * b->nphases, s);
+  if (e == cudaSuccess)
+    e = cudaMemsetAsync(b->d_ptime, 0, sizeof(unsigned long long) * (b->nphases + 1), s);
+  Ctl c = control(b);
   if (e == cudaSuccess) {
     void* args[] = {&c};
     e = cudaLaunchCooperativeKernel((const void*)k_batch, dim3(b->blocks), dim3(kThreads), args,
@@ -989,6 +1164,229 @@ cudaError_t enqueue_solve(mg_batch* b, cudaStream_t s) {
     e = cudaMemcpyAsync(b->h_hist, b->d_hist, sizeof(double) * b->ngrids * b->hist_cap,
                         cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->h_err, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
+  return e;
+}
+
+// --- the staged solve -------------------------------------------------------
+
+// The classes of a batch; empty where there are too many for a stream each, or
+// too many grids in one for a launch.
+void make_classes(mg_batch* b, std::vector<int>& order) {
+  using Class = mg_batch::Class;
+  std::vector<Class>& cs = b->classes;
+  std::vector<std::vector<int>> members;
+  for (int g = 0; g < b->ngrids; ++g) {
+    const GridDev& d = b->host_grids[g];
+    size_t q = 0;
+    while (q < cs.size() && !(cs[q].n == d.n && cs[q].bc == d.bc && cs[q].h == d.h)) ++q;
+    if (q == cs.size()) {
+      if (q == (size_t)kMaxClasses) {
+        cs.clear();
+        return;
+      }
+      Class k{};
+      k.n = d.n;
+      k.bc = d.bc;
+      k.L = d.L;
+      k.h = d.h;
+      cs.push_back(k);
+      members.emplace_back();
+    }
+    members[q].push_back(g);
+    if (members[q].size() > 65535) {  // a launch's grid.y
+      cs.clear();
+      return;
+    }
+  }
+  std::vector<size_t> by(cs.size());
+  for (size_t q = 0; q < by.size(); ++q) by[q] = q;
+  std::stable_sort(by.begin(), by.end(), [&](size_t a, size_t c) { return cs[a].n > cs[c].n; });
+  std::vector<Class> sorted;
+  for (size_t q : by) {
+    Class k = cs[q];
+    k.first = (int)order.size();
+    k.count = (int)members[q].size();
+    order.insert(order.end(), members[q].begin(), members[q].end());
+    sorted.push_back(k);
+  }
+  cs = sorted;
+}
+
+// A launch per phase on the class's stream; the first error is kept.
+struct Stage {
+  mg_batch* b;
+  mg_batch::Class* k;
+  Ctl c;
+  cudaError_t e = cudaSuccess;
+
+  const int* grids() const { return b->d_class + k->first; }
+  template <typename... K, typename... A>
+  void go(void (*kernel)(K...), dim3 grid, int threads, size_t smem, A... args) {
+    if (e != cudaSuccess) return;
+    ++g_launches;
+    e = launch_after(kernel, grid, threads, smem, k->s, c, grids(), args...);
+  }
+  template <int TYPE>
+  void chunks() {
+    const int nchunk = (int)(((long long)k->n * k->n * k->n + kChunk - 1) / kChunk);
+    go(k_stage_chunks<TYPE>, dim3(nchunk, k->count), kThreads, 0);
+  }
+  void each(int type) { go(k_stage_grid, k->count, 32, 0, type); }
+
+  template <int MODE, bool ZERO, int PM, int TX>
+  void leg_t(int n, int l) {
+    using S_ = fused::Shape<MODE, TX, 16>;
+    auto kernel = k_stage_leg<MODE, ZERO, PM, TX>;
+    if (e == cudaSuccess) e = allow_smem(kernel, S_::SMEM);
+    const fused::FusedParams p =
+        leg_params(n, k->bc, k->h * (double)(1 << (k->L - 1 - l)), c.omega);
+    go(kernel, dim3((n / TX) * (n / 16) * (n / p.cz), k->count), S_::NT, S_::SMEM, l, p);
+  }
+  template <typename F>
+  static cudaError_t allow_smem(F kernel, size_t bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  }
+  template <int PM, int TX>
+  void leg(bool down, bool zero, int n, int l) {
+    if (!down) leg_t<fused::kUp, false, PM, TX>(n, l);
+    else if (zero) leg_t<fused::kDown, true, PM, TX>(n, l);
+    else leg_t<fused::kDown, false, PM, TX>(n, l);
+  }
+  void leg(bool down, bool zero, int n) {
+    int l = k->L - 1;
+    for (int m = k->n; m > n; m >>= 1) --l;
+    const bool per = k->bc == BC_PERIODIC;
+    if (per && n >= 64) leg<7, 64>(down, zero, n, l);
+    else if (per) leg<7, 32>(down, zero, n, l);
+    else if (n >= 64) leg<0, 64>(down, zero, n, l);
+    else leg<0, 32>(down, zero, n, l);
+  }
+
+  void begin() {
+    chunks<PH_SRC>();
+    each(PH_MEANFIN);
+    chunks<PH_R0>();
+    each(PH_R0FIN);
+  }
+  void iteration(bool first) {
+    const mg_opts& o = b->opts;
+    const int inner = first && o.first_cycles > 0 ? o.first_cycles : 1 + o.inner_cycles;
+    for (int q = 0; q < inner; ++q) {
+      for (int n = k->n; n >= kFusedMinN; n >>= 1)
+        leg(true, n < k->n || (q == 0 && c.inner_zero), n);
+      go(k_stage_bottom, k->count, kBottomThreads, kBottomBytes, q);
+      for (int n = kFusedMinN; n <= k->n; n <<= 1) leg(false, false, n);
+    }
+    if (first) {
+      chunks<PH_EMAX>();
+      each(PH_SETFX);
+      chunks<PH_TOFX>();
+    }
+    const int n = k->n;
+    if (e == cudaSuccess) e = allow_smem(k_stage_fx, kSmem);
+    go(k_stage_fx, dim3((n / fx_tx(n)) * (n / fx_ty(n)) * (n / fx_cz(n)), k->count), kThreads,
+       kSmem, n, first ? 1 : 0);
+    go(k_stage_fin, 1, 128, 0, k->count, b->h_left + (k - b->classes.data()));
+  }
+  void end() {
+    chunks<PH_PSUM>();
+    each(PH_PMEAN);
+    chunks<PH_PSUB>();
+  }
+  // an outer iteration after the first, as a graph from its first use on
+  void replay() {
+    if (!k->iter && e == cudaSuccess) {
+      const long long before = g_launches;
+      e = cudaStreamBeginCapture(k->s, cudaStreamCaptureModeThreadLocal);
+      if (e != cudaSuccess) return;
+      iteration(false);
+      cudaGraph_t graph = nullptr;
+      const cudaError_t ce = cudaStreamEndCapture(k->s, &graph);
+      if (e == cudaSuccess) e = ce;
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&k->iter, graph, 0);
+      if (graph) cudaGraphDestroy(graph);
+      if (e != cudaSuccess) k->iter = nullptr;
+      k->launches = g_launches - before;
+      g_launches = before;
+    }
+    if (e == cudaSuccess) e = cudaGraphLaunch(k->iter, k->s);
+    g_launches += k->launches;
+  }
+};
+
+// The streams and buffers of the staged solve, with its first use.  False
+// where they cannot be had: the persistent kernel then serves.
+bool staged_ready(mg_batch* b) {
+  if (b->start || b->classes.empty()) return b->start_ok;
+  bool ok = cudaEventCreateWithFlags(&b->start, cudaEventDisableTiming) == cudaSuccess;
+  for (auto& k : b->classes)
+    ok = ok && cudaStreamCreateWithFlags(&k.s, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&k.ev, cudaEventDisableTiming) == cudaSuccess;
+  ok = ok && cudaMallocHost(&b->h_left, sizeof(int) * b->classes.size()) == cudaSuccess;
+  if (!ok) cudaGetLastError();
+  b->start_ok = ok;
+  return ok;
+}
+
+cudaError_t staged_solve(mg_batch* b, cudaStream_t s) {
+  std::vector<mg_batch::Class>& cs = b->classes;
+  cudaError_t e = cudaMemcpyAsync(b->d_grids, b->h_grids, sizeof(GridDev) * b->ngrids,
+                                  cudaMemcpyHostToDevice, s);
+  auto also = [&](cudaError_t x) {
+    if (e == cudaSuccess) e = x;
+  };
+  also(cudaMemsetAsync(b->d_work, 0, sizeof(unsigned long long) * (kPhaseTypes + 2), s));
+  also(cudaMemsetAsync(b->d_work + kPhaseTypes, 0xff, sizeof(unsigned long long), s));
+  also(cudaEventRecord(b->start, s));
+  const Ctl c = control(b);
+  size_t open = 0;
+  auto queue = [&](mg_batch::Class& k, int what) {  // 0 start, 1 an iteration, 2 the end
+    if (e != cudaSuccess) return;
+    Stage st{b, &k, c};
+    if (what == 0) {
+      st.e = cudaStreamWaitEvent(k.s, b->start, 0);
+      st.begin();
+      st.iteration(true);
+    } else if (what == 1) {
+      st.replay();
+    } else {
+      st.end();
+    }
+    also(st.e);
+    also(cudaEventRecord(k.ev, k.s));
+    k.done = what == 0 ? 1 : k.done + 1;
+    k.last = what == 2;
+  };
+  for (auto& k : cs) {
+    queue(k, 0);
+    ++open;
+  }
+  std::vector<char> closed(cs.size(), 0);
+  while (e == cudaSuccess && open > 0) {
+    for (size_t q = 0; q < cs.size() && e == cudaSuccess; ++q) {
+      if (closed[q]) continue;
+      const cudaError_t r = cudaEventQuery(cs[q].ev);
+      if (r == cudaErrorNotReady) {
+        cudaGetLastError();
+        continue;
+      }
+      also(r);
+      if (cs[q].last) {
+        closed[q] = 1;
+        --open;
+      } else {
+        const int left = *reinterpret_cast<volatile int*>(b->h_left + q);
+        queue(cs[q], left == 0 || cs[q].done >= b->opts.max_cycles ? 2 : 1);
+      }
+    }
+    std::this_thread::yield();
+  }
+  if (e != cudaSuccess)  // nothing of this solve stays in flight
+    for (auto& k : cs) cudaStreamSynchronize(k.s);
+  also(cudaMemcpyAsync(b->h_grids, b->d_grids, sizeof(GridDev) * b->ngrids, cudaMemcpyDeviceToHost,
+                       s));
+  also(cudaMemcpyAsync(b->h_hist, b->d_hist, sizeof(double) * b->ngrids * b->hist_cap,
+                       cudaMemcpyDeviceToHost, s));
   return e;
 }
 
@@ -1067,7 +1465,11 @@ mg_status mg_batch_create(int n, const int* dims, const double* dx, const mg_bc*
   b->ntiles = tile0;
   std::vector<Phase> phases;
   std::vector<Item> items;
-  if (ok) build_phases(b, phases, items);
+  std::vector<int> order;
+  if (ok) {
+    build_phases(b, phases, items);
+    make_classes(b, order);
+  }
   b->nphases = (int)phases.size();
   b->nitems = (int)items.size();
   if (ok) {
@@ -1084,10 +1486,12 @@ mg_status mg_batch_create(int n, const int* dims, const double* dx, const mg_bc*
     b->d_err = balloc<int>(b, 1);
     b->d_active = balloc<int>(b, b->nphases);
     b->d_ptime = balloc<unsigned long long>(b, b->nphases + 1);
+    b->d_work = balloc<unsigned long long>(b, kPhaseTypes + 2);
+    b->d_class = balloc<int>(b, n);
     ok = b->d_grids && b->d_phases && b->d_items && b->d_part && b->d_part2 && b->d_ipart &&
          b->d_part3 &&
          b->d_hist && b->d_counters &&
-         b->d_bar && b->d_err && b->d_active && b->d_ptime;
+         b->d_bar && b->d_err && b->d_active && b->d_ptime && b->d_work && b->d_class;
     b->host_phases = phases;
   }
   if (ok) {
@@ -1100,6 +1504,8 @@ mg_status mg_batch_create(int n, const int* dims, const double* dx, const mg_bc*
                     cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(b->d_items, items.data(), sizeof(Item) * items.size(),
                     cudaMemcpyHostToDevice) == cudaSuccess &&
+         (order.empty() || cudaMemcpy(b->d_class, order.data(), sizeof(int) * order.size(),
+                                      cudaMemcpyHostToDevice) == cudaSuccess) &&
          cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem) ==
              cudaSuccess;
   }
@@ -1174,7 +1580,13 @@ mg_status mg_batch_solve(mg_batch* b, const double* const* rho, const double* fo
     b->h_grids[g] = d;
   }
   cudaError_t e = cudaSuccess;
-  if (!b->graph_tried) {
+  // The staged solve was faster or as fast at every size (GB300, ms, staged and
+  // persistent: 512 grids of 16-128 25.3, 35.3; one of 128 2.5, 4.3; 64 of 32
+  // 1.8, 3.1; 256 of 16 1.37, 1.36; 16 of 16 0.79, 0.94).  The persistent
+  // kernel serves callers that limit its CTAs or its barriers, and batches of
+  // more classes than streams.
+  b->staged = b->blocks == b->max_blocks && b->bar_cycles == kBarrierCycles && staged_ready(b);
+  if (!b->staged && !b->graph_tried) {
     // Capture the whole solve (upload of the per-grid arguments, counter
     // resets, the persistent kernel, download of the results) once.
     b->graph_tried = true;
@@ -1193,9 +1605,14 @@ mg_status mg_batch_solve(mg_batch* b, const double* const* rho, const double* fo
     }
     cudaGetLastError();  // a failed capture leaves the direct launch path
   }
-  ++g_launches;
-  if (b->exec) e = cudaGraphLaunch(b->exec, s);
-  else e = enqueue_solve(b, s);
+  if (b->staged) {
+    *b->h_err = 0;
+    e = staged_solve(b, s);
+  } else {
+    ++g_launches;
+    if (b->exec) e = cudaGraphLaunch(b->exec, s);
+    else e = enqueue_solve(b, s);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     b->err = std::string("mg_batch_solve: ") + cudaGetErrorString(e);
@@ -1227,10 +1644,24 @@ mg_status mg_batch_destroy(mg_batch* b) {
 
 long long mg_batch_cells(const mg_batch* b) { return b ? b->cells : 0; }
 
-int mg_batch_graph(const mg_batch* b) { return b && b->exec ? 1 : 0; }
+int mg_batch_graph(const mg_batch* b) { return b && (b->staged || b->exec) ? 1 : 0; }
 
 mg_status mg_batch_phase_ms(mg_batch* b, double* ms_by_type, int n_types) {
   if (!b || !ms_by_type || n_types < 1) return MG_ERR_ARG;
+  if (b->staged) {  // the classes overlap: the wall time by shares of the thread-clocks spent
+    unsigned long long w[kPhaseTypes + 2];
+    if (cudaMemcpy(w, b->d_work, sizeof w, cudaMemcpyDeviceToHost) != cudaSuccess) {
+      cudaGetLastError();
+      return MG_ERR_CUDA;
+    }
+    double all = 0.0;
+    for (int k = 0; k < kPhaseTypes; ++k) all += (double)w[k];
+    const double ms = w[kPhaseTypes + 1] > w[kPhaseTypes]
+                          ? (double)(w[kPhaseTypes + 1] - w[kPhaseTypes]) * 1e-6 : 0.0;
+    for (int k = 0; k < n_types; ++k)
+      ms_by_type[k] = k < kPhaseTypes && all > 0.0 ? ms * (double)w[k] / all : 0.0;
+    return MG_OK;
+  }
   std::vector<unsigned long long> t((size_t)b->nphases + 1);
   if (cudaMemcpy(t.data(), b->d_ptime, sizeof(unsigned long long) * t.size(),
                  cudaMemcpyDeviceToHost) != cudaSuccess) {

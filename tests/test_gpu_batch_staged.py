@@ -1,0 +1,64 @@
+"""The staged batched solve (a launch per phase and class of like grids) against
+the persistent kernel, which runs the same programs: the same bits, histories
+and statuses."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2302_13903_gb300 as mg
+from paper_2302_13903_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+RULES = (mg.PERIODIC, mg.FIXED, mg.ZEROGRAD)
+
+
+def solve(b, rhos, tol):
+    phis = [None if r is None else torch.full_like(r, 7.0) for r in rhos]
+    st, hists, sts = b.solve(rhos, phis, 1.0, tol)
+    return phis, st, hists, list(sts)
+
+
+@pytest.mark.parametrize("sizes,spread", [
+    ((2, 4, 8, 16), 1), ((16, 32), 1), ((32, 64, 128), 1), ((128,), 1), ((256, 2), 1),
+    ((8, 16, 32), 9),  # more classes than streams: the persistent kernel by itself
+])
+@pytest.mark.parametrize("tol", [1e-10, 1e-3])
+def test_staged_solve_gives_the_persistent_kernels_bits(sizes, spread, tol):
+    """Every rule at every size, two grids of the first class, one slot empty, a
+    grid with rho = 0; `spread` spacings."""
+    specs = [(n, bc, (1.0 + q) / n) for n in sizes for bc in RULES for q in range(spread)]
+    specs.append(specs[0])
+    rhos, fixed = [], []
+    for k, (n, bc, _) in enumerate(specs):
+        rho = inputs.batch_source(dict(n=n, bc=bc, seed=40 + k, n_blobs=3))
+        rhos.append(torch.from_numpy(rho).cuda())
+        fixed.append(0.3 if bc == mg.FIXED and k % 2 else 0.0)
+    rhos[1] = None
+    rhos[2] = torch.zeros_like(rhos[2])
+    with mg.Batch([n for n, _, _ in specs], [h for _, _, h in specs], [bc for _, bc, _ in specs],
+                  fixed) as b:
+        first = solve(b, rhos, tol)
+        again = solve(b, rhos, tol)  # its graphs replayed
+        b.set_blocks(7)
+        ref = solve(b, rhos, tol)
+    for got in (first, again):
+        assert got[1] == ref[1] and got[3] == ref[3]
+        for p, q, h, k in zip(got[0], ref[0], got[2], ref[2]):
+            assert (p is None and q is None) or torch.equal(p, q)
+            assert np.array_equal(h, k)
+
+
+def test_max_cycles_ends_every_class():
+    specs = [(16, mg.PERIODIC), (64, mg.FIXED), (32, mg.ZEROGRAD)]
+    rhos = [torch.from_numpy(inputs.batch_source(dict(n=n, bc=bc, seed=n, n_blobs=3))).cuda()
+            for n, bc in specs]
+    for m in (1, 2):
+        with mg.Batch([n for n, _ in specs], [1.0 / n for n, _ in specs], [bc for _, bc in specs],
+                      max_cycles=m) as b:
+            got = solve(b, rhos, 1e-13)
+            b.set_blocks(7)
+            ref = solve(b, rhos, 1e-13)
+        assert got[3] == ref[3] and all(len(h) == m for h in got[2])
+        for p, q in zip(got[0], ref[0]):
+            assert torch.equal(p, q)
