@@ -462,7 +462,7 @@ int mg_batch_graph(const mg_batch *batch);
 /* Device time of the last mg_batch_solve by phase kind, in milliseconds (from
  * the GPU's global timer at each grid-wide barrier of the persistent kernel,
  * else the whole solve's time by the shares of the kinds, whose launches
- * overlap, in the thread-clocks spent): ms_by_type[k] for
+ * overlap, in the SM clocks spent): ms_by_type[k] for
  * k < n_types in the order source, mean, first residual, norms of the
  * source and first residual, fused down leg, bottom levels, fused up leg, max |e|,
  * fixed-point scale, conversion to fixed point, outer step (correction and

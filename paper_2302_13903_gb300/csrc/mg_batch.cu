@@ -138,7 +138,7 @@ struct Ctl {
   int max_cycles, inner_zero;
   double stall_ratio;
   long long bar_cycles;  // a barrier wait gives up after this many clock cycles
-  unsigned long long* work;  // staged: [type] thread-clocks spent, then first start, last end (ns)
+  unsigned long long* work;  // staged: [type] SM-clocks spent, then first start, last end (ns)
 };
 
 __device__ bool grid_barrier(const Ctl& c) {
@@ -248,6 +248,7 @@ __device__ void chunk_item(const Ctl& c, GridDev& g, int chunk) {
   const double a0 = fpg * sc, b0 = mean * sc;
   const float bt = (float)(2.0 * bcval * inv_h2 * sc);  // one fixed-value ghost term, scaled
   const double c2 = h * h * two_S;
+  float em = 0.f;
   float af = 0.f, ar = 0.f;  // FP32 sums over at most 8 cells, then added in FP64
   double acc2 = 0.0;
   int nf = 0;
@@ -339,7 +340,7 @@ __device__ void chunk_item(const Ctl& c, GridDev& g, int chunk) {
       mb = b1 > mb ? b1 : mb;
     } else if (TYPE == PH_EMAX) {
       const float2 v = reinterpret_cast<const float2*>(e32)[t2];
-      mx = fmax(mx, (double)fmaxf(fabsf(v.x), fabsf(v.y)));
+      em = fmaxf(em, fmaxf(fabsf(v.x), fabsf(v.y)));
     } else if (TYPE == PH_PSUM) {
       const longlong2 v = reinterpret_cast<const longlong2*>(PHI)[t2];
       s_hi += (v.x >> 32) + (v.y >> 32);
@@ -359,6 +360,7 @@ __device__ void chunk_item(const Ctl& c, GridDev& g, int chunk) {
     if (threadIdx.x == 0) c.part2[g.chunk0 + chunk] = b;
   }
   if (TYPE == PH_SRC) mx = __longlong_as_double((long long)mb);
+  if (TYPE == PH_EMAX) mx = em;
   if (TYPE == PH_SRC || TYPE == PH_EMAX) {
     const double b = block_max(mx);
     if (threadIdx.x == 0) c.part2[g.chunk0 + chunk] = b;
@@ -443,6 +445,17 @@ struct TileRing {
   float he[kRing][kThreads];
 };
 static_assert(kPlaneBytes + sizeof(TileRing) <= kSmem, "outer-step ring exceeds the CTA's smem");
+
+// Sum over a tile's columns of each column's FP32 sum over its planes, in an
+// order that does not depend on which thread had the column; in thread 0.
+__device__ __forceinline__ double column_sum(const float* sq, int cols) {
+  double v = 0.0;
+  if (threadIdx.x < 32) {
+    for (int q = threadIdx.x; q < cols; q += 32) v += sq[q];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  }
+  return v;
+}
 
 __device__ void fx_tile_item(const Ctl& c, GridDev& g, const Item& I, bool zero_in,
                              float4* smem) {
@@ -535,7 +548,7 @@ __device__ void fx_tile_item(const Ctl& c, GridDev& g, const Item& I, bool zero_
     zm[k] = cact[k] ? own_at(k, z0 - 1) : 0;
     self[k] = cact[k] ? own_at(k, z0) : 0;
   }
-  float acc = 0.f;
+  float acc[kFxCols] = {};
   bool bad = false;
   for (int z = z0; z < z1; ++z) {
     issue(z + 2);
@@ -577,7 +590,7 @@ __device__ void fx_tile_item(const Ctl& c, GridDev& g, const Item& I, bool zero_
       const long long R = ring.f[sl][k][tid] - (((xm + xp) + (ym + yp)) + (zmv + zpv) - 6 * sv);
       const float r = __ll2float_rn(R) * rfac;
       r32[o] = r;
-      acc = fmaf(r, r, acc);
+      acc[k] = fmaf(r, r, acc[k]);
       zm[k] = sv;
       self[k] = zp;
     }
@@ -586,8 +599,14 @@ __device__ void fx_tile_item(const Ctl& c, GridDev& g, const Item& I, bool zero_
   }
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   if (bad) atomicOr(&g.fxbad, 1);
-  const double b = block_sum((double)acc);
-  if (threadIdx.x == 0) c.part3[g.part0 + (I.c * (n / TY) + I.b) * (n / TX) + I.a] = b;
+  __syncthreads();  // every thread has read its last plane
+  float* sq = reinterpret_cast<float*>(smem);
+#pragma unroll
+  for (int k = 0; k < kFxCols; ++k)
+    if (cact[k]) sq[tid + k * kThreads] = acc[k];
+  __syncthreads();
+  const double b = column_sum(sq, cols);
+  if (tid == 0) c.part3[g.part0 + (I.c * (n / TY) + I.b) * (n / TX) + I.a] = b;
 }
 
 // Stopping rule of the single-grid solve, after one outer iteration.
@@ -840,20 +859,22 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(Ctl c) {
 // SM) and constants, and one class's last wave is filled by the others.  The
 // items are the persistent kernel's programs: the same bits.
 
-// What the phase cost, for the shares in mg_batch_phase_ms.
+// What the phase cost, for the shares in mg_batch_phase_ms: the CTA's clocks
+// over the CTAs that fill an SM.
 struct Meter {
   unsigned long long* w;
-  int type;
+  int type, per_sm;
   long long t0;
-  __device__ Meter(const Ctl& c, int type_) {
+  __device__ Meter(const Ctl& c, int type_, int per_sm_) {
     w = c.work;
     type = type_;
+    per_sm = per_sm_;
     t0 = clock64();
     if (threadIdx.x == 0 && type == PH_SRC) atomicMin(w + kPhaseTypes, global_ns());
   }
   __device__ void stop() {
     if (threadIdx.x != 0) return;
-    atomicAdd(w + type, (unsigned long long)(clock64() - t0) * blockDim.x);
+    atomicAdd(w + type, (unsigned long long)(clock64() - t0) / per_sm);
     if (type == PH_PSUB) atomicMax(w + kPhaseTypes + 1, global_ns());
   }
 };
@@ -864,7 +885,7 @@ __global__ void __launch_bounds__(kThreads) k_stage_chunks(const __grid_constant
   dev::after_previous();
   GridDev& g = c.grids[grids[blockIdx.y]];
   if (!runs(g, TYPE)) return;
-  Meter m(c, TYPE);
+  Meter m(c, TYPE, 9);
   chunk_item<TYPE>(c, g, blockIdx.x);
   m.stop();
 }
@@ -874,7 +895,7 @@ __global__ void k_stage_grid(const __grid_constant__ Ctl c, const int* grids, in
   const int gi = grids[blockIdx.x];
   GridDev& g = c.grids[gi];
   if (!runs(g, type)) return;
-  Meter m(c, type);
+  Meter m(c, type, 32);
   if (threadIdx.x == 0) grid_item(c, g, type, gi);
   m.stop();
 }
@@ -883,7 +904,7 @@ __global__ void k_stage_grid(const __grid_constant__ Ctl c, const int* grids, in
 // page-locked memory, where the host reads it.
 __global__ void k_stage_fin(const __grid_constant__ Ctl c, const int* grids, int count, int* left) {
   dev::after_previous();
-  Meter m(c, PH_FIN);
+  Meter m(c, PH_FIN, 16);
   int n = 0;
   for (int q = threadIdx.x; q < count; q += blockDim.x) {
     GridDev& g = c.grids[grids[q]];
@@ -903,15 +924,154 @@ __global__ void k_stage_fin(const __grid_constant__ Ctl c, const int* grids, int
   }
 }
 
+// The outer step on grids too small for a tile of 32 x 16 columns.
 __global__ void __launch_bounds__(kThreads) k_stage_fx(const __grid_constant__ Ctl c,
                                                        const int* grids, int n, int zero_in) {
   dev::after_previous();
   extern __shared__ float4 smem[];
   GridDev& g = c.grids[grids[blockIdx.y]];
   if (!runs(g, PH_FXSTEP)) return;
-  Meter m(c, PH_FXSTEP);
+  Meter m(c, PH_FXSTEP, 3);
   const int nx = n / fx_tx(n), ny = n / fx_ty(n), t = blockIdx.x;
   fx_tile_item(c, g, Item{0, t % nx, t / nx % ny, t / (nx * ny)}, zero_in != 0, smem);
+  m.stop();
+}
+
+// fx_tile_item on grids of at least 32 cells a side, as the single-grid step: a
+// column per thread, the ring's slots and the rule known at compile time, the
+// correction rounded in integer arithmetic (with it and the residual's
+// conversion both on the FP64 pipe, that pipe bounds the step).
+constexpr int kFxThreads = 512;  // 32 x 16 columns
+struct FxStageRing {
+  long long p[kRing][kFxThreads], f[kRing][kFxThreads];
+  float e[kRing][kFxThreads];
+  long long hp[kRing][128];
+  float he[kRing][128];
+};
+
+template <bool PER, bool ZERO_IN>
+__global__ void __launch_bounds__(kFxThreads, 3) k_stage_fx_tile(const __grid_constant__ Ctl c,
+                                                                 const int* grids, int n) {
+  dev::after_previous();
+  GridDev& g = c.grids[grids[blockIdx.y]];
+  if (!runs(g, PH_FXSTEP)) return;
+  Meter m(c, PH_FXSTEP, 3);
+  __shared__ long long P[2][18][34];
+  extern __shared__ float4 smem[];
+  FxStageRing& ring = *reinterpret_cast<FxStageRing*>(smem);
+  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+  const int nx = n >> 5, ny = n >> 4;
+  const int x0 = ((int)blockIdx.x & (nx - 1)) << 5;
+  const int y0 = (((int)blockIdx.x / nx) & (ny - 1)) << 4, z0 = (int)blockIdx.x / (nx * ny) * 32;
+  const int z1 = z0 + 32;
+  const int i = x0 + tx, j = y0 + ty;
+  const unsigned plane = (unsigned)n * n, col = (unsigned)j * n + i;
+  const long long* pin = g.cur ? g.fx2 : reinterpret_cast<const long long*>(g.phi);
+  long long* const pout = g.cur ? reinterpret_cast<long long*>(g.phi) : g.fx2;
+  const long long* const FX = reinterpret_cast<const long long*>(g.f64);
+  const float* const e = g.u32[g.L - 1];
+  float* const r32 = g.f32[g.L - 1];
+  const float ce = (float)(g.two_S / g.scale);
+  const float rfac = (float)(1.0 / (g.rn * g.h * g.h * g.two_S));
+  // the ghost across a wall: (self ^ flip) - flip + shift (self, or 2 b - self)
+  const long long flip = g.bc == BC_ZEROGRAD ? 0 : -1, shift = g.bc == BC_ZEROGRAD ? 0 : g.b2;
+  // the halo cell this thread loads: rows -1 and 16 over the full width,
+  // columns -1 and 32 over the tile's rows
+  const bool halo = tid < 2 * 34 + 2 * 16;
+  int ha = 0, hb = 0;
+  if (halo) {
+    if (tid < 34) { ha = tid; }
+    else if (tid < 68) { ha = tid - 34; hb = 17; }
+    else if (tid < 84) { hb = tid - 67; }
+    else { ha = 33; hb = tid - 83; }
+  }
+  int hx = x0 - 1 + ha, hy = y0 - 1 + hb;
+  const bool h_in = halo && (PER || (hx >= 0 && hx < n && hy >= 0 && hy < n));
+  hx &= n - 1;
+  hy &= n - 1;
+  const unsigned hcol = h_in ? (unsigned)hy * n + hx : 0u;
+  // slot of plane q: (q - z0 + 1) mod 4
+  auto issue = [&](auto SLc, int q) {
+    constexpr int sl = decltype(SLc)::value & 3;
+    if (q <= z1) {
+      const bool in = PER || (q >= 0 && q < n);
+      const unsigned o = (unsigned)(q & (n - 1)) * plane + col;
+      if (!ZERO_IN) ring_cp8(&ring.p[sl][tid], pin + o, in ? 8 : 0);
+      ring_cp4(&ring.e[sl][tid], e + o, in ? 4 : 0);
+      if (q >= z0 && q < z1) {
+        ring_cp8(&ring.f[sl][tid], FX + o, 8);
+        if (halo) {
+          const unsigned ho = (unsigned)q * plane + hcol;
+          if (!ZERO_IN) ring_cp8(&ring.hp[sl][tid], pin + ho, h_in ? 8 : 0);
+          ring_cp4(&ring.he[sl][tid], e + ho, h_in ? 4 : 0);
+        }
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  bool bad = false;
+  auto own_at = [&](auto SLc) -> long long {
+    constexpr int sl = decltype(SLc)::value & 3;
+    const float x = ring.e[sl][tid] * ce;
+    bad |= x != x;  // the integer rounding takes NaN to 0
+    return (ZERO_IN ? 0 : ring.p[sl][tid]) + cvt::f2ll_rn(x);
+  };
+  using std::integral_constant;
+  issue(integral_constant<int, 0>{}, z0 - 1);
+  issue(integral_constant<int, 1>{}, z0);
+  issue(integral_constant<int, 2>{}, z0 + 1);
+  asm volatile("cp.async.wait_group 1;\n" ::: "memory");  // planes z0 - 1, z0 landed
+  long long zm = own_at(integral_constant<int, 0>{}), self = own_at(integral_constant<int, 1>{});
+  float acc = 0.f;
+  auto step = [&](auto Jc, int z) {
+    constexpr int J = decltype(Jc)::value, sl = (J + 1) & 3, buf = J & 1;
+    issue(integral_constant<int, J + 3>{}, z + 2);
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");  // every plane up to z + 1
+    const unsigned o = (unsigned)z * plane + col;
+    const long long zp = own_at(integral_constant<int, J + 2>{});
+    P[buf][ty + 1][tx + 1] = self;
+    if (halo) {
+      const long long hv = (ZERO_IN ? 0 : ring.hp[sl][tid]) + cvt::f2ll_rn(ring.he[sl][tid] * ce);
+      P[buf][hb][ha] = h_in ? hv : 0;
+    }
+    pout[o] = self;
+    bad |= (unsigned long long)(self + (1LL << 60)) > (2ULL << 60);  // |PHI'| > 2^60
+    __syncthreads();
+    long long xm = P[buf][ty + 1][tx], xp = P[buf][ty + 1][tx + 2];
+    long long ym = P[buf][ty][tx + 1], yp = P[buf][ty + 2][tx + 1];
+    long long zl = zm, zh = zp;
+    if (!PER) {
+      const long long gh = (self ^ flip) - flip + shift;
+      if (i == 0) xm = gh;
+      if (i == n - 1) xp = gh;
+      if (j == 0) ym = gh;
+      if (j == n - 1) yp = gh;
+      if (z == 0) zl = gh;
+      if (z == n - 1) zh = gh;
+    }
+    const long long R = ring.f[sl][tid] - (((xm + xp) + (ym + yp)) + (zl + zh) - 6 * self);
+    const float r = __ll2float_rn(R) * rfac;
+    r32[o] = r;
+    acc = fmaf(r, r, acc);
+    zm = self;
+    self = zp;
+    // the next plane writes the other half of P; this one is rewritten two
+    // planes on, after every thread has passed the next barrier
+  };
+  for (int z = z0; z < z1; z += 4) {
+    step(integral_constant<int, 0>{}, z);
+    step(integral_constant<int, 1>{}, z + 1);
+    step(integral_constant<int, 2>{}, z + 2);
+    step(integral_constant<int, 3>{}, z + 3);
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  if (bad) atomicOr(&g.fxbad, 1);
+  __syncthreads();
+  float* sq = reinterpret_cast<float*>(P);
+  sq[tid] = acc;
+  __syncthreads();
+  const double b = column_sum(sq, kFxThreads);
+  if (tid == 0) c.part3[g.part0 + blockIdx.x] = b;
   m.stop();
 }
 
@@ -921,7 +1081,7 @@ __global__ void __launch_bounds__(kBottomThreads) k_stage_bottom(const __grid_co
   extern __shared__ float4 smem[];
   const GridDev& g = c.grids[grids[blockIdx.x]];
   if (!runs(g, PH_BOTTOM)) return;
-  Meter m(c, PH_BOTTOM);
+  Meter m(c, PH_BOTTOM, 1);
   bottom_item(c, g, cycle, smem);
   m.stop();
 }
@@ -935,7 +1095,7 @@ __global__ void __maxnreg__((fused::fused_max_regs<MODE, 16, PM>()))
   const GridDev& g = c.grids[grids[blockIdx.y]];
   constexpr int type = MODE == fused::kDown ? PH_DOWN : PH_UP;
   if (!runs(g, type)) return;
-  Meter m(c, type);
+  Meter m(c, type, MODE == fused::kUp && PM == 7 ? 3 : 2);
   const int nx = p.nx / TX, ny = p.nx / 16, t = blockIdx.x;
   constexpr bool UP = MODE == fused::kUp;
   fused::fused_tile<MODE, ZERO, PM, TX, 16>(UP ? g.u32b[l] : g.u32[l], UP ? g.u32[l] : g.u32b[l],
@@ -1283,9 +1443,17 @@ struct Stage {
       chunks<PH_TOFX>();
     }
     const int n = k->n;
-    if (e == cudaSuccess) e = allow_smem(k_stage_fx, kSmem);
-    go(k_stage_fx, dim3((n / fx_tx(n)) * (n / fx_ty(n)) * (n / fx_cz(n)), k->count), kThreads,
-       kSmem, n, first ? 1 : 0);
+    const dim3 tiles((n / fx_tx(n)) * (n / fx_ty(n)) * (n / fx_cz(n)), k->count);
+    if (n >= 32) {
+      const bool per = k->bc == BC_PERIODIC;
+      auto kernel = per ? (first ? k_stage_fx_tile<true, true> : k_stage_fx_tile<true, false>)
+                        : (first ? k_stage_fx_tile<false, true> : k_stage_fx_tile<false, false>);
+      if (e == cudaSuccess) e = allow_smem(kernel, sizeof(FxStageRing));
+      go(kernel, tiles, kFxThreads, sizeof(FxStageRing), n);
+    } else {
+      if (e == cudaSuccess) e = allow_smem(k_stage_fx, kSmem);
+      go(k_stage_fx, tiles, kThreads, kSmem, n, first ? 1 : 0);
+    }
     go(k_stage_fin, 1, 128, 0, k->count, b->h_left + (k - b->classes.data()));
   }
   void end() {
@@ -1648,7 +1816,7 @@ int mg_batch_graph(const mg_batch* b) { return b && (b->staged || b->exec) ? 1 :
 
 mg_status mg_batch_phase_ms(mg_batch* b, double* ms_by_type, int n_types) {
   if (!b || !ms_by_type || n_types < 1) return MG_ERR_ARG;
-  if (b->staged) {  // the classes overlap: the wall time by shares of the thread-clocks spent
+  if (b->staged) {  // the classes overlap: the wall time by shares of the SM clocks spent
     unsigned long long w[kPhaseTypes + 2];
     if (cudaMemcpy(w, b->d_work, sizeof w, cudaMemcpyDeviceToHost) != cudaSuccess) {
       cudaGetLastError();
