@@ -58,7 +58,7 @@ constexpr int kMaxL = 16;
 constexpr int kMaxClasses = 24;  // streams of a staged solve
 constexpr int kChunk = 32768;   // cells per chunk item
 constexpr int kFusedMinN = 32;  // levels of at least 32^3 use the fused tiles
-constexpr int kCz = 64;         // z-chunk of fused tiles
+constexpr int kCz = 64;         // z-chunk of fused tiles (the most, in a staged solve)
 constexpr long long kBarrierCycles = 4000000000LL;  // ~2 s at 2 GHz
 
 struct GridDev {
@@ -1398,8 +1398,17 @@ struct Stage {
     using S_ = fused::Shape<MODE, TX, 16>;
     auto kernel = k_stage_leg<MODE, ZERO, PM, TX>;
     if (e == cudaSuccess) e = allow_smem(kernel, S_::SMEM);
-    const fused::FusedParams p =
+    fused::FusedParams p =
         leg_params(n, k->bc, k->h * (double)(1 << (k->L - 1 - l)), c.omega);
+    // z-chunks of 64 planes, halved down to 8 until the batch's classes, each by
+    // its share of the cells, have four CTAs per SM: shorter chunks recompute
+    // more halo planes, but a march of 64 planes is all the time a leg of few
+    // tiles takes (GB300, ms, always 64 and so: one grid of 128^3 2.48, 1.30; 8
+    // of 64^3 3.05, 1.69; 129 of 16-128 7.46, 6.42; 512 of 16-128 23.9, 23.8;
+    // four per SM for each class: 512 of 16-128 24.9)
+    const double share = (double)k->count * k->n * k->n * k->n / (double)b->cells;
+    const long long cols = (long long)k->count * (n / TX) * (n / 16);
+    while (p.cz > 8 && (double)(cols * (n / p.cz)) < 4.0 * share * sm_count()) p.cz /= 2;
     go(kernel, dim3((n / TX) * (n / 16) * (n / p.cz), k->count), S_::NT, S_::SMEM, l, p);
   }
   template <typename F>
@@ -1749,8 +1758,8 @@ mg_status mg_batch_solve(mg_batch* b, const double* const* rho, const double* fo
   }
   cudaError_t e = cudaSuccess;
   // The staged solve was faster or as fast at every size (GB300, ms, staged and
-  // persistent: 512 grids of 16-128 25.3, 35.3; one of 128 2.5, 4.3; 64 of 32
-  // 1.8, 3.1; 256 of 16 1.37, 1.36; 16 of 16 0.79, 0.94).  The persistent
+  // persistent: 512 grids of 16-128 23.8, 35.5; one of 128 1.30, 4.3; 64 of 32
+  // 1.57, 3.1; 256 of 16 1.38, 1.36; 16 of 16 0.79, 0.94).  The persistent
   // kernel serves callers that limit its CTAs or its barriers, and batches of
   // more classes than streams.
   b->staged = b->blocks == b->max_blocks && b->bar_cycles == kBarrierCycles && staged_ready(b);
