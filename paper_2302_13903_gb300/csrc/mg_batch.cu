@@ -703,40 +703,34 @@ __device__ __forceinline__ bool runs(const GridDev& g, int type) {
   return !g.skip && (type == PH_PSUM ? has_mean : (type > PH_PSUM || g.active));
 }
 
-// The levels of at most 16^3 of one V-cycle, by one CTA, in its dynamic shared
-// memory (kBottomBytes): a chain of some 25 dependent passes over at most 4096
-// cells, so what counts is the latency of a load.
-constexpr size_t kBottomBytes = 2 * (4096 + 512 + 64 + 8 + 1) * sizeof(float);
+// The levels of at most 16^3 of one V-cycle, by one CTA (cf and ih2 of
+// bottom_params).
+constexpr size_t kBottomBytes = bottom::kBytes;
 static_assert(kBottomBytes <= kSmem, "the bottom levels exceed the CTA's smem");
+static_assert(bottom::kTopN == kFusedMinN / 2, "the bottom starts below the fused levels");
 
-__device__ void bottom_item(const Ctl& c, const GridDev& g, int cycle, float4* smem) {
-  // the arguments in shared memory: their per-level arrays are indexed by a
-  // run-time level, which in each thread's own copy would put them in local
-  // memory
-  __shared__ bottom::BottomArgs<float> a;
-  const int top = level_of(g, min(g.n, kFusedMinN / 2));
-  if (threadIdx.x == 0) {
-    for (int l = 0; l < kBottomLevels; ++l) {
-      const bool used = l <= top;
-      a.u[l] = used ? g.u32[l] : nullptr;
-      a.f[l] = used ? g.f32[l] : nullptr;
-      a.n[l] = used ? (g.n >> (g.L - 1 - l)) : 0;
-      a.h[l] = used ? g.h * (double)(1 << (g.L - 1 - l)) : 0.0;
-      a.bc[l] = hom_bc(g);
-    }
-    a.hom = hom_bc(g);
-    a.omega = c.omega;
-    a.pre = 1;
-    a.post = 1;
-    a.top = top;
-    a.fmg = 0;
-    bottom::set_coefficients(a);
-  }
-  __syncthreads();
-  const bool zg = (top < g.L - 1) || (cycle == 0 && c.inner_zero);
-  bottom::in_shared(a, reinterpret_cast<float*>(smem), !zg, [&](const bottom::BottomArgs<float>& b) {
-    bottom::vcycle<float, false>(b, top, b.hom, zg);
-  });
+__device__ __forceinline__ void bottom_item(const Ctl& c, const GridDev& g, int cycle, float cf,
+                                            float ih2, float4* smem) {
+  const int n = min(g.n, bottom::kTopN), top = level_of(g, n);
+  bottom::Args a;
+  a.u = g.u32[top];
+  a.f = g.f32[top];
+  a.zero = top < g.L - 1 || (cycle == 0 && c.inner_zero);
+  a.sgn = g.bc == BC_ZEROGRAD ? 1.f : -1.f;
+  a.cu = (float)(1.0 - c.omega);
+  a.cs = (float)(c.omega / 6.0);
+  a.cf = cf;
+  a.ih2 = ih2;
+  bottom::vcycle(n, g.bc == BC_PERIODIC, reinterpret_cast<float*>(smem), a);
+}
+
+// cf and ih2 of the bottom's top level on a grid of n cells a side.
+struct BottomParams {
+  float cf, ih2;
+};
+__host__ __device__ inline BottomParams bottom_params(int n, double h, double omega) {
+  for (; n > bottom::kTopN; n /= 2) h *= 2.0;
+  return {(float)(-omega * h * h / 6.0), (float)(1.0 / (h * h))};
 }
 
 // The constants of a leg on level l (n^3 cells) of grid g.
@@ -823,7 +817,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(Ctl c) {
             if (g.active) atomicAdd(&c.active_left[ph], 1);
           }
           break;
-        case PH_BOTTOM: bottom_item(c, g, P.cycle, smem); break;
+        case PH_BOTTOM: {
+          __shared__ BottomParams bp;
+          if (threadIdx.x == 0) bp = bottom_params(g.n, g.h, c.omega);
+          __syncthreads();
+          bottom_item(c, g, P.cycle, bp.cf, bp.ih2, smem);
+          break;
+        }
         case PH_DOWN:
         case PH_UP: {
           const int l = level_of(g, P.n);
@@ -1076,13 +1076,14 @@ __global__ void __launch_bounds__(kFxThreads, 3) k_stage_fx_tile(const __grid_co
 }
 
 __global__ void __launch_bounds__(kBottomThreads) k_stage_bottom(const __grid_constant__ Ctl c,
-                                                                 const int* grids, int cycle) {
+                                                                 const int* grids, int cycle,
+                                                                 BottomParams p) {
   dev::after_previous();
   extern __shared__ float4 smem[];
   const GridDev& g = c.grids[grids[blockIdx.x]];
   if (!runs(g, PH_BOTTOM)) return;
-  Meter m(c, PH_BOTTOM, 1);
-  bottom_item(c, g, cycle, smem);
+  Meter m(c, PH_BOTTOM, 2);
+  bottom_item(c, g, cycle, p.cf, p.ih2, smem);
   m.stop();
 }
 
@@ -1443,7 +1444,8 @@ struct Stage {
     for (int q = 0; q < inner; ++q) {
       for (int n = k->n; n >= kFusedMinN; n >>= 1)
         leg(true, n < k->n || (q == 0 && c.inner_zero), n);
-      go(k_stage_bottom, k->count, kBottomThreads, kBottomBytes, q);
+      go(k_stage_bottom, k->count, kBottomThreads, kBottomBytes, q,
+         bottom_params(k->n, k->h, c.omega));
       for (int n = kFusedMinN; n <= k->n; n <<= 1) leg(false, false, n);
     }
     if (first) {
@@ -1758,8 +1760,8 @@ mg_status mg_batch_solve(mg_batch* b, const double* const* rho, const double* fo
   }
   cudaError_t e = cudaSuccess;
   // The staged solve was faster or as fast at every size (GB300, ms, staged and
-  // persistent: 512 grids of 16-128 23.8, 35.5; one of 128 1.30, 4.3; 64 of 32
-  // 1.57, 3.1; 256 of 16 1.38, 1.36; 16 of 16 0.79, 0.94).  The persistent
+  // persistent: 512 grids of 16-128 22.8, 34.2; one of 128 1.13, 3.9; 64 of 32
+  // 1.39, 2.6; 256 of 16 0.99, 0.99; 16 of 16 0.57, 0.58).  The persistent
   // kernel serves callers that limit its CTAs or its barriers, and batches of
   // more classes than streams.
   b->staged = b->blocks == b->max_blocks && b->bar_cycles == kBarrierCycles && staged_ready(b);

@@ -215,9 +215,6 @@ struct CoarseCall {
 template <typename T>
 cudaError_t launch_coarse(const CoarseCall<T>& q, cudaStream_t s);
 
-// Levels the batched solver's bottom programs hold (mg_bottom.cuh).
-constexpr int kBottomLevels = 6;
-
 // ---------------------------------------------------------------------------
 // Fused FP32 V-cycle legs (homogeneous rules only).  Each reads u_in and
 // writes u_out (distinct buffers).
