@@ -790,11 +790,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(Ctl c) {
       if (threadIdx.x == 0) s_item = (int)atomicAdd(&c.counters[ph], 1u);
       __syncthreads();
       const int it = s_item;
+      const Item I = c.items[P.first + min(it, P.count - 1)];
+      GridDev& g = c.grids[I.grid];
+      const bool run = runs(g, P.type);  // before any thread of this CTA changes it
       __syncthreads();
       if (it >= P.count) break;
-      const Item I = c.items[P.first + it];
-      GridDev& g = c.grids[I.grid];
-      if (!runs(g, P.type)) continue;
+      if (!run) continue;
       switch (P.type) {
         case PH_SRC: chunk_item<PH_SRC>(c, g, I.a); break;
         case PH_R0: chunk_item<PH_R0>(c, g, I.a); break;
