@@ -433,8 +433,8 @@ def run_per_face(args, stream):
 
 
 def run_batched(args, ws, rank, stream):
-    """512 grids of {16,32,64,128}^3 (Zipf weights), mixed rules, one persistent
-    graph-captured launch per solve; under torchrun each rank takes its LPT share."""
+    """512 grids of {16,32,64,128}^3 (Zipf weights), mixed rules, in one
+    mg_batch_solve; under torchrun each rank takes its LPT share."""
     import torch
 
     import paper_2302_13903_gb300 as mg
@@ -471,8 +471,8 @@ def run_batched(args, ws, rank, stream):
             "phase_ms": phases,
             "workload": "512 grids, sizes {16,32,64,128}^3 with Zipf 1/rank weights, rules "
                         "periodic / fixed 0 / zero gradient, 1-8 Gaussian blobs each; FP32 "
-                        "multigrid inside FP64 defect correction to 1e-10; one persistent "
-                        "cooperative launch captured as a CUDA graph"}
+                        "multigrid inside FP64 defect correction to 1e-10; a launch per phase "
+                        "and class of like grids, later outer iterations as CUDA graphs"}
 
 
 def run_serving(args):

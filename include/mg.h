@@ -412,7 +412,7 @@ mg_status mg_op_multipole_moments_noalloc(int nx, int ny, int nz, double h, cons
                                           double *Q_host, void *stream);
 
 /* ------------------------------------------------------------------------
- * Batched solve: many independent grids in one persistent launch.
+ * Batched solve: many independent grids solved together.
  * ---------------------------------------------------------------------- */
 typedef struct mg_batch mg_batch;
 
