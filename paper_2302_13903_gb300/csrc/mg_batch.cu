@@ -374,16 +374,30 @@ __device__ void chunk_item(const Ctl& c, GridDev& g, int chunk) {
   }
 }
 
+// Sum (and maximum) of n partials by warp 0, in an order that depends on n alone;
+// in every lane.  One thread's chain of adds on loads from L2 (64 to 1024 partials)
+// cost two grids of 256^3 5.33 ms a solve against 4.98, one of 128^3 1.12 against
+// 1.09 (GB300).
+template <typename T>
+__device__ __forceinline__ T lane_sum(const T* p, int n, int step = 1) {
+  T v = 0;
+  for (int q = threadIdx.x; q < n; q += 32) v += p[(size_t)q * step];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 __device__ double chunk_max(const Ctl& c, const GridDev& g) {
   double m = 0.0;
-  for (int q = 0; q < g.nchunk; ++q) m = fmax(m, c.part2[g.chunk0 + q]);
+  for (int q = threadIdx.x; q < g.nchunk; q += 32) m = fmax(m, c.part2[g.chunk0 + q]);
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
   return m;
 }
 
 // The fixed-point scale of one grid after its first inner solve: 2^S the
 // largest power of two keeping |PHI| < 2^55 and |h^2 f 2^S| < 2^58.
 __device__ void setfx_item(const Ctl& c, GridDev& g) {
-  const double mphi = chunk_max(c, g) / g.scale;  // phi = e / scale after this step
+  const double me = chunk_max(c, g);
+  if (threadIdx.x != 0) return;
+  const double mphi = me / g.scale;  // phi = e / scale after this step
   const double mfh = g.maxf * g.h * g.h;
   double lim = 0.0;
   if (mphi > 0.0) lim = 36028797018963968.0 / mphi;                    // 2^55
@@ -396,12 +410,6 @@ __device__ void setfx_item(const Ctl& c, GridDev& g) {
   g.two_S = ldexp(1.0, e2 - 1);
   g.b2 = g.bc == BC_FIXED ? __double2ll_rn(2.0 * g.bcval * g.two_S) : 0;
   g.in_fx = 1;
-}
-
-__device__ double chunk_total(const Ctl& c, const GridDev& g) {
-  double s = 0.0;
-  for (int q = 0; q < g.nchunk; ++q) s += c.part[g.chunk0 + q];
-  return s;
 }
 
 // Tile sizes of the fixed-point step: TX x TY columns, FXCZ planes.
@@ -609,12 +617,12 @@ __device__ void fx_tile_item(const Ctl& c, GridDev& g, const Item& I, bool zero_
   if (tid == 0) c.part3[g.part0 + (I.c * (n / TY) + I.b) * (n / TX) + I.a] = b;
 }
 
-// Stopping rule of the single-grid solve, after one outer iteration.
+// Stopping rule of the single-grid solve, after one outer iteration (by warp 0).
 __device__ void fin_item(const Ctl& c, GridDev& g, int gi) {
   const double N = (double)g.n * g.n * g.n;
   // the outer step summed the squares of r32 = r / rn_previous, per tile
-  double tot = 0.0;
-  for (int q = 0; q < g.ntile; ++q) tot += c.part3[g.part0 + q];
+  const double tot = lane_sum(c.part3 + g.part0, g.ntile);
+  if (threadIdx.x != 0) return;
   const double rn = sqrt(tot / N) * g.rn;
   g.cur ^= 1;  // the step wrote the other integer buffer
   double r = rn / g.fnorm;
@@ -638,22 +646,24 @@ __device__ void fin_item(const Ctl& c, GridDev& g, int gi) {
   }
 }
 
-// The phases that are one thread's work on one grid (index gi).
+// The phases that are warp 0's work on one grid (index gi).
 __device__ void grid_item(const Ctl& c, GridDev& g, int type, int gi) {
   const double N = (double)g.n * g.n * g.n;
   switch (type) {
-    case PH_MEANFIN:
-      g.mean = (g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD) ? g.fpg * (chunk_total(c, g) / N) : 0.0;
+    case PH_MEANFIN: {
+      const double total = lane_sum(c.part + g.chunk0, g.nchunk), mx = chunk_max(c, g);
+      if (threadIdx.x != 0) break;
+      g.mean = (g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD) ? g.fpg * (total / N) : 0.0;
       // max |f - mean| <= |4 pi G| max |rho| + |mean|: the scale of r32 and of 2^S
-      g.maxf = fabs(g.fpg) * chunk_max(c, g) + fabs(g.mean);
+      g.maxf = fabs(g.fpg) * mx + fabs(g.mean);
       g.scale = g.maxf > 0.0 ? 1.0 / g.maxf : 1.0;
       break;
+    }
     case PH_R0FIN: {
-      double fs = 0.0, rs = 0.0;  // sums of ((f - mean) sc)^2 and (r0 sc)^2
-      for (int q = 0; q < g.nchunk; ++q) {
-        fs += c.part[g.chunk0 + q];
-        rs += c.part2[g.chunk0 + q];
-      }
+      // sums of ((f - mean) sc)^2 and (r0 sc)^2
+      const double fs = lane_sum(c.part + g.chunk0, g.nchunk);
+      const double rs = lane_sum(c.part2 + g.chunk0, g.nchunk);
+      if (threadIdx.x != 0) break;
       g.fnorm = sqrt(fs / N) / g.scale;
       g.rn = sqrt(rs / N) / g.scale;
       if (g.fnorm == 0.0) g.fnorm = g.rn > 0.0 ? g.rn : 1.0;
@@ -667,14 +677,14 @@ __device__ void grid_item(const Ctl& c, GridDev& g, int type, int gi) {
     }
     case PH_SETFX: setfx_item(c, g); break;
     case PH_PMEAN: {
+      // exact integer total, independent of the chunking
+      const bool fx = (g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD) && g.in_fx;
+      const long long th = fx ? lane_sum(c.ipart + 2 * (size_t)g.chunk0, g.nchunk, 2) : 0;
+      const long long tl = fx ? lane_sum(c.ipart + 2 * (size_t)g.chunk0 + 1, g.nchunk, 2) : 0;
+      if (threadIdx.x != 0) break;
       double m = 0.0;
       if (g.bc == BC_PERIODIC || g.bc == BC_ZEROGRAD) {
-        if (g.in_fx) {  // exact integer total, independent of the chunking
-          long long th = 0, tl = 0;
-          for (int q = 0; q < g.nchunk; ++q) {
-            th += c.ipart[2 * (g.chunk0 + q)];
-            tl += c.ipart[2 * (g.chunk0 + q) + 1];
-          }
+        if (fx) {
           m = ((double)th * 4294967296.0 + (double)tl) / (N * g.two_S);
           // the same mean as an integer, exactly: the 128-bit sum th 2^32 + tl
           // over N = 2^(3 lg) cells, rounded (ties up)
@@ -810,12 +820,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(Ctl c) {
         case PH_PMEAN:
         case PH_R0FIN:
         case PH_SETFX:
-          if (threadIdx.x == 0) grid_item(c, g, P.type, I.grid);
+          if (threadIdx.x < 32) grid_item(c, g, P.type, I.grid);
           break;
         case PH_FIN:
-          if (threadIdx.x == 0) {
+          if (threadIdx.x < 32) {
             fin_item(c, g, I.grid);
-            if (g.active) atomicAdd(&c.active_left[ph], 1);
+            if (threadIdx.x == 0 && g.active) atomicAdd(&c.active_left[ph], 1);
           }
           break;
         case PH_BOTTOM: {
@@ -897,32 +907,29 @@ __global__ void k_stage_grid(const __grid_constant__ Ctl c, const int* grids, in
   GridDev& g = c.grids[gi];
   if (!runs(g, type)) return;
   Meter m(c, type, 32);
-  if (threadIdx.x == 0) grid_item(c, g, type, gi);
+  grid_item(c, g, type, gi);
   m.stop();
 }
 
-// The stopping rule of a class's grids; the number still active goes to
-// page-locked memory, where the host reads it.
-__global__ void k_stage_fin(const __grid_constant__ Ctl c, const int* grids, int count, int* left) {
+// The stopping rule of a class's grids, a warp each; the last one writes the
+// number still active to page-locked memory, where the host reads it.  sync:
+// arrivals and active grids, 0 before and after.
+__global__ void __launch_bounds__(32) k_stage_fin(const __grid_constant__ Ctl c, const int* grids,
+                                                  int* sync, int* left) {
   dev::after_previous();
-  Meter m(c, PH_FIN, 16);
-  int n = 0;
-  for (int q = threadIdx.x; q < count; q += blockDim.x) {
-    GridDev& g = c.grids[grids[q]];
-    if (!runs(g, PH_FIN)) continue;
-    fin_item(c, g, grids[q]);
-    n += g.active;
-  }
-  __shared__ int total;
-  if (threadIdx.x == 0) total = 0;
-  __syncthreads();
-  atomicAdd(&total, n);
-  __syncthreads();
+  Meter m(c, PH_FIN, 32);
+  const int gi = grids[blockIdx.x];
+  GridDev& g = c.grids[gi];
+  const bool run = runs(g, PH_FIN);
+  if (run) fin_item(c, g, gi);
   m.stop();
-  if (threadIdx.x == 0) {
-    *reinterpret_cast<volatile int*>(left) = total;
-    __threadfence_system();
-  }
+  if (threadIdx.x != 0) return;
+  if (run && g.active) atomicAdd(sync + 1, 1);
+  __threadfence();
+  if (atomicAdd(sync, 1) != (int)gridDim.x - 1) return;
+  sync[0] = 0;
+  *reinterpret_cast<volatile int*>(left) = atomicExch(sync + 1, 0);
+  __threadfence_system();
 }
 
 // The outer step on grids too small for a tile of 32 x 16 columns.
@@ -1162,6 +1169,7 @@ struct mg_batch {
   std::vector<Class> classes;
   int* d_class = nullptr;
   unsigned long long* d_work = nullptr;
+  int* d_fin = nullptr;   // two counters per class
   int* h_left = nullptr;  // pinned: grids of each class still active
   cudaEvent_t start = nullptr;
   bool start_ok = false;    // the streams, events and h_left are there
@@ -1466,7 +1474,8 @@ struct Stage {
       if (e == cudaSuccess) e = allow_smem(k_stage_fx, kSmem);
       go(k_stage_fx, tiles, kThreads, kSmem, n, first ? 1 : 0);
     }
-    go(k_stage_fin, 1, 128, 0, k->count, b->h_left + (k - b->classes.data()));
+    const int q = (int)(k - b->classes.data());
+    go(k_stage_fin, k->count, 32, 0, b->d_fin + 2 * q, b->h_left + q);
   }
   void end() {
     chunks<PH_PSUM>();
@@ -1517,6 +1526,7 @@ cudaError_t staged_solve(mg_batch* b, cudaStream_t s) {
   };
   also(cudaMemsetAsync(b->d_work, 0, sizeof(unsigned long long) * (kPhaseTypes + 2), s));
   also(cudaMemsetAsync(b->d_work + kPhaseTypes, 0xff, sizeof(unsigned long long), s));
+  also(cudaMemsetAsync(b->d_fin, 0, sizeof(int) * 2 * kMaxClasses, s));
   also(cudaEventRecord(b->start, s));
   const Ctl c = control(b);
   size_t open = 0;
@@ -1668,10 +1678,11 @@ mg_status mg_batch_create(int n, const int* dims, const double* dx, const mg_bc*
     b->d_ptime = balloc<unsigned long long>(b, b->nphases + 1);
     b->d_work = balloc<unsigned long long>(b, kPhaseTypes + 2);
     b->d_class = balloc<int>(b, n);
+    b->d_fin = balloc<int>(b, 2 * kMaxClasses);
     ok = b->d_grids && b->d_phases && b->d_items && b->d_part && b->d_part2 && b->d_ipart &&
          b->d_part3 &&
          b->d_hist && b->d_counters &&
-         b->d_bar && b->d_err && b->d_active && b->d_ptime && b->d_work && b->d_class;
+         b->d_bar && b->d_err && b->d_active && b->d_ptime && b->d_work && b->d_class && b->d_fin;
     b->host_phases = phases;
   }
   if (ok) {
