@@ -1772,7 +1772,7 @@ mg_status mg_batch_solve(mg_batch* b, const double* const* rho, const double* fo
   }
   cudaError_t e = cudaSuccess;
   // The staged solve was faster or as fast at every size (GB300, ms, staged and
-  // persistent: 512 grids of 16-128 22.8, 34.2; one of 128 1.13, 3.9; 64 of 32
+  // persistent: 512 grids of 16-128 22.8, 34.2; one of 128 1.09, 3.8; 64 of 32
   // 1.39, 2.6; 256 of 16 0.99, 0.99; 16 of 16 0.57, 0.58).  The persistent
   // kernel serves callers that limit its CTAs or its barriers, and batches of
   // more classes than streams.
