@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <utility>
 
 #include "mg_device.cuh"
 #include "mg_internal.h"
@@ -548,11 +549,17 @@ struct Prog {
 
 template <typename T, bool PER, int MODE>
 __global__ void __launch_bounds__(kThreads<T>) k_coarse(const __grid_constant__ CoarseArgs<T> a) {
+  // a CTA's shared memory may be stored into once that CTA has started: the
+  // cluster meets before the first put().  Arriving first, waiting last, the
+  // barrier passes while the kernel before this one runs and the slabs are made.
+  cg::cluster_group cl = cg::this_cluster();
+  auto started = cl.barrier_arrive();
   dev::after_previous();
   extern __shared__ double coarse_smem[];
   __shared__ Slab<T> slabs[2][kCoarseLevels];
   Prog<T, PER> p(a, reinterpret_cast<T*>(coarse_smem), slabs);
   __syncthreads();
+  cl.barrier_wait(std::move(started));
   if constexpr (MODE == COARSE_FMG) p.run_fmg();
   else if constexpr (MODE == COARSE_BASIS) p.run_basis();
   else p.run_vcycles();

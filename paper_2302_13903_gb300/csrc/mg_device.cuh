@@ -23,9 +23,10 @@
 namespace mg {
 namespace dev {
 
-// First statement of every kernel launched by launch_after: waits until the
-// kernel before it in the stream is complete and its stores are visible, then
-// lets the next one be placed on free SMs, where it waits in turn.  So the next
+// First statement (but for a cluster barrier's arrival) of every kernel launched
+// by launch_after: waits until the kernel before it in the stream is complete
+// and its stores are visible, then lets the next one be placed on free SMs,
+// where it waits in turn.  So the next
 // kernel's launch latency (1-1.5 us of a 4-5 us kernel on the small levels)
 // passes while this one runs.  Waiting first keeps at most one kernel placed
 // ahead, and no kernel touches memory before its predecessor is done.
