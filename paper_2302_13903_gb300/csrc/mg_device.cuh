@@ -29,7 +29,11 @@ namespace dev {
 // where it waits in turn.  So the next
 // kernel's launch latency (1-1.5 us of a 4-5 us kernel on the small levels)
 // passes while this one runs.  Waiting first keeps at most one kernel placed
-// ahead, and no kernel touches memory before its predecessor is done.
+// ahead, and no kernel touches memory before its predecessor is done.  The
+// kernel's inputs may still be written while it waits, so it takes no pointer as
+// `const T* __restrict__`: that would let the compiler read through it as data
+// that is constant from the launch on, before the wait or past the coherent
+// caches.
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -60,7 +60,7 @@ __device__ __forceinline__ double block_reduce(double v) {
 // max |a| of FP32 values.  VEC (16-byte aligned): four values per 16-byte
 // load, four loads in flight per thread.
 template <bool VEC>
-__global__ void k_absmax(const float* __restrict__ a, long long n, double* __restrict__ partials) {
+__global__ void k_absmax(const float* a, long long n, double* __restrict__ partials) {
   dev::after_previous();
   float m = 0.f;
   auto take = [&](float x) {
@@ -106,7 +106,7 @@ __global__ void k_absmax(const float* __restrict__ a, long long n, double* __res
 // held the pass to 1.3 TB/s (0.81 ms at 512^3).  Two values per 16-byte load,
 // four loads in flight.
 template <bool PAIRS>
-__global__ void k_absmax_bits(const unsigned long long* __restrict__ a, long long n,
+__global__ void k_absmax_bits(const unsigned long long* a, long long n,
                               double* __restrict__ partials) {
   dev::after_previous();
   unsigned long long m = 0;
@@ -142,7 +142,7 @@ __global__ void k_absmax_bits(const unsigned long long* __restrict__ a, long lon
   if (threadIdx.x == 0) partials[blockIdx.x] = r;
 }
 
-__global__ void k_finish_max(const double* __restrict__ partials, int nb, double* out) {
+__global__ void k_finish_max(const double* partials, int nb, double* out) {
   dev::after_previous();
   double m = 0.0;
   for (int t = threadIdx.x; t < nb; t += blockDim.x) m = fmax(m, partials[t]);
@@ -187,7 +187,7 @@ inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 // ADD: plus b (one rounding more, as a pass of its own would).
 template <bool PAIRS, bool ADD>
 __global__ void k_fx_to_f64(const long long* q, double* out, long long n, int S,
-                            const long long* __restrict__ mean, double b) {
+                            const long long* mean, double b) {
   dev::after_previous();
   const long long M = mean ? mean[0] : 0;
   stream8<PAIRS>(reinterpret_cast<const unsigned long long*>(q),
@@ -283,7 +283,7 @@ __device__ __forceinline__ double exact_value(const ExactSum& a) {
 // double whose bits are the largest |rho| pattern); two cells per step.
 // With `copy`, rho is read from host memory and each value is also stored
 // into copy (the device array the later passes read).
-__global__ void k_rho_stats(const double2* __restrict__ rho, long long n2,
+__global__ void k_rho_stats(const double2* rho, long long n2,
                             double* __restrict__ sum, double* __restrict__ mx,
                             double2* __restrict__ copy) {
   dev::after_previous();
@@ -331,8 +331,8 @@ __global__ void k_rho_stats(const double2* __restrict__ rho, long long n2,
 // integer conversion.
 // From the device: a and b (as doubles holding FP32 values) in ab[0], ab[1]
 // when ab is given, else the arguments.
-__global__ void k_rho_to_r32(const double2* __restrict__ rho, float2* __restrict__ r32,
-                             long long n2, float a_arg, float b_arg, const double* __restrict__ ab,
+__global__ void k_rho_to_r32(const double2* rho, float2* __restrict__ r32,
+                             long long n2, float a_arg, float b_arg, const double* ab,
                              double* __restrict__ sum, double* __restrict__ mx) {
   dev::after_previous();
   const float a = ab ? (float)ab[0] : a_arg, b = ab ? (float)ab[1] : b_arg;
@@ -356,7 +356,7 @@ __global__ void k_rho_to_r32(const double2* __restrict__ rho, float2* __restrict
 
 // In place into the integer array q: round(a rho - b) (the fixed-point h^2 f).
 template <bool PAIRS>
-__global__ void k_rho_to_fx(const double* __restrict__ rho, long long* __restrict__ q, long long n,
+__global__ void k_rho_to_fx(const double* rho, long long* __restrict__ q, long long n,
                             double a, double b) {
   dev::after_previous();
   stream8<PAIRS>(reinterpret_cast<const unsigned long long*>(rho),
@@ -365,7 +365,7 @@ __global__ void k_rho_to_fx(const double* __restrict__ rho, long long* __restric
                  });
 }
 
-__global__ void k_finish_sum_max(const double* __restrict__ sum, const double* __restrict__ mx,
+__global__ void k_finish_sum_max(const double* sum, const double* mx,
                                  int nb, double* __restrict__ out) {
   dev::after_previous();
   double a = 0.0, m = 0.0;
@@ -383,7 +383,7 @@ __global__ void k_finish_sum_max(const double* __restrict__ sum, const double* _
 
 // PHI += round(e * c) (the FP32 correction on the fixed-point grid); flags a
 // value above 2^60, past which neighbour sums could overflow.
-__global__ void k_fx_correct(long long* __restrict__ phi, const float* __restrict__ e, long long n,
+__global__ void k_fx_correct(long long* __restrict__ phi, const float* e, long long n,
                              float c, int* __restrict__ flag) {
   dev::after_previous();
   bool bad = false;
@@ -507,8 +507,8 @@ constexpr int fx_min_blocks() {
 // PM: the periodic axes (bit 0 x, 1 y, 2 z).
 template <int PM, bool ZERO_IN>
 __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
-    k_fx_step(const long long* __restrict__ phi_in, long long* __restrict__ phi_out,
-              const float* __restrict__ e, float c, const long long* __restrict__ F,
+    k_fx_step(const long long* phi_in, long long* __restrict__ phi_out,
+              const float* e, float c, const long long* F,
               float* __restrict__ r32, Grid g, FxBc bc, float factor, int cz,
               double* __restrict__ partials, long long* __restrict__ psum,
               int* __restrict__ flag) {
@@ -681,7 +681,7 @@ __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
 // lo) and their mean rounded to an integer, exactly: N = 2^log2n cells, so the
 // mean is the 128-bit sum shifted right with rounding (ties up).  out[0]: the
 // sum as a double; out[1]: the mean's bits as a long long.
-__global__ void k_finish_fx_sum(const long long* __restrict__ psum, int nb, int log2n,
+__global__ void k_finish_fx_sum(const long long* psum, int nb, int log2n,
                                 double* __restrict__ out) {
   dev::after_previous();
   __shared__ long long sh[kThreads], sl[kThreads];
@@ -723,9 +723,9 @@ __global__ void k_finish_fx_sum(const long long* __restrict__ psum, int nb, int 
 // two face accelerations, which on the integer grid is the exact difference
 // -(PHI_{i+1} - PHI_{i-1}) rounded once and scaled by 2^-S / (2 h).
 // Writes phi (as doubles, into a different buffer than q) and g = [gx|gy|gz].
-__global__ void k_fx_finish_gravity(const long long* __restrict__ q, double* __restrict__ phi,
+__global__ void k_fx_finish_gravity(const long long* q, double* __restrict__ phi,
                                     double* __restrict__ g, Grid gr, FxBc bc, int S,
-                                    double cg, const long long* __restrict__ mean) {
+                                    double cg, const long long* mean) {
   dev::after_previous();
   const long long M = mean ? mean[0] : 0;
   const long long N = gr.cells();
@@ -791,7 +791,7 @@ cudaError_t launch_fx_to_f64(const long long* q, double* out, long long n, int S
 }
 
 template <int KIND>
-__global__ void k_convert(const void* __restrict__ in, void* __restrict__ out, long long n) {
+__global__ void k_convert(const void* in, void* __restrict__ out, long long n) {
   dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
@@ -847,7 +847,7 @@ cudaError_t launch_rho_stats_copy(const double* host_rho, double* dev, long long
 // out[1] = scale = 1 / (|4 pi G| max|rho| + |mu|), out[2], out[3] = the FP32
 // a = 4 pi G scale and b = mu scale of launch_rho_to_r32 -- each one IEEE
 // operation in the order the host would take them.
-__global__ void k_source_scale(const double* __restrict__ st, long long n, double four_pi_G,
+__global__ void k_source_scale(const double* st, long long n, double four_pi_G,
                                int has_mean, double* __restrict__ out) {
   dev::after_previous();
   const double mu = has_mean ? __dmul_rn(four_pi_G, __ddiv_rn(st[0], (double)n)) : 0.0;

@@ -828,8 +828,8 @@ constexpr int fused_max_regs() {
 
 template <int MODE, bool ZERO, int PM, int TX, int TY>
 __global__ void __maxnreg__((fused_max_regs<MODE, TY, PM>()))
-    k_fused(const float* __restrict__ u_in, float* __restrict__ u_out, const float* __restrict__ f,
-            const float* __restrict__ ec, float* __restrict__ fc, FusedParams p) {
+    k_fused(const float* u_in, float* __restrict__ u_out, const float* f,
+            const float* ec, float* __restrict__ fc, FusedParams p) {
   dev::after_previous();
   extern __shared__ float4 smem[];
   fused_tile<MODE, ZERO, PM, TX, TY>(u_in, u_out, f, ec, fc, p, blockIdx.x, blockIdx.y, blockIdx.z,

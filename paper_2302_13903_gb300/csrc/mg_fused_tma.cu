@@ -35,8 +35,8 @@ constexpr int kPrefetch = ZERO ? 2 : 0;
 
 template <bool ZERO>
 __global__ void __maxnreg__((fused::fused_max_regs<fused::kDown, 32>()))
-    k_fused_down_tma(const float* __restrict__ u_in, float* __restrict__ u_out,
-                     const float* __restrict__ f, float* __restrict__ fc, FusedParams p,
+    k_fused_down_tma(const float* u_in, float* __restrict__ u_out,
+                     const float* f, float* __restrict__ fc, FusedParams p,
                      const __grid_constant__ CUtensorMap tmu,
                      const __grid_constant__ CUtensorMap tmf, int* err) {
   dev::after_previous();
@@ -53,8 +53,8 @@ __global__ void __maxnreg__((fused::fused_max_regs<fused::kDown, 32>()))
 constexpr int kPrefetchUp = 0;
 
 __global__ void __maxnreg__((fused::fused_max_regs<fused::kUp, 16>()))
-    k_fused_up_tma(const float* __restrict__ u_in, float* __restrict__ u_out,
-                   const float* __restrict__ f, const float* __restrict__ ec, FusedParams p,
+    k_fused_up_tma(const float* u_in, float* __restrict__ u_out,
+                   const float* f, const float* ec, FusedParams p,
                    const __grid_constant__ CUtensorMap tmu,
                    const __grid_constant__ CUtensorMap tmf, int* err) {
   dev::after_previous();

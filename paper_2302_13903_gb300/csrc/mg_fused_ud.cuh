@@ -302,8 +302,8 @@ constexpr int updown_max_regs() {
 
 template <int PM, int TX, int TY>
 __global__ void __maxnreg__((updown_max_regs<TY>()))
-    k_updown(const float* __restrict__ u_in, float* __restrict__ u_out,
-             const float* __restrict__ f, const float* __restrict__ ec, float* __restrict__ fc,
+    k_updown(const float* u_in, float* __restrict__ u_out,
+             const float* f, const float* ec, float* __restrict__ fc,
              FusedParams p) {
   dev::after_previous();
   extern __shared__ float4 smem[];

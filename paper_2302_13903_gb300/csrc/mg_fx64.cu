@@ -591,7 +591,7 @@ constexpr size_t up_smem() {
 // F = round(a rho - b) less round(2 b_face 2^S) for each of the cell's fixed and
 // open faces (c2 = 2^(S+1)), b = c *mu; per-block sums of F^2 without the
 // faces' part (the norm of f).
-__global__ void __launch_bounds__(256) k_fx64_source(const double* __restrict__ rho,
+__global__ void __launch_bounds__(256) k_fx64_source(const double* rho,
                                                      long long* __restrict__ F, Grid g, Bc bc,
                                                      double a, double c, const double* mu, double c2,
                                                      double* __restrict__ partials) {
@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(256) k_fx64_source(const double* __restrict__ 
 
 // fc = 4 pi G (mean of rho over the eight children) - *mu: the source of the
 // next level, straight from rho (one FP64 operation per cell).
-__global__ void __launch_bounds__(256) k_fx64_restrict(const double* __restrict__ rho,
+__global__ void __launch_bounds__(256) k_fx64_restrict(const double* rho,
                                                        double* __restrict__ fc, Grid g, double c,
                                                        const double* mu) {
   dev::after_previous();

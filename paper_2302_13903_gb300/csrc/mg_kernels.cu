@@ -311,7 +311,7 @@ bool homogeneous_rule(const Bc& bc) {
 // ---------------------------------------------------------------------------
 // d = f - (sum_nb - 6u) / h^2; optional store and partial sums of d^2.
 template <typename T>
-__global__ void k_defect(const T* __restrict__ u, const T* __restrict__ f, T* __restrict__ d,
+__global__ void k_defect(const T* u, const T* f, T* __restrict__ d,
                          Grid g, Bc bc, T inv_h2, double* __restrict__ partials) {
   dev::after_previous();
   const long long total = g.cells();
@@ -392,7 +392,7 @@ __global__ void k_add_const(double* __restrict__ u, long long n, double v) {
 
 // f = 4 pi G rho and partial sums of f, or of f^2 (SQ).
 template <bool SQ>
-__global__ void k_source(const double* __restrict__ rho, double* __restrict__ f, long long n,
+__global__ void k_source(const double* rho, double* __restrict__ f, long long n,
                          double four_pi_G, double* __restrict__ partials) {
   dev::after_previous();
   double acc = 0.0;
@@ -408,7 +408,7 @@ __global__ void k_source(const double* __restrict__ rho, double* __restrict__ f,
 }
 
 template <typename T>
-__global__ void k_sum(const T* __restrict__ a, long long n, int squares,
+__global__ void k_sum(const T* a, long long n, int squares,
                       double* __restrict__ partials) {
   dev::after_previous();
   double acc = 0.0;
@@ -421,7 +421,7 @@ __global__ void k_sum(const T* __restrict__ a, long long n, int squares,
   if (threadIdx.x == 0) partials[blockIdx.x] = b;
 }
 
-__global__ void k_finish_sum(const double* __restrict__ partials, int nb, double* __restrict__ out) {
+__global__ void k_finish_sum(const double* partials, int nb, double* __restrict__ out) {
   dev::after_previous();
   double acc = 0.0;
 #pragma unroll 8
@@ -433,7 +433,7 @@ __global__ void k_finish_sum(const double* __restrict__ partials, int nb, double
 // a -= total[0] / n (the total was formed on the device in a fixed order);
 // SQ: partial sums of the new a^2.
 template <bool SQ>
-__global__ void k_subtract_mean(double* __restrict__ a, long long n, const double* __restrict__ total,
+__global__ void k_subtract_mean(double* __restrict__ a, long long n, const double* total,
                                 double* __restrict__ partials) {
   dev::after_previous();
   const double mean = total[0] / (double)n;
@@ -453,7 +453,7 @@ __global__ void k_subtract_mean(double* __restrict__ a, long long n, const doubl
 
 // r32 = scale d with d = f - (sum_nb - 6 u) / h^2, partial sums of d^2: for
 // sizes that are not even.
-__global__ void k_outer_residual(const double* __restrict__ u, const double* __restrict__ f,
+__global__ void k_outer_residual(const double* u, const double* f,
                                  float* __restrict__ r32, Grid g, Bc bc, double inv_h2,
                                  double scale, double* __restrict__ partials) {
   dev::after_previous();
@@ -473,7 +473,7 @@ __global__ void k_outer_residual(const double* __restrict__ u, const double* __r
   if (threadIdx.x == 0) partials[blockIdx.x] = b;
 }
 
-__global__ void k_scale_to_f32(const double* __restrict__ a, float* __restrict__ b, long long n,
+__global__ void k_scale_to_f32(const double* a, float* __restrict__ b, long long n,
                                double scale) {
   dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
@@ -481,7 +481,7 @@ __global__ void k_scale_to_f32(const double* __restrict__ a, float* __restrict__
     b[t] = (float)(scale * a[t]);
 }
 
-__global__ void k_correct(double* __restrict__ u, const float* __restrict__ e, long long n,
+__global__ void k_correct(double* __restrict__ u, const float* e, long long n,
                           double inv_scale) {
   dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
@@ -491,7 +491,7 @@ __global__ void k_correct(double* __restrict__ u, const float* __restrict__ e, l
 
 // Algorithm 3 step 5 on a coarse level: f += L ur (the restricted potential's
 // Laplacian with the level's own rule) and the start value u = ur.
-__global__ void k_fas_rhs(const double* __restrict__ ur, double* __restrict__ f,
+__global__ void k_fas_rhs(const double* ur, double* __restrict__ f,
                           double* __restrict__ u, Grid g, Bc bc, double inv_h2) {
   dev::after_previous();
   const long long total = g.cells();
@@ -507,7 +507,7 @@ __global__ void k_fas_rhs(const double* __restrict__ ur, double* __restrict__ f,
 }
 
 // Algorithm 3 step 7: u -= ur (the coarse-grid correction).
-__global__ void k_sub(double* __restrict__ u, const double* __restrict__ ur, long long n) {
+__global__ void k_sub(double* __restrict__ u, const double* ur, long long n) {
   dev::after_previous();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
@@ -517,7 +517,7 @@ __global__ void k_sub(double* __restrict__ u, const double* __restrict__ ur, lon
 // g = -grad phi at cell centres (Sec. 3.2.3): per axis the average of the two
 // face accelerations -(phi_{i+1} - phi_i) / h and -(phi_i - phi_{i-1}) / h,
 // neighbours outside the level from the rule; g = [g_x | g_y | g_z].
-__global__ void k_gravity(const double* __restrict__ u, double* __restrict__ g, Grid gr, Bc bc,
+__global__ void k_gravity(const double* u, double* __restrict__ g, Grid gr, Bc bc,
                           double h) {
   dev::after_previous();
   const long long total = gr.cells();

@@ -34,3 +34,13 @@ def test_a_cluster_meets_before_it_stores_into_its_ctas():
     the whole cluster comes before the programs that store into it."""
     body = {k[1]: k[3] for k in kernels()}["k_coarse"]
     assert 0 <= body.find("barrier_arrive(") < body.find("barrier_wait(") < body.find("p.run_")
+
+
+def test_inputs_of_early_placed_kernels_are_not_read_as_constant():
+    """A kernel placed while its predecessor still writes must not promise that
+    its inputs stay as they are from the launch on (const T* __restrict__)."""
+    early = [k for k in kernels() if "after_previous(" in k[3]]
+    assert len(early) > 40
+    for file, name, params, _ in early:
+        for p in params.split(","):
+            assert not ("const" in p and "__restrict__" in p), (file, name, p.strip())
