@@ -1725,7 +1725,7 @@ void autotune(mg_ctx* c, cudaStream_t s) {
     }
   }
   const Grid g = level_grid(c, F);
-  if (c->fxbuf) {
+  if (c->opts.prec == MG_MIXED && c->fxbuf) {  // (the FP64 path has a buffer of that name too)
     const TuneKey key{prop.multiProcessorCount, prop.major, prop.minor, TUNE_FX, g.nx, g.ny, g.nz,
                       periodic};
     auto hit = g_tune.find(key);

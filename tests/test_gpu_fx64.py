@@ -134,3 +134,14 @@ def test_level_kernels_on_even_sizes(dims, rule, prec):
     got = mg.op_prolong(gc, bc, bc_value=0.0, add=True, uf=torch.from_numpy(fine).cuda())
     ref = orc.prolong(c.astype(np.float64), bc, bc_value=0.0, add=True, uf=fine.astype(np.float64))
     close(got, ref)
+
+
+def test_autotune_after_a_solve():
+    """mg_ctx_autotune has nothing to time on an FP64 context, before a solve or
+    after one."""
+    rho = torch.from_numpy(source((128, 32, 16), 6)).cuda()  # a shape no other test tunes
+    with mg.Solver((128, 32, 16), 1.0 / 128, mg.PERIODIC, prec=mg.FP64) as s:
+        first = s.solve(rho, 1.0, 1e-9)
+        s.autotune()
+        again = s.solve(rho, 1.0, 1e-9)
+    assert torch.equal(first[0], again[0]) and np.array_equal(first[1], again[1])
