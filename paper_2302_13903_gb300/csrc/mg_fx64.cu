@@ -39,6 +39,7 @@
 #include "mg_convert.cuh"
 #include "mg_device.cuh"
 #include "mg_internal.h"
+#include "mg_sums.h"
 
 namespace mg {
 namespace {
@@ -194,14 +195,14 @@ __device__ __forceinline__ bool too_large(long long v, int m) {
 
 // Block sum of doubles and of (hi, lo) integers into one partial per CTA.
 template <int NT>
-__device__ __forceinline__ void block_sums(double v, long long s, bool sums, double* norm,
+__device__ __forceinline__ void block_sums(double v, const SplitSum& s, bool sums, double* norm,
                                            long long* psum) {
   constexpr int NW = (NT + 31) / 32;
   __shared__ double wd[NW];
   __shared__ long long wh[NW], wl[NW];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned mask = w == NT / 32 ? (1u << (NT & 31)) - 1 : 0xffffffffu;  // a partial last warp
-  long long hi = s >> 32, lo = s & 0xffffffffLL;
+  long long hi = s.hi(), lo = s.lo();
   for (int o = 16; o > 0; o >>= 1) {
     const double d = __shfl_down_sync(mask, v, o);
     const long long h = __shfl_down_sync(mask, hi, o), l = __shfl_down_sync(mask, lo, o);
@@ -294,7 +295,8 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     cp_commit();
   };
   long long uP[4] = {}, uQ[4] = {}, fP[4] = {}, fQ[4] = {};
-  long long ud = 0, acc = 0, done = 0, psum = 0;
+  long long ud = 0, acc = 0, done = 0;
+  SplitSum psum;
   // outside the level cells stay 0
   auto delta = [&](long long R) { return !WALLS || p.valid ? weigh(R, a.w) : 0; };
   const int most = 1 << (a.limit - 32);
@@ -327,7 +329,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     if (!COARSE) {
       raw[I0] = uB[J];
       if (framed) frame[I0] = frame_in ? ring.frame[J][t] : 0;
-      if (p.tile && q >= z0 && q < z1) psum += uP[J] + uQ[J];
+      if (p.tile && q >= z0 && q < z1) psum.add(uP[J] + uQ[J]);
     }
     // the block whose last plane was q - 4: its even and odd row's sums
     if (!EVEN && q - 5 >= z0 && q - 5 < z1 && even_row) {
@@ -574,7 +576,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
   }
   cp_wait<0>();
   if (bad) atomicOr(a.flag, 1);
-  if (!COARSE) block_sums<W::NT>(norm.total(), 0, false, a.norm, nullptr);
+  if (!COARSE) block_sums<W::NT>(norm.total(), SplitSum{}, false, a.norm, nullptr);
 }
 
 template <int TX>
@@ -776,9 +778,8 @@ bool fx64_ok(Grid g) {
          g.cells() <= (1LL << 30) && fx64_blocks(g) <= kPartials;
 }
 
-// Planes per CTA: the even count for which the last wave of CTAs
-// is best filled, counting the six planes a chunk's halo costs; at most 128 (a
-// thread's exact sum of its columns' integers must stay below 2^63).
+// Planes per CTA: the even count for which the last wave of CTAs is best filled,
+// counting the six planes a chunk's halo costs; at most 128.
 int fx64_cz(Grid g) {
   const int tx = tile_width(g), wave = sm_count() * (tx == 64 ? 1 : 2);
   const long long cols = (long long)(g.nx / tx) * (g.ny / TY);

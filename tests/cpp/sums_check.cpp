@@ -1,0 +1,37 @@
+// Exact sums of the integer legs (mg_sums.h) against 128-bit ones.
+#include <cstdio>
+#include <initializer_list>
+
+#include "../../paper_2302_13903_gb300/csrc/mg_sums.h"
+
+static int failures = 0;
+#define CHECK(x)                                       \
+  do {                                                 \
+    if (!(x)) {                                        \
+      std::printf("line %d: %s\n", __LINE__, #x);      \
+      ++failures;                                      \
+    }                                                  \
+  } while (0)
+
+// A column of `planes` pairs of one sign, as the down leg's threads sum them: at 2^55
+// and more the plain 64-bit sum of 128 pairs wraps.
+static void split_sum() {
+  for (int bits : {0, 40, 54, 55, 57, 59})
+    for (int sign : {1, -1})
+      for (int planes : {4, 64, 128}) {
+        const long long v = sign * ((1LL << bits) - 1);
+        mg::SplitSum s;
+        __int128 sum = 0;
+        for (int p = 0; p < planes; ++p) {
+          s.add(v + v + (p & 3));
+          sum += v + v + (p & 3);
+        }
+        CHECK((__int128)s.hi() * ((__int128)1 << 32) + s.lo() == sum);
+      }
+}
+
+int main() {
+  split_sum();
+  std::printf(failures ? "FAILED\n" : "ok\n");
+  return failures != 0;
+}
