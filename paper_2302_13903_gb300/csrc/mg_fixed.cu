@@ -19,6 +19,7 @@
 #include "mg_convert.cuh"
 #include "mg_device.cuh"
 #include "mg_internal.h"
+#include "mg_sums.h"
 
 namespace mg {
 namespace {
@@ -197,14 +198,19 @@ __global__ void k_fx_to_f64(const long long* q, double* out, long long n, int S,
                  });
 }
 
-// In place: the double a[t] becomes the integer round(a[t] c).
-template <bool PAIRS>
-__global__ void k_f64_to_fx(double* a, long long n, double c) {
+// In place: the double a[t] becomes the integer round(a[t] c).  CHECK: *flag |= 1
+// where that is 2^bits or more, or not a number.
+template <bool PAIRS, bool CHECK>
+__global__ void k_f64_to_fx(double* a, long long n, double c, int bits, int* flag) {
   dev::after_previous();
   unsigned long long* q = reinterpret_cast<unsigned long long*>(a);
+  bool bad = false;
   stream8<PAIRS>(q, q, n, [&](unsigned long long v) {
-    return (unsigned long long)cvt::d2ll_rn(__longlong_as_double((long long)v) * c);
+    const double x = __longlong_as_double((long long)v) * c;
+    if (CHECK) bad |= past_range((unsigned long long)__double_as_longlong(x), bits);
+    return (unsigned long long)cvt::d2ll_rn(x);
   });
+  if (CHECK && bad) atomicOr(flag, 1);
 }
 
 // |x| as an unsigned integer: for non-negative doubles (and floats) the order
@@ -771,10 +777,13 @@ cudaError_t launch_absmax(const T* a, long long n, double* partials, double* out
 template cudaError_t launch_absmax<double>(const double*, long long, double*, double*, cudaStream_t);
 template cudaError_t launch_absmax<float>(const float*, long long, double*, double*, cudaStream_t);
 
-cudaError_t launch_f64_to_fx(double* a, long long n, double c, cudaStream_t s) {
+cudaError_t launch_f64_to_fx(double* a, long long n, double c, cudaStream_t s, int bits, int* flag) {
   ++g_launches;
-  if (aligned16(a)) launch_after(k_f64_to_fx<true>, grid_for(n / 8), kThreads, 0, s, a, n, c);
-  else launch_after(k_f64_to_fx<false>, grid_for(n), kThreads, 0, s, a, n, c);
+  const bool pairs = aligned16(a);
+  const int blocks = grid_for(pairs ? n / 8 : n);
+  auto kernel = flag ? (pairs ? k_f64_to_fx<true, true> : k_f64_to_fx<false, true>)
+                     : (pairs ? k_f64_to_fx<true, false> : k_f64_to_fx<false, false>);
+  launch_after(kernel, blocks, kThreads, 0, s, a, n, c, bits, flag);
   return cudaGetLastError();
 }
 

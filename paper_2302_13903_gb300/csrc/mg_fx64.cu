@@ -825,7 +825,7 @@ cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s) {
   a.psum = q.psum;
   a.ec = q.ec;
   // with |ec| < 2^56 and its sums of weight 64 below 2^62
-  a.limit = q.coarse ? 56 : 59;
+  a.limit = q.coarse ? kFx64Correction : 59;
   a.flag = q.flag;
   const bool wide = tile_width(q.g) == 64, gd = !down && q.shift != 0;
   if (q.coarse) {

@@ -278,8 +278,10 @@ int* down_tma_op_flag();
 // out[0] = max |a| (deterministic two-stage reduction through partials).
 template <typename T>
 cudaError_t launch_absmax(const T* a, long long n, double* partials, double* out, cudaStream_t s);
-// In place: double -> round(a c) as int64.
-cudaError_t launch_f64_to_fx(double* a, long long n, double c, cudaStream_t s);
+// In place: double -> round(a c) as int64; with `flag`, *flag |= 1 where |a c| is
+// 2^bits or more, or a c is NaN.
+cudaError_t launch_f64_to_fx(double* a, long long n, double c, cudaStream_t s, int bits = 0,
+                             int* flag = nullptr);
 // out[t] = (q[t] - *mean) 2^-S + b (mean may be null: 0); out may alias q.
 cudaError_t launch_fx_to_f64(const long long* q, double* out, long long n, int S,
                              const long long* mean, double b, cudaStream_t s);
@@ -347,9 +349,10 @@ int fx64_blocks(Grid g);
 // norm = sums of (h^2 2^S defect)^2 over the red cells of u_in; psum = sums of
 // u_in.  up: u_out = SMOOTH(u_in + trilinear(ec) 2^-shift); norm = the same
 // over the black cells of u_out.  coarse: a correction level, down from u_in =
-// 0, no norms and sums.  *flag |= 1 where |u_out| passes 2^59 (coarse 2^56) or
-// fci its range.
+// 0, no norms and sums.  *flag |= 1 where |u_out| passes 2^59 (coarse
+// 2^kFx64Correction) or fci its range.
 constexpr int kFx64Guard = 2;  // guard bits of the integer correction levels
+constexpr int kFx64Correction = 56;  // corrections stay below 2^56
 struct Fx64Leg {
   const long long* u_in;
   long long* u_out;

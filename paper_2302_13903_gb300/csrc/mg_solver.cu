@@ -878,7 +878,8 @@ void fp64_correction(mg_ctx* c, int l, const Bc& hom, double h, cudaStream_t s) 
   Pyr<double> P = pyr<double>(c);
   if (l == 0) coarsest_solve<double>(c, P.u[0], P.f[0], hom, false, s);
   else vcycle<double>(c, P, l, hom, hom, true, s);
-  check(c, mg::launch_f64_to_fx(c->u64[l], level_grid(c, l).cells(), 1.0 / (8.0 * h * h), s),
+  check(c, mg::launch_f64_to_fx(c->u64[l], level_grid(c, l).cells(), 1.0 / (8.0 * h * h), s,
+                                mg::kFx64Correction, c->iflag),
         "correction -> fixed point");
 }
 
@@ -913,8 +914,8 @@ void fx64_correction(mg_ctx* c, int l, const Bc& hom, cudaStream_t s) {
 
 // The FP64 solve from an FMG start with the levels from 64^3 up in 64-bit fixed
 // point (mg_fx64.cu).  The finest level's source and start are never formed
-// as doubles.  Returns -1 where the values are not finite or leave the
-// integers' range (nothing but phi is lost then), else the status.
+// as doubles.  Returns -1 where the values are not finite, leave the integers'
+// range or diverge on them (nothing but phi is lost then), else the status.
 int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, double* phi,
                double* gacc, const Bc* bcs, const Bc& hom, double* hist, int hist_cap, int* n_hist,
                cudaStream_t s) {
@@ -1002,6 +1003,7 @@ int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, doubl
       hist[n++] = r;
       rule.record(r);
       st = rule.decide(r, cyc, c->opts.max_cycles, n, hist_cap);
+      if (st == MG_ERR_DIVERGED) return -1;
       if (st >= 0) break;
     }
     replay(c, c->inner[1], true, s, [&]() {

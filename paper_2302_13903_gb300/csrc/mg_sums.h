@@ -1,5 +1,6 @@
-// mg_sums.h -- exact sums a thread of the integer legs keeps (host and device, so
-// that their ranges are tested on the host).
+// mg_sums.h -- exact sums a thread of the integer legs keeps, and the range check
+// of what becomes an integer (host and device, so that they are tested on the
+// host).
 #pragma once
 
 #ifdef __CUDACC__
@@ -26,5 +27,11 @@ struct SplitSum {
   MG_HD long long lo() const { return (long long)(rest() & 0xffffffffu); }
   MG_HD unsigned long long rest() const { return part - ((unsigned long long)(long long)top << 44); }
 };
+
+// Whether a binary64 of these bits is 2^bits or more in magnitude, infinite or
+// NaN (integer arithmetic only).
+MG_HD bool past_range(unsigned long long u, int bits) {
+  return (int)((u >> 52) & 0x7ff) >= 1023 + bits;
+}
 
 }  // namespace mg

@@ -1,5 +1,7 @@
-// Exact sums of the integer legs (mg_sums.h) against 128-bit ones.
+// Exact sums and range checks of the integer legs (mg_sums.h).
+#include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <initializer_list>
 
 #include "../../paper_2302_13903_gb300/csrc/mg_sums.h"
@@ -30,8 +32,28 @@ static void split_sum() {
       }
 }
 
+static void range() {
+  const double limit = std::ldexp(1.0, 56);
+  for (int sign : {1, -1}) {
+    const double out[] = {limit, 1.5 * limit, 1e300, INFINITY, NAN};
+    const double in[] = {0.0, 5e-324, 1.0, std::nextafter(limit, 0.0)};
+    unsigned long long u;
+    for (double x : out) {
+      x = std::copysign(x, sign);
+      std::memcpy(&u, &x, 8);
+      CHECK(mg::past_range(u, 56));
+    }
+    for (double x : in) {
+      x = std::copysign(x, sign);
+      std::memcpy(&u, &x, 8);
+      CHECK(!mg::past_range(u, 56));
+    }
+  }
+}
+
 int main() {
   split_sum();
+  range();
   std::printf(failures ? "FAILED\n" : "ok\n");
   return failures != 0;
 }

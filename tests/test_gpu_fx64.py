@@ -145,3 +145,16 @@ def test_autotune_after_a_solve():
         s.autotune()
         again = s.solve(rho, 1.0, 1e-9)
     assert torch.equal(first[0], again[0]) and np.array_equal(first[1], again[1])
+
+
+@pytest.mark.parametrize("rule", ["periodic", "fixed"])
+def test_a_solve_that_diverges_is_the_general_path(rule):
+    """Where the relaxation diverges the integers' ranges end first: status,
+    history and phi are those of the FP64 kernels (as for a misaligned phi)."""
+    rho = source((64, 64, 64), 7)
+    odd = torch.zeros(rho.size + 1, dtype=torch.float64, device="cuda")[1:].view(rho.shape)
+    ref, h0, st0 = gpu(rho, rule, tol=1e-10, phi=odd, omega=1.999, stall_ratio=NO_STALL)
+    phi, hist, st = gpu(rho, rule, tol=1e-10, omega=1.999, stall_ratio=NO_STALL)
+    assert st == st0
+    if st == 5:  # MG_ERR_DIVERGED
+        assert np.array_equal(hist, h0) and np.array_equal(phi, ref)
