@@ -166,28 +166,6 @@ __device__ __forceinline__ long long residual(const long long* o, long long self
   return (((mate + o[xo]) + (o[-PW] + o[PW])) + (zl + zh)) - n * self - F;
 }
 
-// Sum of squares of integers |R| < 2^63 in two floats (relative error about
-// 2^-44), scaled by 2^-24: FP32 and integer instructions only.  A conversion
-// and a multiply-add per cell on the FP64 units, 64 clocks of a scheduler each,
-// set the pace of the legs otherwise.
-struct Squares {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(long long r) {
-    // of |r|: its three parts then never cancel, so hi is |R| to 2^-24
-    const unsigned long long R = (unsigned long long)(r < 0 ? -r : r);
-    const float x2 = (float)(int)(R >> 40) * 0x1p28f;
-    const float x1 = (float)(int)((unsigned)(R >> 20) & 0xfffffu) * 0x1p8f;
-    const float x0 = (float)(int)((unsigned)R & 0xfffffu) * 0x1p-12f;
-    const float lo = x1 + x0, hi = x2 + lo;        // R 2^-12 = hi + rem
-    const float rem = ((x2 - hi) + x1) + x0;
-    const float q = hi * hi, e = fmaf(hi + hi, rem, fmaf(hi, hi, -q));
-    const float t = s + q, b = t - s;
-    c += ((s - (t - b)) + (q - b)) + e;
-    s = t;
-  }
-  __device__ __forceinline__ double total() const { return ((double)s + (double)c) * 0x1p24; }
-};
-
 // |v| at or past 2^32 m, by the high word.
 __device__ __forceinline__ bool too_large(long long v, int m) {
   return (unsigned)((int)(v >> 32) + m) >= 2u * m;
@@ -300,7 +278,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
   // outside the level cells stay 0
   auto delta = [&](long long R) { return !WALLS || p.valid ? weigh(R, a.w) : 0; };
   const int most = 1 << (a.limit - 32);
-  Squares norm;
+  SquareSum norm;
   bool bad = false;
   using std::integral_constant;
   issue(integral_constant<int, 0>{}, z0 - 3);
@@ -496,7 +474,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
   const int most = 1 << (a.limit - 32);
   constexpr int bits = 6 + GUARD;
   constexpr long long half = 1LL << (bits - 1);
-  Squares norm;
+  SquareSum norm;
   bool bad = false;
   using std::integral_constant;
   issue(integral_constant<int, 0>{}, z0 - 2);
@@ -601,7 +579,7 @@ __global__ void __launch_bounds__(256) k_fx64_source(const double* rho,
   const dev::Split sp(g.nx, g.ny);
   const double b = c * mu[0];
   const bool faces = bc.kind != BC_PERIODIC && bc.kind != BC_ZEROGRAD;
-  Squares sum;
+  SquareSum sum;
 #pragma unroll 4
   for (long long t = blockIdx.x * 256LL + threadIdx.x; t < g.cells(); t += gridDim.x * 256LL) {
     long long v = cvt::d2ll_rn(fma(a, rho[t], -b));

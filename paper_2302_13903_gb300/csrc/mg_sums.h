@@ -28,6 +28,39 @@ struct SplitSum {
   MG_HD unsigned long long rest() const { return part - ((unsigned long long)(long long)top << 44); }
 };
 
+// Sum of squares of integers |r| < 2^63, exactly, as top 2^128 + hi 2^64 + lo: 32-bit
+// integer instructions only.  A conversion and a multiply-add per cell on the FP64
+// units, 64 clocks of a scheduler each, set the pace of the integer legs otherwise.
+struct SquareSum {
+  unsigned long long lo = 0, hi = 0;
+  unsigned top = 0;
+  MG_HD void add(long long r) {
+    const unsigned long long a = r < 0 ? 0ull - (unsigned long long)r : (unsigned long long)r;
+    const unsigned h = (unsigned)(a >> 32), l = (unsigned)a;
+    const unsigned long long ll = (unsigned long long)l * l, hh = (unsigned long long)h * h;
+    const unsigned long long m = (unsigned long long)l * h;  // r^2 = hh 2^64 + m 2^33 + ll
+    sum(ll, hh);
+    sum(m << 33, m >> 31);
+  }
+  MG_HD double total() const {
+    return ((double)top * 0x1p64 + (double)hi) * 0x1p64 + (double)lo;
+  }
+
+ private:
+  MG_HD void sum(unsigned long long l, unsigned long long h) {
+#ifdef __CUDA_ARCH__
+    asm("add.cc.u64 %0, %0, %3;\n\taddc.cc.u64 %1, %1, %4;\n\taddc.u32 %2, %2, 0;"
+        : "+l"(lo), "+l"(hi), "+r"(top)
+        : "l"(l), "l"(h));
+#else
+    lo += l;
+    const unsigned long long c = lo < l, k = hi + h;
+    hi = k + c;
+    top += (k < h) + (hi < c);
+#endif
+  }
+};
+
 // Whether a binary64 of these bits is 2^bits or more in magnitude, infinite or
 // NaN (integer arithmetic only).
 MG_HD bool past_range(unsigned long long u, int bits) {

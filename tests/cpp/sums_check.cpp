@@ -32,6 +32,31 @@ static void split_sum() {
       }
 }
 
+// Against 64-bit pieces of the exact sum, for values up to the largest the legs
+// form and as many of them as a thread of the source pass adds.
+static void square_sum() {
+  for (int bits : {0, 1, 24, 31, 32, 33, 48, 53, 58, 62, 63})
+    for (int count : {1, 2, 128, 4096}) {
+      mg::SquareSum s;
+      unsigned __int128 low = 0;  // sums of the squares' lower and upper 64 bits
+      unsigned __int128 high = 0;
+      for (int q = 0; q < count; ++q) {
+        const long long v = (long long)((1ull << bits) - 1 - (unsigned long long)(q % 3)) * (q % 2 ? 1 : -1);
+        const long long r = bits < 2 ? (long long)((1ull << bits) - 1) : v;
+        s.add(r);
+        const unsigned __int128 a = r < 0 ? -(__int128)r : (__int128)r, sq = a * a;
+        low += (unsigned long long)sq;
+        high += (unsigned long long)(sq >> 64);
+      }
+      high += (unsigned long long)(low >> 64);
+      CHECK(s.lo == (unsigned long long)low);
+      CHECK(s.hi == (unsigned long long)high);
+      CHECK(s.top == (unsigned)(high >> 64));
+      const double want = (double)high * 0x1p64 + (double)(unsigned long long)low;
+      CHECK(std::fabs(s.total() - want) <= 0x1p-52 * want);
+    }
+}
+
 static void range() {
   const double limit = std::ldexp(1.0, 56);
   for (int sign : {1, -1}) {
@@ -53,6 +78,7 @@ static void range() {
 
 int main() {
   split_sum();
+  square_sum();
   range();
   std::printf(failures ? "FAILED\n" : "ok\n");
   return failures != 0;
