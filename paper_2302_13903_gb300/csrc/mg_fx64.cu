@@ -62,8 +62,7 @@ struct Fx64Args {
   Weight w;
   double* norm;  // per-CTA sum of R^2: red cells of u_in (down), black cells of u_out (up)
   double* fc;           // down: coarse right-hand side, -sum of R, as doubles,
-  long long* fci;       //   or on the coarse level's integer grid (fc null)
-  int shift;            // down: -sum of R 2^shift is F there
+  long long* fci;       //   or half of it, as F of an integer level (fc null)
   long long* psum;      // down: per-CTA exact sum of u_in, (hi, lo) pairs
   const long long* ec;  // up: coarse correction on the integer grid
   int limit;            // log2 of the largest |U|
@@ -314,9 +313,9 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
       const long long sum = -(done + odd[W::PW]);
       const size_t o = (size_t)((q - 5) >> 1) * (plane >> 2) + colc;
       if (a.fci) {
-        const long long f = a.shift >= 0 ? sum << a.shift : (sum + 1) >> 1;
+        const long long f = (sum + ((sum >> 1) & 1)) >> 1;  // ties to even: no bias
         a.fci[o] = f;
-        bad |= too_large(f, 1 << 27) || too_large(sum, 1 << 26);
+        bad |= too_large(f, 1 << 28);
       } else {
         a.fc[o] = cvt::ll2d_rn(sum);
       }
@@ -385,8 +384,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
 // q - 2, then final and written.  The correction of a pair is interpolated
 // along y, then x, then z with weights 3 and 1 on the integer grid and rounded
 // once by the division by 64.  Unrolled by four as the down leg.
-// GUARD: ec's guard bits.
-template <bool WALLS, int TX, bool COARSE, int GUARD>
+template <bool WALLS, int TX, bool COARSE>
 __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
     k_fx64_up(const __grid_constant__ Fx64Args a) {
   dev::after_previous();
@@ -472,8 +470,6 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
   // outside the level cells stay 0
   auto delta = [&](long long R) { return !WALLS || p.valid ? weigh(R, a.w) : 0; };
   const int most = 1 << (a.limit - 32);
-  constexpr int bits = 6 + GUARD;
-  constexpr long long half = 1LL << (bits - 1);
   SquareSum norm;
   bool bad = false;
   using std::integral_constant;
@@ -512,7 +508,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
     }
     if (!WALLS || p.valid) {
       const longlong2 v = ring.u[J][t], f = ring.f[J][t];
-      const long long v0 = v.x + ((d0 + half) >> bits), v1 = v.y + ((d1 + half) >> bits);
+      const long long v0 = v.x + ((d0 + 32) >> 6), v1 = v.y + ((d1 + 32) >> 6);
       uP[J] = p.swap ? v1 : v0;
       uQ[J] = p.swap ? v0 : v1;
       fP[J] = p.swap ? f.y : f.x;
@@ -730,19 +726,14 @@ cudaError_t launch_leg(K* kernel, std::atomic<int>* configured, size_t smem, int
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// guard: up from a level with guard bits to one without.
 template <bool WALLS, int TX, bool COARSE>
-cudaError_t launch(const Fx64Args& a, bool down, bool guard, cudaStream_t s) {
-  static std::atomic<int> configured[3][64];
+cudaError_t launch(const Fx64Args& a, bool down, cudaStream_t s) {
+  static std::atomic<int> configured[2][64];
   if (down)
     return launch_leg(k_fx64_down<WALLS, TX, COARSE>, configured[0], down_smem<TX>(), Down<TX>::NT,
                       TX, a, s);
-  if constexpr (!COARSE)
-    if (guard)
-      return launch_leg(k_fx64_up<WALLS, TX, false, kFx64Guard>, configured[2], up_smem<TX>(),
-                        Up<TX>::NT, TX, a, s);
-  return launch_leg(k_fx64_up<WALLS, TX, COARSE, 0>, configured[1], up_smem<TX>(), Up<TX>::NT, TX,
-                    a, s);
+  return launch_leg(k_fx64_up<WALLS, TX, COARSE>, configured[1], up_smem<TX>(), Up<TX>::NT, TX, a,
+                    s);
 }
 
 // Tile width: 64 cells, one CTA per SM, or on levels that would leave SMs
@@ -799,19 +790,18 @@ cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s) {
   a.norm = q.norm;
   a.fc = q.fc;
   a.fci = q.fci;
-  a.shift = q.shift;
   a.psum = q.psum;
   a.ec = q.ec;
   // with |ec| < 2^56 and its sums of weight 64 below 2^62
   a.limit = q.coarse ? kFx64Correction : 59;
   a.flag = q.flag;
-  const bool wide = tile_width(q.g) == 64, gd = !down && q.shift != 0;
+  const bool wide = tile_width(q.g) == 64;
   if (q.coarse) {
-    if (a.fk) return wide ? launch<true, 64, true>(a, down, gd, s) : launch<true, 32, true>(a, down, gd, s);
-    return wide ? launch<false, 64, true>(a, down, gd, s) : launch<false, 32, true>(a, down, gd, s);
+    if (a.fk) return wide ? launch<true, 64, true>(a, down, s) : launch<true, 32, true>(a, down, s);
+    return wide ? launch<false, 64, true>(a, down, s) : launch<false, 32, true>(a, down, s);
   }
-  if (a.fk) return wide ? launch<true, 64, false>(a, down, gd, s) : launch<true, 32, false>(a, down, gd, s);
-  return wide ? launch<false, 64, false>(a, down, gd, s) : launch<false, 32, false>(a, down, gd, s);
+  if (a.fk) return wide ? launch<true, 64, false>(a, down, s) : launch<true, 32, false>(a, down, s);
+  return wide ? launch<false, 64, false>(a, down, s) : launch<false, 32, false>(a, down, s);
 }
 
 cudaError_t launch_fx64_source(const double* rho, long long* F, Grid g, const Bc& bc,

@@ -345,13 +345,12 @@ bool fx64_ok(Grid g);
 int fx64_cz(Grid g);
 int fx64_blocks(Grid g);
 // down: u_out = SMOOTH(u_in); fc = the restricted defect times 8 h^2 2^S, or
-// fci = that divided by 8 times 2^(3 + shift), F of an integer coarse level;
+// fci = half of it, F of an integer coarse level;
 // norm = sums of (h^2 2^S defect)^2 over the red cells of u_in; psum = sums of
-// u_in.  up: u_out = SMOOTH(u_in + trilinear(ec) 2^-shift); norm = the same
+// u_in.  up: u_out = SMOOTH(u_in + trilinear(ec)); norm = the same
 // over the black cells of u_out.  coarse: a correction level, down from u_in =
 // 0, no norms and sums.  *flag |= 1 where |u_out| passes 2^59 (coarse
 // 2^kFx64Correction) or fci its range.
-constexpr int kFx64Guard = 2;  // guard bits of the integer correction levels
 constexpr int kFx64Correction = 56;  // corrections stay below 2^56
 struct Fx64Leg {
   const long long* u_in;
@@ -361,7 +360,6 @@ struct Fx64Leg {
   Bc hom;
   double omega;
   bool coarse;
-  int shift;
   double* fc;
   long long* fci;
   const long long* ec;

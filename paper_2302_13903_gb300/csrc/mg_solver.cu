@@ -884,8 +884,8 @@ void fp64_correction(mg_ctx* c, int l, const Bc& hom, double h, cudaStream_t s) 
 }
 
 // The correction of level l < F of the integer FP64 path from F in f64[l] into
-// u64[l] (both as integers with kFx64Guard guard bits): the levels with a
-// second buffer as integers, the ones below in FP64.
+// u64[l] (both as integers): the levels with a second buffer as integers, the
+// ones below in FP64.
 void fx64_correction(mg_ctx* c, int l, const Bc& hom, cudaStream_t s) {
   const Grid g = level_grid(c, l);
   const double h = level_h(c, l);
@@ -898,7 +898,6 @@ void fx64_correction(mg_ctx* c, int l, const Bc& hom, cudaStream_t s) {
   leg.coarse = true;
   leg.flag = c->iflag;
   leg.u_out = c->ub64[l];
-  leg.shift = -1;
   const bool below = c->ub64[l - 1] != nullptr;
   leg.fc = below ? nullptr : c->f64[l - 1];
   leg.fci = below ? q(c->f64[l - 1]) : nullptr;
@@ -908,7 +907,6 @@ void fx64_correction(mg_ctx* c, int l, const Bc& hom, cudaStream_t s) {
   leg.u_in = c->ub64[l];
   leg.u_out = q(c->u64[l]);
   leg.ec = q(c->u64[l - 1]);
-  leg.shift = 0;
   check(c, mg::launch_fx64(leg, false, s), "up leg");
 }
 
@@ -934,7 +932,7 @@ int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, doubl
   open_boundary(c, rho, four_pi_G, true, s);
   check(c, cudaMemsetAsync(c->scal + 50, 0, 2 * sizeof(double), s), "zero");
   fmg_below<double>(c, pyr<double>(c), bcs, hom, true, s);
-  // 2^S: |phi| < 2^54 (five bits of room before 2^59) and |h^2 f| < 2^55; I'
+  // 2^S: |phi| < 2^57 (two bits of room before 2^59) and |h^2 f| < 2^58; I'
   // raises max |u| by (38 / 32)^3 < 2 at most
   check(c, mg::launch_absmax<double>(c->u64[F - 1], gc.cells(), c->partials, c->scal + 50, s),
         "max |phi|");
@@ -955,7 +953,7 @@ int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, doubl
   int ep = 0, ef = 0;
   std::frexp(mphi, &ep);  // mphi < 2^ep
   std::frexp(mfh, &ef);
-  const int S = std::min(54 - ep, 55 - ef);
+  const int S = std::min(57 - ep, 58 - ef);
   if (S < -900 || S > 900) return -1;
   const double two_S = std::ldexp(1.0, S);
   long long *cur = reinterpret_cast<long long*>(phi), *alt = c->fxbuf;
@@ -989,7 +987,6 @@ int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, doubl
       leg.u_in = cur;
       leg.u_out = alt;
       leg.norm = red;
-      leg.shift = mg::kFx64Guard - 1;
       check(c, mg::launch_fx64(leg, true, s), "down leg");
     }
     if (cyc >= 0) {  // the norm of the last cycle's phi (the leg above ran ahead of the test)
@@ -1014,7 +1011,6 @@ int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, doubl
     leg.u_in = alt;
     leg.u_out = cur;
     leg.norm = black;
-    leg.shift = below ? mg::kFx64Guard : 0;
     check(c, mg::launch_fx64(leg, false, s), "up leg");
   }
   const long long* mean = nullptr;

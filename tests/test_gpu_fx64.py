@@ -158,3 +158,113 @@ def test_a_solve_that_diverges_is_the_general_path(rule):
     assert st == st0
     if st == 5:  # MG_ERR_DIVERGED
         assert np.array_equal(hist, h0) and np.array_equal(phi, ref)
+
+
+# --- the rounding floor: errors against the discrete solution in double-double ---
+
+def two_sum(a, b):
+    s = a + b
+    t = s - a
+    return s, (a - (s - t)) + (b - t)
+
+
+def dd(*parts):
+    """Sum of (high, low) pairs."""
+    hi, lo = parts[0]
+    for h, l in parts[1:]:
+        hi, e = two_sum(hi, h)
+        hi, lo = two_sum(hi, lo + e + l)
+    return hi, lo
+
+
+def neighbours(t, kind):
+    """The six neighbours of every cell under one homogeneous rule."""
+    for d in range(3):
+        for end in (0, t.shape[d] - 1):
+            r = torch.roll(t, 1 if end == 0 else -1, d)
+            if kind != P:
+                own = t.narrow(d, end, 1)
+                r.narrow(d, end, 1).copy_(own if kind == Z else -own)
+            yield r
+
+
+def modes(m, kind, h):
+    """Eigenvalues and orthonormal eigenvectors of the second difference."""
+    a = -2.0 * np.eye(m) + np.eye(m, k=1) + np.eye(m, k=-1)
+    if kind == P:
+        a[0, -1] += 1
+        a[-1, 0] += 1
+    else:
+        a[0, 0] += 1 if kind == Z else -1
+        a[-1, -1] += 1 if kind == Z else -1
+    w, v = np.linalg.eigh(a)
+    return torch.from_numpy(w / h ** 2).cuda(), torch.from_numpy(v).cuda()
+
+
+def discrete_solution(rho, kind, h):
+    """(high, low) of phi with L phi = rho, by refinement on exact residuals."""
+    free = kind != F
+    axes = [modes(m, kind, h) for m in rho.shape]
+    lam = axes[0][0][:, None, None] + axes[1][0][:, None] + axes[2][0]
+    null = lam.abs() < 1e-6 * lam.abs().max() if free else torch.zeros_like(lam, dtype=torch.bool)
+    lam = torch.where(null, 1.0, lam)
+
+    def minus_mean(x):
+        if not free:
+            return x
+        m = np.sum(x[0].cpu().numpy().astype(np.longdouble)) + np.sum(x[1].cpu().numpy().astype(np.longdouble))
+        m /= x[0].numel()
+        hi = float(m)
+        return dd(x, (torch.full_like(x[0], -hi), torch.full_like(x[0], -float(m - hi))))
+
+    zero = torch.zeros_like(rho)
+    f, phi = minus_mean((rho, zero)), (zero, zero)
+    for _ in range(4):
+        lap = dd((-4 * phi[0], -4 * phi[1]), (-2 * phi[0], -2 * phi[1]),
+                 *zip(neighbours(phi[0], kind), neighbours(phi[1], kind)))
+        r = sum(dd(f, (-lap[0] / h ** 2, -lap[1] / h ** 2)))  # h is a power of two
+        t = torch.einsum("zyx,za,yb,xc->abc", r, *(v for _, v in axes))
+        t = torch.where(null, 0.0, t / lam)
+        phi = dd(phi, (torch.einsum("abc,za,yb,xc->zyx", t, *(v for _, v in axes)), zero))
+    return minus_mean(phi)
+
+
+def blobs(n, count, kind):
+    """Gaussian blobs of width 0.02 to 0.08 of the side (tails wrapped if periodic)."""
+    rng = np.random.default_rng(count)
+    x = (np.arange(n) + 0.5) / n
+    rho = np.zeros((n, n, n))
+    for _ in range(count):
+        s, amp, c = rng.uniform(0.02, 0.08), rng.lognormal(), rng.random(3)
+        d = [x - v for v in c]
+        if kind == P:
+            d = [v - np.round(v) for v in d]
+        g = [np.exp(-0.5 * (v / s) ** 2) for v in d]
+        rho += amp * g[2][:, None, None] * g[1][:, None] * g[0]
+    return torch.from_numpy(rho - (rho.mean() if kind != F else 0.0)).cuda()
+
+
+FLOOR_SIZES = [64]
+
+
+@pytest.mark.parametrize("count", [4, 64])
+@pytest.mark.parametrize("kind", [P, F, Z])
+@pytest.mark.parametrize("n", FLOOR_SIZES)
+def test_rounding_floor_is_that_of_doubles(n, kind, count):
+    """Iterated until it stalls, the solve on the integer grid is as near the
+    discrete solution as the FP64 kernels (an 8-byte aligned phi takes those),
+    to one bit, by the largest and by the mean error of phi and of g."""
+    rho = blobs(n, count, kind)
+    hi, lo = discrete_solution(rho, kind, 1.0 / n)
+    err = []
+    for off in (0, 1):
+        phi = torch.zeros(rho.numel() + 1, dtype=torch.float64, device="cuda")[off:off + rho.numel()].view(rho.shape)
+        with mg.Solver(n, 1.0 / n, kind, prec=mg.FP64) as s:
+            phi, g, _, st = s.solve_gravity(rho, 1.0, 0.0, phi=phi)
+        assert st == 0
+        e = (phi - hi) - lo
+        nb = list(zip(neighbours(hi, kind), neighbours(lo, kind)))
+        eg = [g[a] - sum(dd(nb[4 - 2 * a], (-nb[5 - 2 * a][0], -nb[5 - 2 * a][1]))) * (0.5 * n) for a in range(3)]
+        err.append([e.abs().max(), e.norm(), max(x.abs().max() for x in eg), sum(x.norm() ** 2 for x in eg) ** 0.5])
+    for a, b in zip(*err):
+        assert float(a) <= 2.0 * float(b), [[float(x) for x in row] for row in err]
