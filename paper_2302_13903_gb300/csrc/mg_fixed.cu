@@ -682,6 +682,51 @@ __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
   }
 }
 
+// Exact sums of q per block as pairs (hi, lo).  A pass of its own at the end of
+// an FP64 solve (0.17 ms at 512^3): summed in the down legs, whose registers are
+// all in use, it cost each of ten some 0.13 ms there.  Bound by bytes: four
+// 16-byte loads in flight.
+__global__ void __launch_bounds__(kThreads) k_fx_sum(const longlong2* q, long long n2,
+                                                     long long* __restrict__ psum) {
+  dev::after_previous();
+  SplitSum sum;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  for (; t + 3 * stride < n2; t += 4 * stride) {
+    longlong2 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = q[t + k * stride];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      sum.add(v[k].x);
+      sum.add(v[k].y);
+    }
+  }
+  for (; t < n2; t += stride) {
+    sum.add(q[t].x);
+    sum.add(q[t].y);
+  }
+  __shared__ long long wh[kThreads / 32], wl[kThreads / 32];
+  long long hi = sum.hi(), lo = sum.lo();
+  for (int o = 16; o > 0; o >>= 1) {
+    hi += __shfl_down_sync(0xffffffffu, hi, o);
+    lo += __shfl_down_sync(0xffffffffu, lo, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    wh[threadIdx.x >> 5] = hi;
+    wl[threadIdx.x >> 5] = lo;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kThreads / 32; ++w) {
+      hi += wh[w];
+      lo += wl[w];
+    }
+    psum[2 * blockIdx.x] = hi;
+    psum[2 * blockIdx.x + 1] = lo;
+  }
+}
+
 // out[0] = the total of the (hi, lo) pairs as a double, summed exactly.
 // The integers' sum from the per-block (hi, lo) partials (value = hi 2^32 +
 // lo) and their mean rounded to an integer, exactly: N = 2^log2n cells, so the
@@ -999,6 +1044,14 @@ cudaError_t launch_fx_finish_gravity(const long long* q, double* phi, double* g,
   const FxBc b = fx_bc(bc, two_pow_S);
   ++g_launches;
   launch_after(k_fx_finish_gravity, grid_for(gr.cells()), kThreads, 0, s, q, phi, g, gr, b, S, 1.0 / (2.0 * h * two_pow_S), mean);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fx_sum(const long long* q, long long n, long long* psum, cudaStream_t s) {
+  if (n % 2) return cudaErrorInvalidValue;
+  ++g_launches;
+  launch_after(k_fx_sum, reduce_blocks(n), kThreads, 0, s, reinterpret_cast<const longlong2*>(q),
+               n / 2, psum);
   return cudaGetLastError();
 }
 

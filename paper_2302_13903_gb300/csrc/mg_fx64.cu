@@ -63,7 +63,6 @@ struct Fx64Args {
   double* norm;  // per-CTA sum of R^2: red cells of u_in (down), black cells of u_out (up)
   double* fc;           // down: coarse right-hand side, -sum of R, as doubles,
   long long* fci;       //   or half of it, as F of an integer level (fc null)
-  long long* psum;      // down: per-CTA exact sum of u_in, (hi, lo) pairs
   const long long* ec;  // up: coarse correction on the integer grid
   int limit;            // log2 of the largest |U|
   int* flag;            // |U| or |F| of the coarse level passed its limit
@@ -170,44 +169,23 @@ __device__ __forceinline__ bool too_large(long long v, int m) {
   return (unsigned)((int)(v >> 32) + m) >= 2u * m;
 }
 
-// Block sum of doubles and of (hi, lo) integers into one partial per CTA.
+// Block sum into one partial per CTA.
 template <int NT>
-__device__ __forceinline__ void block_sums(double v, const SplitSum& s, bool sums, double* norm,
-                                           long long* psum) {
+__device__ __forceinline__ void block_sum(double v, double* norm) {
   constexpr int NW = (NT + 31) / 32;
   __shared__ double wd[NW];
-  __shared__ long long wh[NW], wl[NW];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned mask = w == NT / 32 ? (1u << (NT & 31)) - 1 : 0xffffffffu;  // a partial last warp
-  long long hi = s.hi(), lo = s.lo();
   for (int o = 16; o > 0; o >>= 1) {
     const double d = __shfl_down_sync(mask, v, o);
-    const long long h = __shfl_down_sync(mask, hi, o), l = __shfl_down_sync(mask, lo, o);
-    const bool in = lane + o < 32 && (int)threadIdx.x + o < NT;
-    v += in ? d : 0.0;
-    hi += in ? h : 0;
-    lo += in ? l : 0;
+    v += lane + o < 32 && (int)threadIdx.x + o < NT ? d : 0.0;
   }
-  if (lane == 0) {
-    wd[w] = v;
-    wh[w] = hi;
-    wl[w] = lo;
-  }
+  if (lane == 0) wd[w] = v;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    long long th = 0, tl = 0;
-    for (int q = 0; q < NW; ++q) {
-      t += wd[q];
-      th += wh[q];
-      tl += wl[q];
-    }
-    const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    norm[b] = t;
-    if (sums) {
-      psum[2 * b] = th;
-      psum[2 * b + 1] = tl;
-    }
+    for (int q = 0; q < NW; ++q) t += wd[q];
+    norm[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = t;
   }
 }
 
@@ -227,7 +205,7 @@ __device__ __forceinline__ int plane_of(int q, int nz, bool pz) {
 // cell); [C] red defects of q - 3.  The march is unrolled by four, so that ring
 // slots and the registers of the four planes in hand are fixed: plane q is in
 // slot J, planes q - 1, q - 2, q - 3 in J - 1, J - 2, J - 3 (mod 4).
-// COARSE: a correction level, from u = 0 and without the norm and the sum.
+// COARSE: a correction level, from u = 0 and without the norm.
 template <bool WALLS, int TX, bool COARSE>
 __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     k_fx64_down(const __grid_constant__ Fx64Args a) {
@@ -273,7 +251,6 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
   };
   long long uP[4] = {}, uQ[4] = {}, fP[4] = {}, fQ[4] = {};
   long long ud = 0, acc = 0, done = 0;
-  SplitSum psum;
   // outside the level cells stay 0
   auto delta = [&](long long R) { return !WALLS || p.valid ? weigh(R, a.w) : 0; };
   const int most = 1 << (a.limit - 32);
@@ -306,7 +283,6 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
     if (!COARSE) {
       raw[I0] = uB[J];
       if (framed) frame[I0] = frame_in ? ring.frame[J][t] : 0;
-      if (p.tile && q >= z0 && q < z1) psum.add(uP[J] + uQ[J]);
     }
     // the block whose last plane was q - 4: its even and odd row's sums
     if (!EVEN && q - 5 >= z0 && q - 5 < z1 && even_row) {
@@ -375,7 +351,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
   }
   cp_wait<0>();
   if (bad) atomicOr(a.flag, 1);
-  if (!COARSE) block_sums<W::NT>(norm.total(), psum, true, a.norm, a.psum);
+  if (!COARSE) block_sum<W::NT>(norm.total(), a.norm);
 }
 
 // ---------------------------------------------------------------------------
@@ -550,7 +526,7 @@ __global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
   }
   cp_wait<0>();
   if (bad) atomicOr(a.flag, 1);
-  if (!COARSE) block_sums<W::NT>(norm.total(), SplitSum{}, false, a.norm, nullptr);
+  if (!COARSE) block_sum<W::NT>(norm.total(), a.norm);
 }
 
 template <int TX>
@@ -790,7 +766,6 @@ cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s) {
   a.norm = q.norm;
   a.fc = q.fc;
   a.fci = q.fci;
-  a.psum = q.psum;
   a.ec = q.ec;
   // with |ec| < 2^56 and its sums of weight 64 below 2^62
   a.limit = q.coarse ? kFx64Correction : 59;

@@ -332,7 +332,9 @@ cudaError_t launch_fx_step(const long long* phi_in, long long* phi_out, const fl
 cudaError_t launch_fx_finish_gravity(const long long* q, double* phi, double* g, Grid gr,
                                      const Bc& bc, double h, int S, const long long* mean,
                                      cudaStream_t s);
-// out[0] = sum over nb blocks of the pairs launch_fx_step wrote, as a double;
+// reduce_blocks(n) partial sums of q, exact, as pairs (hi, lo); n even.
+cudaError_t launch_fx_sum(const long long* q, long long n, long long* psum, cudaStream_t s);
+// out[0] = sum over nb blocks of the pairs of one of the two, as a double;
 // out[1] (as a long long) = that sum over n = 2^k cells, rounded to an integer.
 cudaError_t launch_finish_fx_sum(const long long* psum, int nb, long long n, double* out,
                                  cudaStream_t s);
@@ -340,14 +342,13 @@ cudaError_t launch_finish_fx_sum(const long long* psum, int nb, long long n, dou
 // ---------------------------------------------------------------------------
 // The FP64 path's finest level in 64-bit fixed point (mg_fx64.cu).  Levels
 // with nx a multiple of 64, ny of 16 and nz even (fx64_ok); per-CTA sums in
-// arrays of fx64_blocks(g) entries (psum: pairs).
+// arrays of fx64_blocks(g) entries.
 bool fx64_ok(Grid g);
 int fx64_cz(Grid g);
 int fx64_blocks(Grid g);
 // down: u_out = SMOOTH(u_in); fc = the restricted defect times 8 h^2 2^S, or
 // fci = half of it, F of an integer coarse level;
-// norm = sums of (h^2 2^S defect)^2 over the red cells of u_in; psum = sums of
-// u_in.  up: u_out = SMOOTH(u_in + trilinear(ec)); norm = the same
+// norm = sums of (h^2 2^S defect)^2 over the red cells of u_in.  up: u_out = SMOOTH(u_in + trilinear(ec)); norm = the same
 // over the black cells of u_out.  coarse: a correction level, down from u_in =
 // 0, no norms and sums.  *flag |= 1 where |u_out| passes 2^59 (coarse
 // 2^kFx64Correction) or fci its range.
@@ -364,7 +365,6 @@ struct Fx64Leg {
   long long* fci;
   const long long* ec;
   double* norm;
-  long long* psum;
   int* flag;
 };
 cudaError_t launch_fx64(const Fx64Leg& q, bool down, cudaStream_t s);

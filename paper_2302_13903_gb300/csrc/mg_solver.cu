@@ -269,9 +269,8 @@ void alloc_hierarchy(mg_ctx* c) {
     const int nb = mg::fx_step_blocks(level_grid(c, F), 0);
     if (nb > c->partials_cap) c->partials_cap = nb;
   }
-  const bool fx64 = fx64_wanted(c);
   // partials, then room for two integers per block of the fixed-point step
-  c->partials = dalloc<double>(c, (fx64 ? 4 : 3) * (size_t)c->partials_cap);
+  c->partials = dalloc<double>(c, 3 * (size_t)c->partials_cap);
   // scalars, then the flags, then the dense matrix
   const size_t dense = dense_level(c) > 0 ? (size_t)mg::kDense * mg::kDense : 0;
   c->scal = dalloc<double>(c, 66 + dense);
@@ -957,7 +956,7 @@ int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, doubl
   if (S < -900 || S > 900) return -1;
   const double two_S = std::ldexp(1.0, S);
   long long *cur = reinterpret_cast<long long*>(phi), *alt = c->fxbuf;
-  double *red = c->partials, *black = c->partials + 3 * (size_t)c->partials_cap;
+  double *red = c->partials, *black = c->partials + c->partials_cap;
   const int nb = mg::fx64_blocks(g);
   check(c, mg::launch_fx64_source(rho, reinterpret_cast<long long*>(c->f64[F]), g, bc, four_pi_G, mu,
                                   h * h * two_S, two_S, c->partials, s),
@@ -977,7 +976,6 @@ int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, doubl
   leg.fc = below ? nullptr : c->f64[F - 1];
   leg.fci = below ? reinterpret_cast<long long*>(c->f64[F - 1]) : nullptr;
   leg.ec = reinterpret_cast<const long long*>(c->u64[F - 1]);
-  leg.psum = reinterpret_cast<long long*>(c->partials + c->partials_cap);
   leg.flag = c->iflag;
   StopRule rule{tol, c->opts.stall_ratio};
   int n = 0, st = -1;
@@ -1015,7 +1013,10 @@ int solve_fx64(mg_ctx* c, const double* rho, double four_pi_G, double tol, doubl
   }
   const long long* mean = nullptr;
   if (mean_free(c)) {
-    check(c, mg::launch_finish_fx_sum(leg.psum, nb, N, c->scal + 56, s), "finish sum phi");
+    long long* psum = reinterpret_cast<long long*>(c->partials);
+    check(c, mg::launch_fx_sum(cur, N, psum, s), "sum phi");
+    check(c, mg::launch_finish_fx_sum(psum, mg::reduce_blocks(N), N, c->scal + 56, s),
+          "finish sum phi");
     mean = reinterpret_cast<const long long*>(c->scal + 57);
   }
   if (gacc) {
