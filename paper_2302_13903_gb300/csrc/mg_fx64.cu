@@ -540,21 +540,31 @@ constexpr size_t up_smem() {
   return sizeof(Ring<W::NT, 1>) + 4 * (size_t)W::PLANE * sizeof(long long);
 }
 
-// F = round(a rho - b) less round(2 b_face 2^S) for each of the cell's fixed and
+// F = a rho - b, rounded, less round(2 b_face 2^S) for each of the cell's fixed and
 // open faces (c2 = 2^(S+1)), b = c *mu; per-block sums of F^2 without the
-// faces' part (the norm of f).
+// faces' part (the norm of f).  Rounding to nearest gives regions of constant rho
+// (the background of compact objects, less its mean) one and the same error, and
+// an error that is smooth is what the inverse of L blows up: at 256^3, four
+// blobs, it was most of the solution's.  So a rho - b is formed to 1/16 and rounded
+// down after the addition of 0 .. 15 sixteenths, each to one cell of 16
+// neighbouring ones, which makes their mean exact; red and black cells take
+// halves of the offsets, so that what is left is as rough as it can be.
 __global__ void __launch_bounds__(256) k_fx64_source(const double* rho,
                                                      long long* __restrict__ F, Grid g, Bc bc,
                                                      double a, double c, const double* mu, double c2,
                                                      double* __restrict__ partials) {
   dev::after_previous();
   const dev::Split sp(g.nx, g.ny);
-  const double b = c * mu[0];
+  a *= 16.0;
+  const double b = 16.0 * c * mu[0];
   const bool faces = bc.kind != BC_PERIODIC && bc.kind != BC_ZEROGRAD;
   SquareSum sum;
 #pragma unroll 4
   for (long long t = blockIdx.x * 256LL + threadIdx.x; t < g.cells(); t += gridDim.x * 256LL) {
-    long long v = cvt::d2ll_rn(fma(a, rho[t], -b));
+    // the last bits of i, i ^ j and i ^ j ^ k, and the next one of the latter
+    const unsigned q = (unsigned)t, xy = q ^ q >> sp.lx, xyz = xy ^ q >> sp.lxy;
+    const unsigned offset = (xyz & 1) << 3 | (xy & 1) << 2 | (q & 1) << 1 | (xyz >> 1 & 1);
+    long long v = (cvt::d2ll_rn(fma(a, rho[t], -b)) + offset) >> 4;
     sum.add(v);
     if (faces) {
       int i, j, k;

@@ -244,7 +244,7 @@ def blobs(n, count, kind):
     return torch.from_numpy(rho - (rho.mean() if kind != F else 0.0)).cuda()
 
 
-FLOOR_SIZES = [64]
+FLOOR_SIZES = [64, 128]
 
 
 @pytest.mark.parametrize("count", [4, 64])
