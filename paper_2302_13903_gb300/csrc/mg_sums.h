@@ -28,36 +28,43 @@ struct SplitSum {
   MG_HD unsigned long long rest() const { return part - ((unsigned long long)(long long)top << 44); }
 };
 
-// Sum of squares of integers |r| < 2^63, exactly, as top 2^128 + hi 2^64 + lo: 32-bit
-// integer instructions only.  A conversion and a multiply-add per cell on the FP64
+// Sum of squares of integers |r| < 2^63, exactly, in five 32-bit words: integer
+// instructions only.  A conversion and a multiply-add per cell on the FP64
 // units, 64 clocks of a scheduler each, set the pace of the integer legs otherwise.
 struct SquareSum {
-  unsigned long long lo = 0, hi = 0;
-  unsigned top = 0;
+  unsigned w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0;
   MG_HD void add(long long r) {
     const unsigned long long a = r < 0 ? 0ull - (unsigned long long)r : (unsigned long long)r;
-    const unsigned h = (unsigned)(a >> 32), l = (unsigned)a;
-    const unsigned long long ll = (unsigned long long)l * l, hh = (unsigned long long)h * h;
-    const unsigned long long m = (unsigned long long)l * h;  // r^2 = hh 2^64 + m 2^33 + ll
-    sum(ll, hh);
-    sum(m << 33, m >> 31);
-  }
-  MG_HD double total() const {
-    return ((double)top * 0x1p64 + (double)hi) * 0x1p64 + (double)lo;
-  }
-
- private:
-  MG_HD void sum(unsigned long long l, unsigned long long h) {
+    const unsigned h = (unsigned)(a >> 32), l = (unsigned)a, h2 = 2 * h;  // h < 2^31
 #ifdef __CUDA_ARCH__
-    asm("add.cc.u64 %0, %0, %3;\n\taddc.cc.u64 %1, %1, %4;\n\taddc.u32 %2, %2, 0;"
-        : "+l"(lo), "+l"(hi), "+r"(top)
-        : "l"(l), "l"(h));
+    asm("mad.lo.cc.u32 %0, %5, %5, %0;\n\tmadc.hi.cc.u32 %1, %5, %5, %1;\n\t"
+        "addc.cc.u32 %2, %2, 0;\n\taddc.cc.u32 %3, %3, 0;\n\taddc.u32 %4, %4, 0;"
+        : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3), "+r"(w4)
+        : "r"(l));
+    if (h)
+      asm("mad.lo.cc.u32 %0, %4, %6, %0;\n\tmadc.hi.cc.u32 %1, %4, %6, %1;\n\t"
+        "addc.cc.u32 %2, %2, 0;\n\taddc.u32 %3, %3, 0;\n\t"
+        "mad.lo.cc.u32 %1, %5, %5, %1;\n\tmadc.hi.cc.u32 %2, %5, %5, %2;\n\taddc.u32 %3, %3, 0;"
+        : "+r"(w1), "+r"(w2), "+r"(w3), "+r"(w4)
+        : "r"(l), "r"(h), "r"(h2));
 #else
-    lo += l;
-    const unsigned long long c = lo < l, k = hi + h;
-    hi = k + c;
-    top += (k < h) + (hi < c);
+    const unsigned long long ll = (unsigned long long)l * l, hh = (unsigned long long)h * h;
+    const unsigned long long m = (unsigned long long)l * h2;
+    unsigned long long c = (unsigned long long)w0 + (unsigned)ll;
+    w0 = (unsigned)c;
+    c = (c >> 32) + w1 + (ll >> 32) + (unsigned)m;
+    w1 = (unsigned)c;
+    c = (c >> 32) + w2 + (unsigned)hh + (m >> 32);
+    w2 = (unsigned)c;
+    c = (c >> 32) + w3 + (hh >> 32);
+    w3 = (unsigned)c;
+    w4 += (unsigned)(c >> 32);
 #endif
+  }
+  MG_HD unsigned long long lo() const { return (unsigned long long)w1 << 32 | w0; }
+  MG_HD unsigned long long hi() const { return (unsigned long long)w3 << 32 | w2; }
+  MG_HD double total() const {
+    return ((double)w4 * 0x1p64 + (double)hi()) * 0x1p64 + (double)lo();
   }
 };
 

@@ -49,9 +49,9 @@ static void square_sum() {
         high += (unsigned long long)(sq >> 64);
       }
       high += (unsigned long long)(low >> 64);
-      CHECK(s.lo == (unsigned long long)low);
-      CHECK(s.hi == (unsigned long long)high);
-      CHECK(s.top == (unsigned)(high >> 64));
+      CHECK(s.lo() == (unsigned long long)low);
+      CHECK(s.hi() == (unsigned long long)high);
+      CHECK(s.w4 == (unsigned)(high >> 64));
       const double want = (double)high * 0x1p64 + (double)(unsigned long long)low;
       CHECK(std::fabs(s.total() - want) <= 0x1p-52 * want);
     }
