@@ -137,7 +137,9 @@ void mg_opts_init(mg_opts *opts);
  * side has one cell (Sec. 3.2.1): for a cube the coarsest level is one cell,
  * solved exactly; for a box it has several, smoothed by N_0,max Gauss-Seidel
  * sweeps (Sec. 2.3.2).  The level hierarchy and all scratch are allocated on
- * the current device here.  opts may be NULL for defaults; it is copied.  On
+ * the current device here, but for two things that the first solve which uses
+ * them allocates: an MG_FP64 solve's integer buffers (mg_solve_bytes) and
+ * mg_solve_host's device copies of rho and phi.  opts may be NULL for defaults; it is copied.  On
  * success *ctx owns the device memory until mg_destroy.  Errors: MG_ERR_ARG
  * (sizes, kinds, options), MG_ERR_OOM, MG_ERR_CUDA. */
 mg_status mg_create(int nx, int ny, int nz, double dx, mg_bc bc, const mg_opts *opts,
@@ -175,10 +177,30 @@ mg_status mg_solve_gravity(mg_ctx *ctx, const double *rho_dev, double four_pi_G,
 
 /* Device bytes mg_create would allocate for this grid and these options
  * (the level hierarchy and scratch, as requested from cudaMalloc; the
- * allocator's rounding is not included).  Allocates nothing.  Errors:
- * MG_ERR_ARG as mg_create. */
+ * allocator's rounding is not included).  What the first solve adds is
+ * mg_solve_bytes.  Allocates nothing.  Errors: MG_ERR_ARG as mg_create. */
 mg_status mg_required_bytes(int nx, int ny, int nz, mg_bc bc, const mg_opts *opts,
                             size_t *bytes);
+
+/* Device bytes the first mg_solve of such a context adds: the second buffers of
+ * the levels that an MG_FP64 solve runs in 64-bit fixed point (levels from 64^3
+ * up, of a solve from an FMG start with pre = post = 1, fas = coarse_literal =
+ * 0), up to 9.1 bytes per cell; 0 for other solves.  They are taken once and
+ * kept, and only where they are at most half of the device's free memory;
+ * without them the same solve runs on the FP64 kernels, three to four times
+ * slower at 512^3, to the same tolerance but not to the same bits.  Allocates
+ * nothing.  Errors: MG_ERR_ARG (sizes, options). */
+mg_status mg_solve_bytes(int nx, int ny, int nz, const mg_opts *opts, size_t *bytes);
+
+/* Whether solves of this context may take those buffers.  on = 0: never; what
+ * it holds is freed.  1 (default): the next solve that would use them asks for
+ * them, also after an earlier solve did not get them.  Errors: MG_ERR_ARG. */
+mg_status mg_ctx_set_solve_buffers(mg_ctx *ctx, int on);
+
+/* 1 where the last solve of this context ran its upper levels in fixed point
+ * (MG_FP64: on the integer buffers; MG_MIXED: the outer loop), 0 where it ran
+ * in floating point throughout. */
+int mg_ctx_fixed_point(const mg_ctx *ctx);
 
 /* Solve for phi given rho: f = four_pi_G * rho; for periodic and
  * zero-gradient grids the mean of f is removed and the returned phi has zero
@@ -208,7 +230,8 @@ mg_status mg_solve_host(mg_ctx *ctx, const double *rho, double four_pi_G, double
 /* Release the context and its device memory.  NULL is accepted. */
 mg_status mg_destroy(mg_ctx *ctx);
 
-/* Bytes of device memory the context holds. */
+/* Bytes of device memory the context holds now: mg_required_bytes after
+ * mg_create, more after the solves that allocate (see there). */
 size_t mg_ctx_device_bytes(const mg_ctx *ctx);
 
 /* Number of kernel launches issued by the last mg_solve / mg_solve_host of
@@ -225,8 +248,9 @@ typedef enum {
   MG_K_OUTER_RESIDUAL = 5,  /* MIXED: FP64 residual -> FP32                       */
   MG_K_CORRECT = 6,         /* MIXED: FP64 correction update                      */
   MG_K_SOURCE = 7,          /* f = 4 pi G rho and its sums                         */
-  MG_K_FUSED_DOWN = 8,      /* FP32 fused SMOOTH + defect + restriction           */
-  MG_K_FUSED_UP = 9,        /* FP32 fused prolongation + correction + SMOOTH      */
+  MG_K_FUSED_DOWN = 8,      /* FP32 fused SMOOTH + defect + restriction; MG_FP64  */
+                            /* in fixed point: the same leg on 64-bit integers    */
+  MG_K_FUSED_UP = 9,        /* fused prolongation + correction + SMOOTH, as above */
   MG_K_GRAVITY = 10,        /* acceleration g = -grad phi (mg_solve_gravity)       */
   MG_K_FUSED_DOWN0 = 11,    /* MG_K_FUSED_DOWN from a zero start (reads f only)   */
   MG_K_FUSED_UPDOWN = 12,   /* FP32 up leg of one V-cycle and down leg of the     */

@@ -34,7 +34,7 @@ EXPORTS = [
     "mg_server_create", "mg_server_submit", "mg_server_poll", "mg_server_wait",
     "mg_server_get_stats", "mg_server_destroy", "mg_server_last_error", "mg_op_convert",
     "mg_op_fused_leg", "mg_op_fx_step", "mg_batch_set_barrier_limit", "mg_batch_set_blocks",
-    "mg_ctx_tensor_copies",
+    "mg_ctx_tensor_copies", "mg_solve_bytes", "mg_ctx_set_solve_buffers", "mg_ctx_fixed_point",
 ]
 KERNELS = ["sor", "defect_restrict", "prolong", "fmg_prolong", "defect_norm", "outer_residual",
            "correct", "source", "fused_down", "fused_up", "gravity", "fused_down0",
@@ -196,6 +196,12 @@ def lib():
             L.mg_ctx_tile_config.restype = i
             L.mg_required_bytes.argtypes = [i, i, i, i, ctypes.POINTER(Opts), ctypes.POINTER(sz)]
             L.mg_required_bytes.restype = i
+            L.mg_solve_bytes.argtypes = [i, i, i, ctypes.POINTER(Opts), ctypes.POINTER(sz)]
+            L.mg_solve_bytes.restype = i
+            L.mg_ctx_set_solve_buffers.argtypes = [p, i]
+            L.mg_ctx_set_solve_buffers.restype = i
+            L.mg_ctx_fixed_point.argtypes = [p]
+            L.mg_ctx_fixed_point.restype = i
             L.mg_server_create.argtypes = [sz, i, i, ctypes.POINTER(Opts), ctypes.POINTER(p)]
             L.mg_server_create.restype = i
             L.mg_server_submit.argtypes = [p, ctypes.POINTER(Request),
@@ -306,6 +312,15 @@ class Solver:
     @property
     def device_bytes(self):
         return lib().mg_ctx_device_bytes(self.ctx)
+
+    def set_solve_buffers(self, on):
+        """Whether FP64 solves may take their integer buffers (mg_ctx_set_solve_buffers)."""
+        _check(lib().mg_ctx_set_solve_buffers(self.ctx, int(on)), self.ctx)
+
+    @property
+    def fixed_point(self):
+        """Whether the last solve ran its upper levels in fixed point."""
+        return bool(lib().mg_ctx_fixed_point(self.ctx))
 
     @property
     def last_launches(self):
@@ -686,6 +701,14 @@ def required_bytes(n, bc=PERIODIC, **opts) -> int:
     o = default_opts(**opts)
     b = ctypes.c_size_t(0)
     _check(lib().mg_required_bytes(n, n, n, bc, ctypes.byref(o), ctypes.byref(b)))
+    return b.value
+
+
+def solve_bytes(n, **opts) -> int:
+    """Device bytes the first solve of an n^3 grid adds (mg_solve_bytes)."""
+    o = default_opts(**opts)
+    b = ctypes.c_size_t(0)
+    _check(lib().mg_solve_bytes(n, n, n, ctypes.byref(o), ctypes.byref(b)))
     return b.value
 
 

@@ -69,11 +69,8 @@ mg_status solve_host_copies(mg_ctx* c, const double* rho, double four_pi_G, doub
                             double* phi, double* hist, int hist_cap, int* n_hist,
                             cudaStream_t s, double* copy_ms = nullptr);
 
-// Device bytes the first mg_solve of a context of this shape adds to what
-// mg_create allocated (mg_required_bytes): the FP64 path's integer buffers.
+// mg_solve_bytes (0 for sizes no context takes).
 size_t solve_buffer_bytes(int nx, int ny, int nz, const mg_opts& opts);
-// Solves of this context do without them (in FP64 throughout).
-void no_solve_buffers(mg_ctx* c);
 
 // Record the message mg_last_error(NULL) returns on this thread (entry points
 // that have no context report their failures through it).

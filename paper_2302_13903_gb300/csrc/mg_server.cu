@@ -169,7 +169,7 @@ mg_status create_hier(mg_server* S, const Request* r, cudaStream_t stream, Hier*
                            r->req.face_value, &o, &h->ctx);
     else
       st = mg_create(r->req.nx, r->req.ny, r->req.nz, r->req.dx, r->req.bc, &o, &h->ctx);
-    if (st == MG_OK && r->plain) mg::no_solve_buffers(h->ctx);
+    if (st == MG_OK && r->plain) mg_ctx_set_solve_buffers(h->ctx, 0);
     if (st == MG_OK) mg_ctx_autotune(h->ctx, stream);  // shapes, cached per process
   }
   if (st != MG_OK) {

@@ -50,7 +50,8 @@ struct mg_ctx {
   double* faces[kMaxLevels] = {};  // open / fixed-face boundary values per level
   double* ur64[kMaxLevels] = {};   // FAS: restricted potential per coarse level
   long long* ub64[kMaxLevels] = {};  // second buffer of the integer correction levels
-  bool fx64_tried = false;           // whether those buffers were asked for
+  bool fx64_tried = false;           // those buffers are not to be asked for (again)
+  bool fixed_point = false;          // the last solve ran on integers
   // FP32 hierarchy (mixed precision); u32b is the second buffer of levels the
   // fused kernels handle (they read one buffer and write the other).
   float* u32[kMaxLevels] = {};
@@ -217,11 +218,19 @@ bool fx64_wanted(const mg_ctx* c) {
 
 // The integer levels' second buffers (the first ones are phi's own storage and
 // the FP64 levels'), 9.1 bytes per finest cell: allocated by the first solve
-// that uses them and kept; where they do not fit, the solve runs in FP64.
+// that uses them and kept; where they do not fit, or would take more than half
+// of the free memory, which the caller may have planned to use, the solve runs
+// in FP64.
 bool fx64_buffers(mg_ctx* c) {
   if (c->fxbuf) return true;
   if (c->fx64_tried || !fx64_wanted(c)) return false;
   c->fx64_tried = true;
+  size_t unused = 0, total = 0;
+  if (cudaMemGetInfo(&unused, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (mg::solve_buffer_bytes(c->n, c->ny, c->nz, c->opts) > unused / 2) return false;
   const size_t had = c->allocs.size(), bytes = c->bytes;
   try {
     for (int l = c->L - 2; l > 0 && mg::fx64_ok(level_grid(c, l)); --l)
@@ -1055,6 +1064,7 @@ mg_status solve_fp64(mg_ctx* c, const double* rho, double four_pi_G, double tol,
   if (((pp | pr) & 15u) == 0 && apart && fx64_buffers(c)) {
     const int st = solve_fx64(c, rho, four_pi_G, tol, phi, gacc, bcs, hom, hist, hist_cap, n_hist, s);
     if (st >= 0) {
+      c->fixed_point = true;
       c->u64[F] = nullptr;
       return (mg_status)st;
     }
@@ -1333,6 +1343,7 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
     if (st >= 0) break;
   }
   int late = 0;  // iflag[1]
+  c->fixed_point = in_fx;
   if (in_fx) {
     // phi = (PHI - M) 2^-S, M the integers' mean (periodic / zero gradient)
     // rounded to an integer, from the last step's exact integer sums
@@ -1777,8 +1788,6 @@ size_t mg::solve_buffer_bytes(int nx, int ny, int nz, const mg_opts& o) {
   return cells * sizeof(long long);
 }
 
-void mg::no_solve_buffers(mg_ctx* c) { c->fx64_tried = true; }
-
 extern "C" {
 
 void mg_opts_init(mg_opts* o) {
@@ -2033,6 +2042,39 @@ mg_status mg_required_bytes(int nx, int ny, int nz, mg_bc bc, const mg_opts* opt
   return MG_OK;
 }
 
+mg_status mg_solve_bytes(int nx, int ny, int nz, const mg_opts* opts, size_t* bytes) {
+  if (!bytes) return MG_ERR_ARG;
+  *bytes = 0;
+  mg_opts o;
+  if (opts) o = *opts;
+  else mg_opts_init(&o);
+  if (!dims_ok(nx, ny, nz) || validate_opts(o) != MG_OK) {
+    g_err = "mg_solve_bytes: invalid argument";
+    return MG_ERR_ARG;
+  }
+  *bytes = mg::solve_buffer_bytes(nx, ny, nz, o);
+  return MG_OK;
+}
+
+mg_status mg_ctx_set_solve_buffers(mg_ctx* c, int on) {
+  if (!c || (on != 0 && on != 1)) return MG_ERR_ARG;
+  c->fx64_tried = on == 0;
+  if (on != 0 || c->opts.prec != MG_FP64 || !c->fxbuf) return MG_OK;
+  drop_inner_graph(c);  // it holds the buffers' addresses
+  auto give_back = [&](long long*& p, int l) {
+    if (!p) return;
+    cudaFree(p);
+    c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), static_cast<void*>(p)));
+    c->bytes -= (size_t)level_grid(c, l).cells() * sizeof(long long);
+    p = nullptr;
+  };
+  for (int l = 0; l < c->L; ++l) give_back(c->ub64[l], l);
+  give_back(c->fxbuf, c->L - 1);
+  return MG_OK;
+}
+
+int mg_ctx_fixed_point(const mg_ctx* c) { return c && c->fixed_point ? 1 : 0; }
+
 // The stream a solve given stream s runs on: s, or for the legacy default
 // stream (whose launches cannot be captured as a graph) the context's own,
 // ordered after what the default stream holds now.  The solve synchronises it
@@ -2065,6 +2107,7 @@ mg_status mg_solve_gravity(mg_ctx* c, const double* rho, double four_pi_G, doubl
     return MG_ERR_ARG;
   }
   *n_hist = 0;
+  c->fixed_point = false;
   cudaStream_t s = (cudaStream_t)stream;
   mg::g_launches = 0;
   mg_status st;

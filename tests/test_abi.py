@@ -91,6 +91,22 @@ def test_required_bytes_counts_the_hierarchy():
     assert L.mg_required_bytes(8, 8, 8, 0, ctypes.byref(o), None) == 1
 
 
+def test_solve_bytes_counts_the_integer_buffers():
+    """A second 64-bit buffer for the finest level and each one down to 64^3 of an
+    FP64 solve from an FMG start with V(1,1); nothing else allocates in a solve."""
+    assert mg.solve_bytes(128, prec=mg.FP64) == 8 * (128 ** 3 + 64 ** 3)
+    assert mg.solve_bytes(64, prec=mg.FP64) == 8 * 64 ** 3
+    assert mg.solve_bytes(32, prec=mg.FP64) == 0
+    for kw in (dict(prec=mg.MIXED), dict(mode_fmg=0), dict(fas=1), dict(pre=2),
+               dict(coarse_literal=1)):
+        assert mg.solve_bytes(128, **kw) == 0, kw
+    L = mg.lib()
+    b, o = ctypes.c_size_t(0), mg.default_opts()
+    assert L.mg_solve_bytes(12, 12, 12, ctypes.byref(o), ctypes.byref(b)) == 1
+    assert L.mg_solve_bytes(8, 8, 8, None, None) == 1
+    assert L.mg_ctx_set_solve_buffers(None, 1) == 1 and L.mg_ctx_fixed_point(None) == 0
+
+
 def test_server_argument_validation_needs_no_gpu():
     L = mg.lib()
     h = ctypes.c_void_p()

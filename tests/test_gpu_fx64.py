@@ -160,6 +160,46 @@ def test_a_solve_that_diverges_is_the_general_path(rule):
         assert np.array_equal(hist, h0) and np.array_equal(phi, ref)
 
 
+def test_solve_buffers_are_counted_and_can_be_declined():
+    """The first solve adds mg_solve_bytes to the context, or with the buffers
+    declined nothing, and runs on the FP64 kernels (as for a misaligned phi)."""
+    rho = source((64, 64, 64), 8)
+    odd = torch.zeros(rho.size + 1, dtype=torch.float64, device="cuda")[1:].view(rho.shape)
+    plain = gpu(rho, "periodic", tol=1e-9, phi=odd)[0]
+    dev = torch.from_numpy(rho).cuda()
+    with mg.Solver(64, 1.0 / 64, P, prec=mg.FP64) as s:
+        need, extra = mg.required_bytes(64, P, prec=mg.FP64), mg.solve_bytes(64, prec=mg.FP64)
+        assert s.device_bytes == need
+        first = s.solve(dev, 1.0, 1e-9)[0]
+        assert s.device_bytes == need + extra and s.fixed_point
+        s.set_solve_buffers(False)
+        assert s.device_bytes == need
+        for _ in range(3):  # launch by launch, captured, replayed
+            assert np.array_equal(s.solve(dev, 1.0, 1e-9)[0].cpu().numpy(), plain)
+            assert s.device_bytes == need and not s.fixed_point
+        s.set_solve_buffers(True)
+        for _ in range(3):
+            assert torch.equal(s.solve(dev, 1.0, 1e-9)[0], first)
+            assert s.device_bytes == need + extra and s.fixed_point
+
+
+def test_server_counts_the_solve_buffers_or_does_without():
+    """A budget that holds them: a solve's own bits; one that holds the hierarchy
+    alone: accepted, with the FP64 kernels' bits."""
+    rho = source((64, 64, 64), 9)
+    odd = torch.zeros(rho.size + 1, dtype=torch.float64, device="cuda")[1:].view(rho.shape)
+    plain, fixed = gpu(rho, "periodic", tol=1e-9, phi=odd)[0], gpu(rho, "periodic", tol=1e-9)[0]
+    need = mg.required_bytes(64, P, prec=mg.FP64)
+    for budget, want in ((need + mg.solve_bytes(64, prec=mg.FP64), fixed), (need, plain)):
+        with mg.Server(budget, slots=1, prec=mg.FP64) as s:
+            phi = torch.zeros(rho.shape, dtype=torch.float64, device="cuda")
+            for _ in range(2):
+                t = s.submit(torch.from_numpy(rho).cuda(), phi, bc=P, tol=1e-9)
+                assert s.wait(t, 60)[0].status == 0
+                assert np.array_equal(phi.cpu().numpy(), want)
+            assert s.stats()["peak_bytes"] == budget
+
+
 # --- the rounding floor: errors against the discrete solution in double-double ---
 
 def two_sum(a, b):
