@@ -462,8 +462,9 @@ mg_status mg_batch_create(int n, const int *dims, const double *dx, const mg_bc 
  * form a class; the classes run side by side on streams of the batch's own,
  * ordered after `stream`, a launch per phase and class, each outer iteration
  * after a class's first as a CUDA graph (so make the call outside any capture
- * of your own).  After mg_batch_set_blocks or mg_batch_set_barrier_limit, and
- * for more than 24 classes, one persistent cooperative kernel runs every phase
+ * of your own).  After mg_batch_set_blocks or mg_batch_set_barrier_limit, for
+ * more than 24 classes, and where a grid's phi lies in memory that another class
+ * reads as rho (every rho is read before any phi is written), one persistent cooperative kernel runs every phase
  * of every grid instead, captured by the first call and replayed by later
  * ones: the same bits.  Each grid stops by the rule of mg_solve (Sec. 2.3.7).  hist (host, n * hist_cap, may be NULL)
  * receives each grid's ||d||/||f|| after every outer iteration, n_hist[g] the

@@ -41,6 +41,7 @@
 #include "mg_device.cuh"
 #include "mg_fused.cuh"
 #include "mg_internal.h"
+#include "mg_spans.h"
 
 namespace mg {
 namespace batch {
@@ -1167,6 +1168,7 @@ struct mg_batch {
     bool last = false;               // its final phases are queued
   };
   std::vector<Class> classes;
+  std::vector<int> class_of;  // each grid's class
   int* d_class = nullptr;
   unsigned long long* d_work = nullptr;
   int* d_fin = nullptr;   // two counters per class
@@ -1344,6 +1346,7 @@ cudaError_t enqueue_solve(mg_batch* b, cudaStream_t s) {
 void make_classes(mg_batch* b, std::vector<int>& order) {
   using Class = mg_batch::Class;
   std::vector<Class>& cs = b->classes;
+  b->class_of.assign((size_t)b->ngrids, 0);
   std::vector<std::vector<int>> members;
   for (int g = 0; g < b->ngrids; ++g) {
     const GridDev& d = b->host_grids[g];
@@ -1376,6 +1379,7 @@ void make_classes(mg_batch* b, std::vector<int>& order) {
     Class k = cs[q];
     k.first = (int)order.size();
     k.count = (int)members[q].size();
+    for (int g : members[q]) b->class_of[(size_t)g] = (int)sorted.size();
     order.insert(order.end(), members[q].begin(), members[q].end());
     sorted.push_back(k);
   }
@@ -1515,6 +1519,22 @@ bool staged_ready(mg_batch* b) {
   if (!ok) cudaGetLastError();
   b->start_ok = ok;
   return ok;
+}
+
+// Whether a grid's phi lies in memory that another class reads as rho.  A class
+// writes its phi while others may not have read their rho yet; the persistent
+// kernel reads every rho before it writes any phi.
+bool phi_over_rho(const mg_batch* b) {
+  std::vector<Span> out, in;
+  for (int g = 0; g < b->ngrids; ++g) {
+    const GridDev& d = b->h_grids[g];
+    if (d.skip) continue;
+    const size_t bytes = sizeof(double) * (size_t)d.n * d.n * d.n;
+    const uintptr_t p = (uintptr_t)d.phi, r = (uintptr_t)d.rho;
+    out.push_back({p, p + bytes, b->class_of[(size_t)g]});
+    in.push_back({r, r + bytes, b->class_of[(size_t)g]});
+  }
+  return spans_cross(out, std::move(in));
 }
 
 cudaError_t staged_solve(mg_batch* b, cudaStream_t s) {
@@ -1774,9 +1794,10 @@ mg_status mg_batch_solve(mg_batch* b, const double* const* rho, const double* fo
   // The staged solve was faster or as fast at every size (GB300, ms, staged and
   // persistent: 512 grids of 16-128 22.8, 34.2; one of 128 1.09, 3.8; 64 of 32
   // 1.39, 2.6; 256 of 16 0.99, 0.99; 16 of 16 0.57, 0.58).  The persistent
-  // kernel serves callers that limit its CTAs or its barriers, and batches of
-  // more classes than streams.
-  b->staged = b->blocks == b->max_blocks && b->bar_cycles == kBarrierCycles && staged_ready(b);
+  // kernel serves callers that limit its CTAs or its barriers, batches of more
+  // classes than streams, and solves with a phi in another class's rho.
+  b->staged = b->blocks == b->max_blocks && b->bar_cycles == kBarrierCycles && staged_ready(b) &&
+              !(b->classes.size() > 1 && phi_over_rho(b));
   if (!b->staged && !b->graph_tried) {
     // Capture the whole solve (upload of the per-grid arguments, counter
     // resets, the persistent kernel, download of the results) once.

@@ -62,3 +62,30 @@ def test_max_cycles_ends_every_class():
         assert got[3] == ref[3] and all(len(h) == m for h in got[2])
         for p, q in zip(got[0], ref[0]):
             assert torch.equal(p, q)
+
+
+def test_phi_in_another_grids_source():
+    """Every rho is read before any phi is written, also where they share memory
+    across sizes: the results are those of separate arrays."""
+    specs = [(64, mg.PERIODIC), (16, mg.FIXED), (32, mg.ZEROGRAD)]
+    rhos = [torch.from_numpy(inputs.batch_source(dict(n=n, bc=bc, seed=n, n_blobs=3))).cuda()
+            for n, bc in specs]
+    with mg.Batch([n for n, _ in specs], [1.0 / n for n, _ in specs],
+                  [bc for _, bc in specs]) as b:
+        ref, st, hists, sts = solve(b, rhos, 1e-10)
+        # the small grids' phi in the large grid's rho, the large one's over both
+        # small sources
+        big = rhos[0].clone().view(-1)
+        both = torch.zeros(64 ** 3, dtype=torch.float64, device="cuda")
+        both[:16 ** 3] = rhos[1].view(-1)
+        both[16 ** 3:16 ** 3 + 32 ** 3] = rhos[2].view(-1)
+        src = [big.view(64, 64, 64), both[:16 ** 3].view(16, 16, 16),
+               both[16 ** 3:16 ** 3 + 32 ** 3].view(32, 32, 32)]
+        out = [both.view(64, 64, 64), big[:16 ** 3].view(16, 16, 16),
+               big[16 ** 3:16 ** 3 + 32 ** 3].view(32, 32, 32)]
+        # (the large grid's phi is written over the small ones' sources, theirs
+        # over its source)
+        got = b.solve(src, out, 1.0, 1e-10)
+        assert got[0] == st and list(got[2]) == sts
+        for p, q, h, k in zip(out, ref, got[1], hists):
+            assert torch.equal(p, q) and np.array_equal(h, k)
