@@ -466,7 +466,9 @@ mg_status mg_batch_create(int n, const int *dims, const double *dx, const mg_bc 
  * more than 24 classes, and where a grid's phi lies in memory that another class
  * reads as rho (every rho is read before any phi is written), one persistent cooperative kernel runs every phase
  * of every grid instead, captured by the first call and replayed by later
- * ones: the same bits.  Each grid stops by the rule of mg_solve (Sec. 2.3.7).  hist (host, n * hist_cap, may be NULL)
+ * ones: the same bits.  The calling thread waits as the device's scheduling flag
+ * says (cudaDeviceScheduleBlockingSync: it blocks or sleeps; else it polls).
+ * Each grid stops by the rule of mg_solve (Sec. 2.3.7).  hist (host, n * hist_cap, may be NULL)
  * receives each grid's ||d||/||f|| after every outer iteration, n_hist[g] the
  * count, status[g] its result.  Returns MG_OK when every grid converged, else
  * the first failing grid's status, MG_ERR_TIMEOUT if a grid-wide barrier wait

@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1571,8 +1572,19 @@ cudaError_t staged_solve(mg_batch* b, cudaStream_t s) {
     queue(k, 0);
     ++open;
   }
+  // The host waits for whichever class is done first.  The driver's own wait takes
+  // over where that is one class, and follows the device's scheduling flag; for
+  // several the host polls, or sleeps in between where that flag asks for waits
+  // that block.
+  unsigned flags = 0;
+  also(cudaGetDeviceFlags(&flags));
+  const bool block = (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
   std::vector<char> closed(cs.size(), 0);
   while (e == cudaSuccess && open > 0) {
+    if (open == 1) {
+      const size_t q = (size_t)(std::find(closed.begin(), closed.end(), 0) - closed.begin());
+      also(cudaStreamSynchronize(cs[q].s));
+    }
     for (size_t q = 0; q < cs.size() && e == cudaSuccess; ++q) {
       if (closed[q]) continue;
       const cudaError_t r = cudaEventQuery(cs[q].ev);
@@ -1589,7 +1601,10 @@ cudaError_t staged_solve(mg_batch* b, cudaStream_t s) {
         queue(cs[q], left == 0 || cs[q].done >= b->opts.max_cycles ? 2 : 1);
       }
     }
-    std::this_thread::yield();
+    if (open > 1) {
+      if (block) std::this_thread::sleep_for(std::chrono::microseconds(50));
+      else std::this_thread::yield();
+    }
   }
   if (e != cudaSuccess)  // nothing of this solve stays in flight
     for (auto& k : cs) cudaStreamSynchronize(k.s);

@@ -89,3 +89,42 @@ def test_phi_in_another_grids_source():
         assert got[0] == st and list(got[2]) == sts
         for p, q, h, k in zip(out, ref, got[1], hists):
             assert torch.equal(p, q) and np.array_equal(h, k)
+
+
+BLOCKING = r"""
+import ctypes, sys, time
+sys.path.insert(0, sys.argv[1])
+cu = ctypes.CDLL("libcuda.so.1")
+assert cu.cuInit(0) == 0
+assert cu.cuDevicePrimaryCtxSetFlags_v2(0, 4) == 0  # CU_CTX_SCHED_BLOCKING_SYNC, of this process
+import torch
+import paper_2302_13903_gb300 as mg
+from paper_2302_13903_gb300 import inputs
+specs = [(256, mg.PERIODIC), (256, mg.FIXED), (128, mg.FIXED)][:int(sys.argv[2])]
+rhos = [torch.from_numpy(inputs.batch_source(dict(n=n, bc=bc, seed=n, n_blobs=3))).cuda()
+        for n, bc in specs]
+phis = [torch.zeros_like(r) for r in rhos]
+with mg.Batch([n for n, _ in specs], [1.0 / n for n, _ in specs], [bc for _, bc in specs]) as b:
+    for _ in range(3):
+        b.solve(rhos, phis, 1.0, 1e-10)
+    torch.cuda.synchronize()
+    wall, cpu = time.perf_counter(), time.thread_time()
+    for _ in range(10):
+        b.solve(rhos, phis, 1.0, 1e-10)
+    wall, cpu = time.perf_counter() - wall, time.thread_time() - cpu
+print(cpu / wall)
+"""
+
+
+@pytest.mark.parametrize("classes", [1, 3])
+def test_a_blocking_process_blocks(classes):
+    """Where the process asked for waits that block, the calling thread is idle for
+    most of a solve of large grids (its launches take some tenths of it)."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", BLOCKING, root, str(classes)], capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    assert float(r.stdout) < 0.6, r.stdout
