@@ -2081,10 +2081,10 @@ int mg_ctx_fixed_point(const mg_ctx* c) { return c && c->fixed_point ? 1 : 0; }
 // before it returns, so later work on any stream comes after it.
 static cudaStream_t capturable_stream(mg_ctx* c, cudaStream_t s) {
   if (s != nullptr && s != cudaStreamLegacy) return s;
-  if (!c->own_stream) {
+  if (!c->own_stream)
     check(c, cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking), "stream");
+  if (!c->own_event)
     check(c, cudaEventCreateWithFlags(&c->own_event, cudaEventDisableTiming), "event");
-  }
   check(c, cudaEventRecord(c->own_event, s), "record");
   check(c, cudaStreamWaitEvent(c->own_stream, c->own_event, 0), "wait");
   return c->own_stream;

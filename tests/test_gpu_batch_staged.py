@@ -128,3 +128,21 @@ def test_a_blocking_process_blocks(classes):
                        text=True, timeout=300)
     assert r.returncode == 0, r.stderr
     assert float(r.stdout) < 0.6, r.stdout
+
+
+def test_phase_times_after_set_blocks_and_back():
+    """The shares of a staged solve, the barrier times of a persistent one, and the
+    former again: no negative time, and no more in all than the call took."""
+    import time
+    rhos = [torch.from_numpy(inputs.batch_source(dict(n=n, bc=bc, seed=n, n_blobs=3))).cuda()
+            for n, bc in ((64, mg.PERIODIC), (32, mg.FIXED))]
+    with mg.Batch([64, 32], [1 / 64, 1 / 32], [mg.PERIODIC, mg.FIXED]) as b:
+        for blocks in (0, 7, 0):
+            b.set_blocks(blocks)
+            for _ in range(2):
+                t = time.perf_counter()
+                solve(b, rhos, 1e-10)
+                wall = 1e3 * (time.perf_counter() - t)
+                ms = b.phase_ms()
+                ms = list(ms.values()) if isinstance(ms, dict) else list(ms)
+                assert min(ms) >= 0.0 and 0.0 < sum(ms) <= wall
