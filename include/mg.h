@@ -139,9 +139,10 @@ void mg_opts_init(mg_opts *opts);
  * sweeps (Sec. 2.3.2).  The level hierarchy and all scratch are allocated on
  * the current device here, but for two things that the first solve which uses
  * them allocates: an MG_FP64 solve's integer buffers (mg_solve_bytes) and
- * mg_solve_host's device copies of rho and phi.  opts may be NULL for defaults; it is copied.  On
- * success *ctx owns the device memory until mg_destroy.  Errors: MG_ERR_ARG
- * (sizes, kinds, options), MG_ERR_OOM, MG_ERR_CUDA. */
+ * mg_solve_host's device copies of rho and phi.  opts may be NULL for
+ * defaults; it is copied.  On success *ctx owns the device memory until
+ * mg_destroy.  Errors: MG_ERR_ARG (sizes, kinds, options), MG_ERR_OOM,
+ * MG_ERR_CUDA. */
 mg_status mg_create(int nx, int ny, int nz, double dx, mg_bc bc, const mg_opts *opts,
                     mg_ctx **ctx);
 
@@ -158,7 +159,7 @@ mg_status mg_create(int nx, int ny, int nz, double dx, mg_bc bc, const mg_opts *
  * faces too).  Six equal rules (and, if fixed, equal values) give the
  * context mg_create gives for that rule; otherwise the context's rule is
  * MG_BC_MIXED.  Its levels run with the face rules in their ghost synthesis
- * (the fused FP32 legs, the single-CTA coarse levels and MG_MIXED's exact
+ * (the fused FP32 legs, the coarse levels in one launch and MG_MIXED's exact
  * fixed-point outer step for any combination of periodic axes).  Other
  * arguments and errors as mg_create. */
 mg_status mg_create_faces(int nx, int ny, int nz, double dx, const mg_bc *face_bc,
@@ -463,16 +464,17 @@ mg_status mg_batch_create(int n, const int *dims, const double *dx, const mg_bc 
  * ordered after `stream`, a launch per phase and class, each outer iteration
  * after a class's first as a CUDA graph (so make the call outside any capture
  * of your own).  After mg_batch_set_blocks or mg_batch_set_barrier_limit, for
- * more than 24 classes, and where a grid's phi lies in memory that another class
- * reads as rho (every rho is read before any phi is written), one persistent cooperative kernel runs every phase
- * of every grid instead, captured by the first call and replayed by later
- * ones: the same bits.  The calling thread waits as the device's scheduling flag
- * says (cudaDeviceScheduleBlockingSync: it blocks or sleeps; else it polls).
- * Each grid stops by the rule of mg_solve (Sec. 2.3.7).  hist (host, n * hist_cap, may be NULL)
- * receives each grid's ||d||/||f|| after every outer iteration, n_hist[g] the
- * count, status[g] its result.  Returns MG_OK when every grid converged, else
- * the first failing grid's status, MG_ERR_TIMEOUT if a grid-wide barrier wait
- * ran out (about 2 s), MG_ERR_CUDA.  Synchronises `stream`. */
+ * more than 24 classes, and where a grid's phi lies in memory that another
+ * class reads as rho (every rho is read before any phi is written), one
+ * persistent cooperative kernel runs every phase of every grid instead,
+ * captured by the first call and replayed by later ones: the same bits.  The
+ * calling thread waits as the device's scheduling flag says
+ * (cudaDeviceScheduleBlockingSync: it blocks or sleeps; else it polls). Each
+ * grid stops by the rule of mg_solve (Sec. 2.3.7).  hist (host, n * hist_cap,
+ * may be NULL) receives each grid's ||d||/||f|| after every outer iteration,
+ * n_hist[g] the count, status[g] its result.  Returns MG_OK when every grid
+ * converged, else the first failing grid's status, MG_ERR_TIMEOUT if a grid-
+ * wide barrier wait ran out (about 2 s), MG_ERR_CUDA.  Synchronises `stream`. */
 mg_status mg_batch_solve(mg_batch *batch, const double *const *rho_dev, const double *four_pi_G,
                          const double *tol, double *const *phi_dev, double *hist, int hist_cap,
                          int *n_hist, mg_status *status, void *stream);
@@ -499,16 +501,17 @@ int mg_batch_graph(const mg_batch *batch);
 mg_status mg_batch_phase_ms(mg_batch *batch, double *ms_by_type, int n_types);
 
 /* CTAs of the persistent launch: 0 (default) no limit, else at most that many
- * (fewer CTAs leave SMs to other streams' work, for a batch of small grids).  Takes effect at the next mg_batch_solve,
- * which captures its CUDA graph again.  Errors: MG_ERR_ARG (blocks < 0). */
+ * (fewer CTAs leave SMs to other streams' work, for a batch of small grids).
+ * Takes effect at the next mg_batch_solve, which captures its CUDA graph again.
+ * Errors: MG_ERR_ARG (blocks < 0). */
 mg_status mg_batch_set_blocks(mg_batch *batch, int blocks);
 
-/* Limit of one wait at the persistent kernel's grid-wide barriers, in GPU
- * clock cycles (default 4e9, about 2 s at 2 GHz; any other value chooses that
- * kernel); a wait that runs out makes
- * every block return and mg_batch_solve report MG_ERR_TIMEOUT, leaving the
- * batch usable.  Takes effect at the next mg_batch_solve, which captures its
- * CUDA graph again.  Errors: MG_ERR_ARG (cycles < 0). */
+/* Limit of one wait at the persistent kernel's grid-wide barriers, in GPU clock
+ * cycles (default 4e9, about 2 s at 2 GHz; any other value chooses that kernel);
+ * a wait that runs out makes every block return and mg_batch_solve report
+ * MG_ERR_TIMEOUT, leaving the batch usable.  Takes effect at the next
+ * mg_batch_solve, which captures its CUDA graph again.  Errors: MG_ERR_ARG
+ * (cycles < 0). */
 mg_status mg_batch_set_barrier_limit(mg_batch *batch, long long cycles);
 
 const char *mg_batch_last_error(const mg_batch *batch);

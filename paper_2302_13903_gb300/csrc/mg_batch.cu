@@ -18,8 +18,8 @@
 // Work items by phase:
 //   source: f = 4 pi G rho, mean removal, ||f||     (chunks of 32768 cells)
 //   first residual r = f - L(0), FP32 copy           (chunks)
-//   per V-cycle: down legs on levels >= 64^3 (fused tiles), one CTA per grid
-//     for the levels <= 32^3 (whole coarse cycle), up legs on levels >= 64^3
+//   per V-cycle: down legs on levels >= 32^3 (fused tiles), one CTA per grid
+//     for the levels <= 16^3 (whole coarse cycle), up legs on levels >= 32^3
 //   correction phi += e / scale, FP64 residual + norm (chunks), stopping rule
 //     (one item per grid)
 //   at the end: <phi> = 0 for periodic and zero-gradient grids (chunks)
@@ -94,7 +94,7 @@ enum PhaseType : int {
   PH_R0,           // chunk: r = f - mean - L(0) -> r32 (scaled), sums of (f - mean)^2, r^2
   PH_R0FIN,        // grid: ||f||, rn
   PH_DOWN,         // tile: fused down leg on level size `n`
-  PH_BOTTOM,       // grid: levels <= 32^3 of one V-cycle
+  PH_BOTTOM,       // grid: levels <= 16^3 of one V-cycle
   PH_UP,           // tile: fused up leg on level size `n`
   PH_EMAX,         // chunk: max |e| (first outer iteration)
   PH_SETFX,        // grid: the fixed-point scale 2^S

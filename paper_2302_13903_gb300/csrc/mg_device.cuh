@@ -1,5 +1,5 @@
-// mg_device.cuh -- device helpers shared by the per-level kernels, the
-// single-CTA bottom solver and the batched solver.
+// mg_device.cuh -- device helpers shared by the per-level kernels, the coarse
+// levels' one launch (mg_coarse.cu) and the batched solver.
 //
 // Layout: every level is an nx*ny*nz array of active cells, z-major, x
 // fastest; there are no ghost cells in memory.  A neighbour outside the level

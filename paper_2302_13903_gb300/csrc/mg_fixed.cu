@@ -878,7 +878,8 @@ cudaError_t launch_rho_stats(const double* rho, long long n, double* partials, d
   // at most 2^14 values per thread in the exact sums (2^32 cells, 34 GB of rho)
   if (n > (long long)nb * kThreads * 16384) return cudaErrorInvalidValue;
   ++g_launches;
-  launch_after(k_rho_stats, nb, kThreads, 0, s, reinterpret_cast<const double2*>(rho), n / 2, partials, partials + nb, nullptr);
+  launch_after(k_rho_stats, nb, kThreads, 0, s, reinterpret_cast<const double2*>(rho), n / 2,
+               partials, partials + nb, nullptr);
   ++g_launches;
   launch_after(k_finish_sum_max, 1, kThreads, 0, s, partials, partials + nb, nb, out);
   return cudaGetLastError();
@@ -890,7 +891,8 @@ cudaError_t launch_rho_stats_copy(const double* host_rho, double* dev, long long
   const int nb = reduce_blocks(n / 2);
   if (n > (long long)nb * kThreads * 16384) return cudaErrorInvalidValue;
   ++g_launches;
-  launch_after(k_rho_stats, nb, kThreads, 0, s, reinterpret_cast<const double2*>(host_rho), n / 2, partials, partials + nb, reinterpret_cast<double2*>(dev));
+  launch_after(k_rho_stats, nb, kThreads, 0, s, reinterpret_cast<const double2*>(host_rho), n / 2,
+               partials, partials + nb, reinterpret_cast<double2*>(dev));
   ++g_launches;
   launch_after(k_finish_sum_max, 1, kThreads, 0, s, partials, partials + nb, nb, out);
   return cudaGetLastError();
@@ -926,7 +928,9 @@ cudaError_t launch_rho_to_r32(const double* rho, float* r32, long long n, double
   if (n % 2) return cudaErrorInvalidValue;
   const int nb = reduce_blocks(n / 2);
   ++g_launches;
-  launch_after(k_rho_to_r32, nb, kThreads, 0, s, reinterpret_cast<const double2*>(rho), reinterpret_cast<float2*>(r32), n / 2, (float)a, (float)b, ab_dev, partials, partials + nb);
+  launch_after(k_rho_to_r32, nb, kThreads, 0, s, reinterpret_cast<const double2*>(rho),
+               reinterpret_cast<float2*>(r32), n / 2, (float)a, (float)b, ab_dev, partials,
+               partials + nb);
   ++g_launches;
   launch_after(k_finish_sum_max, 1, kThreads, 0, s, partials, partials + nb, nb, out);
   return cudaGetLastError();
@@ -1033,7 +1037,8 @@ cudaError_t launch_fx_step(const long long* phi_in, long long* phi_out, const fl
     configured[dev].store(1);
   }
   const Kf kf = kfs[pm][zero_in ? 1 : 0];
-  launch_after(kf, grid, FX_TX * FX_TY, kFxSmem, s, phi_in, phi_out, e, c, F, r32, g, b, factor, cz, partials, psum, flag);
+  launch_after(kf, grid, FX_TX * FX_TY, kFxSmem, s, phi_in, phi_out, e, c, F, r32, g, b, factor, cz,
+               partials, psum, flag);
   return cudaGetLastError();
 }
 
@@ -1043,7 +1048,8 @@ cudaError_t launch_fx_finish_gravity(const long long* q, double* phi, double* g,
   const double two_pow_S = std::ldexp(1.0, S);
   const FxBc b = fx_bc(bc, two_pow_S);
   ++g_launches;
-  launch_after(k_fx_finish_gravity, grid_for(gr.cells()), kThreads, 0, s, q, phi, g, gr, b, S, 1.0 / (2.0 * h * two_pow_S), mean);
+  launch_after(k_fx_finish_gravity, grid_for(gr.cells()), kThreads, 0, s, q, phi, g, gr, b, S,
+               1.0 / (2.0 * h * two_pow_S), mean);
   return cudaGetLastError();
 }
 

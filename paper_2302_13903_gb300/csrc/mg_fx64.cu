@@ -1,10 +1,15 @@
-// mg_fx64.cu -- the finest level of the FP64 path in exact 64-bit fixed point.
+// mg_fx64.cu -- the levels of the FP64 path from 64^3 up in exact 64-bit fixed
+// point.
 //
 // An SM issues two FP64 operations per clock, so a V(1,1) cycle's 25-30 FP64
 // operations per cell take several times as long as its bytes.  Here phi and
-// h^2 f of the finest level are 64-bit integers scaled by 2^S with |phi| <
-// 2^54: a quantum of at most 2^-53 max|phi|, the spacing of doubles there.
-// With U and F those integers,
+// h^2 f of the finest level are 64-bit integers scaled by 2^S, S so large that
+// twice the largest |phi| of the FMG start on the next level lies between 2^56
+// and 2^57 (or h^2 max|f| between 2^57 and 2^58): a quantum of 2^-56 to 2^-55
+// of max|phi|, an eighth to a quarter of the spacing of doubles there.  Cells
+// more than that below max|phi| have fewer bits than doubles have; every cell's
+// update carries an eighth of the rounding that an FP64 update carries where |phi| is
+// largest.  With U and F those integers,
 //   R = (sum of the six neighbours of U) - 6 U - F       (exactly)
 //   SMOOTH: U += round(R omega / 6)                      (Eqs. rbsor1-rbsor2)
 //   defect: f - L u = -R / (h^2 2^S)                     (Eq. defect)
@@ -13,10 +18,15 @@
 // constant and is folded into F (F - round(2 b 2^S)) when F is formed, so the
 // sweeps run the homogeneous rule.
 //
-// The levels below, down to 64^3, hold the correction on the same grid with two
-// guard bits (2^(S+2)): with h_c = 2 h their right-hand side is F_c = -(sum of
-// R) / 2 in quanta of their own, so no scale has to be found, and a correction
-// is known to a quarter of a quantum of the phi it is added to.
+// The levels below, down to 64^3, hold the correction on the same grid: with h_c
+// = 2 h their right-hand side is F_c = -(sum of R) / 2, so no scale has to be
+// found, and a correction has the quantum of the phi it is added to.
+//
+// Ranges: |U| < 2^59 on the finest level and |F| < 2^60 keep |R| below 2^63; the
+// flag is raised where a U passes that, a correction 2^56 (its interpolation has
+// weights of 64 in all) or a coarse F 2^60, and the solve then runs in FP64.  The
+// sum of R over eight cells is not checked on its own: past 2^63 it is one wrong
+// correction, which the next norm, exact always, shows.
 //
 // Two z-marching kernels, like the FP32 legs: down = one SMOOTH and the
 // restricted defect, up = the prolonged correction and one SMOOTH.  A CTA
@@ -723,7 +733,10 @@ cudaError_t launch(const Fx64Args& a, bool down, cudaStream_t s) {
 }
 
 // Tile width: 64 cells, one CTA per SM, or on levels that would leave SMs
-// without one, 32 cells and two CTAs per SM (more halo, shorter chains).
+// without one, 32 cells and two CTAs per SM (more halo, shorter chains).  Solves
+// with the wide tiles at 64^3 as well, as here, with the narrow ones up to 128^3 and
+// up to 256^3 (GB300, periodic, us): 64^3 971, 963, 963, 963; 128^3 1526, 1493,
+// 1560, 1560; 256^3 4840, 4832, 4858, 5248.
 int tile_width(Grid g) { return g.cells() <= (1LL << 18) ? 32 : 64; }
 
 }  // namespace

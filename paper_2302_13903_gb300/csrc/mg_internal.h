@@ -337,18 +337,18 @@ cudaError_t launch_finish_fx_sum(const long long* psum, int nb, long long n, dou
                                  cudaStream_t s);
 
 // ---------------------------------------------------------------------------
-// The FP64 path's finest level in 64-bit fixed point (mg_fx64.cu).  Levels
+// The FP64 path's levels from 64^3 up in 64-bit fixed point (mg_fx64.cu).  Levels
 // with nx a multiple of 64, ny of 16 and nz even (fx64_ok); per-CTA sums in
 // arrays of fx64_blocks(g) entries.
 bool fx64_ok(Grid g);
 int fx64_cz(Grid g);
 int fx64_blocks(Grid g);
-// down: u_out = SMOOTH(u_in); fc = the restricted defect times 8 h^2 2^S, or
-// fci = half of it, F of an integer coarse level;
-// norm = sums of (h^2 2^S defect)^2 over the red cells of u_in.  up: u_out = SMOOTH(u_in + trilinear(ec)); norm = the same
-// over the black cells of u_out.  coarse: a correction level, down from u_in =
-// 0, no norms and sums.  *flag |= 1 where |u_out| passes 2^59 (coarse
-// 2^kFx64Correction) or fci its range.
+// down: u_out = SMOOTH(u_in); fc = the restricted defect times 8 h^2 2^S, or fci
+// = half of it, F of an integer coarse level; norm = sums of (h^2 2^S defect)^2
+// over the red cells of u_in.  up: u_out = SMOOTH(u_in + trilinear(ec)); norm = the
+// same over the black cells of u_out.  coarse: a correction level, down from u_in
+// = 0, no norms.  *flag |= 1 where |u_out| passes 2^59 (coarse 2^kFx64Correction)
+// or fci its range.
 constexpr int kFx64Correction = 56;  // corrections stay below 2^56
 struct Fx64Leg {
   const long long* u_in;

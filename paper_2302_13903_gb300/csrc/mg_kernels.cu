@@ -58,7 +58,8 @@ int grid_for(long long work) {
 
 // Threads per block of a level kernel with `work` items: 256, or 64 where blocks
 // of 256 would leave SMs, and with them FP64 units, without one (32^3: 32
-// blocks on 152 SMs).
+// blocks on 152 SMs).  FP64 solves with 64 there and with 256 everywhere (GB300, us):
+// 32^3 fixed 1098, 1148; 64^3 periodic 964, 991; 128^3 1493, 1532; 256^3 4832, 4889.
 int threads_for(long long work) { return work < 256LL * sm_count() ? 64 : kThreads; }
 int blocks_for(long long work) {
   const int t = threads_for(work);
@@ -451,28 +452,6 @@ __global__ void k_subtract_mean(double* __restrict__ a, long long n, const doubl
   }
 }
 
-// r32 = scale d with d = f - (sum_nb - 6 u) / h^2, partial sums of d^2: for
-// sizes that are not even.
-__global__ void k_outer_residual(const double* u, const double* f,
-                                 float* __restrict__ r32, Grid g, Bc bc, double inv_h2,
-                                 double scale, double* __restrict__ partials) {
-  dev::after_previous();
-  const long long total = g.cells();
-  double acc = 0.0;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(t % g.nx);
-    const long long r = t / g.nx;
-    const int j = (int)(r % g.ny), k = (int)(r / g.ny);
-    const double s = dev::neighbour_sum(u, i, j, k, g, bc);
-    const double d = f[t] - (s - 6.0 * u[t]) * inv_h2;
-    r32[t] = (float)(d * scale);
-    acc += d * d;
-  }
-  const double b = block_sum(acc);
-  if (threadIdx.x == 0) partials[blockIdx.x] = b;
-}
-
 __global__ void k_scale_to_f32(const double* a, float* __restrict__ b, long long n,
                                double scale) {
   dev::after_previous();
@@ -574,9 +553,11 @@ cudaError_t launch_sor(T* u, const T* f, Grid g, double h, Bc bc, double omega, 
   ++g_launches;
   if (g.nx % 2 == 0 && g.ny % 2 == 0) {
     if (bc.kind == BC_PERIODIC)
-      launch_after(k_sor_patch<T, true>, blocks_for(work / 2), threads_for(work / 2), 0, s, u, f, g, bc, cu, cs, cf, colour);
+      launch_after(k_sor_patch<T, true>, blocks_for(work / 2), threads_for(work / 2), 0, s, u, f, g,
+                   bc, cu, cs, cf, colour);
     else
-      launch_after(k_sor_patch<T, false>, blocks_for(work / 2), threads_for(work / 2), 0, s, u, f, g, bc, cu, cs, cf, colour);
+      launch_after(k_sor_patch<T, false>, blocks_for(work / 2), threads_for(work / 2), 0, s, u, f,
+                   g, bc, cu, cs, cf, colour);
   } else {
     launch_after(k_sor<T>, grid_for(work), kThreads, 0, s, u, f, g, bc, cu, cs, cf, colour);
   }
@@ -587,7 +568,8 @@ template <typename T>
 cudaError_t launch_sor_red_zero(T* u, const T* f, Grid g, double h, double omega,
                                 cudaStream_t s) {
   ++g_launches;
-  launch_after(k_sor_red_zero<T>, blocks_for(g.cells()), threads_for(g.cells()), 0, s, u, f, g, (T)(-omega * h * h / 6.0));
+  launch_after(k_sor_red_zero<T>, blocks_for(g.cells()), threads_for(g.cells()), 0, s, u, f, g,
+               (T)(-omega * h * h / 6.0));
   return cudaGetLastError();
 }
 
@@ -599,9 +581,11 @@ cudaError_t launch_defect(const T* u, const T* f, T* d, Grid g, double h, Bc bc,
   if (partials && !d && g.nx % 2 == 0 && g.ny % 2 == 0) {
     const T ih2 = (T)(1.0 / (h * h));
     if (bc.kind == BC_PERIODIC)
-      launch_after(k_defect_norm<T, true, false>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials, nullptr, 0.0);
+      launch_after(k_defect_norm<T, true, false>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials,
+                   nullptr, 0.0);
     else
-      launch_after(k_defect_norm<T, false, false>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials, nullptr, 0.0);
+      launch_after(k_defect_norm<T, false, false>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials,
+                   nullptr, 0.0);
     return cudaGetLastError();
   }
   launch_after(k_defect<T>, nb, kThreads, 0, s, u, f, d, g, bc, (T)(1.0 / (h * h)), partials);
@@ -616,9 +600,11 @@ cudaError_t launch_defect_restrict(const T* u, const T* f, T* fc, Grid g, double
   if (!even_sizes(g))
     launch_after(k_defect_restrict<T>, grid_for(g.cells() / 8), kThreads, 0, s, u, f, fc, g, bc, ih2);
   else if (bc.kind == BC_PERIODIC)
-    launch_after(k_defect_restrict_block<T, true>, blocks_for(g.cells() / 4), threads_for(g.cells() / 4), 0, s, u, f, fc, g, bc, ih2);
+    launch_after(k_defect_restrict_block<T, true>, blocks_for(g.cells() / 4),
+                 threads_for(g.cells() / 4), 0, s, u, f, fc, g, bc, ih2);
   else
-    launch_after(k_defect_restrict_block<T, false>, blocks_for(g.cells() / 4), threads_for(g.cells() / 4), 0, s, u, f, fc, g, bc, ih2);
+    launch_after(k_defect_restrict_block<T, false>, blocks_for(g.cells() / 4),
+                 threads_for(g.cells() / 4), 0, s, u, f, fc, g, bc, ih2);
   return cudaGetLastError();
 }
 
@@ -634,18 +620,23 @@ cudaError_t launch_prolong(const T* uc, T* uf, Grid gf, Bc bc_coarse, int high_o
                            cudaStream_t s) {
   ++g_launches;
   // z-chunks of coarse columns: 8 planes each while that leaves about 2^16
-  // work items (three FP64 warps per scheduler), fewer on small levels
+  // work items (three FP64 warps per scheduler), fewer on small levels.  With 2^18
+  // FP64 solves took (GB300) 256^3 periodic 4853 us instead of 4832, fixed 7128
+  // instead of 7090, the smaller ones the same
   const long long cols = (long long)(gf.nx / 2) * (gf.ny / 2);
   const int cnz = gf.nz / 2;
   int cz = 8;
   while (cz > 1 && cols * ((cnz + cz - 1) / cz) < (1LL << 16)) cz /= 2;
   const long long items = cols * ((cnz + cz - 1) / cz);
   if (!high_order && add && homogeneous_rule(bc_coarse))
-    launch_after(k_prolong_add<T>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf, bc_coarse, cz, items);
+    launch_after(k_prolong_add<T>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf,
+                 bc_coarse, cz, items);
   else if (high_order)
-    launch_after(k_prolong<T, true>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf, bc_coarse, add, cz, items);
+    launch_after(k_prolong<T, true>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf,
+                 bc_coarse, add, cz, items);
   else
-    launch_after(k_prolong<T, false>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf, bc_coarse, add, cz, items);
+    launch_after(k_prolong<T, false>, blocks_for(items), threads_for(items), 0, s, uc, uf, gf,
+                 bc_coarse, add, cz, items);
   return cudaGetLastError();
 }
 
@@ -718,16 +709,11 @@ cudaError_t launch_finish_sum(const double* partials, int nb, double* out, cudaS
 cudaError_t launch_outer_residual(const double* u, const double* f, float* r32, Grid g, double h,
                                   Bc bc, double scale, double* partials, cudaStream_t s) {
   ++g_launches;
-  const int nb = reduce_blocks(g.cells());
-  const double ih2 = 1.0 / (h * h);
-  if (g.nx % 2 == 0 && g.ny % 2 == 0) {
-    if (bc.kind == BC_PERIODIC)
-      launch_after(k_defect_norm<double, true, true>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials, r32, scale);
-    else
-      launch_after(k_defect_norm<double, false, true>, nb, kThreads, 0, s, u, f, g, bc, ih2, partials, r32, scale);
-  } else {
-    launch_after(k_outer_residual, nb, kThreads, 0, s, u, f, r32, g, bc, ih2, scale, partials);
-  }
+  if (g.nx % 2 || g.ny % 2) return cudaErrorInvalidValue;  // levels have sides 2^k >= 2
+  auto kernel = bc.kind == BC_PERIODIC ? k_defect_norm<double, true, true>
+                                       : k_defect_norm<double, false, true>;
+  launch_after(kernel, reduce_blocks(g.cells()), kThreads, 0, s, u, f, g, bc, 1.0 / (h * h),
+               partials, r32, scale);
   return cudaGetLastError();
 }
 

@@ -315,9 +315,9 @@ __device__ __forceinline__ double binom(int n, int k) {
 // fixed order), then the centre of mass (thread 0), the moments about it (one
 // monomial per thread) and Q_lm (one per thread).
 constexpr int kFinishThreads = 512;
-__global__ void __launch_bounds__(kFinishThreads) k_moments_finish(const double* __restrict__ partials, int nb, double h, int lmax,
-                                 int use_com, double ox, double oy, double oz,
-                                 double* __restrict__ out) {
+__global__ void __launch_bounds__(kFinishThreads)
+    k_moments_finish(const double* __restrict__ partials, int nb, double h, int lmax, int use_com,
+                     double ox, double oy, double oz, double* __restrict__ out) {
   __shared__ double M[kMono];
   __shared__ double Cs[kMono];
   __shared__ double P[3][5];  // (-o)^p per axis, p = 0..4

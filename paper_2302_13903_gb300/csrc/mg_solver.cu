@@ -1549,7 +1549,7 @@ void autotune(mg_ctx* c, cudaStream_t s) {
       if (!c->u32b[l] || !mg::fused_ok(g, hom)) continue;
       // a level whose u (both buffers) and f stay in L2 from leg to leg is
       // timed with them there: flushed, the launch that moves the fewest bytes
-      // wins, which at 128^3 was the up-down pass (29.5 us against 21 us for
+      // wins, which at 128^3 was the up-down pass (29.5 us against 24 us for
       // the two legs inside a solve)
       const bool resident = 12 * (size_t)g.cells() <= (size_t)prop.l2CacheSize / 4 * 3;
       void* const cold = resident ? nullptr : flush;

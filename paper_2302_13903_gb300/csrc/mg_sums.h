@@ -1,6 +1,6 @@
-// mg_sums.h -- exact sums a thread of the integer legs keeps, and the range check
-// of what becomes an integer (host and device, so that they are tested on the
-// host).
+// mg_sums.h -- exact sums that threads of the FP64 path's integer kernels keep, and
+// the range check of what becomes an integer (host and device, so that they are
+// tested on the host).
 #pragma once
 
 #ifdef __CUDACC__

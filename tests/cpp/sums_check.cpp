@@ -15,12 +15,12 @@ static int failures = 0;
     }                                                  \
   } while (0)
 
-// A column of `planes` pairs of one sign, as the down leg's threads sum them: at 2^55
-// and more the plain 64-bit sum of 128 pairs wraps.
+// Pairs of values of one sign, up to the 4096 a thread of the sum pass adds: at
+// 2^55 and more the plain 64-bit sum of 128 pairs wraps.
 static void split_sum() {
   for (int bits : {0, 40, 54, 55, 57, 59})
     for (int sign : {1, -1})
-      for (int planes : {4, 64, 128}) {
+      for (int planes : {4, 64, 128, 4096}) {
         const long long v = sign * ((1LL << bits) - 1);
         mg::SplitSum s;
         __int128 sum = 0;
