@@ -217,7 +217,7 @@ __device__ __forceinline__ int plane_of(int q, int nz, bool pz) {
 // slot J, planes q - 1, q - 2, q - 3 in J - 1, J - 2, J - 3 (mod 4).
 // COARSE: a correction level, from u = 0 and without the norm.
 template <bool WALLS, int TX, bool COARSE>
-__global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
+__global__ void __launch_bounds__(Down<TX>::NT)
     k_fx64_down(const __grid_constant__ Fx64Args a) {
   dev::after_previous();
   using W = Down<TX>;
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(Down<TX>::NT, TX == 64 ? 1 : 2)
 // along y, then x, then z with weights 3 and 1 on the integer grid and rounded
 // once by the division by 64.  Unrolled by four as the down leg.
 template <bool WALLS, int TX, bool COARSE>
-__global__ void __launch_bounds__(Up<TX>::NT, TX == 64 ? 1 : 2)
+__global__ void __launch_bounds__(Up<TX>::NT)
     k_fx64_up(const __grid_constant__ Fx64Args a) {
   dev::after_previous();
   using W = Up<TX>;
@@ -732,11 +732,13 @@ cudaError_t launch(const Fx64Args& a, bool down, cudaStream_t s) {
                     s);
 }
 
-// Tile width: 64 cells, one CTA per SM, or on levels that would leave SMs
-// without one, 32 cells and two CTAs per SM (more halo, shorter chains).  Solves
-// with the wide tiles at 64^3 as well, as here, with the narrow ones up to 128^3 and
-// up to 256^3 (GB300, periodic, us): 64^3 971, 963, 963, 963; 128^3 1526, 1493,
-// 1560, 1560; 256^3 4840, 4832, 4858, 5248.
+// Tile width: 64 cells, or on levels that would leave SMs without a CTA, 32 cells
+// (more halo, shorter chains); one CTA per SM either way, so that the threads of the
+// narrow tiles (400, at most 128 CTAs of at least four planes) may have the
+// registers they ask for: held to two CTAs they spilled 100-190 bytes, 64^3 fixed
+// 1560 us instead of 1394.  Solves with the wide tiles at 64^3 as well, as here, and
+// with the narrow ones up to 128^3 (GB300, periodic, us): 64^3 966, 889, 890; 128^3
+// 1514, 1477, 1526; 256^3 4830, 4791, 4946.
 int tile_width(Grid g) { return g.cells() <= (1LL << 18) ? 32 : 64; }
 
 }  // namespace
@@ -749,7 +751,7 @@ bool fx64_ok(Grid g) {
 // Planes per CTA: the even count for which the last wave of CTAs is best filled,
 // counting the six planes a chunk's halo costs; at most 128.
 int fx64_cz(Grid g) {
-  const int tx = tile_width(g), wave = sm_count() * (tx == 64 ? 1 : 2);
+  const int tx = tile_width(g), wave = sm_count();
   const long long cols = (long long)(g.nx / tx) * (g.ny / TY);
   int best = 0;
   long long least = 0;
