@@ -588,10 +588,10 @@ __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
   cp_wait<1>();  // planes z0 - 1 and z0 have landed
   long long zm = own_at(I0{}), self = own_at(I1{});
   float acc = 0.f;
-  // exact sum of this column's PHI' (|PHI'| <= 2^60 and at most 128 planes per
-  // CTA, so no overflow); split into hi 2^32 + lo for the block sums
+  // sum of this column's PHI', exact while |PHI'| < 2^56 (at most 128 planes per
+  // CTA); split into hi 2^32 + lo for the block sums
   long long csum = 0;
-  bool bad = false;
+  unsigned big = 0;  // the upper words' bits that differ from the sign, of all planes
   // plane z = z0 + J (mod 4): its slot is J + 1, z + 1's is J + 2, z + 2's J + 3
   auto step = [&](auto Jc, int z) {
     constexpr int J = decltype(Jc)::value;
@@ -608,7 +608,8 @@ __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
     }
     phi_out[o] = self;
     csum += self;
-    bad |= (unsigned long long)(self + (1LL << 60)) > (2ULL << 60);  // |PHI'| > 2^60
+    const int top = (int)(self >> 32);
+    big |= (unsigned)(top ^ (top >> 31));
     __syncthreads();
     long long xm = P[buf][ty + 1][tx], xp = P[buf][ty + 1][tx + 2];
     long long ym = P[buf][ty][tx + 1], yp = P[buf][ty + 2][tx + 1];
@@ -644,7 +645,7 @@ __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
     step(std::integral_constant<int, 3>{}, z + 3);
   }
   cp_wait<0>();
-  if (bad) atomicOr(flag, 1);
+  if (big >> 24) atomicOr(flag, big >> 28 ? 3 : 2);  // past 2^56, past 2^60
   // deterministic block sums, then one partial per block (blocks in launch
   // order); the sums of PHI' stay exact integers, so their total does not
   // depend on the blocking
@@ -683,19 +684,26 @@ __global__ void __launch_bounds__(FX_TX* FX_TY, fx_min_blocks<PM>())
 }
 
 // Exact sums of q per block as pairs (hi, lo).  A pass of its own at the end of
-// an FP64 solve (0.17 ms at 512^3): summed in the down legs, whose registers are
-// all in use, it cost each of ten some 0.13 ms there.  Bound by bytes: four
-// 16-byte loads in flight.
-__global__ void __launch_bounds__(kThreads) k_fx_sum(const longlong2* q, long long n2,
+// an FP64 solve (0.15 ms at 512^3): summed in the down legs, whose registers are
+// all in use, it cost each of ten some 0.13 ms there.  Also of a mixed solve whose
+// steps saw values their own sums do not hold.  Bound by bytes: four 16-byte loads
+// in flight.
+// PAIRS: q is 16-byte aligned.
+template <bool PAIRS>
+__global__ void __launch_bounds__(kThreads) k_fx_sum(const long long* q1, long long n2,
                                                      long long* __restrict__ psum) {
   dev::after_previous();
   SplitSum sum;
+  const longlong2* q = reinterpret_cast<const longlong2*>(q1);
+  auto load = [&](long long t) {
+    return PAIRS ? q[t] : make_longlong2(q1[2 * t], q1[2 * t + 1]);
+  };
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   for (; t + 3 * stride < n2; t += 4 * stride) {
     longlong2 v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = q[t + k * stride];
+    for (int k = 0; k < 4; ++k) v[k] = load(t + k * stride);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       sum.add(v[k].x);
@@ -703,8 +711,9 @@ __global__ void __launch_bounds__(kThreads) k_fx_sum(const longlong2* q, long lo
     }
   }
   for (; t < n2; t += stride) {
-    sum.add(q[t].x);
-    sum.add(q[t].y);
+    const longlong2 v = load(t);
+    sum.add(v.x);
+    sum.add(v.y);
   }
   __shared__ long long wh[kThreads / 32], wl[kThreads / 32];
   long long hi = sum.hi(), lo = sum.lo();
@@ -960,7 +969,7 @@ bool fx_step_ok(Grid g) {
 
 // Planes per CTA: the given cz, else the largest of 64 .. 4 that still
 // gives four CTAs per SM; at most 128 (a thread's exact sum of its column's
-// integers, each below 2^55, must stay below 2^63).
+// integers, each below 2^56, must stay below 2^63).
 int fx_step_cz(Grid g, int cz) {
   const long long cols = (long long)(g.nx / FX_TX) * (g.ny / FX_TY);
   if (cz <= 0) {
@@ -1056,7 +1065,7 @@ cudaError_t launch_fx_finish_gravity(const long long* q, double* phi, double* g,
 cudaError_t launch_fx_sum(const long long* q, long long n, long long* psum, cudaStream_t s) {
   if (n % 2) return cudaErrorInvalidValue;
   ++g_launches;
-  launch_after(k_fx_sum, reduce_blocks(n), kThreads, 0, s, reinterpret_cast<const longlong2*>(q),
+  launch_after(aligned16(q) ? k_fx_sum<true> : k_fx_sum<false>, reduce_blocks(n), kThreads, 0, s, q,
                n / 2, psum);
   return cudaGetLastError();
 }

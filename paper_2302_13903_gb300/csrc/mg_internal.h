@@ -152,9 +152,10 @@ cudaError_t launch_subtract_mean(double* a, long long n, double* partials, int n
 // Partial sums of a[i] (FP64) and of a[i]^2.
 template <typename T>
 cudaError_t launch_sum(const T* a, long long n, int squares, double* partials, cudaStream_t s);
-// out[0] = sum(partials[0..nb)) in a fixed order (out may be page-locked host
-// memory).
-cudaError_t launch_finish_sum(const double* partials, int nb, double* out, cudaStream_t s);
+// out[0] = sum(partials[0..nb)) in a fixed order, out[1] = *flag when flag is given
+// (out may be page-locked host memory).
+cudaError_t launch_finish_sum(const double* partials, int nb, double* out, cudaStream_t s,
+                              const int* flag = nullptr);
 // FAS (Algorithm 3): f += L ur and u = ur (step 5); u -= ur (step 7).
 cudaError_t launch_fas_rhs(const double* ur, double* f, double* u, Grid g, double h, Bc bc,
                            cudaStream_t s);
@@ -311,7 +312,8 @@ cudaError_t launch_fx_correct(long long* phi, const float* e, long long n, float
 // null means PHI_in = 0), then r32 = (F - (sum_nb PHI_out - 6 PHI_out)) *
 // factor exactly in integers, one partial sum of r32^2 per block in partials
 // (count in *nb_out, at most nb_max) and, when psum is given, the exact sum of
-// PHI_out per block as a (hi 2^32, lo) pair of integers (2 nb_max entries).
+// PHI_out per block as a (hi 2^32, lo) pair of integers (2 nb_max entries), for
+// |PHI_out| < 2^56.  *flag |= 2 where that is passed, |= 1 where 2^60 is.
 // Requires nx % 32 == 0 and ny % 16 == 0 (fx_step_ok).
 // cz = 0 takes the built-in planes per CTA; fx_step_blocks(g, 0) bounds the
 // block count of every cz >= kFxMinCz.

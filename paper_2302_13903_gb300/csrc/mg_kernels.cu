@@ -422,13 +422,18 @@ __global__ void k_sum(const T* a, long long n, int squares,
   if (threadIdx.x == 0) partials[blockIdx.x] = b;
 }
 
-__global__ void k_finish_sum(const double* partials, int nb, double* __restrict__ out) {
+// flag: also *flag, as a double, into out[1].
+__global__ void k_finish_sum(const double* partials, int nb, double* __restrict__ out,
+                             const int* flag) {
   dev::after_previous();
   double acc = 0.0;
 #pragma unroll 8
   for (int t = threadIdx.x; t < nb; t += kThreads) acc += partials[t];
   const double b = block_sum(acc);
-  if (threadIdx.x == 0) out[0] = b;
+  if (threadIdx.x == 0) {
+    out[0] = b;
+    if (flag) out[1] = (double)*flag;
+  }
 }
 
 // a -= total[0] / n (the total was formed on the device in a fixed order);
@@ -665,7 +670,7 @@ cudaError_t launch_source(const double* rho, double* f, long long n, double four
 cudaError_t launch_subtract_mean(double* a, long long n, double* partials, int nb,
                                  double* total_slot, bool squares, cudaStream_t s) {
   ++g_launches;
-  launch_after(k_finish_sum, 1, kThreads, 0, s, partials, nb, total_slot);
+  launch_after(k_finish_sum, 1, kThreads, 0, s, partials, nb, total_slot, nullptr);
   ++g_launches;
   if (squares)
     launch_after(k_subtract_mean<true>, reduce_blocks(n), kThreads, 0, s, a, n, total_slot, partials);
@@ -700,9 +705,10 @@ cudaError_t launch_gravity(const double* u, double* g, Grid gr, double h, Bc bc,
   return cudaGetLastError();
 }
 
-cudaError_t launch_finish_sum(const double* partials, int nb, double* out, cudaStream_t s) {
+cudaError_t launch_finish_sum(const double* partials, int nb, double* out, cudaStream_t s,
+                              const int* flag) {
   ++g_launches;
-  launch_after(k_finish_sum, 1, kThreads, 0, s, partials, nb, out);
+  launch_after(k_finish_sum, 1, kThreads, 0, s, partials, nb, out, flag);
   return cudaGetLastError();
 }
 

@@ -778,9 +778,10 @@ void fmg_fas(mg_ctx* c, const Bc* bcs, const Bc& hom, cudaStream_t s) {
 }
 
 // The sum of nb partial sums, in a fixed order, written to page-locked host
-// memory by the kernel that forms it (a copy behind it costs 3-4 us).
-double read_sum(mg_ctx* c, int nb, cudaStream_t s) {
-  check(c, mg::launch_finish_sum(c->partials, nb, c->pinned, s), "finish sum");
+// memory by the kernel that forms it (a copy behind it costs 3-4 us); with `flag`,
+// that flag into pinned[1].
+double read_sum(mg_ctx* c, int nb, cudaStream_t s, const int* flag = nullptr) {
+  check(c, mg::launch_finish_sum(c->partials, nb, c->pinned, s, flag), "finish sum");
   check(c, cudaStreamSynchronize(s), "sync");
   return c->pinned[0];
 }
@@ -1241,6 +1242,7 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
   // per-block exact sums of the integer phi, (hi, lo) pairs
   long long* psum = reinterpret_cast<long long*>(c->partials + c->partials_cap);
   int nbs = 0;
+  bool sums_hold = true;  // the steps saw no integer past 2^56
   const long long* FX = reinterpret_cast<const long long*>(f);
   for (int it = 0;; ++it) {
     if (rn == 0.0) {  // exact already (zero source with a homogeneous rule)
@@ -1334,7 +1336,8 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
       }
       phi_zero = false;
       std::swap(cur, alt);
-      rn = std::sqrt(read_sum(c, nbs, s) / (double)N) / scale;
+      rn = std::sqrt(read_sum(c, nbs, s, c->iflag) / (double)N) / scale;
+      sums_hold = c->pinned[1] == 0.0;
     }
     const double r = rn / fnorm;
     hist[n++] = r;
@@ -1346,9 +1349,14 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
   c->fixed_point = in_fx;
   if (in_fx) {
     // phi = (PHI - M) 2^-S, M the integers' mean (periodic / zero gradient)
-    // rounded to an integer, from the last step's exact integer sums
+    // rounded to an integer, from the last step's exact integer sums, or from
+    // phi itself where they may have passed 2^63
     const long long* mean = nullptr;
     if (has_mean) {
+      if (!sums_hold) {
+        check(c, mg::launch_fx_sum(cur, N, psum, s), "sum phi");
+        nbs = mg::reduce_blocks(N);
+      }
       check(c, mg::launch_finish_fx_sum(psum, nbs, N, c->scal + 56, s), "finish sum phi");
       mean = reinterpret_cast<const long long*>(c->scal + 57);
     }
@@ -1377,7 +1385,7 @@ mg_status solve_mixed(mg_ctx* c, const double* rho, double four_pi_G, double tol
     check(c, cudaStreamSynchronize(s), "sync");
     std::memcpy(flags, c->pinned + 60, 2 * sizeof(int));
     late = flags[1];
-    if (flags[0]) {
+    if (flags[0] & 1) {
       c->err = "fixed-point outer loop: |phi| passed 2^60 (the solve diverged)";
       st = MG_ERR_DIVERGED;
     }
