@@ -387,21 +387,6 @@ __global__ void k_finish_sum_max(const double* sum, const double* mx,
   }
 }
 
-// PHI += round(e * c) (the FP32 correction on the fixed-point grid); flags a
-// value above 2^60, past which neighbour sums could overflow.
-__global__ void k_fx_correct(long long* __restrict__ phi, const float* e, long long n,
-                             float c, int* __restrict__ flag) {
-  dev::after_previous();
-  bool bad = false;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long v = phi[t] + __float2ll_rn(e[t] * c);
-    phi[t] = v;
-    bad |= (v > (1LL << 60)) || (v < -(1LL << 60));
-  }
-  if (bad) atomicOr(flag, 1);
-}
-
 // The rule on the integer grid.  A MIXED rule (kinds per face in fk, as in
 // Bc) takes its fixed faces' values from the face array like OPEN, or 0
 // where there is none (the homogeneous rule).
@@ -952,13 +937,6 @@ cudaError_t launch_rho_to_fx(const double* rho, long long* q, long long n, doubl
     launch_after(k_rho_to_fx<true>, grid_for(n / 8), kThreads, 0, s, rho, q, n, a, b);
   else
     launch_after(k_rho_to_fx<false>, grid_for(n), kThreads, 0, s, rho, q, n, a, b);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fx_correct(long long* phi, const float* e, long long n, float c, int* flag,
-                              cudaStream_t s) {
-  ++g_launches;
-  launch_after(k_fx_correct, grid_for(n), kThreads, 0, s, phi, e, n, c, flag);
   return cudaGetLastError();
 }
 

@@ -305,9 +305,6 @@ cudaError_t launch_rho_to_r32(const double* rho, float* r32, long long n, double
 // q = round(a rho - b) as int64.
 cudaError_t launch_rho_to_fx(const double* rho, long long* q, long long n, double a, double b,
                              cudaStream_t s);
-// PHI += round(e * c); *flag |= 1 if |PHI| passes 2^60.
-cudaError_t launch_fx_correct(long long* phi, const float* e, long long n, float c, int* flag,
-                              cudaStream_t s);
 // Fused outer step: PHI_out = PHI_in + round(e * c) (e must not be null; phi_in
 // null means PHI_in = 0), then r32 = (F - (sum_nb PHI_out - 6 PHI_out)) *
 // factor exactly in integers, one partial sum of r32^2 per block in partials
